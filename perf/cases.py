@@ -1,0 +1,371 @@
+"""What is timed: the calls that a program built on this framework makes, from the smallest to the largest.
+
+Prefill of prompts through whole blocks (attention, score, halting rule, feed-forward, compaction, KV cache), the attention
+half of a block on its own (one block, a cascade that halts tokens after every block, the small fp32 shape), the sparse
+pipeline over given projections (score -> threshold -> compaction -> attention over what stays), and the decoding stage over
+the caches a halted prefill leaves.  Shapes are the ones of paper_2604_18103_b200/workloads.py; lengths are those of the
+benchmark (8192, 32768, 131072 tokens), of vision prompts (about 1300 tokens) and odd ones.
+
+Inputs.  Hidden states of a trained model share a common direction and differ in norm by a factor of a few; here
+H_t = s_t (mu + z_t) / sqrt(2) with mu one direction per case and z_t ~ N(0, I), and the norms s_t lie in bands: tokens that a block
+halts have norms half again those of the tokens that pass it.  The relative update ||U_t|| / ||H_t|| then falls apart into groups
+with a gap between them and the halting rule cuts in the gap, so that the set of tokens that stays does not hang on the last bit of a
+score.  Weights are N(0, 0.02^2), those that write into the residual stream 1 / sqrt(2 * 28) of that (28 blocks with two such matrices
+each), norm weights near one.  The first 64 and last 32 tokens of a prompt always stay.
+"""
+import math
+
+import torch
+
+from paper_2604_18103_b200 import dash
+from paper_2604_18103_b200 import workloads as wl
+
+KEEP_FIRST, KEEP_LAST = 64, 32
+SHAPES = {"qwen": wl.QWEN, "tiny": wl.TINY}
+OUT_SCALE = 1.0 / math.sqrt(2 * 28)
+# ||U_t|| / ||H_t|| of a first block on such inputs for s_t = 1, away from the first tokens: what places a threshold in the gap
+UPDATE = {"qwen": 1.02 * OUT_SCALE, "tiny": 0.0715 * OUT_SCALE}
+BAND = 1.5                     # ratio of the norms of neighbouring bands
+
+
+def listed():
+    return [
+        # a small fp32 model's layer: every launch and conversion counts
+        {"name": "layer_tiny_fp32", "kind": "layer", "shape": "tiny", "seqs": 1, "tokens": 1024, "blocks": 1, "keep": 0.5, "rule": "threshold"},
+        # one layer of the 7B shape, threshold rule: the benchmark's headline step
+        {"name": "layer_8192", "kind": "layer", "shape": "qwen", "seqs": 1, "tokens": 8192, "blocks": 1, "keep": 0.6, "rule": "threshold"},
+        # multi-shot halting: several layers, each keeps a count of the original tokens; three prompts of odd lengths
+        {"name": "cascade_ragged", "kind": "layer", "shape": "qwen", "seqs": 3, "tokens": 12345, "blocks": 4, "keep": 0.35, "rule": "count"},
+        # one short prompt through three blocks (a full one, the one that selects, one on what is left): latency
+        {"name": "prefill_701", "kind": "prefill", "seqs": 1, "tokens": 701, "keep": 0.333},
+        # a batch of vision prompts, 20 % of the tokens stay
+        {"name": "prefill_vision_batch", "kind": "prefill", "seqs": 5, "tokens": 6683, "keep": 0.2},
+        # the paper's setting at its shortest and at a long prompt length
+        {"name": "prefill_8192", "kind": "prefill", "seqs": 1, "tokens": 8192, "keep": 0.333},
+        {"name": "prefill_32768", "kind": "prefill", "seqs": 1, "tokens": 32768, "keep": 0.333},
+        # projections given: score, threshold, compaction of states, Q, K and V, attention over the 20 % that stay
+        {"name": "sparse_131072", "kind": "sparse", "seqs": 1, "tokens": 131072, "keep": 0.2, "indexed": False},
+        # a packed multimodal batch, query rows left in place and fetched by index
+        {"name": "sparse_multimodal", "kind": "sparse", "seqs": 4, "tokens": 49664, "keep": 0.3, "indexed": True},
+        # decoding: attention of one new token per sequence over every block's own cache
+        {"name": "decode_8192", "kind": "decode", "seqs": 1, "tokens": 8192, "keep": 0.333, "full_blocks": 11, "cut_blocks": 17},
+        {"name": "decode_131072", "kind": "decode", "seqs": 1, "tokens": 131072, "keep": 0.333, "full_blocks": 2, "cut_blocks": 3},
+        {"name": "decode_batch", "kind": "decode", "seqs": 24, "tokens": 75001, "keep": 0.333, "full_blocks": 2, "cut_blocks": 3},
+    ]
+
+
+def _log_uniform(rng, lo, hi):
+    return int(round(math.exp(rng.uniform(math.log(lo), math.log(hi)))))
+
+
+def draw(rng):
+    kind = rng.choice(["layer", "layer", "prefill", "prefill", "sparse", "decode", "decode"])
+    if kind == "layer":
+        if rng.random() < 0.3:
+            return {"kind": kind, "shape": "tiny", "seqs": rng.randint(1, 3), "tokens": _log_uniform(rng, 600, 4000), "blocks": 1,
+                    "keep": round(rng.uniform(0.3, 0.8), 3), "rule": "threshold"}
+        rule = rng.choice(["threshold", "count"])
+        return {"kind": kind, "shape": "qwen", "seqs": rng.randint(1, 4), "tokens": _log_uniform(rng, 1500, 24000),
+                "blocks": 1 if rule == "threshold" else rng.randint(1, 4), "keep": round(rng.uniform(0.3, 0.8), 3), "rule": rule}
+    if kind == "prefill":
+        seqs = rng.choice([1, 1, rng.randint(2, 6)])
+        return {"kind": kind, "seqs": seqs, "tokens": _log_uniform(rng, 500 * seqs, 24000), "keep": round(rng.uniform(0.2, 0.6), 3)}
+    if kind == "sparse":
+        seqs = rng.randint(1, 5)
+        return {"kind": kind, "seqs": seqs, "tokens": _log_uniform(rng, 8000, 131072), "keep": round(rng.uniform(0.1, 0.4), 3),
+                "indexed": rng.random() < 0.5}
+    seqs = rng.choice([1, rng.randint(2, 32), rng.randint(33, 96)])
+    return {"kind": kind, "seqs": seqs, "tokens": _log_uniform(rng, 1000 * min(seqs, 40), 131072), "keep": round(rng.uniform(0.2, 0.6), 3),
+            "full_blocks": rng.randint(1, 3), "cut_blocks": rng.randint(1, 4)}
+
+
+# ---- lengths -----------------------------------------------------------------
+def _lengths(case):
+    """Ragged lengths of the case's sequences: fixed by the case, about equal in the mean, within a factor of three of each other."""
+    S, T = case["seqs"], case["tokens"]
+    if S == 1:
+        return [T]
+    g = torch.Generator().manual_seed(T * 131 + S)
+    w = torch.rand(S, generator=g, dtype=torch.float64) + 0.5
+    cut = [0] + [int(round(float(x) * T)) for x in torch.cumsum(w, 0) / w.sum()]
+    cut[-1] = T
+    return [cut[i + 1] - cut[i] for i in range(S)]
+
+
+def _kept(n, keep):
+    """Tokens of a prompt of n that stay: the given share, never fewer than the protected ones."""
+    return min(n, max(KEEP_FIRST + KEEP_LAST, int(keep * n)))
+
+
+def _cascade_shares(case):
+    """Share of the original tokens that stays after each block: evenly spaced down to case["keep"]."""
+    b = case["blocks"]
+    return [1.0 - (1.0 - case["keep"]) * (l + 1) / b for l in range(b)]
+
+
+# ---- inputs -------------------------------------------------------------------
+def _gen(seed, dev):
+    g = torch.Generator(device=dev)
+    g.manual_seed(seed)
+    return g
+
+
+def _hidden(lengths, shares, d, dtype, g, dev):
+    """Hidden states [T, d] whose norms put every token into the band of the block that halts it (shares: what stays after each
+    block); the protected tokens of every prompt are in the last band."""
+    T = sum(lengths)
+    s = torch.empty(T, device=dev)
+    a = 0
+    for n in lengths:
+        band = torch.full((n,), float(len(shares)), device=dev)                 # passes every block
+        kf, kl = min(KEEP_FIRST, n), min(KEEP_LAST, max(0, n - KEEP_FIRST))
+        free = kf + torch.randperm(n - kf - kl, generator=g, device=dev)         # tokens a block may halt, in a random order
+        done = 0
+        for l, f in enumerate(shares):
+            upto = min(n - _kept(n, f), free.numel())
+            band[free[done:upto]] = float(l)
+            done = max(done, upto)
+        s[a:a + n] = BAND ** -band
+        a += n
+    s = s * torch.exp(0.02 * (2 * torch.rand(T, generator=g, device=dev) - 1))
+    mu = torch.randn(d, generator=g, device=dev)
+    z = torch.randn(T, d, generator=g, device=dev)
+    return (z.add_(mu).mul_((s / math.sqrt(2.0))[:, None])).to(dtype)
+
+
+def _weights(shape, g, dev, ffn):
+    def mat(a, b, scale=1.0):
+        return (torch.randn(a, b, generator=g, device=dev) * (0.02 * scale)).to(shape.dtype)
+
+    def norm():
+        return (1.0 + 0.1 * torch.randn(shape.d, generator=g, device=dev)).to(shape.dtype)
+
+    w = {"Wq": mat(shape.d, shape.Hq * shape.D), "Wk": mat(shape.d, shape.Hkv * shape.D), "Wv": mat(shape.d, shape.Hkv * shape.D),
+         "Wo": mat(shape.Hq * shape.D, shape.d, OUT_SCALE), "rms_w": norm()}
+    if ffn:
+        w.update(Wg=mat(shape.d, shape.m), Wu=mat(shape.d, shape.m), Wd=mat(shape.m, shape.d, OUT_SCALE), rms2_w=norm())
+    return w
+
+
+def _int32(x, dev):
+    return torch.tensor(x, dtype=torch.int32, device=dev)
+
+
+class _StepBuffers:
+    """What one block step writes."""
+
+    def __init__(self, n, S, d, dtype, dev):
+        self.H = torch.zeros(n, d, dtype=dtype, device=dev)
+        self.tok = torch.zeros(n, dtype=torch.int32, device=dev)
+        self.pos = torch.zeros(n, dtype=torch.int32, device=dev)
+        self.cu = torch.zeros(S + 1, dtype=torch.int32, device=dev)
+        self.n = torch.zeros(1, dtype=torch.int32, device=dev)
+        self.r = torch.zeros(n, dtype=torch.float32, device=dev)
+        self.mask = torch.zeros(n, dtype=torch.uint8, device=dev)
+
+
+def _prepare_layer(case, seed, dev):
+    shape, lengths, g = SHAPES[case["shape"]], _lengths(case), _gen(seed, dev)
+    S, T, shares = len(lengths), sum(lengths), _cascade_shares(case)
+    cu = wl.cu_from_lengths(lengths)
+    st = {"H": _hidden(lengths, shares, shape.d, shape.dtype, g, dev), "tok": torch.arange(T, dtype=torch.int32, device=dev),
+          "pos": wl.positions(cu).to(dev), "cu": cu.to(dev), "x_full": torch.zeros(T, shape.d, dtype=shape.dtype, device=dev)}
+    st["layers"], st["out"], st["n"], st["longest"] = [], [], [], []
+    table, now = None, list(lengths)
+    for l in range(case["blocks"]):
+        stays = [_kept(n, shares[l]) for n in lengths]
+        rule = {"tau": UPDATE[case["shape"]] * math.sqrt(BAND)} if case["rule"] == "threshold" else \
+            {"sel_mode": dash.SEL_KEEP_COUNT, "keep_counts": _int32(stays, dev)}
+        layer = dash.Layer(shape, _weights(shape, g, dev, False), dev, keep_first=KEEP_FIRST, keep_last=KEEP_LAST, **rule)
+        if layer.rms_folded:
+            table = dash.dash_rope_table(shape.rope_base, shape.D, max(lengths), dev) if table is None else table
+            layer.set_handover(table)
+        n_l = sum(now)
+        st["layers"].append(layer); st["out"].append(_StepBuffers(n_l, S, shape.d, shape.dtype, dev))
+        st["n"].append(n_l); st["longest"].append(max(now))
+        now = stays
+    st["ws"] = dash.workspace(dash.dash_layer_workspace(st["layers"][0], T, S).total, dev)
+    return st
+
+
+def _run_layer(st):
+    H, tok, pos, cu = st["H"], st["tok"], st["pos"], st["cu"]
+    for layer, o, n, longest in zip(st["layers"], st["out"], st["n"], st["longest"]):
+        dash.dash_layer_step(layer, H[:n], tok[:n], pos[:n], cu, longest, st["x_full"], o.H, o.tok, o.pos, o.cu, o.n, o.r, o.mask, st["ws"])
+        H, tok, pos, cu = o.H, o.tok, o.pos, o.cu
+    last = st["out"][-1]
+    return {"x_full": st["x_full"], "H": last.H, "tok": last.tok, "pos": last.pos, "cu": last.cu, "n": last.n,
+            "r": [o.r for o in st["out"]], "mask": [o.mask for o in st["out"]]}
+
+
+def _prepare_prefill(case, seed, dev):
+    """Three blocks in a row: one that passes every token on (threshold rule, nothing halts), the selecting block (a count stays),
+    one on the tokens that are left; rotary table and row factors handed from block to block, every block fills its KV cache."""
+    shape, lengths, g = SHAPES["qwen"], _lengths(case), _gen(seed, dev)
+    S, T = len(lengths), sum(lengths)
+    cu = wl.cu_from_lengths(lengths)
+    stays = [_kept(n, case["keep"]) for n in lengths]
+    st = {"H": _hidden(lengths, [case["keep"]], shape.d, shape.dtype, g, dev), "tok": torch.arange(T, dtype=torch.int32, device=dev),
+          "pos": wl.positions(cu).to(dev), "cu": cu.to(dev), "x_full": torch.zeros(T, shape.d, dtype=shape.dtype, device=dev)}
+    counts = _int32(stays, dev)
+    table = dash.dash_rope_table(shape.rope_base, shape.D, max(lengths), dev)
+    st["n"], st["longest"] = [T, T, sum(stays)], [max(lengths), max(lengths), max(stays)]
+    st["blocks"], st["out"], st["inv"], st["kv"] = [], [], [], []
+    for l in range(3):
+        b = dash.Block(shape, _weights(shape, g, dev, True), dev, tau=0.0, keep_first=KEEP_FIRST, keep_last=KEEP_LAST)
+        if l == 1:
+            b.set_keep_counts(counts, dash.SEL_KEEP_COUNT)
+        n = st["n"][l]
+        st["inv"].append(torch.zeros(n, dtype=torch.float32, device=dev))
+        b.set_handover(table, st["inv"][l - 1] if l else None, st["inv"][l])
+        st["kv"].append([torch.zeros(n, shape.Hkv, shape.D, dtype=shape.dtype, device=dev) for _ in range(2)])
+        b.set_kv_cache(*st["kv"][l])
+        st["blocks"].append(b); st["out"].append(_StepBuffers(n, S, shape.d, shape.dtype, dev))
+    st["ws"] = dash.workspace(dash.dash_block_workspace(st["blocks"][0], T, S).total, dev)
+    return st
+
+
+def _run_prefill(st):
+    H, tok, pos, cu = st["H"], st["tok"], st["pos"], st["cu"]
+    for b, o, n, longest in zip(st["blocks"], st["out"], st["n"], st["longest"]):
+        dash.dash_block_step(b, H[:n], tok[:n], pos[:n], cu, longest, st["x_full"], o.H, o.tok, o.pos, o.cu, o.n, o.r, o.mask, st["ws"])
+        H, tok, pos, cu = o.H, o.tok, o.pos, o.cu
+    last = st["out"][-1]
+    return {"x_full": st["x_full"], "H": last.H, "tok": last.tok, "pos": last.pos, "cu": last.cu, "r": [o.r for o in st["out"]],
+            "mask": [o.mask for o in st["out"]], "kv": st["kv"], "inv_rms": st["inv"][-1]}
+
+
+def _prepare_sparse(case, seed, dev):
+    shape, lengths, g = SHAPES["qwen"], _lengths(case), _gen(seed, dev)
+    S, T, d = len(lengths), sum(lengths), shape.d
+    cu = wl.cu_from_lengths(lengths)
+
+    def normal(*size):
+        return torch.randn(*size, generator=g, device=dev, dtype=torch.float32)
+
+    H = normal(T, d).to(shape.dtype)
+    size = torch.exp(normal(T) - 3.0)                              # heavy-tailed update sizes
+    U = (normal(T, d) * size[:, None]).to(shape.dtype)
+    # a threshold that keeps about the given share: in the middle of the widest of the gaps between the scores around that rank
+    r = torch.cat([torch.linalg.vector_norm(u.double(), dim=1) / torch.linalg.vector_norm(h.double(), dim=1)
+                   for u, h in zip(U.split(8192), H.split(8192))])
+    top = torch.topk(r, int(case["keep"] * T) + 32).values[-64:]
+    cut = int(torch.argmax(top[:-1] - top[1:]))
+    tau = float(0.5 * (top[cut] + top[cut + 1]))
+    dt, i32 = {"dtype": shape.dtype, "device": dev}, {"dtype": torch.int32, "device": dev}
+    Q, K, V = (normal(T, h, shape.D).to(shape.dtype) for h in (shape.Hq, shape.Hkv, shape.Hkv))
+    st = {"U": U, "H": H, "Q": Q, "K": K, "V": V, "tau": tau, "cu": cu.to(dev), "pos": wl.positions(cu).to(dev),
+          "tok": torch.arange(T, **i32), "longest": max(lengths), "indexed": case["indexed"],
+          "r": torch.empty(T, dtype=torch.float32, device=dev), "mask": torch.empty(T, dtype=torch.uint8, device=dev), "Ht": torch.empty(T, d, **dt),
+          "H_next": torch.zeros(T, d, **dt), "K_next": torch.zeros_like(K).view(T, -1), "V_next": torch.zeros_like(V).view(T, -1),
+          "O": torch.zeros(T, shape.Hq, shape.D, **dt)}
+    if not case["indexed"]:
+        st["Q_next"] = torch.zeros_like(Q).view(T, -1)
+    st["lists"] = {"idx": torch.zeros(T, **i32), "pos_out": torch.zeros(T, **i32), "tok_out": torch.zeros(T, **i32),
+                   "cu_out": torch.zeros(S + 1, **i32), "n_out": torch.zeros(1, **i32)}
+    st["ws_c"] = dash.workspace(dash.dash_workspace_bytes(dash.WS_COMPACT, T, S), dev)
+    st["ws_a"] = dash.workspace(dash.dash_workspace_bytes(dash.WS_ATTENTION, T, S, shape.Hq, shape.Hkv, shape.D), dev)
+    return st
+
+
+def _run_sparse(st):
+    dash.dash_delta_norm(st["U"], st["H"], r_out=st["r"], Hres_out=st["Ht"], tau=st["tau"], cu_seqlens=st["cu"], keep_first=KEEP_FIRST,
+                         keep_last=KEEP_LAST, mask_out=st["mask"])
+    T, (_, Hq, D), Hkv = st["Ht"].shape[0], st["Q"].shape, st["K"].shape[1]
+    rows, out = [st["Ht"], st["K"].view(T, -1), st["V"].view(T, -1)], [st["H_next"], st["K_next"], st["V_next"]]
+    if not st["indexed"]:
+        rows.append(st["Q"].view(T, -1)); out.append(st["Q_next"])
+    c = dash.dash_compact(st["mask"], st["cu"], rows=rows, rows_out=out, pos_in=st["pos"], tok_in=st["tok"], outputs=st["lists"], ws=st["ws_c"])
+    K, V = st["K_next"].view(T, Hkv, D), st["V_next"].view(T, Hkv, D)
+    if st["indexed"]:
+        dash.dash_varlen_attention_indexed(st["Q"], K, V, c["idx"], c["cu_out"], st["longest"], kv_packed=True, O=st["O"], ws=st["ws_a"])
+    else:
+        dash.dash_varlen_attention(st["Q_next"].view(T, Hq, D), K, V, c["cu_out"], st["longest"], O=st["O"], ws=st["ws_a"])
+    return {"Ht": st["Ht"], "r": st["r"], "mask": st["mask"], "H_next": st["H_next"], "K_next": st["K_next"], "V_next": st["V_next"], "O": st["O"],
+            **st["lists"]}
+
+
+def _prepare_decode(case, seed, dev):
+    shape, lengths, g = SHAPES["qwen"], _lengths(case), _gen(seed, dev)
+    S = len(lengths)
+
+    def normal(*size):
+        return torch.randn(*size, generator=g, device=dev, dtype=torch.float32).to(shape.dtype)
+
+    st = {"calls": []}
+    for l in range(case["full_blocks"] + case["cut_blocks"]):
+        n = lengths if l < case["full_blocks"] else [_kept(n, case["keep"]) for n in lengths]
+        st["calls"].append({"q": normal(S, shape.Hq, shape.D), "K": normal(sum(n), shape.Hkv, shape.D), "V": normal(sum(n), shape.Hkv, shape.D),
+                            "cu": wl.cu_from_lengths(n).to(dev), "out": torch.zeros(S, shape.Hq, shape.D, dtype=shape.dtype, device=dev)})
+    st["ws"] = dash.workspace(dash.dash_workspace_bytes(dash.WS_DECODE, sum(lengths), S, shape.Hq, shape.Hkv, shape.D), dev)
+    return st
+
+
+def _run_decode(st):
+    for c in st["calls"]:
+        dash.dash_decode_attention(c["q"], c["K"], c["V"], c["cu"], out=c["out"], ws=st["ws"])
+    return [c["out"] for c in st["calls"]]
+
+
+_KINDS = {"layer": (_prepare_layer, _run_layer), "prefill": (_prepare_prefill, _run_prefill), "sparse": (_prepare_sparse, _run_sparse),
+          "decode": (_prepare_decode, _run_decode)}
+
+
+def prepare(case, seed):
+    st = _KINDS[case["kind"]][0](case, seed, "cuda")
+    st["kind"] = case["kind"]
+    return st
+
+
+def run(state):
+    return _KINDS[state["kind"]][1](state)
+
+
+# ---- work and tolerance ----------------------------------------------------------
+def _causal_flops(lengths, shape):
+    return sum(2.0 * shape.Hq * shape.D * n * (n + 1) for n in lengths)
+
+
+def work(case):
+    lengths = _lengths(case)
+    T, S, kind = sum(lengths), len(lengths), case["kind"]
+    shape = SHAPES[case.get("shape", "qwen")]
+    es, hd, nq = torch.empty(0, dtype=shape.dtype).element_size(), shape.Hq * shape.D, (shape.Hq + 2 * shape.Hkv) * shape.D
+    kept = [_kept(n, case["keep"]) for n in lengths]
+    row, b, f = shape.d * es, 0.0, 0.0
+    if kind == "layer":
+        now = lengths
+        for share in _cascade_shares(case):
+            n, after = sum(now), [_kept(x, share) for x in lengths]
+            f += 2.0 * n * shape.d * (nq + hd) + _causal_flops(now, shape)
+            b += shape.d * (nq + hd) * es + n * (2 * row + 8 + 5) + sum(after) * (row + 8)      # weights, H, x_full, r, mask, what goes on
+            now = after
+    elif kind == "prefill":
+        for now, after in ((lengths, lengths), (lengths, kept), (kept, kept)):
+            n = sum(now)
+            f += 2.0 * n * shape.d * (nq + hd + 3 * shape.m) + _causal_flops(now, shape)
+            b += shape.d * (nq + hd + 3 * shape.m) * es + n * (2 * row + 8 + 5 + 2 * shape.Hkv * shape.D * es) + sum(after) * (row + 8 + 4)
+    elif kind == "sparse":
+        m = int(case["keep"] * T)
+        per = [m // S] * S
+        f = _causal_flops(per, shape) + 6.0 * T * shape.d
+        b = T * (3 * row + 5 + 8) + m * (2 * row + 2 * 2 * shape.Hkv * shape.D * es + 2 * hd * es + 12) + (0 if case["indexed"] else m * 2 * hd * es)
+    else:
+        for n in [lengths] * case["full_blocks"] + [kept] * case["cut_blocks"]:
+            b += sum(n) * 2 * shape.Hkv * shape.D * es + 2 * S * hd * es
+            f += 4.0 * sum(n) * hd
+    return {"bytes": b, "flops": f}
+
+
+def tolerance(case):
+    """About four times what is seen between two correct ways through the same bf16 roundings: one block with its norm as a pass of its
+    own instead of folded into the projection (relative error 0.0014, largest 0.008 of a value), four such blocks (0.0046, 0.04),
+    three whole blocks (0.0061, 0.04); attention against 64-bit sums (0.0023, 0.007).  The fp32 layer multiplies bf16 copies of its
+    operands, which moves its scores by about 1e-4.  Decisions and index lists are the same in every one of these comparisons."""
+    if case["kind"] == "layer" and case["shape"] == "tiny":
+        return {"rel": 0.001, "max": 0.005, "differ": 0.0}
+    if case["kind"] == "layer":
+        return {"rel": 0.006 if case["blocks"] == 1 else 0.018, "max": 0.032 if case["blocks"] == 1 else 0.16, "differ": 0.0}
+    if case["kind"] == "prefill":
+        return {"rel": 0.024, "max": 0.16, "differ": 0.0}
+    return {"rel": 0.009, "max": 0.03, "differ": 0.0}
