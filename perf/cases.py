@@ -170,13 +170,14 @@ def _prepare_layer(case, seed, dev):
     cu = wl.cu_from_lengths(lengths)
     st = {"H": _hidden(lengths, shares, shape.d, shape.dtype, g, dev), "tok": torch.arange(T, dtype=torch.int32, device=dev),
           "pos": wl.positions(cu).to(dev), "cu": cu.to(dev), "x_full": torch.zeros(T, shape.d, dtype=shape.dtype, device=dev)}
-    st["layers"], st["out"], st["n"], st["longest"] = [], [], [], []
+    st["layers"], st["out"], st["n"], st["longest"], st["weights"] = [], [], [], [], []
     table, now = None, list(lengths)
     for l in range(case["blocks"]):
         stays = [_kept(n, shares[l]) for n in lengths]
         rule = {"tau": UPDATE[case["shape"]] * math.sqrt(BAND)} if case["rule"] == "threshold" else \
             {"sel_mode": dash.SEL_KEEP_COUNT, "keep_counts": _int32(stays, dev)}
-        layer = dash.Layer(shape, _weights(shape, g, dev, False), dev, keep_first=KEEP_FIRST, keep_last=KEEP_LAST, **rule)
+        st["weights"].append(_weights(shape, g, dev, False))
+        layer = dash.Layer(shape, st["weights"][l], dev, keep_first=KEEP_FIRST, keep_last=KEEP_LAST, **rule)
         if layer.rms_folded:
             table = dash.dash_rope_table(shape.rope_base, shape.D, max(lengths), dev) if table is None else table
             layer.set_handover(table)
@@ -210,9 +211,10 @@ def _prepare_prefill(case, seed, dev):
     counts = _int32(stays, dev)
     table = dash.dash_rope_table(shape.rope_base, shape.D, max(lengths), dev)
     st["n"], st["longest"] = [T, T, sum(stays)], [max(lengths), max(lengths), max(stays)]
-    st["blocks"], st["out"], st["inv"], st["kv"] = [], [], [], []
+    st["blocks"], st["out"], st["inv"], st["kv"], st["weights"] = [], [], [], [], []
     for l in range(3):
-        b = dash.Block(shape, _weights(shape, g, dev, True), dev, tau=0.0, keep_first=KEEP_FIRST, keep_last=KEEP_LAST)
+        st["weights"].append(_weights(shape, g, dev, True))
+        b = dash.Block(shape, st["weights"][l], dev, tau=0.0, keep_first=KEEP_FIRST, keep_last=KEEP_LAST)
         if l == 1:
             b.set_keep_counts(counts, dash.SEL_KEEP_COUNT)
         n = st["n"][l]
@@ -319,6 +321,126 @@ def prepare(case, seed):
 
 def run(state):
     return _KINDS[state["kind"]][1](state)
+
+
+# ---- the same in 64 bits -------------------------------------------------------
+def _rows_apart(rows, lengths):
+    out, a = [], 0
+    for n in lengths:
+        out.append(rows[a:a + n])
+        a += n
+    return out
+
+
+def _attention64(q, K, V, lengths, causal=True):
+    """softmax(q K^T / sqrt(D)) V per packed sequence, in 64 bits; causal: query i of a sequence sees its keys 0..i, else every key is seen."""
+    Hq, D = q.shape[1:]
+    G, out, a = Hq // K.shape[1], torch.zeros(q.shape, dtype=torch.float64, device=q.device), 0
+    for i, n in enumerate(lengths):
+        rows = range(a, a + n, 1024) if causal else (i,)
+        for h in range(Hq):
+            k, v = K[a:a + n, h // G].double(), V[a:a + n, h // G].double()
+            for t in rows:
+                e = min(t + 1024, a + n) if causal else t + 1
+                seen = e - a if causal else n
+                s = q[t:e, h].double() @ k[:seen].T / math.sqrt(D)
+                if causal:
+                    s.masked_fill_(torch.arange(seen, device=q.device)[None, :] > torch.arange(t - a, e - a, device=q.device)[:, None], -math.inf)
+                out[t:e, h] = torch.softmax(s, dim=1) @ v[:seen]
+        a += n
+    return out
+
+
+def _norm64(x, w, eps):
+    return x * torch.rsqrt(x.square().mean(1, keepdim=True) + eps) * w.double()
+
+
+def _rotate64(x, pos, base):
+    half = x.shape[2] // 2
+    ang = pos.double()[:, None] * base ** (-torch.arange(half, dtype=torch.float64, device=x.device) / half)
+    c, s = ang.cos()[:, None], ang.sin()[:, None]
+    return torch.cat([x[..., :half] * c - x[..., half:] * s, x[..., half:] * c + x[..., :half] * s], dim=2)
+
+
+def _keep64(r, lengths, tau=None, counts=None):
+    """Which rows stay: scores not below tau, or the counts[s] highest of sequence s; the protected ends always."""
+    keep = []
+    for i, x in enumerate(_rows_apart(r, lengths)):
+        x = x.clone()
+        x[:KEEP_FIRST] = math.inf
+        x[max(0, len(x) - KEEP_LAST):] = math.inf
+        if counts is None:
+            keep.append(x >= tau)
+        else:
+            m = torch.zeros(len(x), dtype=torch.bool, device=r.device)
+            m[torch.topk(x, counts[i]).indices] = True
+            keep.append(m)
+    return torch.cat(keep)
+
+
+def _steps64(st, shape, rules, ffn):
+    """The blocks in a row in 64 bits on the given bf16 / fp32 inputs and weights.  rules[l] gives block l's rule for the lengths that enter it."""
+    H, tok, pos = st["H"].double(), st["tok"], st["pos"]
+    cu = st["cu"].tolist()
+    lengths = [b - a for a, b in zip(cu, cu[1:])]
+    x_full, steps = torch.zeros_like(H), []
+    for w, rule in zip(st["weights"], rules):
+        n, Hn = H.shape[0], _norm64(H, w["rms_w"], shape.rms_eps)
+        q, k, v = ((Hn @ w[x].double()).view(n, -1, shape.D) for x in ("Wq", "Wk", "Wv"))
+        q, k = _rotate64(q, pos, shape.rope_base), _rotate64(k, pos, shape.rope_base)
+        U = _attention64(q, k, v, lengths).view(n, -1) @ w["Wo"].double()
+        r = U.norm(dim=1) / H.norm(dim=1)
+        H = H + U
+        if ffn:
+            y = _norm64(H, w["rms2_w"], shape.rms_eps)
+            H = H + (torch.nn.functional.silu(y @ w["Wg"].double()) * (y @ w["Wu"].double())) @ w["Wd"].double()
+        x_full[tok.long()] = H
+        keep = rule(r, lengths)
+        lengths = [int(m.sum()) for m in _rows_apart(keep, lengths)]
+        H, tok, pos = H[keep], tok[keep], pos[keep]
+        steps.append({"r": r, "mask": keep.to(torch.uint8), "k": k, "v": v})
+    cu = wl.cu_from_lengths(lengths).to(H.device)
+    return x_full, steps, H, tok, pos, cu
+
+
+def _padded(x, n):
+    return torch.cat([x, x.new_zeros((n - x.shape[0], *x.shape[1:]))])
+
+
+def exact(case, seed):
+    st, shape = prepare(case, seed), SHAPES[case.get("shape", "qwen")]
+    lengths = _lengths(case)
+    if case["kind"] == "decode":
+        return [_attention64(c["q"], c["K"], c["V"], (c["cu"][1:] - c["cu"][:-1]).tolist(), causal=False) for c in st["calls"]]
+    if case["kind"] == "sparse":
+        Ht, T = st["H"].double() + st["U"].double(), st["H"].shape[0]
+        r = torch.cat([u.double().norm(dim=1) / h.double().norm(dim=1) for u, h in zip(st["U"].split(8192), st["H"].split(8192))])
+        keep = _keep64(r, lengths, tau=st["tau"])
+        now = [int(m.sum()) for m in _rows_apart(keep, lengths)]
+        K, V = st["K"][keep], st["V"][keep]
+        m = sum(now)
+        return {"Ht": Ht, "r": r, "mask": keep.to(torch.uint8), "H_next": _padded(Ht[keep], T), "K_next": _padded(K.double().view(m, -1), T),
+                "V_next": _padded(V.double().view(m, -1), T), "O": _padded(_attention64(st["Q"][keep], K, V, now), T),
+                "idx": _padded(st["tok"][keep], T), "pos_out": _padded(st["pos"][keep], T), "tok_out": _padded(st["tok"][keep], T),
+                "cu_out": wl.cu_from_lengths(now).to(r.device), "n_out": _int32([m], r.device)}
+    if case["kind"] == "layer":
+        if case["rule"] == "threshold":
+            tau = UPDATE[case["shape"]] * math.sqrt(BAND)
+            rules = [lambda r, now: _keep64(r, now, tau=tau)]
+        else:
+            rules = [lambda r, now, f=f: _keep64(r, now, counts=[_kept(n, f) for n in lengths]) for f in _cascade_shares(case)]
+        x_full, steps, H, tok, pos, cu = _steps64(st, shape, rules, False)
+        n = st["n"][-1]
+        return {"x_full": x_full, "H": _padded(H, n), "tok": _padded(tok, n), "pos": _padded(pos, n), "cu": cu, "n": cu[-1:],
+                "r": [s["r"] for s in steps], "mask": [s["mask"] for s in steps]}
+
+    def every(r, now):
+        return torch.ones_like(r, dtype=torch.bool)
+
+    rules = [every, lambda r, now: _keep64(r, now, counts=[_kept(n, case["keep"]) for n in now]), every]
+    x_full, steps, H, tok, pos, cu = _steps64(st, shape, rules, True)
+    return {"x_full": x_full, "H": H, "tok": tok, "pos": pos, "cu": cu, "r": [s["r"] for s in steps], "mask": [s["mask"] for s in steps],
+            "kv": [[s["k"], s["v"]] for s in steps], "inv_rms": torch.rsqrt(H.square().mean(1) + shape.rms_eps)}
 
 
 # ---- work and tolerance ----------------------------------------------------------
