@@ -12,8 +12,15 @@
 // One CTA per SM, in clusters of two: a pair computes a 256 x 256 tile with tcgen05.mma.cta_group::2 -- CTA r holds rows
 // 128 r .. of the A tile and columns 128 r .. of the W tile, so every SM loads only half of the W operand.  K in steps of 64
 // through a 6-stage TMA ring; warp 0 of each CTA issues its loads (their bytes are counted on the pair's even CTA), warp 1 of
-// the even CTA issues the MMAs and releases stages / hands over accumulators in both CTAs with multicast commits, warps 2-5
+// the even CTA issues the MMAs and releases stages / hands over accumulators in both CTAs with multicast commits, warps 2-9
 // of each CTA read their 128 accumulator rows (two TMEM buffers, so a tile's epilogue overlaps the next tile's MMAs).
+//
+// Epilogue.  A TMEM row belongs to a lane, a row of the output to 8 lanes: every warp turns its 32 x 32 fp32 (or 32 x 64 bf16) piece
+// through 4 KB of shared memory of its own, so that the rows of H, x_full, C and the rotary table are touched in pieces of 32 to
+// 128 contiguous bytes, and what an epilogue reads is asked for a piece ahead.  With a lane per row in the loads and stores too (and
+// four warps) an epilogue took 23-30 thousand cycles (ROPE), 18-22 (RESID), 15 (SWIGLU), 7 (PLAIN) against 31 thousand of a
+// 3584-deep tile's MMAs: the QKV projection waited for it at every tile (41.9 thousand cycles per tile), and the last tile's showed
+// in every launch.
 #include <math.h>
 
 #include "common.cuh"
@@ -26,7 +33,9 @@ using namespace ptx;
 
 constexpr int kGM = 128, kGN = 256, kGK = 64, kGStages = 6;      // kGM: rows per CTA (256 per pair)
 constexpr int kGABytes = kGM * kGK * 2, kGBBytes = kGK * (kGN / 2) * 2, kGStageBytes = kGABytes + kGBBytes;   // per CTA
-constexpr int kGThreads = 192;
+constexpr int kGEpiWarps = 8;                // two per TMEM lane quarter, each with one half of the tile's columns
+constexpr int kGThreads = 64 + 32 * kGEpiWarps;
+constexpr int kGEpiBytes = 4096;             // staging per epilogue warp: 32 rows of 128 bytes
 constexpr int kGGroupN = 16;                 // n tiles per group of the tile order
 constexpr long long kGWait = 4000000000LL;
 
@@ -86,12 +95,45 @@ struct GemmArgs {
     GemmEpilogue e;
 };
 
+// ---- epilogue pieces -----------------------------------------------------------
+// A warp's staging block holds 32 rows of 128 bytes; 16-byte chunk c of row r sits at chunk c ^ (r & 7), so that a lane per row
+// (writes) and eight lanes per row (reads) are both free of bank conflicts.
+__device__ __forceinline__ uint32_t stage_addr(uint32_t stage, int row, int chunk) { return stage + row * 128 + ((chunk ^ (row & 7)) << 4); }
+__device__ __forceinline__ void sts_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+__device__ __forceinline__ uint4 lds_v4(uint32_t addr) {
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint2 ld_v2(const void* p) {       // coherent: x_full may be H itself
+    uint2 v;
+    asm volatile("ld.global.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_v2(void* p, uint32_t a, uint32_t b) {
+    asm volatile("st.global.v2.u32 [%0], {%1,%2};" ::"l"(p), "r"(a), "r"(b) : "memory");
+}
+// v[i] summed over the eight lanes that share lane >> 3; lane j of them is left with v[j & 7]'s total (in v[0])
+__device__ __forceinline__ void reduce_rows8(float (&v)[8], int lane) {
+#pragma unroll
+    for (int w = 4; w >= 1; w >>= 1) {
+        const bool up = (lane & w) != 0;
+#pragma unroll
+        for (int i = 0; i < w; ++i) {
+            const float send = up ? v[i] : v[i + w], keep = up ? v[i + w] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, w);
+        }
+    }
+}
+
 template <int EPI>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGThreads, 1)
 gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapW, const GemmArgs g) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    const uint32_t bars = base + kGStages * kGStageBytes;
+    const uint32_t bars = base + kGStages * kGStageBytes + kGEpiWarps * kGEpiBytes;
     auto full = [&](int s) { return bars + 8 * s; };
     auto empty = [&](int s) { return bars + 8 * (kGStages + s); };
     auto acc_full = [&](int b) { return bars + 8 * (2 * kGStages + b); };
@@ -106,7 +148,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
     if (warp == 1) {
         if (lane == 0) {
             for (int s = 0; s < kGStages; ++s) { mbar_init(full(s), 1); mbar_init(empty(s), 1); }
-            for (int b = 0; b < 2; ++b) { mbar_init(acc_full(b), 1); mbar_init(acc_empty(b), 256); }
+            for (int b = 0; b < 2; ++b) { mbar_init(acc_full(b), 1); mbar_init(acc_empty(b), 2 * kGEpiWarps); }
             fence_barrier_init();
             fence_proxy_async_smem();
         }
@@ -180,139 +222,249 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
             if (!ok) atomicExch(g.status, DASH_ERR_TIMEOUT);
         }
     } else {
-        // ---- epilogue: thread <-> row of the tile (TMEM lane), 256 fp32 accumulators read 32 at a time ----
-        const int q = warp & 3;                                   // TMEM lane quarter this warp may read
+        // ---- epilogue: warp (q, half) holds rows 32 q .. of this CTA's 128 and columns 128 half .. of the tile's 256 (SWIGLU: gate and
+        // up columns of features 64 half ..) ----
+        const int q = warp & 3, half = (warp - 2) >> 2;           // q: the TMEM lane quarter this warp may read
         const uint32_t lane_base = (uint32_t)(q * 32) << 16;
+        const uint32_t stage = base + kGStages * kGStageBytes + (warp - 2) * kGEpiBytes;
         int n_true = g.n;
         if (g.n_dev) { const int nd = *g.n_dev; if (nd < n_true) n_true = nd; }
+        const int r8 = lane >> 3, c8 = lane & 7;                  // eight lanes per row: row r8 + 4 i, chunk c8
         uint32_t tl = 0;
         bool ok = true;
         for (int t = pair; t < tiles; t += n_pairs, ++tl) {
             const int b = tl & 1;
             int mt, nt;
             tile_coords(t, m_tiles, n_tiles, mt, nt);
-            ok = mbar_wait(acc_full(b), (tl >> 1) & 1, kGWait);
-            if (!ok) break;
-            tc_fence_after();
-            const int row = mt * 2 * kGM + rank * kGM + q * 32 + lane;
-            const bool live = row < n_true;
+            const int row0 = mt * 2 * kGM + rank * kGM + q * 32;  // first row of this warp's 32
             const uint32_t tD = tmem + b * kGN + lane_base;
+            auto wait_acc = [&]() { ok = __all_sync(0xffffffffu, mbar_wait(acc_full(b), (tl >> 1) & 1, kGWait)); tc_fence_after(); };
+            // every TMEM read of this warp for the tile has completed: the buffer goes back to the MMA thread
+            auto release_acc = [&]() {
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) arrive_on_leader(acc_empty(b));
+            };
+            auto stage_f32 = [&](const uint32_t* o) {             // 32 columns of this lane's row
+#pragma unroll
+                for (int c = 0; c < 8; ++c) sts_v4(stage_addr(stage, lane, c), o[4 * c], o[4 * c + 1], o[4 * c + 2], o[4 * c + 3]);
+                __syncwarp();
+            };
             if (EPI == GEMM_PLAIN) {
                 // columns at or past N (a last, partial tile) are not stored; N is a multiple of 8 (bf16) / 4 (fp32)
-                const int col0 = nt * kGN;
+                const int col0 = nt * kGN + half * 128;
+                wait_acc();
+                if (!ok) break;
+                if (g.out_f32) {
 #pragma unroll
-                for (int c = 0; c < kGN / 32; ++c) {
-                    uint32_t o[32];
-                    tmem_ld32(tD + c * 32, o);
-                    tmem_wait_ld();
-                    if (live && g.out_f32) {
-                        float* dst = reinterpret_cast<float*>(g.C) + (int64_t)row * g.ldc + col0 + c * 32;
+                    for (int k = 0; k < 4; ++k) {
+                        uint32_t o[32];
+                        tmem_ld32(tD + half * 128 + k * 32, o);
+                        tmem_wait_ld();
+                        if (k == 3) release_acc();
+                        stage_f32(o);
+                        const int col = col0 + k * 32 + c8 * 4;
 #pragma unroll
-                        for (int e = 0; e < 32; e += 4)
-                            if (col0 + c * 32 + e < g.N) st_v4(dst + e, make_uint4(o[e], o[e + 1], o[e + 2], o[e + 3]));
-                    } else if (live) {
-                        __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(g.C) + (int64_t)row * g.ldc + col0 + c * 32;
+                        for (int i = 0; i < 8; ++i) {
+                            const int r = r8 + 4 * i, row = row0 + r;
+                            const uint4 v = lds_v4(stage_addr(stage, r, c8));
+                            if (row < n_true && col < g.N) st_v4(reinterpret_cast<float*>(g.C) + (int64_t)row * g.ldc + col, v);
+                        }
+                        __syncwarp();
+                    }
+                } else {
 #pragma unroll
-                        for (int e = 0; e < 32; e += 8)
-                            if (col0 + c * 32 + e < g.N)
-                                st_v4(dst + e, make_uint4(pack_bf16(__uint_as_float(o[e]), __uint_as_float(o[e + 1])),
-                                                          pack_bf16(__uint_as_float(o[e + 2]), __uint_as_float(o[e + 3])),
-                                                          pack_bf16(__uint_as_float(o[e + 4]), __uint_as_float(o[e + 5])),
-                                                          pack_bf16(__uint_as_float(o[e + 6]), __uint_as_float(o[e + 7]))));
+                    for (int k = 0; k < 2; ++k) {
+                        uint32_t o[64];
+                        tmem_ld32(tD + half * 128 + k * 64, o);
+                        tmem_ld32(tD + half * 128 + k * 64 + 32, o + 32);
+                        tmem_wait_ld();
+                        if (k == 1) release_acc();
+                        auto pk = [&](int e) { return pack_bf16(__uint_as_float(o[e]), __uint_as_float(o[e + 1])); };
+#pragma unroll
+                        for (int c = 0; c < 8; ++c) sts_v4(stage_addr(stage, lane, c), pk(8 * c), pk(8 * c + 2), pk(8 * c + 4), pk(8 * c + 6));
+                        __syncwarp();
+                        const int col = col0 + k * 64 + c8 * 8;
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            const int r = r8 + 4 * i, row = row0 + r;
+                            const uint4 v = lds_v4(stage_addr(stage, r, c8));
+                            if (row < n_true && col < g.N) st_v4(reinterpret_cast<__nv_bfloat16*>(g.C) + (int64_t)row * g.ldc + col, v);
+                        }
+                        __syncwarp();
                     }
                 }
             } else if (EPI == GEMM_ROPE) {
-                // heads of D columns; inside a head of Q or K the pair (i, i + D/2) is rotated by the angle of (row, i)
-                __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(g.C) + (int64_t)row * g.ldc + nt * kGN;
-                const int D = g.e.D, half = D >> 1;
-                int64_t trow = row;                                            // (cos, sin) of this row: its own entry, or its position's
-                if (g.e.rope_pos) { trow = live ? g.e.rope_pos[row] : 0; if (trow >= g.e.rope_len) trow = g.e.rope_len - 1; if (trow < 0) trow = 0; }
-                const float2* cs = g.e.rope_table + trow * half;
-                const float rsc = (g.e.row_scale && live) ? g.e.row_scale[row] : 1.0f;
-                for (int h0 = 0; h0 < kGN; h0 += D) {
-                    const bool rotate = (nt * kGN + h0) < g.e.n_rot_cols;
-                    // D = 128: two 32-column chunks per half; D = 64: one
-                    for (int c = 0; c < half; c += 32) {
-                        uint32_t x1[32], x2[32];
-                        tmem_ld32(tD + h0 + c, x1);
-                        tmem_ld32(tD + h0 + half + c, x2);
-                        tmem_wait_ld();
-                        if (live) {
-                            float y1[32], y2[32];
+                // heads of D columns; inside a head of Q or K the pair (i, i + D/2) is rotated by the angle of (row, i).  A piece is 16
+                // pairs of a head: four lanes per row, four pairs each; rows in the order 0, 4, 1, 5, 2, 6, 3, 7 so that the two rows of
+                // a quarter warp lie in different halves of the banks.
+                const int D = g.e.D, hd2 = D >> 1, c4 = lane & 3, rr = (lane >> 3) + 4 * ((lane >> 2) & 1);
+                float rsc[4];
+                int tab[4];                                       // (cos, sin) entry of this row: its own, or its position's
 #pragma unroll
-                            for (int e = 0; e < 32; ++e) {
-                                const float a = __uint_as_float(x1[e]) * rsc, bb = __uint_as_float(x2[e]) * rsc;
-                                if (rotate) {
-                                    const float2 t2 = cs[c + e];
-                                    y1[e] = a * t2.x - bb * t2.y;
-                                    y2[e] = bb * t2.x + a * t2.y;
-                                } else { y1[e] = a; y2[e] = bb; }
-                            }
+                for (int i = 0; i < 4; ++i) {
+                    const int row = row0 + rr + 8 * i;
+                    const bool live = row < n_true;
+                    int64_t trow = live ? row : 0;
+                    if (g.e.rope_pos) { trow = live ? g.e.rope_pos[row] : 0; if (trow >= g.e.rope_len) trow = g.e.rope_len - 1; if (trow < 0) trow = 0; }
+                    tab[i] = (int)trow;
+                    rsc[i] = (g.e.row_scale && live) ? g.e.row_scale[row] : 1.0f;
+                }
+                const int colw = nt * kGN + half * 128;           // first column of this warp
+                auto head_of = [&](int k) { return D == 128 ? 0 : (k >> 1) * 64; };
+                auto pair_of = [&](int k) { return D == 128 ? k * 16 : (k & 1) * 16; };
+                const bool tab16 = (reinterpret_cast<uint64_t>(g.e.rope_table) & 15u) == 0;
+                uint4 cs[8];
+                auto fetch_cs = [&](int k) {
+                    if (colw + head_of(k) < g.e.n_rot_cols) {
 #pragma unroll
-                            for (int e = 0; e < 32; e += 8) {
-                                st_v4(dst + h0 + c + e, make_uint4(pack_bf16(y1[e], y1[e + 1]), pack_bf16(y1[e + 2], y1[e + 3]),
-                                                                   pack_bf16(y1[e + 4], y1[e + 5]), pack_bf16(y1[e + 6], y1[e + 7])));
-                                st_v4(dst + h0 + half + c + e, make_uint4(pack_bf16(y2[e], y2[e + 1]), pack_bf16(y2[e + 2], y2[e + 3]),
-                                                                          pack_bf16(y2[e + 4], y2[e + 5]), pack_bf16(y2[e + 6], y2[e + 7])));
+                        for (int i = 0; i < 4; ++i) {
+                            const float2* p = g.e.rope_table + (int64_t)tab[i] * hd2 + pair_of(k) + c4 * 4;
+                            if (tab16) {
+                                cs[2 * i] = __ldg(reinterpret_cast<const uint4*>(p));
+                                cs[2 * i + 1] = __ldg(reinterpret_cast<const uint4*>(p) + 1);
+                            } else {                              // a caller's table need only be 8-byte aligned
+                                const uint2* p2 = reinterpret_cast<const uint2*>(p);
+                                const uint2 a0 = __ldg(p2), a1 = __ldg(p2 + 1), a2 = __ldg(p2 + 2), a3 = __ldg(p2 + 3);
+                                cs[2 * i] = make_uint4(a0.x, a0.y, a1.x, a1.y);
+                                cs[2 * i + 1] = make_uint4(a2.x, a2.y, a3.x, a3.y);
                             }
                         }
                     }
+                };
+                fetch_cs(0);
+                wait_acc();
+                if (!ok) break;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int h0 = head_of(k), c = pair_of(k), colh = colw + h0;
+                    uint32_t o[32];
+                    tmem_ld16(tD + half * 128 + h0 + c, o);
+                    tmem_ld16(tD + half * 128 + h0 + hd2 + c, o + 16);
+                    tmem_wait_ld();
+                    if (k == 3) release_acc();
+                    stage_f32(o);
+                    const bool rotate = colh < g.e.n_rot_cols;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int r = rr + 8 * i, row = row0 + r;
+                        const uint4 v1 = lds_v4(stage_addr(stage, r, c4)), v2 = lds_v4(stage_addr(stage, r, 4 + c4));
+                        const float x1[4] = {__uint_as_float(v1.x) * rsc[i], __uint_as_float(v1.y) * rsc[i], __uint_as_float(v1.z) * rsc[i], __uint_as_float(v1.w) * rsc[i]};
+                        const float x2[4] = {__uint_as_float(v2.x) * rsc[i], __uint_as_float(v2.y) * rsc[i], __uint_as_float(v2.z) * rsc[i], __uint_as_float(v2.w) * rsc[i]};
+                        float y1[4], y2[4];
+                        if (rotate) {
+                            const uint32_t t[8] = {cs[2 * i].x, cs[2 * i].y, cs[2 * i].z, cs[2 * i].w, cs[2 * i + 1].x, cs[2 * i + 1].y, cs[2 * i + 1].z, cs[2 * i + 1].w};
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                const float cv = __uint_as_float(t[2 * e]), sv = __uint_as_float(t[2 * e + 1]);
+                                y1[e] = x1[e] * cv - x2[e] * sv;
+                                y2[e] = x2[e] * cv + x1[e] * sv;
+                            }
+                        } else {
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) { y1[e] = x1[e]; y2[e] = x2[e]; }
+                        }
+                        if (row < n_true) {
+                            __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(g.C) + (int64_t)row * g.ldc + colh + c + c4 * 4;
+                            st_v2(dst, pack_bf16(y1[0], y1[1]), pack_bf16(y1[2], y1[3]));
+                            st_v2(dst + hd2, pack_bf16(y2[0], y2[1]), pack_bf16(y2[2], y2[3]));
+                        }
+                    }
+                    if (k < 3) fetch_cs(k + 1);
+                    __syncwarp();
                 }
             } else if (EPI == GEMM_RESID) {
-                // H~ = H + U (U in fp32, one rounding) to x_full[tok[row]]; sums of u^2 and h^2 over this tile's 256 columns
-                const __nv_bfloat16* hsrc = reinterpret_cast<const __nv_bfloat16*>(g.e.H) + (int64_t)row * g.e.ldh + nt * kGN;
-                __nv_bfloat16* dst = live ? reinterpret_cast<__nv_bfloat16*>(g.e.x_full) + (int64_t)(g.e.tok_index ? g.e.tok_index[row] : row) * g.e.ldx + nt * kGN : nullptr;
-                float su = 0.f, sh = 0.f, st2 = 0.f;
+                // H~ = H + U (U in fp32, one rounding) to x_full[tok[row]]; sums of u^2, h^2 and (h+u)^2 over this warp's 128 columns
+                const int col0 = nt * kGN + half * 128 + c8 * 4;
+                const __nv_bfloat16* hsrc = reinterpret_cast<const __nv_bfloat16*>(g.e.H) + col0;
+                __nv_bfloat16* xdst = reinterpret_cast<__nv_bfloat16*>(g.e.x_full) + col0;
+                int tok[8];
+                uint2 hv[8];
 #pragma unroll
-                for (int c = 0; c < kGN / 32; ++c) {
+                for (int i = 0; i < 8; ++i) {
+                    const int row = row0 + r8 + 4 * i;
+                    tok[i] = row < n_true ? (g.e.tok_index ? g.e.tok_index[row] : row) : 0;
+                }
+                auto fetch_h = [&](int k) {
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const int row = row0 + r8 + 4 * i;
+                        if (row < n_true) hv[i] = ld_v2(hsrc + (int64_t)row * g.e.ldh + k * 32);
+                    }
+                };
+                fetch_h(0);
+                float su[8], sh[8], st2[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) su[i] = sh[i] = st2[i] = 0.f;
+                wait_acc();
+                if (!ok) break;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
                     uint32_t o[32];
-                    tmem_ld32(tD + c * 32, o);
+                    tmem_ld32(tD + half * 128 + k * 32, o);
                     tmem_wait_ld();
-                    if (live) {
+                    if (k == 3) release_acc();
+                    stage_f32(o);
+                    uint2 hc[8];
 #pragma unroll
-                        for (int e = 0; e < 32; e += 8) {
-                            const uint4 hv = ld_v4(hsrc + c * 32 + e);        // coherent: x_full may be H itself (identity token rows)
-                            const float hf[8] = {bf16lo(hv.x), bf16hi(hv.x), bf16lo(hv.y), bf16hi(hv.y), bf16lo(hv.z), bf16hi(hv.z), bf16lo(hv.w), bf16hi(hv.w)};
-                            float y[8];
+                    for (int i = 0; i < 8; ++i) hc[i] = hv[i];
+                    if (k < 3) fetch_h(k + 1);
 #pragma unroll
-                            for (int i = 0; i < 8; ++i) {
-                                const float u = __uint_as_float(o[e + i]);
-                                su += u * u;
-                                sh += hf[i] * hf[i];
-                                y[i] = hf[i] + u;
-                                st2 += y[i] * y[i];
+                    for (int i = 0; i < 8; ++i) {
+                        const int r = r8 + 4 * i, row = row0 + r;
+                        const uint4 v = lds_v4(stage_addr(stage, r, c8));
+                        if (row < n_true) {
+                            const float u[4] = {__uint_as_float(v.x), __uint_as_float(v.y), __uint_as_float(v.z), __uint_as_float(v.w)};
+                            const float h[4] = {bf16lo(hc[i].x), bf16hi(hc[i].x), bf16lo(hc[i].y), bf16hi(hc[i].y)};
+                            float y[4];
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                su[i] += u[e] * u[e];
+                                sh[i] += h[e] * h[e];
+                                y[e] = h[e] + u[e];
+                                st2[i] += y[e] * y[e];
                             }
-                            st_v4(dst + c * 32 + e, make_uint4(pack_bf16(y[0], y[1]), pack_bf16(y[2], y[3]), pack_bf16(y[4], y[5]), pack_bf16(y[6], y[7])));
+                            st_v2(xdst + (int64_t)tok[i] * g.e.ldx + k * 32, pack_bf16(y[0], y[1]), pack_bf16(y[2], y[3]));
                         }
                     }
+                    __syncwarp();
                 }
-                if (live) g.e.sums[(int64_t)row * n_tiles + nt] = make_float4(su, sh, st2, 0.f);
+                reduce_rows8(su, lane); reduce_rows8(sh, lane); reduce_rows8(st2, lane);
+                const int row = row0 + r8 + 4 * c8;               // this lane holds the sums of row r8 + 4 c8
+                if (row < n_true) g.e.sums[(int64_t)row * (2 * n_tiles) + 2 * nt + half] = make_float4(su[0], sh[0], st2[0], 0.f);
             } else {
                 // SWIGLU: columns 0-127 gate, 128-255 up of the same 128 features
-                __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(g.C) + (int64_t)row * g.ldc + nt * 128;
-                const float rsc = (g.e.row_scale && live) ? g.e.row_scale[row] : 1.0f;
+                const float rsc = (g.e.row_scale && row0 + lane < n_true) ? g.e.row_scale[row0 + lane] : 1.0f;
+                wait_acc();
+                if (!ok) break;
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
+                for (int k = 0; k < 2; ++k) {
                     uint32_t gt[32], up[32];
-                    tmem_ld32(tD + c * 32, gt);
-                    tmem_ld32(tD + 128 + c * 32, up);
+                    tmem_ld32(tD + half * 64 + k * 32, gt);
+                    tmem_ld32(tD + 128 + half * 64 + k * 32, up);
                     tmem_wait_ld();
-                    if (live) {
-                        float a[32];
+                    if (k == 1) release_acc();
+                    float a[32];
 #pragma unroll
-                        for (int e = 0; e < 32; ++e) {
-                            const float z = __uint_as_float(gt[e]) * rsc;
-                            a[e] = z / (1.0f + __expf(-z)) * (__uint_as_float(up[e]) * rsc);
-                        }
-#pragma unroll
-                        for (int e = 0; e < 32; e += 8)
-                            st_v4(dst + c * 32 + e, make_uint4(pack_bf16(a[e], a[e + 1]), pack_bf16(a[e + 2], a[e + 3]),
-                                                               pack_bf16(a[e + 4], a[e + 5]), pack_bf16(a[e + 6], a[e + 7])));
+                    for (int e = 0; e < 32; ++e) {
+                        const float z = __uint_as_float(gt[e]) * rsc;
+                        a[e] = z / (1.0f + __expf(-z)) * (__uint_as_float(up[e]) * rsc);
                     }
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+                        sts_v4(stage_addr(stage, lane, k * 4 + c), pack_bf16(a[8 * c], a[8 * c + 1]), pack_bf16(a[8 * c + 2], a[8 * c + 3]),
+                               pack_bf16(a[8 * c + 4], a[8 * c + 5]), pack_bf16(a[8 * c + 6], a[8 * c + 7]));
                 }
+                __syncwarp();
+                __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(g.C) + nt * 128 + half * 64 + c8 * 8;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int r = r8 + 4 * i, row = row0 + r;
+                    const uint4 v = lds_v4(stage_addr(stage, r, c8));
+                    if (row < n_true) st_v4(dst + (int64_t)row * g.ldc, v);
+                }
+                __syncwarp();
             }
-            tc_fence_before();
-            arrive_on_leader(acc_empty(b));
         }
         if (!ok && lane == 0) atomicExch(g.status, DASH_ERR_TIMEOUT);
     }
@@ -386,7 +538,7 @@ static int make_map_2d_bf16(CUtensorMap* map, const void* basep, uint64_t inner,
 
 template <int EPI>
 static int launch_gemm(const CUtensorMap& ma, const CUtensorMap& mw, const GemmArgs& g, cudaStream_t st) {
-    const int smem = kGStages * kGStageBytes + 1024 + 256;
+    const int smem = kGStages * kGStageBytes + kGEpiWarps * kGEpiBytes + 1024 + 256;
     static std::atomic<uint64_t> configured{0};
     if (!set_max_smem_once(gemm_kernel<EPI>, smem, configured)) return DASH_ERR_CUDA;
     const int tiles = ((g.n + 2 * kGM - 1) / (2 * kGM)) * g.n_tiles;

@@ -19,8 +19,8 @@ struct GemmEpilogue {
     // ROPE, SWIGLU: row_scale (null: none) multiplies the accumulators of a row first -- 1 / rms(row) when the RMSNorm in front of the
     // projection is folded into it (its weight into W, its row factor here)
     const float* row_scale = nullptr;
-    // RESID: x_full[tok_index[row]] (tok_index null: row) = H[row] + (A W)[row]; sums [n, N/256] = (sum u^2, sum h^2, sum (h+u)^2, 0)
-    // per column tile
+    // RESID: x_full[tok_index[row]] (tok_index null: row) = H[row] + (A W)[row]; sums [n, N/128] = (sum u^2, sum h^2, sum (h+u)^2, 0)
+    // per 128 columns
     const void* H = nullptr; int64_t ldh = 0;
     const int32_t* tok_index = nullptr;
     void* x_full = nullptr; int64_t ldx = 0;

@@ -265,7 +265,7 @@ extern "C" int dash_layer_workspace(const dash_layer_cfg* cfg, int64_t n, int S,
     off += align_up(dash_workspace_bytes(DASH_WS_COMPACT, n, S, 0, 0, 0, cfg->dt), 256);
     off += align_up(dash_workspace_bytes(DASH_WS_ATTENTION, n, S, cfg->Hq, cfg->Hkv, cfg->D, cfg->dt), 256);
     off += align_up((size_t)n * (cfg->D / 2) * sizeof(float2), 256);              // (cos, sin) of every row for the QKV epilogue
-    off += align_up((size_t)n * ((cfg->d + 255) / 256) * sizeof(float4), 256);    // per-row partial sums of the output-projection epilogue
+    off += align_up((size_t)n * ((cfg->d + 127) / 128) * sizeof(float4), 256);    // per-row partial sums of the output-projection epilogue
     off += 2 * align_up((size_t)n * sizeof(float), 256);                          // row factors of the two folded norms
     out->total = off;
     return DASH_OK;
@@ -304,7 +304,7 @@ static int carve_ws(const dash_layer_cfg* cfg, int64_t n, int S, void* ws, StepW
     out->attn_bytes = dash_workspace_bytes(DASH_WS_ATTENTION, n, S, cfg->Hq, cfg->Hkv, cfg->D, cfg->dt);
     out->rope_tab = (float2*)(out->attn_ws + align_up(out->attn_bytes, 256));
     out->sums = (float4*)((char*)out->rope_tab + align_up((size_t)n * (cfg->D / 2) * sizeof(float2), 256));
-    out->inv_rms = (float*)((char*)out->sums + align_up((size_t)n * ((cfg->d + 255) / 256) * sizeof(float4), 256));
+    out->inv_rms = (float*)((char*)out->sums + align_up((size_t)n * ((cfg->d + 127) / 128) * sizeof(float4), 256));
     out->inv_rms2 = (float*)((char*)out->inv_rms + align_up((size_t)n * sizeof(float), 256));
     return DASH_OK;
 }
@@ -450,7 +450,7 @@ extern "C" int dash_layer_step(const dash_layer_cfg* cfg, const void* H_in, cons
             // halting rule and the compaction of the rows that stay (from x_full) in one pass
             rc = out_proj_residual(cfg, H_in, tok_index_in, x_full, cu_in, S, n, W, st);
             if (rc == DASH_OK)
-                return launch_delta_tail(nullptr, nullptr, nullptr, W.sums, d / 256, n, d, cfg->dt, cfg->norm_mode, cfg->norm_eps, cfg->tau,
+                return launch_delta_tail(nullptr, nullptr, nullptr, W.sums, d / 128, n, d, cfg->dt, cfg->norm_mode, cfg->norm_eps, cfg->tau,
                                          cfg->keep_first, cfg->keep_last, cu_in, S, tok_index_in, pos_in, x_full, H_next, r_out, mask_out,
                                          tok_index_next, pos_next, cu_next, n_next_dev, W.compact_ws, W.compact_bytes, true, st,
                                          cfg->inv_rms_next, cfg->rms_eps);
@@ -536,7 +536,7 @@ extern "C" int dash_block_step(const dash_block_cfg* cfg, const void* H_in, cons
         // H~ came out of the projection's epilogue (into W.Ht) with the row sums: finish the score, then the rule
         dash_threshold ft = {a->tau, a->keep_first, a->keep_last, cu_in, S, mask_out};
         have_inv_rms2 = cfg->rms2_folded != 0;
-        if ((rc = launch_sums_to_score(W.sums, d / 256, n, a->norm_mode, a->norm_eps, r_out, a->sel_mode == DASH_SEL_THRESHOLD ? &ft : nullptr,
+        if ((rc = launch_sums_to_score(W.sums, d / 128, n, a->norm_mode, a->norm_eps, r_out, a->sel_mode == DASH_SEL_THRESHOLD ? &ft : nullptr,
                                        n_dev, have_inv_rms2 ? W.inv_rms2 : nullptr, d, a->rms_eps, st)) != DASH_OK) return rc;
         if (a->sel_mode != DASH_SEL_THRESHOLD &&
             (rc = dash_select(r_out, n, cu_in, S, a->sel_mode, a->tau, a->keep_counts, a->keep_first, a->keep_last, mask_out, st)) != DASH_OK)
