@@ -37,6 +37,10 @@ constexpr int kGEpiWarps = 8;                // two per TMEM lane quarter, each 
 constexpr int kGThreads = 64 + 32 * kGEpiWarps;
 constexpr int kGEpiBytes = 4096;             // staging per epilogue warp: 32 rows of 128 bytes
 constexpr int kGGroupN = 16;                 // n tiles per group of the tile order
+constexpr int kGSplitMaxRounds = 4;          // tiles may be cut along K where whole tiles take up to so many rounds
+constexpr int kGSplitMaxParts = 4;           // parts of a tile, on the average
+constexpr int kGSplitMinShare = 6;           // K steps of a pair's share, at least
+constexpr int kGSplitCost = 60;              // K steps that a cut costs
 constexpr long long kGWait = 4000000000LL;
 
 constexpr uint32_t kPeerMask = 0xFEFFFFFFu;   // clears the CTA-rank bit of a shared::cluster address: the pair's even CTA
@@ -85,6 +89,41 @@ __device__ __forceinline__ void tile_coords(int t, int m_tiles, int n_tiles, int
     nt = g * kGGroupN + r % gw;
 }
 
+template <int N> struct Width { static constexpr int value = N; };
+
+// What a pair of CTAs works on.  Whole tiles: t = pair, pair + P, .. in the order of tile_coords.  Cut along K (groups > 0): the pairs form
+// `groups` groups with one pair per row of tiles; the K steps of all column tiles are dealt out evenly to the groups, in order, so that
+// a group's share begins and ends anywhere inside a tile, and its pairs go through the same part of W at the same time (W comes from
+// HBM once: with the tiles' K steps simply dealt out to the pairs, a 136 MB weight matrix was read 3.6 times for three rows of tiles).
+struct Work {
+    int t, tiles, P, m_tiles, n_tiles, ksteps, mt;
+    long long u, u1;
+    bool cut;
+    __device__ __forceinline__ Work(int pair, int P_, int m_tiles_, int n_tiles_, int ksteps_, int groups)
+        : t(pair), tiles(m_tiles_ * n_tiles_), P(P_), m_tiles(m_tiles_), n_tiles(n_tiles_), ksteps(ksteps_), mt(0), u(0), u1(0), cut(groups > 0) {
+        if (cut) {
+            const int grp = pair / m_tiles;
+            const long long U = (long long)n_tiles * ksteps;
+            mt = pair % m_tiles;
+            if (grp < groups) { u = grp * U / groups; u1 = (grp + 1) * U / groups; }
+        }
+    }
+    __device__ __forceinline__ bool next(int& m, int& n, int& k0, int& k1) {
+        if (!cut) {
+            if (t >= tiles) return false;
+            tile_coords(t, m_tiles, n_tiles, m, n);
+            k0 = 0; k1 = ksteps; t += P;
+            return true;
+        }
+        if (u >= u1) return false;
+        n = (int)(u / ksteps); m = mt;
+        k0 = (int)(u - (long long)n * ksteps);
+        k1 = (int)min((long long)ksteps, k0 + (u1 - u));
+        u += k1 - k0;
+        return true;
+    }
+};
+
 struct GemmArgs {
     int n, N, K;                 // rows (upper bound), columns of W that one tile row of the output spans, depth
     int n_tiles;                 // tiles along the output columns
@@ -92,6 +131,9 @@ struct GemmArgs {
     int out_f32;                 // PLAIN: C is fp32 (else bf16)
     const int32_t* n_dev;        // device: true number of rows (<= n), or null
     int* status;
+    int groups;                  // > 0: tiles are cut along K (see Work)
+    float* part;                 // partial tiles of the pairs: two of 256 x 256 fp32 each
+    unsigned int* arrived;       // per tile, CTA of the pair and epilogue warp: parts that are in `part`
     GemmEpilogue e;
 };
 
@@ -163,7 +205,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
     cluster_sync_all();                                    // the peer's barriers exist before anything is signalled across
     tc_fence_after();
     const uint32_t tmem = *slot_gen;
-    const int m_tiles = (g.n + 2 * kGM - 1) / (2 * kGM), n_tiles = g.n_tiles, tiles = m_tiles * n_tiles, ksteps = (g.K + kGK - 1) / kGK;
+    const int m_tiles = (g.n + 2 * kGM - 1) / (2 * kGM), n_tiles = g.n_tiles, ksteps = (g.K + kGK - 1) / kGK;
     const int n_pairs = (int)gridDim.x / 2, pair = (int)blockIdx.x / 2;
     constexpr uint32_t idesc = idesc_bf16_f32(2 * kGM, kGN, false, true);
     constexpr uint32_t hi = smem_desc_hi_sw128(1024);
@@ -173,11 +215,11 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
         if (lane == 0) {
             uint32_t it = 0;
             bool ok = true;
-            for (int t = pair; t < tiles && ok; t += n_pairs) {
-                int mt, nt;
-                tile_coords(t, m_tiles, n_tiles, mt, nt);
+            Work w(pair, n_pairs, m_tiles, n_tiles, ksteps, g.groups);
+            int mt, nt, k0, k1;
+            while (ok && w.next(mt, nt, k0, k1)) {
                 const int m0 = mt * 2 * kGM + rank * kGM;
-                for (int k = 0; k < ksteps && ok; ++k, ++it) {
+                for (int k = k0; k < k1 && ok; ++k, ++it) {
                     const int s = it % kGStages;
                     if (it >= kGStages) ok = mbar_wait(empty(s), ((it / kGStages) - 1) & 1, kGWait);
                     if (!ok) break;
@@ -199,13 +241,15 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
         if (lane == 0 && rank == 0) {
             uint32_t it = 0, tl = 0;
             bool ok = true;
-            for (int t = pair; t < tiles && ok; t += n_pairs, ++tl) {
+            Work w(pair, n_pairs, m_tiles, n_tiles, ksteps, g.groups);
+            int mt, nt, k0, k1;
+            for (; ok && w.next(mt, nt, k0, k1); ++tl) {
                 const int b = tl & 1;
                 if (tl >= 2) ok = mbar_wait(acc_empty(b), ((tl >> 1) - 1) & 1, kGWait);
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t tD = tmem + b * kGN;
-                for (int k = 0; k < ksteps && ok; ++k, ++it) {
+                for (int k = k0; k < k1 && ok; ++k, ++it) {
                     const int s = it % kGStages;
                     ok = mbar_wait(full(s), (it / kGStages) & 1, kGWait);
                     if (!ok) break;
@@ -214,7 +258,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                     const uint32_t a_lo = smem_desc_lo(sA, 16), b_lo = smem_desc_lo(sB, kGK * 128);
 #pragma unroll
                     for (int kk = 0; kk < kGK / 16; ++kk)
-                        mma_ss_lh(tD, a_lo + ((kk * 32) >> 4), hi, b_lo + ((kk * 2048) >> 4), hi, idesc, (k > 0) || (kk > 0));
+                        mma_ss_lh(tD, a_lo + ((kk * 32) >> 4), hi, b_lo + ((kk * 2048) >> 4), hi, idesc, (k > k0) || (kk > 0));
                     commit_pair(empty(s));
                 }
                 commit_pair(acc_full(b));
@@ -232,10 +276,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
         const int r8 = lane >> 3, c8 = lane & 7;                  // eight lanes per row: row r8 + 4 i, chunk c8
         uint32_t tl = 0;
         bool ok = true;
-        for (int t = pair; t < tiles; t += n_pairs, ++tl) {
+        Work w(pair, n_pairs, m_tiles, n_tiles, ksteps, g.groups);
+        int mt, nt, k0, k1;
+        for (; w.next(mt, nt, k0, k1); ++tl) {
             const int b = tl & 1;
-            int mt, nt;
-            tile_coords(t, m_tiles, n_tiles, mt, nt);
             const int row0 = mt * 2 * kGM + rank * kGM + q * 32;  // first row of this warp's 32
             const uint32_t tD = tmem + b * kGN + lane_base;
             auto wait_acc = [&]() { ok = __all_sync(0xffffffffu, mbar_wait(acc_full(b), (tl >> 1) & 1, kGWait)); tc_fence_after(); };
@@ -245,6 +289,83 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                 __syncwarp();
                 if (lane == 0) arrive_on_leader(acc_empty(b));
             };
+            // A tile that was cut along K: every pair leaves its partial sums in `part` (a lane's row in 16-byte pieces, so that a warp's
+            // piece is 512 contiguous bytes), the last one to do so adds them up in the order of K and goes on as with a whole tile.
+            // Nobody waits for anybody.  Warp by warp: the same warp of every pair holds the same rows and columns.
+            int n_parts = 1, first_grp = 0;
+            auto part_of = [&](int grp, int col) {
+                const long long U = (long long)n_tiles * ksteps;
+                const int seg = (int)((grp * U / g.groups) / ksteps) == nt ? 0 : 1;      // the tile its share begins in, or the one it ends in
+                return reinterpret_cast<float4*>(g.part) + (size_t)(2 * (grp * m_tiles + mt) + seg) * (2 * kGM * kGN / 4) + (size_t)(col >> 2) * (2 * kGM) +
+                       rank * kGM + q * 32 + lane;
+            };
+            auto leave_part = [&]() -> bool {                     // true: the tile is left to another pair
+                const long long U = (long long)n_tiles * ksteps, u0 = (long long)nt * ksteps;
+                first_grp = (int)(((u0 + 1) * g.groups - 1) / U);
+                n_parts = (int)(((u0 + ksteps) * g.groups - 1) / U) - first_grp + 1;
+                unsigned int* cnt = g.arrived + (size_t)((nt * m_tiles + mt) * 2 + rank) * kGEpiWarps + (warp - 2);
+                if (row0 >= g.n) return true;                     // no rows here: nothing to add up, nothing to store
+                float4* dst0 = part_of(pair / m_tiles, 0);
+#pragma unroll 1
+                for (int k = 0; k < 4; ++k) {
+                    const int col = EPI == GEMM_SWIGLU ? (k >> 1) * 128 + half * 64 + (k & 1) * 32 : half * 128 + k * 32;
+                    uint32_t o[32];
+                    tmem_ld32(tD + col, o);
+                    tmem_wait_ld();
+                    float4* dst = dst0 + (size_t)(col >> 2) * (2 * kGM);
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) st_v4(dst + c * (2 * kGM), make_uint4(o[4 * c], o[4 * c + 1], o[4 * c + 2], o[4 * c + 3]));
+                }
+                __threadfence();
+                __syncwarp();
+                unsigned int in = 0;
+                if (lane == 0) in = atomicAdd(cnt, 1u);
+                in = __shfl_sync(0xffffffffu, in, 0);
+                if (in != (unsigned int)(n_parts - 1)) return true;
+                __threadfence();
+                if (lane == 0) *cnt = 0u;                         // for the next launch
+                return false;
+            };
+            // o[0 .. N) and o[N .. 2N): N columns of this lane's row from columns col0 and col1 of the tile
+            auto load_acc = [&](auto width, int col0, int col1, uint32_t* o) {
+                constexpr int N = decltype(width)::value;
+                if (n_parts == 1) {
+                    if constexpr (N == 32) { tmem_ld32(tD + col0, o); tmem_ld32(tD + col1, o + 32); }
+                    else { tmem_ld16(tD + col0, o); tmem_ld16(tD + col1, o + 16); }
+                    tmem_wait_ld();
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 2 * N; ++e) o[e] = 0u;
+#pragma unroll 1
+                    for (int p = 0; p < n_parts; p += 2) {        // two parts' loads in flight
+                        const bool two = p + 1 < n_parts;
+                        const float4* s0 = part_of(first_grp + p, 0);
+                        const float4* s1 = two ? part_of(first_grp + p + 1, 0) : s0;
+#pragma unroll
+                        for (int h = 0; h < N / 16; ++h) {
+                            float4 v[16];
+#pragma unroll
+                            for (int c = 0; c < 16; ++c) {
+                                const int cc = h * 8 + (c & 7);
+                                const int col = (cc < N / 4 ? col0 + 4 * cc : col1 + 4 * (cc - N / 4));
+                                v[c] = __ldcg((c < 8 ? s0 : s1) + (size_t)(col >> 2) * (2 * kGM));
+                            }
+#pragma unroll
+                            for (int c = 0; c < 16; ++c) {
+                                if (c < 8 || two) {
+                                    const float add[4] = {v[c].x, v[c].y, v[c].z, v[c].w};
+#pragma unroll
+                                    for (int e = 0; e < 4; ++e) {
+                                        uint32_t& x = o[(h * 8 + (c & 7)) * 4 + e];
+                                        x = __float_as_uint(__uint_as_float(x) + add[e]);
+                                    }
+                                }
+                            }
+                        }
+                    }
+                }
+            };
+            const Width<16> w16; const Width<32> w32;
             auto stage_f32 = [&](const uint32_t* o) {             // 32 columns of this lane's row
 #pragma unroll
                 for (int c = 0; c < 8; ++c) sts_v4(stage_addr(stage, lane, c), o[4 * c], o[4 * c + 1], o[4 * c + 2], o[4 * c + 3]);
@@ -255,12 +376,12 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                 const int col0 = nt * kGN + half * 128;
                 wait_acc();
                 if (!ok) break;
+                if (k1 - k0 != ksteps && leave_part()) { release_acc(); continue; }
                 if (g.out_f32) {
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
                         uint32_t o[32];
-                        tmem_ld32(tD + half * 128 + k * 32, o);
-                        tmem_wait_ld();
+                        load_acc(w16, half * 128 + k * 32, half * 128 + k * 32 + 16, o);
                         if (k == 3) release_acc();
                         stage_f32(o);
                         const int col = col0 + k * 32 + c8 * 4;
@@ -276,9 +397,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
 #pragma unroll
                     for (int k = 0; k < 2; ++k) {
                         uint32_t o[64];
-                        tmem_ld32(tD + half * 128 + k * 64, o);
-                        tmem_ld32(tD + half * 128 + k * 64 + 32, o + 32);
-                        tmem_wait_ld();
+                        load_acc(w32, half * 128 + k * 64, half * 128 + k * 64 + 32, o);
                         if (k == 1) release_acc();
                         auto pk = [&](int e) { return pack_bf16(__uint_as_float(o[e]), __uint_as_float(o[e + 1])); };
 #pragma unroll
@@ -335,13 +454,12 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                 fetch_cs(0);
                 wait_acc();
                 if (!ok) break;
+                if (k1 - k0 != ksteps && leave_part()) { release_acc(); continue; }
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     const int h0 = head_of(k), c = pair_of(k), colh = colw + h0;
                     uint32_t o[32];
-                    tmem_ld16(tD + half * 128 + h0 + c, o);
-                    tmem_ld16(tD + half * 128 + h0 + hd2 + c, o + 16);
-                    tmem_wait_ld();
+                    load_acc(w16, half * 128 + h0 + c, half * 128 + h0 + hd2 + c, o);
                     if (k == 3) release_acc();
                     stage_f32(o);
                     const bool rotate = colh < g.e.n_rot_cols;
@@ -398,24 +516,20 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                 for (int i = 0; i < 8; ++i) su[i] = sh[i] = st2[i] = 0.f;
                 wait_acc();
                 if (!ok) break;
+                if (k1 - k0 != ksteps && leave_part()) { release_acc(); continue; }
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     uint32_t o[32];
-                    tmem_ld32(tD + half * 128 + k * 32, o);
-                    tmem_wait_ld();
+                    load_acc(w16, half * 128 + k * 32, half * 128 + k * 32 + 16, o);
                     if (k == 3) release_acc();
                     stage_f32(o);
-                    uint2 hc[8];
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) hc[i] = hv[i];
-                    if (k < 3) fetch_h(k + 1);
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
                         const int r = r8 + 4 * i, row = row0 + r;
                         const uint4 v = lds_v4(stage_addr(stage, r, c8));
                         if (row < n_true) {
                             const float u[4] = {__uint_as_float(v.x), __uint_as_float(v.y), __uint_as_float(v.z), __uint_as_float(v.w)};
-                            const float h[4] = {bf16lo(hc[i].x), bf16hi(hc[i].x), bf16lo(hc[i].y), bf16hi(hc[i].y)};
+                            const float h[4] = {bf16lo(hv[i].x), bf16hi(hv[i].x), bf16lo(hv[i].y), bf16hi(hv[i].y)};
                             float y[4];
 #pragma unroll
                             for (int e = 0; e < 4; ++e) {
@@ -427,6 +541,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                             st_v2(xdst + (int64_t)tok[i] * g.e.ldx + k * 32, pack_bf16(y[0], y[1]), pack_bf16(y[2], y[3]));
                         }
                     }
+                    if (k < 3) fetch_h(k + 1);
                     __syncwarp();
                 }
                 reduce_rows8(su, lane); reduce_rows8(sh, lane); reduce_rows8(st2, lane);
@@ -437,12 +552,12 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                 const float rsc = (g.e.row_scale && row0 + lane < n_true) ? g.e.row_scale[row0 + lane] : 1.0f;
                 wait_acc();
                 if (!ok) break;
+                if (k1 - k0 != ksteps && leave_part()) { release_acc(); continue; }
 #pragma unroll
                 for (int k = 0; k < 2; ++k) {
-                    uint32_t gt[32], up[32];
-                    tmem_ld32(tD + half * 64 + k * 32, gt);
-                    tmem_ld32(tD + 128 + half * 64 + k * 32, up);
-                    tmem_wait_ld();
+                    uint32_t gu[64];
+                    const uint32_t *gt = gu, *up = gu + 32;
+                    load_acc(w32, half * 64 + k * 32, 128 + half * 64 + k * 32, gu);
                     if (k == 1) release_acc();
                     float a[32];
 #pragma unroll
@@ -536,14 +651,34 @@ static int make_map_2d_bf16(CUtensorMap* map, const void* basep, uint64_t inner,
                ? DASH_OK : DASH_ERR_CUDA;
 }
 
+// Scratch of tiles cut along K: two partial tiles per pair; a counter per tile, CTA and epilogue warp
+size_t gemm_split_part_bytes() { return (size_t)(sm_count() / 2) * 2 * (2 * kGM * kGN) * sizeof(float); }
+size_t gemm_split_count_bytes() { return align_up((size_t)(sm_count() / 2) * kGSplitMaxRounds * 2 * kGEpiWarps * sizeof(unsigned int), 256); }
+
+// Into how many groups of pairs the K steps are dealt out (0: whole tiles).  Whole tiles take ceil(tiles / P) rounds of `ksteps` steps, the last
+// of which may be nearly empty; cut, a pair takes n_tiles / groups tiles' worth of steps.  What the cut costs, partial tiles out and
+// in again, is worth about kGSplitCost steps.
+static int gemm_groups(int m_tiles, int n_tiles, int ksteps, int P, bool can) {
+    const long long tiles = (long long)m_tiles * n_tiles;
+    if (!can || m_tiles > P || tiles > (long long)kGSplitMaxRounds * P) return 0;
+    int groups = P / m_tiles;
+    const int most = (int)min((long long)n_tiles * kGSplitMaxParts, (long long)n_tiles * ksteps / kGSplitMinShare);
+    if (groups > most) groups = most;
+    if (groups < 1) return 0;
+    const long long whole = (tiles + P - 1) / P * ksteps, cut = ((long long)n_tiles * ksteps + groups - 1) / groups;
+    return cut + kGSplitCost < whole ? groups : 0;
+}
+
 template <int EPI>
-static int launch_gemm(const CUtensorMap& ma, const CUtensorMap& mw, const GemmArgs& g, cudaStream_t st) {
+static int launch_gemm(const CUtensorMap& ma, const CUtensorMap& mw, GemmArgs g, cudaStream_t st) {
     const int smem = kGStages * kGStageBytes + kGEpiWarps * kGEpiBytes + 1024 + 256;
     static std::atomic<uint64_t> configured{0};
     if (!set_max_smem_once(gemm_kernel<EPI>, smem, configured)) return DASH_ERR_CUDA;
-    const int tiles = ((g.n + 2 * kGM - 1) / (2 * kGM)) * g.n_tiles;
+    const int m_tiles = (g.n + 2 * kGM - 1) / (2 * kGM), tiles = m_tiles * g.n_tiles;
     int pairs = sm_count() / 2;
-    if (pairs > tiles) pairs = tiles;
+    g.groups = gemm_groups(m_tiles, g.n_tiles, (g.K + kGK - 1) / kGK, pairs, g.part != nullptr);
+    if (g.groups) pairs = g.groups * m_tiles;
+    else if (pairs > tiles) pairs = tiles;
     gemm_kernel<EPI><<<2 * pairs, kGThreads, smem, st>>>(ma, mw, g);
     return cudaGetLastError() == cudaSuccess ? DASH_OK : DASH_ERR_CUDA;
 }
@@ -560,7 +695,7 @@ bool gemm_shape_ok(GemmEpilogueKind kind, int64_t n, int64_t N, int64_t K, int64
 }
 
 int gemm_bf16(GemmEpilogueKind kind, const void* A, int64_t lda, const void* W, int64_t ldw, void* C, int64_t ldc, int64_t n, int64_t N,
-              int64_t K, const GemmEpilogue& e, const int32_t* n_dev, cudaStream_t st, bool out_f32) {
+              int64_t K, const GemmEpilogue& e, const int32_t* n_dev, cudaStream_t st, bool out_f32, const GemmSplit* sc) {
     if (!gemm_shape_ok(kind, n, N, K, lda, ldw, e)) return DASH_ERR_UNSUPPORTED;
     if (!aligned16(A) || !aligned16(W)) return DASH_ERR_INVALID_ARG;
     if (out_f32 && kind != GEMM_PLAIN) return DASH_ERR_UNSUPPORTED;
@@ -573,6 +708,7 @@ int gemm_bf16(GemmEpilogueKind kind, const void* A, int64_t lda, const void* W, 
     g.n = (int)n; g.N = (int)N; g.K = (int)K;
     g.n_tiles = kind == GEMM_SWIGLU ? e.m / 128 : (int)((N + kGN - 1) / kGN);
     g.C = C; g.ldc = ldc; g.n_dev = n_dev; g.e = e; g.out_f32 = out_f32 ? 1 : 0;
+    g.part = sc ? sc->part : nullptr; g.arrived = sc ? sc->arrived : nullptr; g.groups = 0;
     g.status = status_word_ptr();
     if (!g.status) return DASH_ERR_CUDA;
     switch (kind) {

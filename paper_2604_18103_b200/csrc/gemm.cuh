@@ -29,14 +29,20 @@ struct GemmEpilogue {
     int m = 0;
 };
 
+// Scratch of one GEMM at a time on one stream: part 16-byte aligned, gemm_split_part_bytes(); arrived gemm_split_count_bytes(), zero before the
+// first GEMM that uses it (every GEMM leaves it zero again).
+struct GemmSplit { float* part; unsigned int* arrived; };
+size_t gemm_split_part_bytes();
+size_t gemm_split_count_bytes();
+
 // true if the kernel takes this problem with this epilogue.  PLAIN: any N % 4 == 0, K % 8 == 0 (rows on 16-byte boundaries); the
 // fused epilogues: whole 256-column tiles (SWIGLU: m % 128 == 0) and K in steps of 64 -- otherwise the caller runs the projection
 // PLAIN and the element-wise work as passes of their own.
 bool gemm_shape_ok(GemmEpilogueKind kind, int64_t n, int64_t N, int64_t K, int64_t lda, int64_t ldw, const GemmEpilogue& e);
 // C (or the epilogue's outputs) = A[n, K] W[K, N], A and W bf16; ld* in elements; n_dev: device true row count or null;
-// out_f32 (PLAIN only): C is fp32 instead of bf16
+// out_f32 (PLAIN only): C is fp32 instead of bf16; sc: scratch that lets the kernel cut tiles along K (null: whole tiles only)
 int gemm_bf16(GemmEpilogueKind kind, const void* A, int64_t lda, const void* W, int64_t ldw, void* C, int64_t ldc, int64_t n, int64_t N,
-              int64_t K, const GemmEpilogue& e, const int32_t* n_dev, cudaStream_t st, bool out_f32 = false);
+              int64_t K, const GemmEpilogue& e, const int32_t* n_dev, cudaStream_t st, bool out_f32 = false, const GemmSplit* sc = nullptr);
 // dst (bf16, row stride ld_dst) = src (fp32, row stride ld_src) rounded to nearest even; cols % 4 == 0
 int launch_f32_to_bf16(const float* src, int64_t ld_src, void* dst, int64_t ld_dst, int64_t rows, int64_t cols, cudaStream_t st);
 // per row: (cos, sin) of pos * base^(-2i/D) into table [n, D/2] (table null: not formed; pos null: the row number is the position);

@@ -855,10 +855,17 @@ __global__ void __launch_bounds__(256)
 sums_to_score_kernel(const float4* __restrict__ sums, int n_sum_tiles, int64_t n, int mode, float eps, float* __restrict__ r_out,
                      FusedThreshold ft, const int32_t* __restrict__ n_dev, float* __restrict__ inv_rms_out, float inv_d, float rms_eps) {
     if (n_dev) { int64_t nd = *n_dev; if (nd < n) n = nd; }
-    for (int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; row < n; row += (int64_t)gridDim.x * blockDim.x) {
-        float su = 0.f, sh = 0.f;
-        float st2 = 0.f;
-        for (int i = 0; i < n_sum_tiles; ++i) { const float4 p2 = sums[row * n_sum_tiles + i]; su += p2.x; sh += p2.y; st2 += p2.z; }
+    // eight lanes per row: the row's partial sums lie next to each other
+    const int sub = threadIdx.x & 7;
+    for (int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3; row < n; row += ((int64_t)gridDim.x * blockDim.x) >> 3) {
+        float su = 0.f, sh = 0.f, st2 = 0.f;
+        for (int i = sub; i < n_sum_tiles; i += 8) { const float4 p2 = sums[row * n_sum_tiles + i]; su += p2.x; sh += p2.y; st2 += p2.z; }
+        const unsigned int group = 0xffu << (threadIdx.x & 24);
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) {
+            su += __shfl_xor_sync(group, su, o); sh += __shfl_xor_sync(group, sh, o); st2 += __shfl_xor_sync(group, st2, o);
+        }
+        if (sub != 0) continue;
         if (inv_rms_out) inv_rms_out[row] = rsqrtf(st2 * inv_d + rms_eps);
         const float num = sqrtf(su);
         const float r = (mode == DASH_NORM_ABS) ? num : num / fmaxf(sqrtf(sh), eps);
@@ -876,7 +883,7 @@ int launch_sums_to_score(const float4* sums, int n_sum_tiles, int64_t n, dash_no
                          const int32_t* n_dev, float* inv_rms_out, int d, float rms_eps, cudaStream_t st) {
     FusedThreshold ft = {0.f, 0, 0, nullptr, 0, nullptr};
     if (fused) ft = {fused->tau, fused->keep_first, fused->keep_last, fused->cu_seqlens, fused->S, fused->mask_out};
-    int64_t blocks = (n + 255) / 256, cap = (int64_t)sm_count() * 8;
+    int64_t blocks = (n + 31) / 32, cap = (int64_t)sm_count() * 8;
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
     sums_to_score_kernel<<<(int)blocks, 256, 0, st>>>(sums, n_sum_tiles, n, (int)mode, eps, r_out, ft, n_dev, inv_rms_out, 1.0f / d, rms_eps);
@@ -885,14 +892,9 @@ int launch_sums_to_score(const float4* sums, int n_sum_tiles, int64_t n, dash_no
 
 // Fused tail of the block step (see delta_tail_kernel).  Preconditions checked by the caller: threshold rule, every row
 // scattered, 16-byte aligned rows.  ws: the compaction workspace (ticket + one state word per 32-token tile); ws_is_clear: the
-// caller has already zeroed it on this stream with clear_tail_ws (ahead of the kernels in front, so that this launch follows a
-// kernel directly and may start while that one drains).
-static size_t tail_ws_clear_bytes(int64_t n) { return 256 + (size_t)((n + 31) / 32 > 0 ? (n + 31) / 32 : 1) * 8; }
-int clear_tail_ws(void* ws, size_t ws_bytes, int64_t n, cudaStream_t st) {
-    if (!ws || ((uintptr_t)ws % 256) || ws_bytes < compact_ws_bytes(n)) return DASH_ERR_WORKSPACE;
-    DASH_CUDA_TRY(cudaMemsetAsync(ws, 0, tail_ws_clear_bytes(n), st));
-    return DASH_OK;
-}
+// caller has already zeroed its first tail_ws_clear_bytes(n) on this stream (ahead of the kernels in front, so that this launch
+// follows a kernel directly and may start while that one drains).
+size_t tail_ws_clear_bytes(int64_t n) { return 256 + (size_t)((n + 31) / 32 > 0 ? (n + 31) / 32 : 1) * 8; }
 int launch_delta_tail(const void* U, const void* H, const uint8_t* mask_in, const float4* sums, int n_sum_tiles, int64_t n, int d, dash_dtype dt, dash_norm_mode mode, float eps, float tau,
                       int keep_first, int keep_last, const int32_t* cu_in, int S, const int32_t* tok_in, const int32_t* pos_in,
                       void* x_full, void* H_next, float* r_out, uint8_t* mask_out, int32_t* tok_next, int32_t* pos_next,

@@ -118,7 +118,7 @@ int launch_delta_tail(const void* U, const void* H, const uint8_t* mask_in, cons
                       void* x_full, void* H_next, float* r_out, uint8_t* mask_out, int32_t* tok_next, int32_t* pos_next,
                       int32_t* cu_next, int32_t* n_next, void* ws, size_t ws_bytes, bool ws_is_clear, cudaStream_t st, float* inv_next,
                       float rms_eps);
-int clear_tail_ws(void* ws, size_t ws_bytes, int64_t n, cudaStream_t st);
+size_t tail_ws_clear_bytes(int64_t n);
 int attention_plan(const int32_t* cu_seqlens, int S, int64_t n, int Hq, void* ws, size_t ws_bytes, cudaStream_t st);
 int attention_planned(const void* Q, const void* K, const void* V, void* O, float* lse, int64_t ldq, int64_t ldk, int64_t ldv, int64_t ldo,
                       const int32_t* cu_seqlens, int S, int64_t n, int64_t max_seqlen, int Hq, int Hkv, int D, float scale, dash_dtype dt,
@@ -132,9 +132,9 @@ static size_t conv_w_bytes(int64_t k, int64_t n_cols) { return align_up((size_t)
 // C = A W (plain).  bf16: the GEMM of gemm.cu as it is.  fp32: its operands are rounded to bf16 copies first (what the
 // attention kernel does with Q, K, V), the product accumulates in fp32 and is stored as fp32.
 static int project(dash_dtype dt, const void* A, int64_t lda, const void* W, int64_t ldw, void* C, int64_t ldc, int64_t n, int64_t N, int64_t K,
-                   const int32_t* n_dev, const ConvScratch& cs, cudaStream_t st) {
+                   const int32_t* n_dev, const ConvScratch& cs, const GemmSplit& split, cudaStream_t st) {
     GemmEpilogue e;
-    if (dt == DASH_BF16) return gemm_bf16(GEMM_PLAIN, A, lda, W, ldw, C, ldc, n, N, K, e, n_dev, st);
+    if (dt == DASH_BF16) return gemm_bf16(GEMM_PLAIN, A, lda, W, ldw, C, ldc, n, N, K, e, n_dev, st, false, &split);
     if ((K % 8) || (N % 4)) return DASH_ERR_UNSUPPORTED;
     const int64_t lda_b = K, ldw_b = (int64_t)align_up((size_t)N, 8);
     if ((size_t)n * lda_b * 2 > cs.a_bytes || (size_t)K * ldw_b * 2 > cs.w_bytes) return DASH_ERR_WORKSPACE;
@@ -262,6 +262,7 @@ extern "C" int dash_layer_workspace(const dash_layer_cfg* cfg, int64_t n, int S,
         off += conv_a_bytes(n, cfg->d > hd ? cfg->d : hd);
         off += conv_w_bytes(cfg->d, (int64_t)nq > cfg->d ? (int64_t)nq : cfg->d) > conv_w_bytes(hd, cfg->d) ? conv_w_bytes(cfg->d, (int64_t)nq > cfg->d ? (int64_t)nq : cfg->d) : conv_w_bytes(hd, cfg->d);
     }
+    if (cfg->dt == DASH_BF16) off += gemm_split_part_bytes() + gemm_split_count_bytes();      // tiles of the projections cut along K
     off += align_up(dash_workspace_bytes(DASH_WS_COMPACT, n, S, 0, 0, 0, cfg->dt), 256);
     off += align_up(dash_workspace_bytes(DASH_WS_ATTENTION, n, S, cfg->Hq, cfg->Hkv, cfg->D, cfg->dt), 256);
     off += align_up((size_t)n * (cfg->D / 2) * sizeof(float2), 256);              // (cos, sin) of every row for the QKV epilogue
@@ -277,6 +278,7 @@ struct StepWs {
     dash_layer_ws_layout L;
     char *Hn, *QKV, *O, *U, *Ht, *compact_ws, *attn_ws;
     ConvScratch conv;
+    GemmSplit split;                 // part == null: fp32 tensors
     size_t compact_bytes, attn_bytes;
     float2* rope_tab;
     float4* sums;
@@ -298,6 +300,13 @@ static int carve_ws(const dash_layer_cfg* cfg, int64_t n, int S, void* ws, StepW
         out->conv = {after, ab, after + ab, wb};
         after += ab + wb;
     }
+    out->split = {nullptr, nullptr};
+    if (cfg->dt == DASH_BF16) {
+        out->split.part = (float*)after;
+        after += gemm_split_part_bytes();
+        out->split.arrived = (unsigned int*)after;         // directly in front of the look-back words: one clear takes both
+        after += gemm_split_count_bytes();
+    }
     out->compact_ws = after;
     out->compact_bytes = align_up(dash_workspace_bytes(DASH_WS_COMPACT, n, S, 0, 0, 0, cfg->dt), 256);
     out->attn_ws = out->compact_ws + out->compact_bytes;
@@ -306,6 +315,14 @@ static int carve_ws(const dash_layer_cfg* cfg, int64_t n, int S, void* ws, StepW
     out->sums = (float4*)((char*)out->rope_tab + align_up((size_t)n * (cfg->D / 2) * sizeof(float2), 256));
     out->inv_rms = (float*)((char*)out->sums + align_up((size_t)n * ((cfg->d + 127) / 128) * sizeof(float4), 256));
     out->inv_rms2 = (float*)((char*)out->inv_rms + align_up((size_t)n * sizeof(float), 256));
+    return DASH_OK;
+}
+
+// Zeroed up front, in one go: the arrival counters of projections cut along K and the tail pass's look-back words (whose launch
+// then follows the projection in front of it directly)
+static int clear_step_words(const StepWs& W, int64_t n, bool tail_pass, cudaStream_t st) {
+    const size_t front = W.split.part ? gemm_split_count_bytes() : 0, tail = tail_pass ? tail_ws_clear_bytes(n) : 0;
+    if (front + tail) DASH_CUDA_TRY(cudaMemsetAsync(W.compact_ws - front, 0, front + tail, st));
     return DASH_OK;
 }
 
@@ -347,16 +364,16 @@ static int attention_to_O(const dash_layer_cfg* cfg, const void* H_in, const int
             if (rc != DASH_OK) return rc;
         }
         e.row_scale = cfg->inv_rms_in ? cfg->inv_rms_in : W.inv_rms;
-        if ((rc = gemm_bf16(GEMM_ROPE, H_in, d, cfg->Wqkv, nq, W.QKV, nq, n, nq, d, e, n_dev, st)) != DASH_OK) return rc;
+        if ((rc = gemm_bf16(GEMM_ROPE, H_in, d, cfg->Wqkv, nq, W.QKV, nq, n, nq, d, e, n_dev, st, false, &W.split)) != DASH_OK) return rc;
     } else if (fused) {
         // LN (read as RMSNorm), then Q | K | V = Hn Wqkv with the Q and K heads rotated on the accumulators
         if ((rc = launch_rmsnorm(cfg->dt, H_in, cfg->rms_weight, W.Hn, n, d, cfg->rms_eps, n_dev, st)) != DASH_OK) return rc;
         if ((rc = launch_row_prep(pos_in, n, D, cfg->rope_base, W.rope_tab, nullptr, 0, d, 0.f, nullptr, n_dev, st)) != DASH_OK) return rc;
-        if ((rc = gemm_bf16(GEMM_ROPE, W.Hn, d, cfg->Wqkv, nq, W.QKV, nq, n, nq, d, e, n_dev, st)) != DASH_OK) return rc;
+        if ((rc = gemm_bf16(GEMM_ROPE, W.Hn, d, cfg->Wqkv, nq, W.QKV, nq, n, nq, d, e, n_dev, st, false, &W.split)) != DASH_OK) return rc;
     } else {
         if (cfg->rms_folded) return DASH_ERR_UNSUPPORTED;      // folded weights need the fused projection (bf16, 256-column tiles)
         if ((rc = launch_rmsnorm(cfg->dt, H_in, cfg->rms_weight, W.Hn, n, d, cfg->rms_eps, n_dev, st)) != DASH_OK) return rc;
-        if ((rc = project(cfg->dt, W.Hn, d, cfg->Wqkv, nq, W.QKV, nq, n, nq, d, n_dev, W.conv, st)) != DASH_OK) return rc;
+        if ((rc = project(cfg->dt, W.Hn, d, cfg->Wqkv, nq, W.QKV, nq, n, nq, d, n_dev, W.conv, W.split, st)) != DASH_OK) return rc;
         // rotary embedding on the Q and K heads
         RopeFreq fr;
         for (int i = 0; i < D / 2; ++i) fr.inv_freq[i] = pow(cfg->rope_base, -2.0 * i / D);
@@ -382,7 +399,7 @@ static int attention_to_O(const dash_layer_cfg* cfg, const void* H_in, const int
 // U = O Wo  (pre-residual attention output, Eq. 1) into W.U
 static int out_proj_U(const dash_layer_cfg* cfg, const int32_t* cu_in, int S, int64_t n, const StepWs& W, cudaStream_t st) {
     const int64_t hd = (int64_t)cfg->Hq * cfg->D;
-    return project(cfg->dt, W.O, hd, cfg->Wo, cfg->d, W.U, cfg->d, n, cfg->d, hd, cu_in + S, W.conv, st);
+    return project(cfg->dt, W.O, hd, cfg->Wo, cfg->d, W.U, cfg->d, n, cfg->d, hd, cu_in + S, W.conv, W.split, st);
 }
 
 // Output projection with the residual in its epilogue: dst[idx[row]] = H + O Wo (idx null: row), per-row sums of u^2, h^2 into W.sums.
@@ -393,7 +410,7 @@ static int out_proj_residual(const dash_layer_cfg* cfg, const void* H_in, const 
     GemmEpilogue e;
     e.H = H_in; e.ldh = cfg->d; e.tok_index = idx; e.x_full = dst; e.ldx = cfg->d; e.sums = W.sums;
     if (cfg->dt != DASH_BF16 || !gemm_shape_ok(GEMM_RESID, n, cfg->d, hd, hd, cfg->d, e)) return DASH_ERR_UNSUPPORTED;
-    return gemm_bf16(GEMM_RESID, W.O, hd, cfg->Wo, cfg->d, nullptr, 0, n, cfg->d, hd, e, cu_in + S, st);
+    return gemm_bf16(GEMM_RESID, W.O, hd, cfg->Wo, cfg->d, nullptr, 0, n, cfg->d, hd, e, cu_in + S, st, false, &W.split);
 }
 
 // r (and, threshold rule, the keep mask) from U and H, H~ = H + U into W.Ht; keep-count rule: the radix select on r
@@ -442,8 +459,7 @@ extern "C" int dash_layer_step(const dash_layer_cfg* cfg, const void* H_in, cons
             (cfg->rms_weight && !aligned16(cfg->rms_weight)))
             return DASH_ERR_INVALID_ARG;
         const bool tail_pass = cfg->sel_mode == DASH_SEL_THRESHOLD && cfg->scatter_which == 2;
-        // the tail pass's look-back words are cleared up front: its launch then follows the output projection directly
-        if (tail_pass && (rc = clear_tail_ws(W.compact_ws, W.compact_bytes, n, st)) != DASH_OK) return rc;
+        if ((rc = clear_step_words(W, n, tail_pass, st)) != DASH_OK) return rc;
         if ((rc = attention_to_O(cfg, H_in, pos_in, cu_in, S, n, max_seqlen, W, st)) != DASH_OK) return rc;
         if (tail_pass) {
             // output projection with H~ = H + U written straight to x_full and the row sums of u^2, h^2 beside it; then the score, the
@@ -526,8 +542,7 @@ extern "C" int dash_block_step(const dash_block_cfg* cfg, const void* H_in, cons
         !aligned16(cfg->Wgu) || !aligned16(cfg->Wd) || (cfg->rms2_weight && !aligned16(cfg->rms2_weight)))
         return DASH_ERR_INVALID_ARG;
     const int32_t* n_dev = cu_in + S;
-    // the tail pass's look-back words are cleared up front: its launch then follows the down projection directly
-    if ((rc = clear_tail_ws(W.compact_ws, W.compact_bytes, n, st)) != DASH_OK) return rc;
+    if ((rc = clear_step_words(W, n, true, st)) != DASH_OK) return rc;
     // U = Attn(LN(H)); score and selection from U; H~ = H + U
     if ((rc = attention_to_O(a, H_in, pos_in, cu_in, S, n, max_seqlen, W, st)) != DASH_OK) return rc;
     bool have_inv_rms2 = false;
@@ -557,9 +572,9 @@ extern "C" int dash_block_step(const dash_block_cfg* cfg, const void* H_in, cons
         // gate | up projection with silu(gate) * up on the accumulators: the [n, 2m] intermediate is never stored; with the norm
         // folded in, the operand is H~ itself and the accumulators take the row factor 1 / rms first
         eg.row_scale = cfg->rms2_folded ? W.inv_rms2 : nullptr;
-        if ((rc = gemm_bf16(GEMM_SWIGLU, cfg->rms2_folded ? W.Ht : W.Hn, d, cfg->Wgu, 2 * (int64_t)m, ACT, m, n, 2 * (int64_t)m, d, eg, n_dev, st)) != DASH_OK) return rc;
+        if ((rc = gemm_bf16(GEMM_SWIGLU, cfg->rms2_folded ? W.Ht : W.Hn, d, cfg->Wgu, 2 * (int64_t)m, ACT, m, n, 2 * (int64_t)m, d, eg, n_dev, st, false, &W.split)) != DASH_OK) return rc;
     } else {
-        if ((rc = project(a->dt, W.Hn, d, cfg->Wgu, 2 * (int64_t)m, GU, 2 * (int64_t)m, n, 2 * (int64_t)m, d, n_dev, conv, st)) != DASH_OK) return rc;
+        if ((rc = project(a->dt, W.Hn, d, cfg->Wgu, 2 * (int64_t)m, GU, 2 * (int64_t)m, n, 2 * (int64_t)m, d, n_dev, conv, W.split, st)) != DASH_OK) return rc;
         const int64_t total = n * (int64_t)(m / (16 / es));
         int64_t blocks = (total + 255) / 256, cap = (int64_t)sm_count() * 16;
         if (blocks > cap) blocks = cap;
@@ -567,7 +582,7 @@ extern "C" int dash_block_step(const dash_block_cfg* cfg, const void* H_in, cons
         else swiglu_kernel<false><<<(int)blocks, 256, 0, st>>>(GU, 2 * (int64_t)m * es, ACT, (int64_t)m * es, n, m, n_dev);
         DASH_CUDA_TRY(cudaGetLastError());
     }
-    if ((rc = project(a->dt, ACT, m, cfg->Wd, d, F, d, n, d, m, n_dev, conv, st)) != DASH_OK) return rc;
+    if ((rc = project(a->dt, ACT, m, cfg->Wd, d, F, d, n, d, m, n_dev, conv, W.split, st)) != DASH_OK) return rc;
     if (cfg->signal == DASH_SIGNAL_BLOCK) {
         // ablation: score = change over the whole block, H' - H = U + F (formed in the gate | up buffer, free by now)
         if ((rc = dash_delta_norm(F, W.U, n, d, d, d, a->dt, DASH_NORM_ABS, a->norm_eps, r_out, GU, d, nullptr, nullptr, n_dev, st)) != DASH_OK) return rc;

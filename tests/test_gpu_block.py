@@ -216,3 +216,32 @@ def test_block_step_shapes_without_whole_tiles(dtype):
     assert k == idx.size and abs(k - K) <= flips
     assert torch.equal(b.H_next[:k].cpu(), x_full.cpu()[idx])
     assert np.array_equal(b.tok_next[:k].cpu().numpy(), idx)
+
+
+@pytest.mark.parametrize("n", [100, 257, 523])
+@pytest.mark.parametrize("which", ["deep_output_and_down", "deep_qkv_and_gate_up"])
+def test_block_step_with_projections_cut_along_k(which, n):
+    """Few column tiles over a deep K: the projections deal their K steps out to several pairs of CTAs, which add their partial tiles up (n: fewer
+    rows than half a tile, one row in a second row of tiles, three rows of tiles).  Two runs on the same workspace are bit-identical."""
+    if which == "deep_output_and_down":
+        sh = wl.LayerShape(d=512, Hq=64, Hkv=8, D=128, rope_base=1.0e6, dtype=torch.bfloat16, m=18944)
+    else:
+        sh = wl.LayerShape(d=8192, Hq=4, Hkv=2, D=64, rope_base=1.0e6, dtype=torch.bfloat16, m=256)
+    H, W, cu = wl.hidden_states(n, sh.d, 51, sh.dtype), _weights(sh, 51), wl.cu_from_lengths([n])
+    if sh.d == 8192:
+        # N(0, 0.02^2) entries over a depth of 8192 give queries and keys of standard deviation 1.8 and scores of 3.3, whose rounding
+        # (half an ulp of q and of k, 2^-9 each) the softmax turns into 5-sigma errors of 2e-2 x RMS; a quarter of it, 0.45 and 0.2,
+        # is what a model's initialisation gives
+        W["Wq"], W["Wk"] = W["Wq"] * 0.25, W["Wk"] * 0.25
+    pos = wl.positions(cu)
+    ref = oc.block_step(H, W, cu, pos, sh, tau=0.0)
+    block = dash.Block(sh, W, DEV, tau=0.0)
+    b = BlockBuffers(block, n, 1)
+    out = []
+    for _ in range(2):
+        x_full = torch.zeros(n, sh.d, dtype=sh.dtype, device=DEV)
+        run_block(block, H.to(DEV), torch.arange(n, dtype=torch.int32, device=DEV), pos.to(DEV), cu.to(DEV), n, x_full, b)
+        out.append((x_full.cpu(), b.r.cpu()))
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+    assert np.max(np.abs(out[0][1].numpy() - ref["r"]) / ref["r"]) < 2e-2
+    assert_close_h1(out[0][0].float().numpy(), ref["H1"], f"H' ({which}, n = {n})")
