@@ -4,7 +4,7 @@
 // head form the (mostly empty) 128-row operand of the tcgen05 MMAs, so K and V tiles stream through
 // shared memory once per KV head; the keys of a sequence are split over persistent CTAs (flash-decoding),
 // whose partial (max, sum, O) results a merge kernel spread over all SMs combines.
-//   plan kernel   : items (sequence, KV head, key-block range), sized so that one item exists per CTA (batches of up to 32 sequences: the CTAs plan for themselves) or four per SM (handed out by ticket)
+//   plan kernel   : items (sequence, KV head, key-block range), sized so that one item exists per CTA (batches of up to 128 sequences: the CTAs plan for themselves) or four per SM (handed out by ticket)
 //   decode kernel : per item  S = Q K_j^T -> masked online softmax (one warp: the rows that exist) -> O += P V_j
 //   merge kernel  : O = sum_i 2^((m_i - m) c) O_i / sum_i 2^((m_i - m) c) l_i
 #include <math.h>
@@ -40,64 +40,65 @@ struct DecParams {
 
 // Batches of up to kSelfPlanSeqs sequences need no plan kernel, no ticket and no scratch clear: every CTA derives the chunk
 // length and its items (item i -> CTA i mod grid; the items are equally long) from cu_seqlens itself, and so does the merge.
-constexpr int kSelfPlanSeqs = 32;
+constexpr int kSelfPlanSeqs = 128;
 __device__ __forceinline__ int dec_blocks(const int32_t* cu, int s) { return (cu[s + 1] - cu[s] + kDecBN - 1) / kDecBN; }
-// The plan of a self-planning launch, built once per CTA in shared memory: thread s fetches sequence s, thread 0 does the few
-// serial steps over at most kSelfPlanSeqs numbers.  (Every thread deriving it on its own from cu_seqlens cost the merge kernel of a
-// 32-sequence batch more than its merging.)
+// The plan of a self-planning launch, built once per CTA in shared memory by its first warp, a lane per sequence (four at most).  With
+// thread 0 going through the sequences one by one, up to nine times, the plan of 24 sequences took 3 us of the decode kernel and
+// again of the merge kernel.
 struct SelfPlan {
-    int nb[kSelfPlanSeqs];        // key blocks of sequence s
-    int first[kSelfPlanSeqs];     // first item of sequence s (its Hkv heads follow each other, `per` items each)
-    int per[kSelfPlanSeqs];       // items per (sequence, KV head)
+    int nb[kSelfPlanSeqs];            // key blocks of sequence s
+    int first[kSelfPlanSeqs + 1];     // first item of sequence s (its Hkv heads follow each other, `per` items each); then the number of items
+    int per[kSelfPlanSeqs];           // items per (sequence, KV head)
     int chunk, n_items;
 };
-__device__ __forceinline__ int self_plan_count(const SelfPlan& sp, int S, int Hkv, int chunk) {
-    int k = 0;
-    for (int s = 0; s < S; ++s) k += ((sp.nb[s] + chunk - 1) / chunk) * Hkv;
-    return k;
-}
 // Called by all threads of the CTA (it synchronises).  `target` is twice the number of CTAs.  Chunk length (key blocks per item):
 // preferred is one item per CTA -- the shortest chunk with at most target / 2 items (the last chunk of every sequence and head is an
 // item of its own, so the first guess can overshoot, and a CTA with a second item would double the kernel's time); half the pipeline
 // ramps and half the partial results to merge.  Taken when it keeps at least 17 of 20 CTAs busy; otherwise about `target` items.
 __device__ __forceinline__ void self_plan_build(SelfPlan& sp, const int32_t* cu, int S, int Hkv, int target) {
-    if ((int)threadIdx.x < S) sp.nb[threadIdx.x] = dec_blocks(cu, (int)threadIdx.x);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        long long all = 0;
-        for (int s = 0; s < S; ++s) all += sp.nb[s];
-        all *= Hkv;
-        long long chunk = (all + target - 1) / target;
-        if (chunk < 1) chunk = 1;
+    if (threadIdx.x < 32) {
+        constexpr int PL = kSelfPlanSeqs / 32;
+        const int lane = threadIdx.x;
+        unsigned int nb[PL], all = 0;
+#pragma unroll
+        for (int j = 0; j < PL; ++j) { const int s = lane + 32 * j; nb[j] = s < S ? (unsigned int)dec_blocks(cu, s) : 0u; all += nb[j]; }
+        all = __reduce_add_sync(0xffffffffu, all) * (unsigned int)Hkv;
+        auto count = [&](unsigned int chunk) {
+            unsigned int k = 0;
+#pragma unroll
+            for (int j = 0; j < PL; ++j)
+                if (32 * j < S) k += (nb[j] + chunk - 1) / chunk;
+            return (int)(__reduce_add_sync(0xffffffffu, k) * (unsigned int)Hkv);
+        };
+        unsigned int chunk = max(1u, (all + (unsigned int)target - 1) / (unsigned int)target);
         const int ctas = target / 2;
-        if (ctas > 0) {
-            long long c1 = (all + ctas - 1) / ctas;
-            if (c1 < 1) c1 = 1;
-            int cnt = self_plan_count(sp, S, Hkv, (int)c1);
-            for (int tries = 0; tries < 8 && cnt > ctas; ++tries) cnt = self_plan_count(sp, S, Hkv, (int)++c1);
-            if (cnt <= ctas && cnt * 20 >= ctas * 17) chunk = c1;
+        unsigned int c1 = max(1u, (all + (unsigned int)ctas - 1) / (unsigned int)ctas);
+        int cnt = count(c1);
+        for (int tries = 0; tries < 8 && cnt > ctas; ++tries) cnt = count(++c1);
+        if (cnt <= ctas && cnt * 20 >= ctas * 17) chunk = c1;
+        int k = 0;                    // items in front of the current group of 32 sequences
+#pragma unroll
+        for (int j = 0; j < PL; ++j) {
+            if (32 * j >= S) break;
+            const int s = lane + 32 * j, per = (int)((nb[j] + chunk - 1) / chunk), mine = per * Hkv;
+            int inc = mine;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) { const int x = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += x; }
+            if (s < S) { sp.nb[s] = (int)nb[j]; sp.per[s] = per; sp.first[s] = k + inc - mine; }
+            k += __shfl_sync(0xffffffffu, inc, 31);
         }
-        int k = 0;
-        for (int s = 0; s < S; ++s) {
-            sp.first[s] = k;
-            sp.per[s] = (sp.nb[s] + (int)chunk - 1) / (int)chunk;
-            k += sp.per[s] * Hkv;
-        }
-        sp.chunk = (int)chunk;
-        sp.n_items = k;
+        if (lane == 0) { sp.chunk = (int)chunk; sp.n_items = k; sp.first[S] = k; }
     }
     __syncthreads();
 }
-__device__ __forceinline__ DecItem self_plan_item(const SelfPlan& sp, int S, int Hkv, int item) {
-    DecItem it = {0, 0, 0, 0};
-    for (int s = 0; s < S; ++s) {
-        const int per = sp.per[s];
-        if (item < sp.first[s] + per * Hkv) {
-            const int r = item - sp.first[s], h = r / per, i = r - h * per;
-            it.s = s; it.kvh = h; it.b0 = i * sp.chunk; it.b1 = min((i + 1) * sp.chunk, sp.nb[s]);
-            return it;
-        }
+__device__ __forceinline__ DecItem self_plan_item(const SelfPlan& sp, int S, int item) {
+    int lo = 0, hi = S;               // first[lo] <= item < first[hi]: the last such lo owns the item (sequences without keys own none)
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (sp.first[mid] <= item) lo = mid; else hi = mid;
     }
+    const unsigned int per = (unsigned int)sp.per[lo], r = (unsigned int)(item - sp.first[lo]), h = r / per, i = r - h * per;
+    DecItem it = {lo, (int)h, (int)i * sp.chunk, min(((int)i + 1) * sp.chunk, sp.nb[lo])};
     return it;
 }
 
@@ -212,7 +213,7 @@ decode_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
         }
         if (item >= n_items || *abort_gen) break;
         tc_fence_after();
-        const DecItem it = self_plan ? self_plan_item(sp, p.S, p.Hkv, item) : p.plan[item];
+        const DecItem it = self_plan ? self_plan_item(sp, p.S, item) : p.plan[item];
         const int seq_a = p.cu[it.s], len = p.cu[it.s + 1] - seq_a;
         const int nblk = it.b1 - it.b0;
         const int last_blk = (len + kDecBN - 1) / kDecBN - 1;       // the block of the sequence with a ragged end
