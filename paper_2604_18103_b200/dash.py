@@ -138,11 +138,13 @@ def _check(status: int, where: str):
 
 
 def _p(t: Optional[torch.Tensor]):
-    return None if t is None else c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()           # ctypes takes an int where the signature says c_void_p
 
 
 def _stream():
-    return c_void_p(torch.cuda.current_stream().cuda_stream)
+    # the handle of torch.cuda.current_stream() without the Stream object around it: a call on a short cache is bound by the host,
+    # and half of its 15 us went into such wrappers
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def dtype_code(t: torch.Tensor) -> int:
@@ -352,7 +354,7 @@ def dash_decode_attention(q: torch.Tensor, Kc: torch.Tensor, Vc: torch.Tensor, c
     """q [S,Hq,D] (one new token per sequence), Kc, Vc [n,Hkv,D] packed caches.  Returns out [S,Hq,D] (and lse [S,Hq])."""
     _dev(q, Kc, Vc, cu_seqlens)
     S, Hq, D = q.shape
-    n, Hkv = Kc.shape[0], Kc.shape[1]
+    n, Hkv = Kc.shape[:2]
     if scale is None:
         scale = 1.0 / (D ** 0.5)
     if out is None:
