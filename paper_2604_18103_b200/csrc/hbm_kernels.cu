@@ -453,6 +453,156 @@ struct TailArgs {
     float* inv_next; float inv_d, rms_eps;     // non-null: 1 / sqrt(mean(row^2) + rms_eps) of every row that goes to H_next, in its order
 };
 
+// Look-back of the fused tail: output base of `tile` from the words of the tiles in front of it (decoupled look-back, called by one warp);
+// agg: rows of this tile that stay.  Publishes this tile's words.
+__device__ __forceinline__ int tail_look_back(unsigned long long* tile_state, int tile, int agg, int* status, int lane) {
+    if (tile == 0) {
+        if (lane == 0) st_state(&tile_state[0], kFlagPrefix | (unsigned int)agg);
+        return 0;
+    }
+    if (lane == 0) st_state(&tile_state[tile], kFlagAgg | (unsigned int)agg);
+    int base = 0, look = tile - 1;
+    bool done = false, timed_out = false;
+    while (!done) {
+        const int j = look - lane;
+        unsigned long long st = kFlagPrefix;
+        uint32_t spins = 0;
+        if (j >= 0) {
+            st = ld_state(&tile_state[j]);
+            while ((st >> 32) == 0) {
+                if (++spins > kSpinLimit) { timed_out = true; break; }
+                __nanosleep(32);
+                st = ld_state(&tile_state[j]);
+            }
+        }
+        if (__any_sync(0xffffffffu, timed_out)) { timed_out = true; break; }
+        const unsigned int has_prefix = __ballot_sync(0xffffffffu, (st >> 32) == 2);
+        const int first = has_prefix ? (__ffs(has_prefix) - 1) : 32;
+        int v = (lane <= first) ? (int)(unsigned int)(st & 0xffffffffu) : 0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        base += v;
+        if (has_prefix) done = true; else look -= 32;
+    }
+    if (timed_out) { if (lane == 0) atomicExch(status, DASH_ERR_TIMEOUT); base = 0; }
+    if (lane == 0) st_state(&tile_state[tile], kFlagPrefix | (unsigned int)(base + agg));
+    return base;
+}
+
+// score and keep decision of a row from its sums of u^2 and h^2
+__device__ __forceinline__ int tail_decide(const TailArgs& a, int64_t row, float su, float sh, int lane) {
+    const float num = sqrtf(su);
+    const float r = (a.mode == DASH_NORM_ABS) ? num : num / fmaxf(sqrtf(sh), a.eps);
+    const int s = find_seq(a.cu_in, a.S, (int)row);
+    const int lp = (int)row - a.cu_in[s], len = a.cu_in[s + 1] - a.cu_in[s];
+    const bool prot = (lp < a.keep_first) || (lp >= len - a.keep_last);
+    const int keep = (prot || !(r < a.tau)) ? 1 : 0;
+    if (lane == 0) { a.r_out[row] = r; a.mask_out[row] = (uint8_t)keep; }
+    return keep;
+}
+
+// The same pass with a row held by its warp from the first load to the last store (rows of up to 32 * NV vectors): tiles of eight rows, a warp
+// each, so that 700 rows are 88 CTAs and not 22, a row's loads go out together (in two halves where there are U and H to add), and what
+// goes on to the next block is written from registers instead of being read back.  Bound by the chain ticket -> rows -> look-back; for
+// inputs whose tiles are all resident.  701 rows of 7 KB took 37 us behind the start of the general kernel's launch, 16 here.
+constexpr int kTailRows = 8;
+template <bool BF16, int NV>
+__global__ void __launch_bounds__(32 * kTailRows, 2)
+delta_tail_rows_kernel(const TailArgs a, int64_t n_upper) {
+    __shared__ int s_keep[kTailRows];
+    __shared__ int s_base, s_count;
+    __shared__ unsigned int s_tile, s_ballot;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    ptx::pdl_wait();                                       // launched to start early: nothing global is touched before the kernel in front is done
+    if (threadIdx.x == 0) s_tile = atomicAdd(a.ticket, 1u);
+    __syncthreads();
+    const int tile = (int)s_tile;
+    int64_t n = a.cu_in[a.S];
+    if (n > n_upper) n = n_upper;
+    const int64_t t_start = (int64_t)tile * kTailRows;
+    if (t_start >= n && tile != 0) return;
+    const int64_t t_end = (t_start + kTailRows < n) ? t_start + kTailRows : n;
+    const bool last_tile = (t_end >= n);
+    const int64_t row = t_start + warp;
+    const bool live = row < n;
+    int keep = 0, tok = 0, pos = 0;
+    float ss = 0.f, su = 0.f, sh = 0.f;                    // ss: sum of squares of the row as it goes on (H~ or H')
+    uint4 z[NV];
+    if (live) {
+        tok = a.tok_in[row];
+        pos = a.pos_in[row];
+        if (a.mask_in) keep = a.mask_in[row] != 0;
+        char* x = a.x_full + (int64_t)tok * a.ldx_b;
+        if (a.U) {
+            const char* u = a.U + row * a.ldU_b;
+            const char* h = a.H + row * a.ldH_b;
+            constexpr int HALF = (NV + 1) / 2;
+#pragma unroll
+            for (int part = 0; part < 2; ++part) {
+                uint4 y[HALF];
+#pragma unroll
+                for (int k = 0; k < HALF; ++k) {
+                    const int i = part * HALF + k, v = i * 32 + lane;
+                    if (i < NV && v < a.nvec) { z[i < NV ? i : 0] = ld_nc_v4(u + ((int64_t)v << 4)); y[k] = ld_nc_v4(h + ((int64_t)v << 4)); }
+                }
+#pragma unroll
+                for (int k = 0; k < HALF; ++k) {
+                    const int i = part * HALF + k, v = i * 32 + lane;
+                    if (i < NV && v < a.nvec) {
+                        uint4& w = z[i < NV ? i : 0];
+                        if (!a.mask_in) { su += sumsq_vec<BF16>(w); sh += sumsq_vec<BF16>(y[k]); }
+                        w = add_vec<BF16>(w, y[k]);
+                        if (a.inv_next) ss += sumsq_vec<BF16>(w);
+                        st_v4(x + ((int64_t)v << 4), w);
+                    }
+                }
+            }
+            if (!a.mask_in) keep = tail_decide(a, row, warp_sum(su), warp_sum(sh), lane);
+        } else {
+            // the row is in x_full already: asked for before its score is known
+#pragma unroll
+            for (int i = 0; i < NV; ++i) { const int v = i * 32 + lane; if (v < a.nvec) z[i] = ld_cg_v4(x + ((int64_t)v << 4)); }
+            if (a.sums) {
+                for (int i = lane; i < a.n_sum_tiles; i += 32) { const float4 p2 = a.sums[row * a.n_sum_tiles + i]; su += p2.x; sh += p2.y; ss += p2.z; }
+                if (!a.mask_in) keep = tail_decide(a, row, warp_sum(su), warp_sum(sh), lane);
+            }
+        }
+    }
+    if (a.inv_next) ss = warp_sum(ss);
+    if (lane == 0) s_keep[warp] = keep;
+    __syncthreads();
+    if (warp == 0) {
+        const unsigned int bal = __ballot_sync(0xffffffffu, lane < kTailRows && s_keep[lane < kTailRows ? lane : 0]);
+        const int agg = __popc(bal), base = tail_look_back(a.tile_state, tile, agg, a.status, lane);
+        if (lane == 0) { s_base = base; s_count = agg; s_ballot = bal; }
+    }
+    __syncthreads();
+    const int base = s_base, count = s_count;
+    const unsigned int bal = s_ballot;
+    if (keep) {
+        const int64_t k = base + __popc(bal & ((1u << warp) - 1u));
+        char* dst = a.H_next + k * a.ldn_b;
+#pragma unroll
+        for (int i = 0; i < NV; ++i) { const int v = i * 32 + lane; if (v < a.nvec) st_v4(dst + ((int64_t)v << 4), z[i]); }
+        if (lane == 0) {
+            a.tok_next[k] = tok;
+            a.pos_next[k] = pos;
+            if (a.inv_next) a.inv_next[k] = rsqrtf(ss * a.inv_d + a.rms_eps);
+        }
+    }
+    for (int s = threadIdx.x; s <= a.S; s += 32 * kTailRows) {
+        int64_t c = a.cu_in[s];
+        if (c > n) c = n;
+        bool mine = (c >= t_start && c < t_end) || (last_tile && c == t_end);
+        if (tile == 0 && n == 0) mine = true;
+        if (mine) {
+            const int v = base + (c >= t_end ? count : __popc(bal & ((1u << (int)(c - t_start)) - 1u)));
+            a.cu_next[s] = v;
+            if (s == a.S && a.n_next) *a.n_next = v;
+        }
+    }
+}
+
 template <bool BF16>
 __global__ void __launch_bounds__(kCompactThreads, 2)
 delta_tail_kernel(const TailArgs a, int64_t n_upper) {
@@ -516,13 +666,7 @@ delta_tail_kernel(const TailArgs a, int64_t n_upper) {
                 }
                 su = warp_sum(su);
                 sh = warp_sum(sh);
-                const float num = sqrtf(su);
-                const float r = (a.mode == DASH_NORM_ABS) ? num : num / fmaxf(sqrtf(sh), a.eps);
-                const int s = find_seq(a.cu_in, a.S, (int)row);
-                const int lp = (int)row - a.cu_in[s], len = a.cu_in[s + 1] - a.cu_in[s];
-                const bool prot = (lp < a.keep_first) || (lp >= len - a.keep_last);
-                keep = (prot || !(r < a.tau)) ? 1 : 0;
-                if (lane == 0) { a.r_out[row] = r; a.mask_out[row] = (uint8_t)keep; }
+                keep = tail_decide(a, row, su, sh, lane);
             }
         }
         if (a.inv_next) ss = warp_sum(ss);
@@ -533,37 +677,7 @@ delta_tail_kernel(const TailArgs a, int64_t n_upper) {
         const int my = s_keep[lane];
         const unsigned int bal = __ballot_sync(0xffffffffu, my);
         const int agg = __popc(bal);
-        int base = 0;
-        if (tile == 0) {
-            if (lane == 0) st_state(&a.tile_state[0], kFlagPrefix | (unsigned int)agg);
-        } else {
-            if (lane == 0) st_state(&a.tile_state[tile], kFlagAgg | (unsigned int)agg);
-            int look = tile - 1;
-            bool done = false, timed_out = false;
-            while (!done) {
-                const int j = look - lane;
-                unsigned long long st = kFlagPrefix;
-                uint32_t spins = 0;
-                if (j >= 0) {
-                    st = ld_state(&a.tile_state[j]);
-                    while ((st >> 32) == 0) {
-                        if (++spins > kSpinLimit) { timed_out = true; break; }
-                        __nanosleep(32);
-                        st = ld_state(&a.tile_state[j]);
-                    }
-                }
-                if (__any_sync(0xffffffffu, timed_out)) { timed_out = true; break; }
-                const unsigned int has_prefix = __ballot_sync(0xffffffffu, (st >> 32) == 2);
-                const int first = has_prefix ? (__ffs(has_prefix) - 1) : 32;
-                int v = (lane <= first) ? (int)(unsigned int)(st & 0xffffffffu) : 0;
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                base += v;
-                if (has_prefix) done = true; else look -= 32;
-            }
-            if (timed_out) { if (lane == 0) atomicExch(a.status, DASH_ERR_TIMEOUT); base = 0; }
-            if (lane == 0) st_state(&a.tile_state[tile], kFlagPrefix | (unsigned int)(base + agg));
-        }
+        const int base = tail_look_back(a.tile_state, tile, agg, a.status, lane);
         if (my) {
             const int k = __popc(bal & ((1u << lane) - 1u));
             const int t = (int)t_start + lane;
@@ -894,15 +1008,15 @@ int launch_sums_to_score(const float4* sums, int n_sum_tiles, int64_t n, dash_no
 // scattered, 16-byte aligned rows.  ws: the compaction workspace (ticket + one state word per 32-token tile); ws_is_clear: the
 // caller has already zeroed its first tail_ws_clear_bytes(n) on this stream (ahead of the kernels in front, so that this launch
 // follows a kernel directly and may start while that one drains).
-size_t tail_ws_clear_bytes(int64_t n) { return 256 + (size_t)((n + 31) / 32 > 0 ? (n + 31) / 32 : 1) * 8; }
+// (tiles of kTailRows rows at the smallest)
+size_t tail_ws_clear_bytes(int64_t n) { return 256 + (size_t)((n + kTailRows - 1) / kTailRows > 0 ? (n + kTailRows - 1) / kTailRows : 1) * 8; }
 int launch_delta_tail(const void* U, const void* H, const uint8_t* mask_in, const float4* sums, int n_sum_tiles, int64_t n, int d, dash_dtype dt, dash_norm_mode mode, float eps, float tau,
                       int keep_first, int keep_last, const int32_t* cu_in, int S, const int32_t* tok_in, const int32_t* pos_in,
                       void* x_full, void* H_next, float* r_out, uint8_t* mask_out, int32_t* tok_next, int32_t* pos_next,
                       int32_t* cu_next, int32_t* n_next, void* ws, size_t ws_bytes, bool ws_is_clear, cudaStream_t st, float* inv_next,
                       float rms_eps) {
     const int es = dt == DASH_BF16 ? 2 : 4;
-    if (!ws || ((uintptr_t)ws % 256) || ws_bytes < compact_ws_bytes(n)) return DASH_ERR_WORKSPACE;
-    const int tiles = (int)((n + 31) / 32) > 0 ? (int)((n + 31) / 32) : 1;
+    if (!ws || ((uintptr_t)ws % 256) || ws_bytes < tail_ws_clear_bytes(n)) return DASH_ERR_WORKSPACE;
     if (!ws_is_clear) DASH_CUDA_TRY(cudaMemsetAsync(ws, 0, tail_ws_clear_bytes(n), st));
     TailArgs a;
     a.mask_in = mask_in; a.sums = sums; a.n_sum_tiles = n_sum_tiles;
@@ -914,6 +1028,18 @@ int launch_delta_tail(const void* U, const void* H, const uint8_t* mask_in, cons
     a.inv_next = inv_next; a.inv_d = 1.0f / (float)d; a.rms_eps = rms_eps;
     a.status = status_word_ptr();
     if (!a.status) return DASH_ERR_CUDA;
+    // a row in a warp's registers: up to 16 vectors (8 KB a row: 4096 columns of bf16) per lane; 4 where that is enough
+    const int nv = (a.nvec + 31) / 32, small = (int)((n + kTailRows - 1) / kTailRows) > 0 ? (int)((n + kTailRows - 1) / kTailRows) : 1;
+    // .. and only while all tiles fit the GPU at once: with more, a tile's registers wait for the look-back chain of up to 1024 others in
+    // front of it (8192 rows: 50 and 98 us against 24 and 45 of the general kernel)
+    if (nv <= 16 && small <= 2 * sm_count()) {
+        if (dt == DASH_BF16 && nv <= 4) DASH_CUDA_TRY(launch_pdl(delta_tail_rows_kernel<true, 4>, small, 32 * kTailRows, 0, st, a, n));
+        else if (dt == DASH_BF16) DASH_CUDA_TRY(launch_pdl(delta_tail_rows_kernel<true, 16>, small, 32 * kTailRows, 0, st, a, n));
+        else if (nv <= 4) DASH_CUDA_TRY(launch_pdl(delta_tail_rows_kernel<false, 4>, small, 32 * kTailRows, 0, st, a, n));
+        else DASH_CUDA_TRY(launch_pdl(delta_tail_rows_kernel<false, 16>, small, 32 * kTailRows, 0, st, a, n));
+        return DASH_OK;
+    }
+    const int tiles = (int)((n + 31) / 32) > 0 ? (int)((n + 31) / 32) : 1;
     if (dt == DASH_BF16) DASH_CUDA_TRY(launch_pdl(delta_tail_kernel<true>, tiles, kCompactThreads, 0, st, a, n));
     else DASH_CUDA_TRY(launch_pdl(delta_tail_kernel<false>, tiles, kCompactThreads, 0, st, a, n));
     return DASH_OK;

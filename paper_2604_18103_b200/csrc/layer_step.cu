@@ -204,6 +204,12 @@ fold_norm_weight_kernel(const char* __restrict__ W, int64_t ldw_b, const char* _
     }
 }
 
+// look-back words of a step's compaction, by dash_compact or by the tail pass
+static size_t step_compact_bytes(int64_t n, int S, dash_dtype dt) {
+    const size_t a = dash_workspace_bytes(DASH_WS_COMPACT, n, S, 0, 0, 0, dt), b = tail_ws_clear_bytes(n);
+    return align_up(a > b ? a : b, 256);
+}
+
 static bool cfg_ok(const dash_layer_cfg* c) {
     if (!c || c->d <= 0 || c->Hq < 1 || c->Hkv < 1 || (c->D != 64 && c->D != 128)) return false;
     if ((c->d % 8) || (c->Hq % c->Hkv)) return false;
@@ -263,7 +269,7 @@ extern "C" int dash_layer_workspace(const dash_layer_cfg* cfg, int64_t n, int S,
         off += conv_w_bytes(cfg->d, (int64_t)nq > cfg->d ? (int64_t)nq : cfg->d) > conv_w_bytes(hd, cfg->d) ? conv_w_bytes(cfg->d, (int64_t)nq > cfg->d ? (int64_t)nq : cfg->d) : conv_w_bytes(hd, cfg->d);
     }
     if (cfg->dt == DASH_BF16) off += gemm_split_part_bytes() + gemm_split_count_bytes();      // tiles of the projections cut along K
-    off += align_up(dash_workspace_bytes(DASH_WS_COMPACT, n, S, 0, 0, 0, cfg->dt), 256);
+    off += step_compact_bytes(n, S, cfg->dt);
     off += align_up(dash_workspace_bytes(DASH_WS_ATTENTION, n, S, cfg->Hq, cfg->Hkv, cfg->D, cfg->dt), 256);
     off += align_up((size_t)n * (cfg->D / 2) * sizeof(float2), 256);              // (cos, sin) of every row for the QKV epilogue
     off += align_up((size_t)n * ((cfg->d + 127) / 128) * sizeof(float4), 256);    // per-row partial sums of the output-projection epilogue
@@ -308,7 +314,7 @@ static int carve_ws(const dash_layer_cfg* cfg, int64_t n, int S, void* ws, StepW
         after += gemm_split_count_bytes();
     }
     out->compact_ws = after;
-    out->compact_bytes = align_up(dash_workspace_bytes(DASH_WS_COMPACT, n, S, 0, 0, 0, cfg->dt), 256);
+    out->compact_bytes = step_compact_bytes(n, S, cfg->dt);
     out->attn_ws = out->compact_ws + out->compact_bytes;
     out->attn_bytes = dash_workspace_bytes(DASH_WS_ATTENTION, n, S, cfg->Hq, cfg->Hkv, cfg->D, cfg->dt);
     out->rope_tab = (float2*)(out->attn_ws + align_up(out->attn_bytes, 256));

@@ -274,3 +274,40 @@ def test_layer_step_rows_beyond_the_packed_end_and_protected_tokens():
     assert np.array_equal(bufs.cu_next.cpu().numpy(), cu_ref)
     if flips == 0:
         assert np.array_equal(mask, ref["mask"])
+
+
+@pytest.mark.parametrize("handover", [False, True], ids=["own_factors", "factors_handed_on"])
+@pytest.mark.parametrize("n", [1, 7, 8, 9, 255, 2368, 2369, 4801])
+def test_layer_step_tail_at_the_edges_of_its_tiles(n, handover):
+    """Row counts around the tail pass's tiles of 8 rows and around the count from which its general form (tiles of 32) takes over: what goes on
+    is exactly the kept rows of x_full in order, with their token and position indices, boundaries and row factors."""
+    sh = wl.MINI
+    lens = [n // 3, 0, n - n // 3]
+    cu = wl.cu_from_lengths(lens)
+    H, pos = wl.hidden_states(n, sh.d, 61, sh.dtype).to(DEV), wl.positions(cu).to(DEV)
+    layer = dash.Layer(sh, wl.layer_weights(sh, 61), DEV, tau=0.0)
+    bufs = StepBuffers(layer, n, 3, n, sh.dtype)
+    g = torch.Generator().manual_seed(n)
+    tok = torch.randperm(n, generator=g).to(torch.int32).to(DEV)
+    table = dash.dash_rope_table(sh.rope_base, sh.D, n, DEV)
+    inv = torch.zeros(n, dtype=torch.float32, device=DEV)
+    if handover:
+        layer.set_handover(table, None, inv)
+    x_full = torch.zeros(n, sh.d, dtype=sh.dtype, device=DEV)
+    run_step(layer, H, tok, pos, cu.to(DEV), max(lens), x_full, bufs)
+    assert int(bufs.n_next.item()) == n and bufs.mask.all() and torch.equal(bufs.H_next, x_full[tok.long()])
+    r = bufs.r.cpu().numpy()
+    layer.set_tau(float(np.median(r)))
+    run_step(layer, H, tok, pos, cu.to(DEV), max(lens), x_full, bufs)
+    assert np.array_equal(bufs.r.cpu().numpy(), r)
+    mask = (~(r < np.float32(layer.cfg.tau))).astype(np.uint8)
+    assert np.array_equal(bufs.mask.cpu().numpy(), mask)
+    idx = torch.from_numpy(np.flatnonzero(mask)).to(DEV)
+    k = idx.numel()
+    assert int(bufs.n_next.item()) == k
+    assert torch.equal(bufs.H_next[:k], x_full[tok.long()][idx]) and torch.equal(bufs.tok_next[:k], tok[idx]) and torch.equal(bufs.pos_next[:k], pos[idx])
+    assert bufs.cu_next.tolist() == [0, int(mask[:lens[0]].sum()), int(mask[:lens[0]].sum()), k]
+    if handover:
+        # fp32 sums of squares of the values before their rounding to bf16 (relative 2^-9 each, averaged over a row of 512)
+        ref = torch.rsqrt(bufs.H_next[:k].double().square().mean(1) + sh.rms_eps)
+        assert ((inv[:k].double() - ref).abs() / ref).max() < 2e-3
