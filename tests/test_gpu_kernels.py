@@ -477,3 +477,25 @@ def test_attention_random_packed_batches_match_oracle_on_sampled_rows():
         D = 128 if trial % 2 else 64
         rows = wl.sample_rows(wl.cu_from_lengths(lengths), 60, seed=trial)
         _attention_case(lengths, Hq, Hkv, D, torch.bfloat16, 100 + trial, rows=rows.numpy(), pad=trial)
+
+
+@pytest.mark.parametrize("n", [2, 1023, 1024, 1025, 5000, 10239, 10240, 10241, 50000])
+@pytest.mark.parametrize("kind", ["scores", "few_values", "wide_with_nan_and_zeros"])
+def test_select_keep_count_at_the_edges_of_its_key_cache(n, kind):
+    """Counts per sequence around the 1024 threads and around the 10240 keys held in shared memory, with ties at the cut that stay, that are cut, and
+    scores over the whole range of fp32; the selection equals the oracle's exactly."""
+    g = torch.Generator().manual_seed(n)
+    if kind == "scores":
+        r = torch.rand(n, generator=g) * 0.1 + 0.05
+    elif kind == "few_values":
+        r = torch.randint(0, 5, (n,), generator=g).float()
+    else:
+        r = torch.randn(n, generator=g) * torch.exp(20 * torch.randn(n, generator=g))
+        r[::7], r[3::11] = 0.0, -0.0
+        r[n // 2] = float("nan")
+    cu = wl.cu_from_lengths([n])
+    for k in sorted({1, n // 3, n // 2, n - 1}):
+        for mode, high in ((dash.SEL_KEEP_COUNT, False), (dash.SEL_KEEP_COUNT_HALT_HIGH, True)):
+            m = dash.dash_select(r.to(DEV), cu.to(DEV), mode, keep_counts=torch.tensor([k], dtype=torch.int32, device=DEV))
+            ref = oc.select(r.numpy(), cu, oc.KEEP_COUNT, keep_counts=[k], halt_high=high)
+            assert np.array_equal(m.cpu().numpy(), ref), (n, kind, k, high)
