@@ -464,8 +464,8 @@ extern "C" int dash_layer_step(const dash_layer_cfg* cfg, const void* H_in, cons
         if (!aligned16(H_in) || !aligned16(x_full) || !aligned16(H_next) || !aligned16(cfg->Wqkv) || !aligned16(cfg->Wo) ||
             (cfg->rms_weight && !aligned16(cfg->rms_weight)))
             return DASH_ERR_INVALID_ARG;
-        const bool tail_pass = cfg->sel_mode == DASH_SEL_THRESHOLD && cfg->scatter_which == 2;
-        if ((rc = clear_step_words(W, n, tail_pass, st)) != DASH_OK) return rc;
+        const bool every_row = cfg->scatter_which == 2, tail_pass = cfg->sel_mode == DASH_SEL_THRESHOLD && every_row;
+        if ((rc = clear_step_words(W, n, every_row, st)) != DASH_OK) return rc;
         if ((rc = attention_to_O(cfg, H_in, pos_in, cu_in, S, n, max_seqlen, W, st)) != DASH_OK) return rc;
         if (tail_pass) {
             // output projection with H~ = H + U written straight to x_full and the row sums of u^2, h^2 beside it; then the score, the
@@ -484,6 +484,18 @@ extern "C" int dash_layer_step(const dash_layer_cfg* cfg, const void* H_in, cons
                                      pos_next, cu_next, n_next_dev, W.compact_ws, W.compact_bytes, true, st, nullptr, cfg->rms_eps);
         }
         if (cfg->inv_rms_next) return DASH_ERR_UNSUPPORTED;      // the row factors come out of the fused tail pass (threshold rule, every row scattered)
+        if (every_row && x_full != H_in &&      // (H~ over H itself in another order: only once every row of H has been read)
+            (rc = out_proj_residual(cfg, H_in, tok_index_in, x_full, cu_in, S, n, W, st)) != DASH_ERR_UNSUPPORTED) {
+            // the other rules, every row's H~ in x_full: the score from the projection's row sums, the rule on the scores, then the tail pass
+            // moves the rows that stay.  (U stored, a score pass over U and H, a scatter and a compaction took 110 us where this
+            // takes 35: 12 345 rows of 7 KB.)
+            if (rc != DASH_OK) return rc;
+            if ((rc = launch_sums_to_score(W.sums, d / 128, n, cfg->norm_mode, cfg->norm_eps, r_out, nullptr, cu_in + S, nullptr, d, cfg->rms_eps, st)) != DASH_OK) return rc;
+            if ((rc = dash_select(r_out, n, cu_in, S, cfg->sel_mode, cfg->tau, cfg->keep_counts, cfg->keep_first, cfg->keep_last, mask_out, st)) != DASH_OK) return rc;
+            return launch_delta_tail(nullptr, nullptr, mask_out, nullptr, 0, n, d, cfg->dt, cfg->norm_mode, cfg->norm_eps, cfg->tau, cfg->keep_first,
+                                     cfg->keep_last, cu_in, S, tok_index_in, pos_in, x_full, H_next, nullptr, nullptr, tok_index_next,
+                                     pos_next, cu_next, n_next_dev, W.compact_ws, W.compact_bytes, true, st, nullptr, cfg->rms_eps);
+        }
         if ((rc = out_proj_U(cfg, cu_in, S, n, W, st)) != DASH_OK) return rc;
         if ((rc = score_and_select(cfg, H_in, cu_in, S, n, r_out, mask_out, W, st)) != DASH_OK) return rc;
         // updated states reach the full-length output (halted tokens stay frozen there from now on)

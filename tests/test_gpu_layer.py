@@ -311,3 +311,33 @@ def test_layer_step_tail_at_the_edges_of_its_tiles(n, handover):
         # fp32 sums of squares of the values before their rounding to bf16 (relative 2^-9 each, averaged over a row of 512)
         ref = torch.rsqrt(bufs.H_next[:k].double().square().mean(1) + sh.rms_eps)
         assert ((inv[:k].double() - ref).abs() / ref).max() < 2e-3
+
+
+@pytest.mark.parametrize("mode", [dash.SEL_KEEP_COUNT, dash.SEL_KEEP_COUNT_HALT_HIGH, dash.SEL_THRESHOLD_HALT_HIGH])
+@pytest.mark.parametrize("n", [1, 129, 700, 2500])
+def test_layer_step_other_rules_with_every_row_written(mode, n):
+    """The rules beside the threshold with every row scattered: score and H~ from the output projection's accumulators, then the rule, then the
+    tail pass.  Decisions equal the oracle's on the step's own scores; scores and H~ match the oracle; indices are exact."""
+    sh = wl.MINI
+    lens = [n // 4, 0, n - n // 4]
+    cu = wl.cu_from_lengths(lens)
+    H, W, pos = wl.hidden_states(n, sh.d, 71, sh.dtype), wl.layer_weights(sh, 71), wl.positions(cu)
+    Ks = [oc.keep_count(x, 0.5, 16, 8, mode=1) for x in lens]
+    layer = dash.Layer(sh, W, DEV, sel_mode=mode, keep_counts=torch.tensor(Ks, dtype=torch.int32, device=DEV), keep_first=16, keep_last=8, tau=0.3)
+    bufs = StepBuffers(layer, n, 3, n, sh.dtype)
+    tok = torch.randperm(n, generator=torch.Generator().manual_seed(n)).to(torch.int32)
+    x_full = torch.zeros(n, sh.d, dtype=sh.dtype, device=DEV)
+    run_step(layer, H.to(DEV), tok.to(DEV), pos.to(DEV), cu.to(DEV), max(lens), x_full, bufs)
+    ref = oc.layer_step(H, W, cu, pos, sh, tau=0.0)
+    r, mask = bufs.r.cpu().numpy(), bufs.mask.cpu().numpy()
+    assert np.max(np.abs(r - ref["r"]) / ref["r"]) < 2e-2
+    base = oc.THRESHOLD if mode == dash.SEL_THRESHOLD_HALT_HIGH else oc.KEEP_COUNT
+    assert np.array_equal(mask, oc.select(r, cu, base, tau=0.3, keep_counts=Ks, keep_first=16, keep_last=8, halt_high=mode != dash.SEL_KEEP_COUNT))
+    xf = x_full.cpu()[tok.long()]
+    assert_close_rms(xf.float().numpy(), ref["Ht"], "H~")
+    idx = np.flatnonzero(mask)
+    k = int(bufs.n_next.item())
+    assert k == idx.size and torch.equal(bufs.H_next[:k].cpu(), xf[idx])
+    assert np.array_equal(bufs.tok_next[:k].cpu().numpy(), tok.numpy()[idx]) and np.array_equal(bufs.pos_next[:k].cpu().numpy(), pos.numpy()[idx])
+    a = int(mask[:lens[0]].sum())
+    assert bufs.cu_next.tolist() == [0, a, a, k]
