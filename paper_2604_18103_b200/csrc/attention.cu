@@ -21,6 +21,7 @@
 #include <math.h>
 
 #include "common.cuh"
+#include "prologue.cuh"
 #include "sm100_ptx.cuh"
 
 namespace dash {
@@ -80,6 +81,7 @@ struct AttnParams {
     float scale;
     void* O;
     int64_t ldo;            // elements
+    __nv_bfloat16* O16;     // OUT_F32: a bf16 copy of O as well ([n, Hq, D]), or null
     float* lse;             // [Hq, n] or null
     int64_t n;
     int* status;
@@ -90,55 +92,12 @@ struct AttnParams {
     int kv_packed;              // GATHER: K and V are packed already ([n, Hkv, D], tiled loads); only Q is fetched by index
 };
 
-// ---- plan: which (sequence, query tile) pairs exist, ordered by falling number of key blocks ----
+// ---- plan kernel of a call that is not part of a block step ----
 __global__ void __launch_bounds__(1024)
 attention_plan_kernel(const int32_t* __restrict__ cu, int S, int Hq, int4* __restrict__ plan, int* __restrict__ n_items,
                       unsigned int* __restrict__ ticket, int64_t max_entries) {
-    __shared__ int s_warp[33];
-    __shared__ int s_max;
-    const int tid = threadIdx.x;
     pdl_launch_dependents();
-    if (tid == 0) s_max = 0;
-    __syncthreads();
-    int mx = 0;
-    for (int s = tid; s < S; s += blockDim.x) mx = max(mx, (cu[s + 1] - cu[s] + kBM - 1) / kBM);
-    atomicMax(&s_max, mx);
-    __syncthreads();
-    const int max_nq = s_max;
-    int64_t offset = 0;
-    for (int top = max_nq - 1; top >= 0; top -= (int)blockDim.x) {
-        const int qt = top - tid;                           // thread 0 takes the heaviest level of this chunk
-        int cnt = 0;
-        if (qt >= 0)
-            for (int s = 0; s < S; ++s) cnt += ((cu[s + 1] - cu[s] + kBM - 1) / kBM > qt);
-        // exclusive scan over the block
-        const int lane = tid & 31, w = tid >> 5;
-        int inc = cnt;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) { int t = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += t; }
-        if (lane == 31) s_warp[w] = inc;
-        __syncthreads();
-        if (w == 0) {
-            int x = s_warp[lane], xi = x;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) { int t = __shfl_up_sync(0xffffffffu, xi, o); if (lane >= o) xi += t; }
-            s_warp[lane] = xi - x;
-            if (lane == 31) s_warp[32] = xi;
-        }
-        __syncthreads();
-        int64_t k = offset + s_warp[w] + inc - cnt;
-        const int chunk_total = s_warp[32];
-        if (qt >= 0)
-            for (int s = 0; s < S; ++s)
-                if ((cu[s + 1] - cu[s] + kBM - 1) / kBM > qt) { if (k < max_entries) plan[k] = make_int4(s, qt, cu[s], cu[s + 1]); ++k; }
-        offset += chunk_total;
-        __syncthreads();
-    }
-    if (tid == 0) {
-        if (offset > max_entries) offset = max_entries;     // cannot happen for cu_seqlens[S] <= n; keeps every read in bounds
-        *n_items = (int)(offset * Hq);
-        *ticket = 0u;
-    }
+    attention_plan_items<1024>(cu, S, Hq, plan, n_items, ticket, max_entries);
 }
 
 template <int D>
@@ -490,6 +449,9 @@ attention_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
                             v.x = __float_as_uint(__uint_as_float(o[e]) * inv); v.y = __float_as_uint(__uint_as_float(o[e + 1]) * inv);
                             v.z = __float_as_uint(__uint_as_float(o[e + 2]) * inv); v.w = __float_as_uint(__uint_as_float(o[e + 3]) * inv);
                             st_v4(dst + e, v);
+                            if (p.O16)
+                                *reinterpret_cast<uint2*>(p.O16 + (grow * p.Hq + h) * D + c * 32 + e) =
+                                    make_uint2(pack_bf16(__uint_as_float(v.x), __uint_as_float(v.y)), pack_bf16(__uint_as_float(v.z), __uint_as_float(v.w)));
                         }
                     } else {
                         __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(p.O) + grow * p.ldo + (int64_t)h * D + c * 32;
@@ -564,9 +526,8 @@ static int launch_attention(const CUtensorMap& mq, const CUtensorMap& mk, const 
     return launch_pdl(attention_kernel<D, OUT_F32, GATHER>, grid, kAttnThreads, (size_t)smem, st, mq, mk, mv, p) == cudaSuccess ? DASH_OK : DASH_ERR_CUDA;
 }
 
-// The item list of a call (see attention_plan_kernel) into the head of its workspace.  A caller that knows cu_seqlens early
-// launches it ahead of the work that produces Q, K, V and then calls attention_planned().
-int attention_plan(const int32_t* cu_seqlens, int S, int64_t n, int Hq, void* ws, size_t ws_bytes, cudaStream_t st) {
+// The item list of a call (see attention_plan_items) into the head of its workspace
+static int attention_plan(const int32_t* cu_seqlens, int S, int64_t n, int Hq, void* ws, size_t ws_bytes, cudaStream_t st) {
     if (!cu_seqlens || S < 1 || n < 0 || n > 0x7fffffffLL || Hq < 1) return DASH_ERR_INVALID_ARG;
     if (n == 0) return DASH_OK;
     if (!ws || ((uintptr_t)ws % 256) || ws_bytes < 256 + plan_bytes(n, S)) return DASH_ERR_WORKSPACE;
@@ -581,7 +542,7 @@ static int attention_impl(const void* Q, const void* K, const void* V, void* O, 
                           const int32_t* cu_seqlens, int S, int64_t n, int64_t max_seqlen,
                           int Hq, int Hkv, int D, float scale, int causal, dash_dtype dt,
                           void* ws, size_t ws_bytes, void* stream, bool planned, const int32_t* idx = nullptr, int64_t n_full = 0,
-                          bool kv_packed = false) {
+                          bool kv_packed = false, void* O16 = nullptr) {
     if (n < 0 || S < 1 || max_seqlen < 0 || Hq < 1 || Hkv < 1 || !cu_seqlens) return DASH_ERR_INVALID_ARG;
     if (dt != DASH_F32 && dt != DASH_BF16) return DASH_ERR_INVALID_ARG;
     if (D != 64 && D != 128) return DASH_ERR_UNSUPPORTED;
@@ -605,6 +566,7 @@ static int attention_impl(const void* Q, const void* K, const void* V, void* O, 
         __nv_bfloat16* qb = (__nv_bfloat16*)((char*)ws + 256 + plan_bytes(n, S));
         __nv_bfloat16* kb = qb + (size_t)n * Hq * D;
         __nv_bfloat16* vb = kb + (size_t)n * Hkv * D;
+        if (!planned) {                          // (a planned call finds its copies there: the step's rotary pass wrote them)
         const int cap = sm_count() * 8;
         auto cvt = [&](const void* src, int64_t ld, __nv_bfloat16* dst, int cols) {
             int64_t total = n * (cols / 4);
@@ -614,6 +576,7 @@ static int attention_impl(const void* Q, const void* K, const void* V, void* O, 
         };
         cvt(Q, ldq, qb, Hq * D); cvt(K, ldk, kb, Hkv * D); cvt(V, ldv, vb, Hkv * D);
         DASH_CUDA_TRY(cudaGetLastError());
+        }
         q = qb; k = kb; v = vb;
         lq = (int64_t)Hq * D; lk = lv = (int64_t)Hkv * D;
     }
@@ -639,7 +602,7 @@ static int attention_impl(const void* Q, const void* K, const void* V, void* O, 
     p.n_qtiles = (int)((max_seqlen + kBM - 1) / kBM);
     p.scale = scale;
     p.scale_log2 = scale * 1.4426950408889634f;
-    p.O = O; p.ldo = ldo; p.lse = lse; p.n = n; p.idx = idx; p.kv_packed = kv_packed ? 1 : 0;
+    p.O = O; p.ldo = ldo; p.O16 = (__nv_bfloat16*)O16; p.lse = lse; p.n = n; p.idx = idx; p.kv_packed = kv_packed ? 1 : 0;
     p.status = status_word_ptr();
     if (!p.status) return DASH_ERR_CUDA;
     p.ticket = (unsigned int*)ws;
@@ -655,11 +618,28 @@ static int attention_impl(const void* Q, const void* K, const void* V, void* O, 
     return dt == DASH_F32 ? launch_attention<64, true, false>(mq, mk, mv, p, grid, st) : launch_attention<64, false, false>(mq, mk, mv, p, grid, st);
 }
 
-// same as dash_varlen_attention for a workspace whose item list attention_plan() has already been asked for on this stream
+int attention_plan_ws(int S, int64_t n, int Hq, int Hkv, int D, dash_dtype dt, void* ws, size_t ws_bytes, AttnPlanWs* out) {
+    if (!ws || ((uintptr_t)ws % 256) || ws_bytes < attention_ws_bytes(n, S, Hq, Hkv, D, dt)) return DASH_ERR_WORKSPACE;
+    if ((int64_t)plan_entries(n, S) * Hq > 0x7fffffffLL) return DASH_ERR_UNSUPPORTED;
+    char* w = (char*)ws;
+    out->ticket = (unsigned int*)w; out->n_items = (int*)(w + 4); out->plan = (int4*)(w + 256);
+    out->max_entries = (int64_t)plan_entries(n, S);
+    out->q = out->k = out->v = nullptr;
+    if (dt == DASH_F32) {
+        out->q = (__nv_bfloat16*)(w + 256 + plan_bytes(n, S));
+        out->k = out->q + (size_t)n * Hq * D;
+        out->v = out->k + (size_t)n * Hkv * D;
+    }
+    return DASH_OK;
+}
+
+// same as dash_varlen_attention for a workspace whose item list (and copies) a kernel in front on this stream has filled in; O16: fp32
+// tensors, a bf16 copy of O as well
 int attention_planned(const void* Q, const void* K, const void* V, void* O, float* lse, int64_t ldq, int64_t ldk, int64_t ldv, int64_t ldo,
                       const int32_t* cu_seqlens, int S, int64_t n, int64_t max_seqlen, int Hq, int Hkv, int D, float scale, dash_dtype dt,
-                      void* ws, size_t ws_bytes, cudaStream_t st) {
-    return attention_impl(Q, K, V, O, lse, ldq, ldk, ldv, ldo, cu_seqlens, S, n, max_seqlen, Hq, Hkv, D, scale, 1, dt, ws, ws_bytes, (void*)st, true);
+                      void* ws, size_t ws_bytes, cudaStream_t st, void* O16) {
+    return attention_impl(Q, K, V, O, lse, ldq, ldk, ldv, ldo, cu_seqlens, S, n, max_seqlen, Hq, Hkv, D, scale, 1, dt, ws, ws_bytes, (void*)st, true,
+                          nullptr, 0, false, O16);
 }
 
 }  // namespace dash

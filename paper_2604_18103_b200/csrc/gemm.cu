@@ -25,6 +25,7 @@
 
 #include "common.cuh"
 #include "gemm.cuh"
+#include "prologue.cuh"
 #include "sm100_ptx.cuh"
 
 namespace dash {
@@ -592,50 +593,12 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
     }
 }
 
-// Per row (one warp): (cos, sin) of pos[t] * base^(-2i/D) for i < D/2, angles formed and reduced in fp64 (positions reach 1e5 rad
-// at i = 0: fp32 would lose the angle), evaluated in fp32 on the reduced angle; and, when asked, the row factor of the RMSNorm, 1 / sqrt(mean(h^2) + eps), from one pass over the bf16 row
-struct RopeFreqs { double inv_freq[64]; };
 __global__ void __launch_bounds__(256)
 row_prep_kernel(const int32_t* __restrict__ pos, int64_t n, int half, RopeFreqs fr, float2* __restrict__ table, const char* __restrict__ H,
                 int64_t ldh_b, int nvec, float inv_d, float eps, float* __restrict__ inv_rms, const int32_t* __restrict__ n_dev) {
     pdl_launch_dependents();
-    if (n_dev) { int64_t nd = *n_dev; if (nd < n) n = nd; }
-    const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
-    for (int64_t t = (int64_t)blockIdx.x * wpb + (threadIdx.x >> 5); t < n; t += (int64_t)gridDim.x * wpb) {
-        float ss = 0.f;
-        if (inv_rms) {
-            const char* h = H + t * ldh_b;
-            for (int base = 0; base < nvec; base += 128) {
-                uint4 x[4];
-#pragma unroll
-                for (int k = 0; k < 4; ++k) { const int v = base + k * 32 + lane; if (v < nvec) x[k] = ld_nc_v4(h + ((int64_t)v << 4)); }
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int v = base + k * 32 + lane;
-                    if (v < nvec) {
-                        const float f[8] = {bf16lo(x[k].x), bf16hi(x[k].x), bf16lo(x[k].y), bf16hi(x[k].y), bf16lo(x[k].z), bf16hi(x[k].z), bf16lo(x[k].w), bf16hi(x[k].w)};
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) ss += f[e] * f[e];
-                    }
-                }
-            }
-        }
-        if (table) {
-            const double ps = pos ? (double)pos[t] : (double)t;
-            for (int i = lane; i < half; i += 32) {
-                // angle formed and reduced to [-pi, pi] in fp64 (three operations), sine and cosine of the reduced angle in fp32
-                const double ang = ps * fr.inv_freq[i];
-                const double red = fma(-6.283185307179586476925286766559, rint(ang * 0.15915494309189533576888376337251), ang);
-                float sn, cs;
-                sincosf((float)red, &sn, &cs);
-                table[t * half + i] = make_float2(cs, sn);
-            }
-        }
-        if (inv_rms) {
-            ss = warp_sum(ss);
-            if (lane == 0) inv_rms[t] = rsqrtf(ss * inv_d + eps);
-        }
-    }
+    const int wpb = blockDim.x >> 5;
+    row_prep_rows(pos, n, half, fr, table, H, ldh_b, nvec, inv_d, eps, inv_rms, n_dev, (int64_t)blockIdx.x * wpb + (threadIdx.x >> 5), (int64_t)gridDim.x * wpb);
 }
 
 static int make_map_2d_bf16(CUtensorMap* map, const void* basep, uint64_t inner, uint64_t outer, uint64_t ld_elems, uint32_t box_inner,
@@ -720,18 +683,12 @@ int gemm_bf16(GemmEpilogueKind kind, const void* A, int64_t lda, const void* W, 
 }
 
 int launch_row_prep(const int32_t* pos, int64_t n, int D, double rope_base, float2* table, const void* H, int64_t ldh, int d, float rms_eps,
-                    float* inv_rms, const int32_t* n_dev, cudaStream_t st, bool beside_front) {
+                    float* inv_rms, const int32_t* n_dev, cudaStream_t st) {
     RopeFreqs fr;
     for (int i = 0; i < D / 2; ++i) fr.inv_freq[i] = pow(rope_base, -2.0 * i / D);
     int64_t blocks = (n + 7) / 8, cap = (int64_t)sm_count() * 8;
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
-    // beside_front: the kernel in front in the stream is one whose output this kernel does not read and that was itself an ordinary
-    // launch (the block step's attention item list): launched to start beside it -- the kernel has no griddepcontrol.wait, and its
-    // inputs were complete before the kernel in front started.
-    if (beside_front)
-        return launch_pdl(row_prep_kernel, (int)blocks, 256, 0, st, pos, n, D / 2, fr, table, (const char*)H, ldh * 2, d * 2 / 16, 1.0f / d,
-                          rms_eps, inv_rms, n_dev) == cudaSuccess ? DASH_OK : DASH_ERR_CUDA;
     row_prep_kernel<<<(int)blocks, 256, 0, st>>>(pos, n, D / 2, fr, table, (const char*)H, ldh * 2, d * 2 / 16, 1.0f / d, rms_eps, inv_rms, n_dev);
     return cudaGetLastError() == cudaSuccess ? DASH_OK : DASH_ERR_CUDA;
 }

@@ -9,6 +9,8 @@
 
 #include "common.cuh"
 #include "gemm.cuh"
+#include "prologue.cuh"
+#include "sm100_ptx.cuh"
 
 namespace dash {
 
@@ -59,12 +61,13 @@ rmsnorm_kernel(const char* __restrict__ X, int64_t ldx_b, const char* __restrict
 // Rotary embedding in place on the first `heads` heads of every row of the fused
 // QKV buffer: pair (i, i + D/2) rotated by pos * inv_freq[i].  One warp per token;
 // the angles are formed and reduced in fp64 (positions reach 1e5 rad at i = 0).
-struct RopeFreq { double inv_freq[64]; };
+// fp32: the bf16 copies of Q, K and V that the attention kernel reads ([n, heads, D] each) are written beside it.
+struct AttnCopies { __nv_bfloat16 *q, *k, *v; int Hq, Hkv; };
 
 template <bool BF16, int D>
 __global__ void __launch_bounds__(256)
-rope_kernel(char* __restrict__ X, int64_t ldx_b, const int32_t* __restrict__ pos, int64_t n, int heads, RopeFreq fr,
-            const int32_t* __restrict__ n_dev) {
+rope_kernel(char* __restrict__ X, int64_t ldx_b, const int32_t* __restrict__ pos, int64_t n, int heads, RopeFreqs fr,
+            const int32_t* __restrict__ n_dev, AttnCopies cp) {
     constexpr int HALF = D / 2;
     __shared__ float s_cos[8][HALF], s_sin[8][HALF];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, wpb = blockDim.x >> 5;
@@ -104,8 +107,18 @@ rope_kernel(char* __restrict__ X, int64_t ldx_b, const int32_t* __restrict__ pos
                 for (int e = 0; e < 4; ++e) { y1[e] = x1[e] * c[e] - x2[e] * s[e]; y2[e] = x2[e] * c[e] + x1[e] * s[e]; }
                 oa = make_uint4(__float_as_uint(y1[0]), __float_as_uint(y1[1]), __float_as_uint(y1[2]), __float_as_uint(y1[3]));
                 ob = make_uint4(__float_as_uint(y2[0]), __float_as_uint(y2[1]), __float_as_uint(y2[2]), __float_as_uint(y2[3]));
+                __nv_bfloat16* c16 = (hd < cp.Hq ? cp.q + (t * cp.Hq + hd) * D : cp.k + (t * cp.Hkv + hd - cp.Hq) * D) + v * EPV;
+                *reinterpret_cast<uint2*>(c16) = make_uint2(pack_bf16(y1[0], y1[1]), pack_bf16(y1[2], y1[3]));
+                *reinterpret_cast<uint2*>(c16 + HALF) = make_uint2(pack_bf16(y2[0], y2[1]), pack_bf16(y2[2], y2[3]));
             }
             *p1 = oa; *p2 = ob;
+        }
+        if (!BF16) {
+            const uint4* pv = reinterpret_cast<const uint4*>(row + (int64_t)heads * D * ES);
+            for (int q = lane; q < cp.Hkv * D / 4; q += 32) {
+                const uint4 a = pv[q];
+                *reinterpret_cast<uint2*>(cp.v + t * cp.Hkv * D + q * 4) = make_uint2(pack_bf16(__uint_as_float(a.x), __uint_as_float(a.y)), pack_bf16(__uint_as_float(a.z), __uint_as_float(a.w)));
+            }
         }
         __syncwarp();
     }
@@ -119,13 +132,12 @@ int launch_delta_tail(const void* U, const void* H, const uint8_t* mask_in, cons
                       int32_t* cu_next, int32_t* n_next, void* ws, size_t ws_bytes, bool ws_is_clear, cudaStream_t st, float* inv_next,
                       float rms_eps);
 size_t tail_ws_clear_bytes(int64_t n);
-int attention_plan(const int32_t* cu_seqlens, int S, int64_t n, int Hq, void* ws, size_t ws_bytes, cudaStream_t st);
 int attention_planned(const void* Q, const void* K, const void* V, void* O, float* lse, int64_t ldq, int64_t ldk, int64_t ldv, int64_t ldo,
                       const int32_t* cu_seqlens, int S, int64_t n, int64_t max_seqlen, int Hq, int Hkv, int D, float scale, dash_dtype dt,
-                      void* ws, size_t ws_bytes, cudaStream_t st);
+                      void* ws, size_t ws_bytes, cudaStream_t st, void* O16 = nullptr);
 
 // Room for the bf16 copies of the operands of a projection on fp32 tensors
-struct ConvScratch { char* a; size_t a_bytes; char* w; size_t w_bytes; };
+struct ConvScratch { char* a; size_t a_bytes; char* w; size_t w_bytes; char* w2 = nullptr; };
 static size_t conv_a_bytes(int64_t n, int64_t k_max) { return align_up((size_t)n * align_up((size_t)k_max, 8) * 2, 256); }
 static size_t conv_w_bytes(int64_t k, int64_t n_cols) { return align_up((size_t)k * align_up((size_t)n_cols, 8) * 2, 256); }
 
@@ -142,6 +154,66 @@ static int project(dash_dtype dt, const void* A, int64_t lda, const void* W, int
     if ((rc = launch_f32_to_bf16((const float*)A, lda, cs.a, lda_b, n, K, st)) != DASH_OK) return rc;
     if ((rc = launch_f32_to_bf16((const float*)W, ldw, cs.w, ldw_b, K, N, st)) != DASH_OK) return rc;
     return gemm_bf16(GEMM_PLAIN, cs.a, lda_b, cs.w, ldw_b, C, ldc, n, N, K, e, n_dev, st, true);
+}
+
+// Everything of a step that waits for nothing in it, in one launch: the attention kernel's item list (first CTA), the words that have to
+// be zero (second), then, shared out over the other CTAs, the rows (their norm factors and rotary angles; fp32: the normalised rows
+// rounded to bf16) and, fp32, the bf16 copies of the two weight matrices.  As launches of their own these were a memset and two
+// kernels per step, and eight more in front of and between the projections of an fp32 layer: 2 to 4 us each, for a microsecond of work.
+struct PrologueArgs {
+    const int32_t* cu; int S, Hq;
+    AttnPlanWs ap;
+    uint4* zero; int n_zero;                 // 16-byte vectors
+    int64_t n; const int32_t* n_dev; const char* H; int64_t ldh_b; int nvec; float inv_d, eps;
+    int row_ctas;
+    // bf16: see row_prep_rows (table and inv_rms null: no rows)
+    const int32_t* pos; int half; float2* table; float* inv_rms;
+    // fp32: Hn16 [n, d] = bf16 of the RMSNorm of H
+    const float* rms_w; __nv_bfloat16* Hn16;
+    const float4 *w0, *w1; uint2 *w0_16, *w1_16; int64_t n_w0, n_w1;      // contiguous matrices, in vectors of four
+};
+__global__ void __launch_bounds__(256)
+prologue_kernel(const PrologueArgs a, const RopeFreqs fr) {
+    ptx::pdl_wait();                         // launched to get onto the SMs while the kernel in front drains
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int cta = (int)blockIdx.x;
+    if (cta == 0) {
+        attention_plan_items<256>(a.cu, a.S, a.Hq, a.ap.plan, a.ap.n_items, a.ap.ticket, a.ap.max_entries);
+        return;
+    }
+    if (cta == 1) {
+        for (int i = threadIdx.x; i < a.n_zero; i += 256) a.zero[i] = make_uint4(0, 0, 0, 0);
+        return;
+    }
+    cta -= 2;
+    if (cta < a.row_ctas) {
+        if (!a.Hn16) {
+            row_prep_rows(a.pos, a.n, a.half, fr, a.table, a.H, a.ldh_b, a.nvec, a.inv_d, a.eps, a.inv_rms, a.n_dev, (int64_t)cta * 8 + warp, (int64_t)a.row_ctas * 8);
+            return;
+        }
+        int64_t n = a.n;
+        if (a.n_dev) { const int64_t nd = *a.n_dev; if (nd < n) n = nd; }
+        for (int64_t t = (int64_t)cta * 8 + warp; t < n; t += (int64_t)a.row_ctas * 8) {
+            const float4* x = reinterpret_cast<const float4*>(a.H + t * a.ldh_b);
+            const float4* w = reinterpret_cast<const float4*>(a.rms_w);
+            uint2* y = reinterpret_cast<uint2*>(a.Hn16) + t * a.nvec;
+            float ss = 0.f;
+            for (int v = lane; v < a.nvec; v += 32) { const float4 c = x[v]; ss += c.x * c.x + c.y * c.y + c.z * c.z + c.w * c.w; }
+            const float rs = rsqrtf(warp_sum(ss) * a.inv_d + a.eps);
+            for (int v = lane; v < a.nvec; v += 32) {
+                const float4 c = x[v], g = w[v];
+                y[v] = make_uint2(pack_bf16(c.x * rs * g.x, c.y * rs * g.y), pack_bf16(c.z * rs * g.z, c.w * rs * g.w));
+            }
+        }
+        return;
+    }
+    cta -= a.row_ctas;
+    const int64_t step = (int64_t)((int)gridDim.x - 2 - a.row_ctas) * 256;
+    for (int64_t i = (int64_t)cta * 256 + threadIdx.x; i < a.n_w0 + a.n_w1; i += step) {
+        const bool second = i >= a.n_w0;
+        const float4 c = second ? a.w1[i - a.n_w0] : a.w0[i];
+        (second ? a.w1_16[i - a.n_w0] : a.w0_16[i]) = make_uint2(pack_bf16(c.x, c.y), pack_bf16(c.z, c.w));
+    }
 }
 
 static int rows_grid8(int64_t n) {
@@ -262,11 +334,11 @@ extern "C" int dash_layer_workspace(const dash_layer_cfg* cfg, int64_t n, int S,
     out->O = off;   off += align_up((size_t)n * cfg->Hq * cfg->D * es, 256);
     out->U = off;   off += align_up((size_t)n * cfg->d * es, 256);
     out->Ht = off;  off += align_up((size_t)n * cfg->d * es, 256);
-    out->scratch = off;                    // fp32 tensors: bf16 copies of a projection's operands (activations, then weights)
+    out->scratch = off;                    // fp32 tensors: bf16 copies of the projections' operands (activations, then both weights)
     if (cfg->dt == DASH_F32) {
         const int64_t hd = (int64_t)cfg->Hq * cfg->D;
         off += conv_a_bytes(n, cfg->d > hd ? cfg->d : hd);
-        off += conv_w_bytes(cfg->d, (int64_t)nq > cfg->d ? (int64_t)nq : cfg->d) > conv_w_bytes(hd, cfg->d) ? conv_w_bytes(cfg->d, (int64_t)nq > cfg->d ? (int64_t)nq : cfg->d) : conv_w_bytes(hd, cfg->d);
+        off += conv_w_bytes(cfg->d, nq) + conv_w_bytes(hd, cfg->d);
     }
     if (cfg->dt == DASH_BF16) off += gemm_split_part_bytes() + gemm_split_count_bytes();      // tiles of the projections cut along K
     off += step_compact_bytes(n, S, cfg->dt);
@@ -301,10 +373,9 @@ static int carve_ws(const dash_layer_cfg* cfg, int64_t n, int S, void* ws, StepW
     if (cfg->dt == DASH_F32) {
         const int64_t hd = (int64_t)cfg->Hq * cfg->D, nq = (int64_t)(cfg->Hq + 2 * cfg->Hkv) * cfg->D;
         const size_t ab = conv_a_bytes(n, cfg->d > hd ? cfg->d : hd);
-        const size_t w1 = conv_w_bytes(cfg->d, nq > cfg->d ? nq : cfg->d), w2 = conv_w_bytes(hd, cfg->d);
-        const size_t wb = w1 > w2 ? w1 : w2;
-        out->conv = {after, ab, after + ab, wb};
-        after += ab + wb;
+        const size_t w1 = conv_w_bytes(cfg->d, nq), w2 = conv_w_bytes(hd, cfg->d);
+        out->conv = {after, ab, after + ab, w1, after + ab + w1};
+        after += ab + w1 + w2;
     }
     out->split = {nullptr, nullptr};
     if (cfg->dt == DASH_BF16) {
@@ -324,14 +395,6 @@ static int carve_ws(const dash_layer_cfg* cfg, int64_t n, int S, void* ws, StepW
     return DASH_OK;
 }
 
-// Zeroed up front, in one go: the arrival counters of projections cut along K and the tail pass's look-back words (whose launch
-// then follows the projection in front of it directly)
-static int clear_step_words(const StepWs& W, int64_t n, bool tail_pass, cudaStream_t st) {
-    const size_t front = W.split.part ? gemm_split_count_bytes() : 0, tail = tail_pass ? tail_ws_clear_bytes(n) : 0;
-    if (front + tail) DASH_CUDA_TRY(cudaMemsetAsync(W.compact_ws - front, 0, front + tail, st));
-    return DASH_OK;
-}
-
 static int launch_rmsnorm(dash_dtype dt, const void* X, const void* weight, void* Y, int64_t n, int d, float eps, const int32_t* n_dev,
                           cudaStream_t st) {
     const int es = dt == DASH_BF16 ? 2 : 4, nvec = d * es / 16;
@@ -343,51 +406,71 @@ static int launch_rmsnorm(dash_dtype dt, const void* X, const void* weight, void
 
 // O = attention(rotary(LN(H) Wqkv)) into W.O: RMSNorm -> Q | K | V projection (rotary embedding in the GEMM epilogue when this
 // library's GEMM takes the shape, else a pass of its own) -> causal attention over the packed active set
+// tail_words: the tail pass of the step looks back over words in the compaction workspace
 static int attention_to_O(const dash_layer_cfg* cfg, const void* H_in, const int32_t* pos_in, const int32_t* cu_in, int S, int64_t n,
-                          int64_t max_seqlen, const StepWs& W, cudaStream_t st) {
+                          int64_t max_seqlen, bool tail_words, const StepWs& W, cudaStream_t st) {
     const int es = cfg->dt == DASH_BF16 ? 2 : 4;
     const bool bf = cfg->dt == DASH_BF16;
     const int d = cfg->d, Hq = cfg->Hq, Hkv = cfg->Hkv, D = cfg->D;
     const int64_t nq = (int64_t)(Hq + 2 * Hkv) * D;
     const int32_t* n_dev = cu_in + S;            // true number of entering tokens lives on the device
     int rc;
-    // the attention kernel's item list needs only cu_seqlens: asked for first, so that the attention kernel directly follows the
-    // projection in the stream (and may set itself up while that one drains)
-    if ((rc = attention_plan(cu_in, S, n, Hq, W.attn_ws, W.attn_bytes, st)) != DASH_OK) return rc;
     GemmEpilogue e;
     e.D = D; e.n_rot_cols = (Hq + Hkv) * D; e.rope_table = W.rope_tab;
     const bool fused = bf && gemm_shape_ok(GEMM_ROPE, n, nq, d, d, nq, e);
     if ((cfg->rope_table || cfg->inv_rms_in || cfg->inv_rms_next) && !(fused && cfg->rms_folded)) return DASH_ERR_UNSUPPORTED;
+    if (!fused && cfg->rms_folded) return DASH_ERR_UNSUPPORTED;      // folded weights need the fused projection (bf16, 256-column tiles)
+    // ---- what waits for nothing: item list, zeroed words (arrival counters of cut projections, look-back words behind them), rows ----
+    PrologueArgs pa = {};
+    RopeFreqs fr;
+    for (int i = 0; i < D / 2; ++i) fr.inv_freq[i] = pow(cfg->rope_base, -2.0 * i / D);
+    if ((rc = attention_plan_ws(S, n, Hq, Hkv, D, cfg->dt, W.attn_ws, W.attn_bytes, &pa.ap)) != DASH_OK) return rc;
+    const size_t front = W.split.part ? gemm_split_count_bytes() : 0, tail = tail_words ? align_up(tail_ws_clear_bytes(n), 16) : 0;
+    pa.cu = cu_in; pa.S = S; pa.Hq = Hq;
+    pa.zero = (uint4*)(W.compact_ws - front); pa.n_zero = (int)((front + tail) / 16);
+    pa.n = n; pa.n_dev = n_dev; pa.H = (const char*)H_in; pa.ldh_b = (int64_t)d * es; pa.nvec = d * es / 16; pa.inv_d = 1.0f / d; pa.eps = cfg->rms_eps;
+    pa.pos = pos_in; pa.half = D / 2;
+    int64_t w_ctas = 0;
+    if (fused) {
+        // rotary angles (none where a table by position is handed in) and, with the norm folded, the rows' factors (none where handed in)
+        pa.table = cfg->rope_table ? nullptr : W.rope_tab;
+        pa.inv_rms = cfg->rms_folded && !cfg->inv_rms_in ? W.inv_rms : nullptr;
+    } else if (!bf) {
+        pa.rms_w = (const float*)cfg->rms_weight; pa.Hn16 = (__nv_bfloat16*)W.conv.a;
+        pa.w0 = (const float4*)cfg->Wqkv; pa.w0_16 = (uint2*)W.conv.w; pa.n_w0 = (int64_t)d * nq / 4;
+        pa.w1 = (const float4*)cfg->Wo; pa.w1_16 = (uint2*)W.conv.w2; pa.n_w1 = (int64_t)Hq * D * d / 4;
+        w_ctas = (pa.n_w0 + pa.n_w1 + 1023) / 1024;
+        if (w_ctas > 4LL * sm_count()) w_ctas = 4LL * sm_count();
+    }
+    pa.row_ctas = pa.table || pa.inv_rms || pa.Hn16 ? rows_grid8(n) : 0;
+    DASH_CUDA_TRY(launch_pdl(prologue_kernel, 2 + pa.row_ctas + (int)w_ctas, 256, 0, st, pa, fr));
     if (fused && cfg->rms_folded) {
         // LN folded into the projection: its weight sits in Wqkv, its row factor 1 / rms is applied to the accumulators.
         // One pass over H gives the row factors and the rotary angles -- unless the caller hands them in (a table of the angles
         // by position, made once per prefill; the row factors as the previous block left them): Q | K | V = (H Wqkv) / rms, Q and
         // K rotated.
         if (cfg->rope_table) { e.rope_table = (const float2*)cfg->rope_table; e.rope_pos = pos_in; e.rope_len = cfg->rope_table_len; }
-        if (!cfg->rope_table || !cfg->inv_rms_in) {
-            rc = launch_row_prep(pos_in, n, D, cfg->rope_base, cfg->rope_table ? nullptr : W.rope_tab, H_in, d, d, cfg->rms_eps,
-                                 cfg->inv_rms_in ? nullptr : W.inv_rms, n_dev, st, true);      // beside the item list in front
-            if (rc != DASH_OK) return rc;
-        }
         e.row_scale = cfg->inv_rms_in ? cfg->inv_rms_in : W.inv_rms;
         if ((rc = gemm_bf16(GEMM_ROPE, H_in, d, cfg->Wqkv, nq, W.QKV, nq, n, nq, d, e, n_dev, st, false, &W.split)) != DASH_OK) return rc;
     } else if (fused) {
         // LN (read as RMSNorm), then Q | K | V = Hn Wqkv with the Q and K heads rotated on the accumulators
         if ((rc = launch_rmsnorm(cfg->dt, H_in, cfg->rms_weight, W.Hn, n, d, cfg->rms_eps, n_dev, st)) != DASH_OK) return rc;
-        if ((rc = launch_row_prep(pos_in, n, D, cfg->rope_base, W.rope_tab, nullptr, 0, d, 0.f, nullptr, n_dev, st)) != DASH_OK) return rc;
         if ((rc = gemm_bf16(GEMM_ROPE, W.Hn, d, cfg->Wqkv, nq, W.QKV, nq, n, nq, d, e, n_dev, st, false, &W.split)) != DASH_OK) return rc;
     } else {
-        if (cfg->rms_folded) return DASH_ERR_UNSUPPORTED;      // folded weights need the fused projection (bf16, 256-column tiles)
-        if ((rc = launch_rmsnorm(cfg->dt, H_in, cfg->rms_weight, W.Hn, n, d, cfg->rms_eps, n_dev, st)) != DASH_OK) return rc;
-        if ((rc = project(cfg->dt, W.Hn, d, cfg->Wqkv, nq, W.QKV, nq, n, nq, d, n_dev, W.conv, W.split, st)) != DASH_OK) return rc;
-        // rotary embedding on the Q and K heads
-        RopeFreq fr;
-        for (int i = 0; i < D / 2; ++i) fr.inv_freq[i] = pow(cfg->rope_base, -2.0 * i / D);
         const int heads = Hq + Hkv;
-        if (bf && D == 128) rope_kernel<true, 128><<<rows_grid8(n), 256, 0, st>>>(W.QKV, nq * es, pos_in, n, heads, fr, n_dev);
-        else if (bf) rope_kernel<true, 64><<<rows_grid8(n), 256, 0, st>>>(W.QKV, nq * es, pos_in, n, heads, fr, n_dev);
-        else if (D == 128) rope_kernel<false, 128><<<rows_grid8(n), 256, 0, st>>>(W.QKV, nq * es, pos_in, n, heads, fr, n_dev);
-        else rope_kernel<false, 64><<<rows_grid8(n), 256, 0, st>>>(W.QKV, nq * es, pos_in, n, heads, fr, n_dev);
+        if (bf) {
+            if ((rc = launch_rmsnorm(cfg->dt, H_in, cfg->rms_weight, W.Hn, n, d, cfg->rms_eps, n_dev, st)) != DASH_OK) return rc;
+            if ((rc = project(cfg->dt, W.Hn, d, cfg->Wqkv, nq, W.QKV, nq, n, nq, d, n_dev, W.conv, W.split, st)) != DASH_OK) return rc;
+        } else {
+            // operands as the prologue left them: bf16 copies, products accumulated and stored in fp32
+            if ((rc = gemm_bf16(GEMM_PLAIN, W.conv.a, d, W.conv.w, nq, W.QKV, nq, n, nq, d, GemmEpilogue(), n_dev, st, true)) != DASH_OK) return rc;
+        }
+        // rotary embedding on the Q and K heads
+        const AttnCopies cp = {pa.ap.q, pa.ap.k, pa.ap.v, Hq, Hkv};
+        if (bf && D == 128) rope_kernel<true, 128><<<rows_grid8(n), 256, 0, st>>>(W.QKV, nq * es, pos_in, n, heads, fr, n_dev, cp);
+        else if (bf) rope_kernel<true, 64><<<rows_grid8(n), 256, 0, st>>>(W.QKV, nq * es, pos_in, n, heads, fr, n_dev, cp);
+        else if (D == 128) rope_kernel<false, 128><<<rows_grid8(n), 256, 0, st>>>(W.QKV, nq * es, pos_in, n, heads, fr, n_dev, cp);
+        else rope_kernel<false, 64><<<rows_grid8(n), 256, 0, st>>>(W.QKV, nq * es, pos_in, n, heads, fr, n_dev, cp);
         DASH_CUDA_TRY(cudaGetLastError());
     }
     if (cfg->k_cache) {
@@ -399,12 +482,13 @@ static int attention_to_O(const dash_layer_cfg* cfg, const void* H_in, const int
     // attention over the packed active set
     return attention_planned(W.QKV, W.QKV + (int64_t)Hq * D * es, W.QKV + (int64_t)(Hq + Hkv) * D * es, W.O, nullptr, nq, nq, nq,
                              (int64_t)Hq * D, cu_in, S, n, max_seqlen, Hq, Hkv, D, 1.0f / sqrtf((float)D), cfg->dt,
-                             W.attn_ws, W.attn_bytes, st);
+                             W.attn_ws, W.attn_bytes, st, bf ? nullptr : W.conv.a);      // fp32: O also as the output projection's bf16 operand
 }
 
 // U = O Wo  (pre-residual attention output, Eq. 1) into W.U
 static int out_proj_U(const dash_layer_cfg* cfg, const int32_t* cu_in, int S, int64_t n, const StepWs& W, cudaStream_t st) {
     const int64_t hd = (int64_t)cfg->Hq * cfg->D;
+    if (cfg->dt == DASH_F32) return gemm_bf16(GEMM_PLAIN, W.conv.a, hd, W.conv.w2, cfg->d, W.U, cfg->d, n, cfg->d, hd, GemmEpilogue(), cu_in + S, st, true);
     return project(cfg->dt, W.O, hd, cfg->Wo, cfg->d, W.U, cfg->d, n, cfg->d, hd, cu_in + S, W.conv, W.split, st);
 }
 
@@ -465,8 +549,7 @@ extern "C" int dash_layer_step(const dash_layer_cfg* cfg, const void* H_in, cons
             (cfg->rms_weight && !aligned16(cfg->rms_weight)))
             return DASH_ERR_INVALID_ARG;
         const bool every_row = cfg->scatter_which == 2, tail_pass = cfg->sel_mode == DASH_SEL_THRESHOLD && every_row;
-        if ((rc = clear_step_words(W, n, every_row, st)) != DASH_OK) return rc;
-        if ((rc = attention_to_O(cfg, H_in, pos_in, cu_in, S, n, max_seqlen, W, st)) != DASH_OK) return rc;
+        if ((rc = attention_to_O(cfg, H_in, pos_in, cu_in, S, n, max_seqlen, every_row, W, st)) != DASH_OK) return rc;
         if (tail_pass) {
             // output projection with H~ = H + U written straight to x_full and the row sums of u^2, h^2 beside it; then the score, the
             // halting rule and the compaction of the rows that stay (from x_full) in one pass
@@ -560,9 +643,8 @@ extern "C" int dash_block_step(const dash_block_cfg* cfg, const void* H_in, cons
         !aligned16(cfg->Wgu) || !aligned16(cfg->Wd) || (cfg->rms2_weight && !aligned16(cfg->rms2_weight)))
         return DASH_ERR_INVALID_ARG;
     const int32_t* n_dev = cu_in + S;
-    if ((rc = clear_step_words(W, n, true, st)) != DASH_OK) return rc;
     // U = Attn(LN(H)); score and selection from U; H~ = H + U
-    if ((rc = attention_to_O(a, H_in, pos_in, cu_in, S, n, max_seqlen, W, st)) != DASH_OK) return rc;
+    if ((rc = attention_to_O(a, H_in, pos_in, cu_in, S, n, max_seqlen, true, W, st)) != DASH_OK) return rc;
     bool have_inv_rms2 = false;
     rc = cfg->signal == DASH_SIGNAL_ATTN ? out_proj_residual(a, H_in, nullptr, W.Ht, cu_in, S, n, W, st) : DASH_ERR_UNSUPPORTED;
     if (rc == DASH_OK) {

@@ -1,0 +1,115 @@
+// Device functions that run as kernels of their own and inside the kernel in front of a block step (layer_step.cu).
+#pragma once
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include "common.cuh"
+
+namespace dash {
+
+constexpr int kPlanRows = 128;           // query rows of an attention item
+
+// Where an attention call's item list goes in its workspace and, fp32 tensors, the bf16 copies of Q, K and V: for a step that fills them
+// in a kernel of its own ahead of attention_planned()
+struct AttnPlanWs { int4* plan; int* n_items; unsigned int* ticket; int64_t max_entries; __nv_bfloat16 *q, *k, *v; };
+int attention_plan_ws(int S, int64_t n, int Hq, int Hkv, int D, dash_dtype dt, void* ws, size_t ws_bytes, AttnPlanWs* out);
+
+// Which (sequence, query tile) pairs exist, ordered by falling number of key blocks; called by all THREADS threads of one CTA
+template <int THREADS>
+__device__ __forceinline__ void attention_plan_items(const int32_t* __restrict__ cu, int S, int Hq, int4* __restrict__ plan, int* __restrict__ n_items,
+                                                     unsigned int* __restrict__ ticket, int64_t max_entries) {
+    constexpr int NW = THREADS / 32;
+    __shared__ int s_warp[33];
+    __shared__ int s_max;
+    const int tid = threadIdx.x;
+    if (tid == 0) s_max = 0;
+    __syncthreads();
+    int mx = 0;
+    for (int s = tid; s < S; s += THREADS) mx = max(mx, (cu[s + 1] - cu[s] + kPlanRows - 1) / kPlanRows);
+    atomicMax(&s_max, mx);
+    __syncthreads();
+    const int max_nq = s_max;
+    int64_t offset = 0;
+    for (int top = max_nq - 1; top >= 0; top -= THREADS) {
+        const int qt = top - tid;                           // thread 0 takes the heaviest level of this chunk
+        int cnt = 0;
+        if (qt >= 0)
+            for (int s = 0; s < S; ++s) cnt += ((cu[s + 1] - cu[s] + kPlanRows - 1) / kPlanRows > qt);
+        // exclusive scan over the block
+        const int lane = tid & 31, w = tid >> 5;
+        int inc = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { int t = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += t; }
+        if (lane == 31) s_warp[w] = inc;
+        __syncthreads();
+        if (w == 0) {
+            int x = lane < NW ? s_warp[lane] : 0, xi = x;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) { int t = __shfl_up_sync(0xffffffffu, xi, o); if (lane >= o) xi += t; }
+            s_warp[lane] = xi - x;
+            if (lane == 31) s_warp[32] = xi;
+        }
+        __syncthreads();
+        int64_t k = offset + s_warp[w] + inc - cnt;
+        const int chunk_total = s_warp[32];
+        if (qt >= 0)
+            for (int s = 0; s < S; ++s)
+                if ((cu[s + 1] - cu[s] + kPlanRows - 1) / kPlanRows > qt) { if (k < max_entries) plan[k] = make_int4(s, qt, cu[s], cu[s + 1]); ++k; }
+        offset += chunk_total;
+        __syncthreads();
+    }
+    if (tid == 0) {
+        if (offset > max_entries) offset = max_entries;     // cannot happen for cu_seqlens[S] <= n; keeps every read in bounds
+        *n_items = (int)(offset * Hq);
+        *ticket = 0u;
+    }
+}
+
+struct RopeFreqs { double inv_freq[64]; };
+
+// Per row (one warp): (cos, sin) of pos[t] * base^(-2i/D) for i < D/2, angles formed and reduced in fp64 (positions reach 1e5 rad
+// at i = 0: fp32 would lose the angle), evaluated in fp32 on the reduced angle; and, when asked, the row factor of the RMSNorm, 1 / sqrt(mean(h^2) + eps), from one pass over the bf16 row.
+// Rows first_warp, first_warp + n_warps, ..
+__device__ __forceinline__ void row_prep_rows(const int32_t* __restrict__ pos, int64_t n, int half, const RopeFreqs& fr, float2* __restrict__ table,
+                                              const char* __restrict__ H, int64_t ldh_b, int nvec, float inv_d, float eps, float* __restrict__ inv_rms,
+                                              const int32_t* __restrict__ n_dev, int64_t first_warp, int64_t n_warps) {
+    if (n_dev) { int64_t nd = *n_dev; if (nd < n) n = nd; }
+    const int lane = threadIdx.x & 31;
+    for (int64_t t = first_warp; t < n; t += n_warps) {
+        float ss = 0.f;
+        if (inv_rms) {
+            const char* h = H + t * ldh_b;
+            for (int base = 0; base < nvec; base += 128) {
+                uint4 x[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) { const int v = base + k * 32 + lane; if (v < nvec) x[k] = ld_nc_v4(h + ((int64_t)v << 4)); }
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int v = base + k * 32 + lane;
+                    if (v < nvec) {
+                        const float f[8] = {bf16lo(x[k].x), bf16hi(x[k].x), bf16lo(x[k].y), bf16hi(x[k].y), bf16lo(x[k].z), bf16hi(x[k].z), bf16lo(x[k].w), bf16hi(x[k].w)};
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) ss += f[e] * f[e];
+                    }
+                }
+            }
+        }
+        if (table) {
+            const double ps = pos ? (double)pos[t] : (double)t;
+            for (int i = lane; i < half; i += 32) {
+                // angle formed and reduced to [-pi, pi] in fp64 (three operations), sine and cosine of the reduced angle in fp32
+                const double ang = ps * fr.inv_freq[i];
+                const double red = fma(-6.283185307179586476925286766559, rint(ang * 0.15915494309189533576888376337251), ang);
+                float sn, cs;
+                sincosf((float)red, &sn, &cs);
+                table[t * half + i] = make_float2(cs, sn);
+            }
+        }
+        if (inv_rms) {
+            ss = warp_sum(ss);
+            if (lane == 0) inv_rms[t] = rsqrtf(ss * inv_d + eps);
+        }
+    }
+}
+
+}  // namespace dash
