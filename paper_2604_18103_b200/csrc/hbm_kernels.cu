@@ -540,14 +540,16 @@ __device__ __forceinline__ int tail_decide(const TailArgs& a, int64_t row, float
     return keep;
 }
 
-// The same pass with a row held by its warp from the first load to the last store (rows of up to 32 * NV vectors): tiles of eight rows, a warp
-// each, so that 700 rows are 88 CTAs and not 22, a row's loads go out together (in two halves where there are U and H to add), and what
-// goes on to the next block is written from registers instead of being read back.  Bound by the chain ticket -> rows -> look-back; for
-// inputs whose tiles are all resident.  701 rows of 7 KB took 37 us behind the start of the general kernel's launch, 16 here.
+// The same pass with a warp per row and tiles of eight rows, so that 700 rows are 88 CTAs and not 22.  Bound by the chain ticket -> rows ->
+// look-back -> copy; for inputs whose tiles are all resident.  Loops of seven vectors per lane (two for a row of 3584 bf16), not
+// unrolled: with the whole row in registers and straight-line code the warps waited 14 us for instructions they run once.
 constexpr int kTailRows = 8;
-template <bool BF16, int NV>
-__global__ void __launch_bounds__(32 * kTailRows, 2)
+constexpr int kTailSmallTiles = 2;          // per SM: with more tiles than fit at once, a tile waits for the look-back chain of up to a
+                                            // thousand others (behind the projection in front, 6683 rows: 64 us against 40 of the general kernel, 8192: 80 against 42)
+template <bool BF16>
+__global__ void __launch_bounds__(32 * kTailRows)
 delta_tail_rows_kernel(const TailArgs a, int64_t n_upper) {
+    constexpr int CH = 7;
     __shared__ int s_keep[kTailRows];
     __shared__ int s_base, s_count;
     __shared__ unsigned int s_tile, s_ballot;
@@ -563,49 +565,45 @@ delta_tail_rows_kernel(const TailArgs a, int64_t n_upper) {
     const int64_t t_end = (t_start + kTailRows < n) ? t_start + kTailRows : n;
     const bool last_tile = (t_end >= n);
     const int64_t row = t_start + warp;
-    const bool live = row < n;
     int keep = 0, tok = 0, pos = 0;
     float ss = 0.f, su = 0.f, sh = 0.f;                    // ss: sum of squares of the row as it goes on (H~ or H')
-    uint4 z[NV];
-    if (live) {
+    char* x = a.x_full;
+    if (row < n) {
         tok = a.tok_in[row];
         pos = a.pos_in[row];
+        x += (int64_t)tok * a.ldx_b;
         if (a.mask_in) keep = a.mask_in[row] != 0;
-        char* x = a.x_full + (int64_t)tok * a.ldx_b;
         if (a.U) {
             const char* u = a.U + row * a.ldU_b;
             const char* h = a.H + row * a.ldH_b;
-            constexpr int HALF = (NV + 1) / 2;
+#pragma unroll 1
+            for (int v0 = lane; v0 < a.nvec; v0 += 32 * CH) {
+                uint4 p[CH], q[CH];
 #pragma unroll
-            for (int part = 0; part < 2; ++part) {
-                uint4 y[HALF];
+                for (int k = 0; k < CH; ++k) {
+                    const int64_t v = v0 + k * 32;
+                    if (v < a.nvec) { p[k] = ld_nc_v4(u + (v << 4)); q[k] = ld_nc_v4(h + (v << 4)); }
+                    else p[k] = q[k] = make_uint4(0, 0, 0, 0);
+                }
+                if (!a.mask_in) {
 #pragma unroll
-                for (int k = 0; k < HALF; ++k) {
-                    const int i = part * HALF + k, v = i * 32 + lane;
-                    if (i < NV && v < a.nvec) { z[i < NV ? i : 0] = ld_nc_v4(u + ((int64_t)v << 4)); y[k] = ld_nc_v4(h + ((int64_t)v << 4)); }
+                    for (int k = 0; k < CH; ++k) { su += sumsq_vec<BF16>(p[k]); sh += sumsq_vec<BF16>(q[k]); }
                 }
 #pragma unroll
-                for (int k = 0; k < HALF; ++k) {
-                    const int i = part * HALF + k, v = i * 32 + lane;
-                    if (i < NV && v < a.nvec) {
-                        uint4& w = z[i < NV ? i : 0];
-                        if (!a.mask_in) { su += sumsq_vec<BF16>(w); sh += sumsq_vec<BF16>(y[k]); }
-                        w = add_vec<BF16>(w, y[k]);
-                        if (a.inv_next) ss += sumsq_vec<BF16>(w);
-                        st_v4(x + ((int64_t)v << 4), w);
-                    }
+                for (int k = 0; k < CH; ++k) {
+                    const int64_t v = v0 + k * 32;
+                    p[k] = add_vec<BF16>(p[k], q[k]);
+                    if (v < a.nvec) st_v4(x + (v << 4), p[k]);
+                }
+                if (a.inv_next) {
+#pragma unroll
+                    for (int k = 0; k < CH; ++k) ss += sumsq_vec<BF16>(p[k]);
                 }
             }
-            if (!a.mask_in) keep = tail_decide(a, row, warp_sum(su), warp_sum(sh), lane);
-        } else {
-            // the row is in x_full already: asked for before its score is known
-#pragma unroll
-            for (int i = 0; i < NV; ++i) { const int v = i * 32 + lane; if (v < a.nvec) z[i] = ld_cg_v4(x + ((int64_t)v << 4)); }
-            if (a.sums) {
-                for (int i = lane; i < a.n_sum_tiles; i += 32) { const float4 p2 = a.sums[row * a.n_sum_tiles + i]; su += p2.x; sh += p2.y; ss += p2.z; }
-                if (!a.mask_in) keep = tail_decide(a, row, warp_sum(su), warp_sum(sh), lane);
-            }
+        } else if (a.sums) {
+            for (int i = lane; i < a.n_sum_tiles; i += 32) { const float4 p2 = a.sums[row * a.n_sum_tiles + i]; su += p2.x; sh += p2.y; ss += p2.z; }
         }
+        if (!a.mask_in) keep = tail_decide(a, row, warp_sum(su), warp_sum(sh), lane);
     }
     if (a.inv_next) ss = warp_sum(ss);
     if (lane == 0) s_keep[warp] = keep;
@@ -621,8 +619,14 @@ delta_tail_rows_kernel(const TailArgs a, int64_t n_upper) {
     if (keep) {
         const int64_t k = base + __popc(bal & ((1u << warp) - 1u));
         char* dst = a.H_next + k * a.ldn_b;
+#pragma unroll 1
+        for (int v0 = lane; v0 < a.nvec; v0 += 32 * CH) {
+            uint4 p[CH];
 #pragma unroll
-        for (int i = 0; i < NV; ++i) { const int v = i * 32 + lane; if (v < a.nvec) st_v4(dst + ((int64_t)v << 4), z[i]); }
+            for (int i = 0; i < CH; ++i) { const int64_t v = v0 + i * 32; if (v < a.nvec) p[i] = ld_cg_v4(x + (v << 4)); }
+#pragma unroll
+            for (int i = 0; i < CH; ++i) { const int64_t v = v0 + i * 32; if (v < a.nvec) st_v4(dst + (v << 4), p[i]); }
+        }
         if (lane == 0) {
             a.tok_next[k] = tok;
             a.pos_next[k] = pos;
@@ -1067,15 +1071,10 @@ int launch_delta_tail(const void* U, const void* H, const uint8_t* mask_in, cons
     a.inv_next = inv_next; a.inv_d = 1.0f / (float)d; a.rms_eps = rms_eps;
     a.status = status_word_ptr();
     if (!a.status) return DASH_ERR_CUDA;
-    // a row in a warp's registers: up to 16 vectors (8 KB a row: 4096 columns of bf16) per lane; 4 where that is enough
-    const int nv = (a.nvec + 31) / 32, small = (int)((n + kTailRows - 1) / kTailRows) > 0 ? (int)((n + kTailRows - 1) / kTailRows) : 1;
-    // .. and only while all tiles fit the GPU at once: with more, a tile's registers wait for the look-back chain of up to 1024 others in
-    // front of it (8192 rows: 50 and 98 us against 24 and 45 of the general kernel)
-    if (nv <= 16 && small <= 2 * sm_count()) {
-        if (dt == DASH_BF16 && nv <= 4) DASH_CUDA_TRY(launch_pdl(delta_tail_rows_kernel<true, 4>, small, 32 * kTailRows, 0, st, a, n));
-        else if (dt == DASH_BF16) DASH_CUDA_TRY(launch_pdl(delta_tail_rows_kernel<true, 16>, small, 32 * kTailRows, 0, st, a, n));
-        else if (nv <= 4) DASH_CUDA_TRY(launch_pdl(delta_tail_rows_kernel<false, 4>, small, 32 * kTailRows, 0, st, a, n));
-        else DASH_CUDA_TRY(launch_pdl(delta_tail_rows_kernel<false, 16>, small, 32 * kTailRows, 0, st, a, n));
+    const int small = (int)((n + kTailRows - 1) / kTailRows) > 0 ? (int)((n + kTailRows - 1) / kTailRows) : 1;
+    if (small <= kTailSmallTiles * sm_count()) {
+        if (dt == DASH_BF16) DASH_CUDA_TRY(launch_pdl(delta_tail_rows_kernel<true>, small, 32 * kTailRows, 0, st, a, n));
+        else DASH_CUDA_TRY(launch_pdl(delta_tail_rows_kernel<false>, small, 32 * kTailRows, 0, st, a, n));
         return DASH_OK;
     }
     const int tiles = (int)((n + 31) / 32) > 0 ? (int)((n + 31) / 32) : 1;
