@@ -20,7 +20,7 @@
 // 128 contiguous bytes, and what an epilogue reads is asked for a piece ahead.  With a lane per row in the loads and stores too (and
 // four warps) an epilogue took 23-30 thousand cycles (ROPE), 18-22 (RESID), 15 (SWIGLU), 7 (PLAIN) against 31 thousand of a
 // 3584-deep tile's MMAs: the QKV projection waited for it at every tile (41.9 thousand cycles per tile), and the last tile's showed
-// in every launch.
+// in every launch.  A tile's pieces come in loops: a launch with a tile per CTA runs their code once, and would wait for the instructions.
 #include <math.h>
 
 #include "common.cuh"
@@ -456,7 +456,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                 wait_acc();
                 if (!ok) break;
                 if (k1 - k0 != ksteps && leave_part()) { release_acc(); continue; }
-#pragma unroll
+#pragma unroll 1
                 for (int k = 0; k < 4; ++k) {
                     const int h0 = head_of(k), c = pair_of(k), colh = colw + h0;
                     uint32_t o[32];
@@ -518,7 +518,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                 wait_acc();
                 if (!ok) break;
                 if (k1 - k0 != ksteps && leave_part()) { release_acc(); continue; }
-#pragma unroll
+#pragma unroll 1
                 for (int k = 0; k < 4; ++k) {
                     uint32_t o[32];
                     load_acc(w16, half * 128 + k * 32, half * 128 + k * 32 + 16, o);
@@ -554,21 +554,20 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                 wait_acc();
                 if (!ok) break;
                 if (k1 - k0 != ksteps && leave_part()) { release_acc(); continue; }
+#pragma unroll 1
+                for (int k = 0; k < 4; ++k) {
+                    uint32_t gu[32];                              // 16 gate, 16 up columns of this lane's row
+                    load_acc(w16, half * 64 + k * 16, 128 + half * 64 + k * 16, gu);
+                    if (k == 3) release_acc();
+                    float a[16];
 #pragma unroll
-                for (int k = 0; k < 2; ++k) {
-                    uint32_t gu[64];
-                    const uint32_t *gt = gu, *up = gu + 32;
-                    load_acc(w32, half * 64 + k * 32, 128 + half * 64 + k * 32, gu);
-                    if (k == 1) release_acc();
-                    float a[32];
-#pragma unroll
-                    for (int e = 0; e < 32; ++e) {
-                        const float z = __uint_as_float(gt[e]) * rsc;
-                        a[e] = z / (1.0f + __expf(-z)) * (__uint_as_float(up[e]) * rsc);
+                    for (int e = 0; e < 16; ++e) {
+                        const float z = __uint_as_float(gu[e]) * rsc;
+                        a[e] = z / (1.0f + __expf(-z)) * (__uint_as_float(gu[16 + e]) * rsc);
                     }
 #pragma unroll
-                    for (int c = 0; c < 4; ++c)
-                        sts_v4(stage_addr(stage, lane, k * 4 + c), pack_bf16(a[8 * c], a[8 * c + 1]), pack_bf16(a[8 * c + 2], a[8 * c + 3]),
+                    for (int c = 0; c < 2; ++c)
+                        sts_v4(stage_addr(stage, lane, k * 2 + c), pack_bf16(a[8 * c], a[8 * c + 1]), pack_bf16(a[8 * c + 2], a[8 * c + 3]),
                                pack_bf16(a[8 * c + 4], a[8 * c + 5]), pack_bf16(a[8 * c + 6], a[8 * c + 7]));
                 }
                 __syncwarp();
