@@ -49,6 +49,7 @@ struct SelfPlan {
     int nb[kSelfPlanSeqs];            // key blocks of sequence s
     int first[kSelfPlanSeqs + 1];     // first item of sequence s (its Hkv heads follow each other, `per` items each); then the number of items
     int per[kSelfPlanSeqs];           // items per (sequence, KV head)
+    int cu[kSelfPlanSeqs + 1];        // the boundaries it was made from
     int chunk, n_items;
 };
 // Called by all threads of the CTA (it synchronises).  `target` is twice the number of CTAs.  Chunk length (key blocks per item):
@@ -61,7 +62,10 @@ __device__ __forceinline__ void self_plan_build(SelfPlan& sp, const int32_t* cu,
         const int lane = threadIdx.x;
         unsigned int nb[PL], all = 0;
 #pragma unroll
-        for (int j = 0; j < PL; ++j) { const int s = lane + 32 * j; nb[j] = s < S ? (unsigned int)dec_blocks(cu, s) : 0u; all += nb[j]; }
+        for (int j = 0; j <= PL; ++j) { const int s = lane + 32 * j; if (s <= S) sp.cu[s] = __ldcg(cu + s); }
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < PL; ++j) { const int s = lane + 32 * j; nb[j] = s < S ? (unsigned int)dec_blocks(sp.cu, s) : 0u; all += nb[j]; }
         all = __reduce_add_sync(0xffffffffu, all) * (unsigned int)Hkv;
         auto count = [&](unsigned int chunk) {
             unsigned int k = 0;
@@ -90,6 +94,12 @@ __device__ __forceinline__ void self_plan_build(SelfPlan& sp, const int32_t* cu,
         if (lane == 0) { sp.chunk = (int)chunk; sp.n_items = k; sp.first[S] = k; }
     }
     __syncthreads();
+}
+// Made ahead of its time, from boundaries that may still change: made again if they did
+__device__ __forceinline__ void self_plan_confirm(SelfPlan& sp, const int32_t* cu, int S, int Hkv, int target) {
+    int changed = 0;
+    for (int s = threadIdx.x; s <= S; s += blockDim.x) changed |= __ldcg(cu + s) != sp.cu[s];
+    if (__syncthreads_or(changed)) self_plan_build(sp, cu, S, Hkv, target);
 }
 __device__ __forceinline__ DecItem self_plan_item(const SelfPlan& sp, int S, int item) {
     int lo = 0, hi = S;               // first[lo] <= item < first[hi]: the last such lo owns the item (sequences without keys own none)
@@ -170,7 +180,6 @@ decode_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
     volatile uint32_t* abort_gen = reinterpret_cast<volatile uint32_t*>(smem_gen + L::kBars + 68);
     volatile int* item_gen = reinterpret_cast<volatile int*>(smem_gen + L::kBars + 72);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    pdl_launch_dependents();                 // the merge kernel may get onto the SMs while this one runs
 
     // rows of the Q tile that no load ever writes must not hold NaN patterns: clear the tile once
     for (int i = tid * 16; i < L::kTileBytes; i += kDecThreads * 16) *reinterpret_cast<uint4*>(smem_gen + L::kQ + i) = make_uint4(0, 0, 0, 0);
@@ -191,14 +200,26 @@ decode_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    const bool self_plan = (p.plan == nullptr);
+    __shared__ SelfPlan sp;
+    if (self_plan) {
+        // While the kernel in front drains (the previous call's merge, in a decoding step): the plan from the boundaries as they stand, and
+        // this CTA's first key block asked into L2.  Nothing of either counts if the boundaries turn out to be others (a prefetch
+        // reads nothing; its rows are those of the map or none).
+        self_plan_build(sp, p.cu, p.S, p.Hkv, p.target);
+        if (tid == 32 && (int)blockIdx.x < sp.n_items) {
+            const DecItem it = self_plan_item(sp, p.S, (int)blockIdx.x);
+            const int row = sp.cu[it.s] + it.b0 * kDecBN;
+            for (int c = 0; c < KCH; ++c) { tma_prefetch_3d(&mapK, c * 64, it.kvh, row); tma_prefetch_3d(&mapV, c * 64, it.kvh, row); }
+        }
+    }
     pdl_wait();                              // set-up done; from here on the kernel in front has completed
+    pdl_launch_dependents();                 // the merge kernel may get onto the SMs now: all in front of this kernel is complete for it too
     const uint32_t tmem = *tmem_slot_gen;
     const uint32_t tS = tmem, tP = tmem, tO = tmem + 128;
     constexpr uint32_t idesc_s = idesc_bf16_f32(128, kDecBN, false, false);
     constexpr uint32_t idesc_o = idesc_bf16_f32(128, D, false, true);
-    const bool self_plan = (p.plan == nullptr);
-    __shared__ SelfPlan sp;
-    if (self_plan) self_plan_build(sp, p.cu, p.S, p.Hkv, p.target);
+    if (self_plan) self_plan_confirm(sp, p.cu, p.S, p.Hkv, p.target);
     const int n_items = self_plan ? sp.n_items : *p.n_items;
     uint32_t blk0 = 0, items_done = 0;       // barrier phases run on across the items of this CTA
 
@@ -490,8 +511,9 @@ decode_merge_kernel(const MergeParams p) {
     __shared__ SelfPlan sp;
     __shared__ float s_acc[kMergeThreads / 32][32];
     pdl_launch_dependents();
-    pdl_wait();                              // started while the decode kernel drains: its partial results are complete from here on
+    // started while the decode kernel runs, which had waited for all in front of it before it let this one start: the boundaries stand
     if (!p.seg) self_plan_build(sp, p.cu, p.S, p.Hkv, p.target);
+    pdl_wait();                              // the decode kernel's partial results are complete from here on
     // warps per unit: as many as the machine has per unit, at most the CTA's eight
     const long long n_units = (long long)p.S * p.Hq * (D / 32), warps = (long long)gridDim.x * (kMergeThreads / 32);
     if (n_units * 16 <= warps) decode_merge_units<D, 8>(p, sp, s_acc);
@@ -599,6 +621,12 @@ extern "C" int dash_decode_attention(const void* q, const void* Kc, const void* 
     long long mgrid = (units * 8 + kMergeThreads / 32 - 1) / (kMergeThreads / 32);
     if (mgrid > sm_count()) mgrid = sm_count();
     if (mgrid < 1) mgrid = 1;
+    if (n == 0) {                             // no decode kernel in front that has waited for what writes the boundaries: in plain stream order
+        if (D == 128) decode_merge_kernel<128><<<(int)mgrid, kMergeThreads, 0, st>>>(mp);
+        else decode_merge_kernel<64><<<(int)mgrid, kMergeThreads, 0, st>>>(mp);
+        DASH_CUDA_TRY(cudaGetLastError());
+        return DASH_OK;
+    }
     if (D == 128) DASH_CUDA_TRY(launch_pdl(decode_merge_kernel<128>, (int)mgrid, kMergeThreads, 0, st, mp));
     else DASH_CUDA_TRY(launch_pdl(decode_merge_kernel<64>, (int)mgrid, kMergeThreads, 0, st, mp));
     return DASH_OK;
