@@ -464,6 +464,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                     if (k == 3) release_acc();
                     stage_f32(o);
                     const bool rotate = colh < g.e.n_rot_cols;
+                    // a head of K or V goes to the caller's cache as well
+                    __nv_bfloat16* cache = nullptr;
+                    if (g.e.k_cache && colh >= g.e.q_cols)
+                        cache = reinterpret_cast<__nv_bfloat16*>(rotate ? g.e.k_cache : g.e.v_cache) + (colh - (rotate ? g.e.q_cols : g.e.n_rot_cols));
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
                         const int r = rr + 8 * i, row = row0 + r;
@@ -484,9 +488,15 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                             for (int e = 0; e < 4; ++e) { y1[e] = x1[e]; y2[e] = x2[e]; }
                         }
                         if (row < n_true) {
+                            const uint32_t a0 = pack_bf16(y1[0], y1[1]), a1 = pack_bf16(y1[2], y1[3]), b0 = pack_bf16(y2[0], y2[1]), b1 = pack_bf16(y2[2], y2[3]);
                             __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(g.C) + (int64_t)row * g.ldc + colh + c + c4 * 4;
-                            st_v2(dst, pack_bf16(y1[0], y1[1]), pack_bf16(y1[2], y1[3]));
-                            st_v2(dst + hd2, pack_bf16(y2[0], y2[1]), pack_bf16(y2[2], y2[3]));
+                            st_v2(dst, a0, a1);
+                            st_v2(dst + hd2, b0, b1);
+                            if (cache) {
+                                __nv_bfloat16* kv = cache + (int64_t)row * g.e.ld_cache + c + c4 * 4;
+                                st_v2(kv, a0, a1);
+                                st_v2(kv + hd2, b0, b1);
+                            }
                         }
                     }
                     if (k < 3) fetch_cs(k + 1);

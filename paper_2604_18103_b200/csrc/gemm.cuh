@@ -16,6 +16,9 @@ struct GemmEpilogue {
     const float2* rope_table = nullptr;
     // rope_pos null: the table holds one entry per row; else one per position and row t uses entry min(rope_pos[t], rope_len - 1)
     const int32_t* rope_pos = nullptr; int64_t rope_len = 0;
+    // ROPE: k_cache / v_cache (null: none): the K and V heads' columns (behind q_cols of Q) once more, rows of ld_cache elements, 8-byte aligned
+    int q_cols = 0;
+    void *k_cache = nullptr, *v_cache = nullptr; int64_t ld_cache = 0;
     // ROPE, SWIGLU: row_scale (null: none) multiplies the accumulators of a row first -- 1 / rms(row) when the RMSNorm in front of the
     // projection is folded into it (its weight into W, its row factor here)
     const float* row_scale = nullptr;

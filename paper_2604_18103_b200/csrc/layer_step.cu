@@ -419,6 +419,10 @@ static int attention_to_O(const dash_layer_cfg* cfg, const void* H_in, const int
     e.D = D; e.n_rot_cols = (Hq + Hkv) * D; e.rope_table = W.rope_tab;
     const bool fused = bf && gemm_shape_ok(GEMM_ROPE, n, nq, d, d, nq, e);
     if ((cfg->rope_table || cfg->inv_rms_in || cfg->inv_rms_next) && !(fused && cfg->rms_folded)) return DASH_ERR_UNSUPPORTED;
+    // this depth's KV cache rows: keys (rotary applied) and values of the entering tokens, packed [n, Hkv, D].  From the fused projection's
+    // epilogue where the buffers allow its 8-byte stores, else copied out of QKV (two launches, 3.5 us each for 701 tokens)
+    const bool cache_fused = fused && cfg->k_cache && !(((uintptr_t)cfg->k_cache | (uintptr_t)cfg->v_cache) & 7);
+    if (cache_fused) { e.q_cols = Hq * D; e.k_cache = cfg->k_cache; e.v_cache = cfg->v_cache; e.ld_cache = (int64_t)Hkv * D; }
     if (!fused && cfg->rms_folded) return DASH_ERR_UNSUPPORTED;      // folded weights need the fused projection (bf16, 256-column tiles)
     // ---- what waits for nothing: item list, zeroed words (arrival counters of cut projections, look-back words behind them), rows ----
     PrologueArgs pa = {};
@@ -473,8 +477,7 @@ static int attention_to_O(const dash_layer_cfg* cfg, const void* H_in, const int
         else rope_kernel<false, 64><<<rows_grid8(n), 256, 0, st>>>(W.QKV, nq * es, pos_in, n, heads, fr, n_dev, cp);
         DASH_CUDA_TRY(cudaGetLastError());
     }
-    if (cfg->k_cache) {
-        // this depth's KV cache rows: keys (rotary applied) and values of the entering tokens, packed [n, Hkv, D]
+    if (cfg->k_cache && !cache_fused) {
         const int64_t kvb = (int64_t)Hkv * D * es;
         if ((rc = dash_scatter(W.QKV + (int64_t)Hq * D * es, n, kvb, nq * es, nullptr, nullptr, 2, n_dev, cfg->k_cache, kvb, st)) != DASH_OK) return rc;
         if ((rc = dash_scatter(W.QKV + (int64_t)(Hq + Hkv) * D * es, n, kvb, nq * es, nullptr, nullptr, 2, n_dev, cfg->v_cache, kvb, st)) != DASH_OK) return rc;

@@ -341,3 +341,28 @@ def test_layer_step_other_rules_with_every_row_written(mode, n):
     assert np.array_equal(bufs.tok_next[:k].cpu().numpy(), tok.numpy()[idx]) and np.array_equal(bufs.pos_next[:k].cpu().numpy(), pos.numpy()[idx])
     a = int(mask[:lens[0]].sum())
     assert bufs.cu_next.tolist() == [0, a, a, k]
+
+
+@pytest.mark.parametrize("offset", [0, 4, 2], ids=["aligned", "8_bytes", "4_bytes"])
+@pytest.mark.parametrize("shape", [wl.LayerShape(d=512, Hq=4, Hkv=4, D=64, rope_base=1.0e4, dtype=torch.bfloat16, m=512),
+                                   wl.LayerShape(d=512, Hq=8, Hkv=2, D=128, rope_base=1.0e6, dtype=torch.bfloat16, m=512)], ids=["heads_of_64", "heads_of_128"])
+def test_kv_cache_rows_are_the_projections_for_every_head_size_and_alignment(shape, offset):
+    """The K and V columns that a step leaves in its workspace and the cache rows are the same bits, whether the projection's epilogue writes
+    them (8-byte aligned buffers) or a copy does; rows past the batch stay untouched."""
+    n, pad = 300, 20
+    cu = wl.cu_from_lengths([n])
+    layer = dash.Layer(shape, wl.layer_weights(shape, 81), DEV, tau=0.0)
+    width = shape.Hkv * shape.D
+    flat = [torch.full(((n + pad) * width + offset,), 7.0, dtype=shape.dtype, device=DEV) for _ in range(2)]
+    K, V = (x[offset:].view(n + pad, shape.Hkv, shape.D) for x in flat)
+    layer.set_kv_cache(K, V)
+    H = wl.hidden_states(n + pad, shape.d, 81, shape.dtype).to(DEV)             # room for more rows than the batch holds
+    pos = torch.arange(n + pad, dtype=torch.int32, device=DEV)
+    bufs = StepBuffers(layer, n + pad, 1, n + pad, shape.dtype)
+    x_full = torch.zeros(n + pad, shape.d, dtype=shape.dtype, device=DEV)
+    run_step(layer, H, pos, pos, cu.to(DEV), n, x_full, bufs)
+    nq = (shape.Hq + 2 * shape.Hkv) * shape.D
+    QKV = bufs.view(bufs.lay.QKV, n + pad, nq, shape.dtype)[:n]
+    q = shape.Hq * shape.D
+    assert torch.equal(K[:n].reshape(n, width), QKV[:, q:q + width]) and torch.equal(V[:n].reshape(n, width), QKV[:, q + width:])
+    assert (K[n:] == 7.0).all() and (V[n:] == 7.0).all()
