@@ -130,6 +130,7 @@ struct GemmArgs {
     int n_tiles;                 // tiles along the output columns
     void* C; int64_t ldc;        // PLAIN / ROPE / SWIGLU output (elements)
     int out_f32;                 // PLAIN: C is fp32 (else bf16)
+    int w_early;                 // W may be read before the kernel in front is complete
     const int32_t* n_dev;        // device: true number of rows (<= n), or null
     int* status;
     int groups;                  // > 0: tiles are cut along K (see Work)
@@ -184,8 +185,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
     const uint32_t slot = bars + 8 * (2 * kGStages + 4);
     volatile uint32_t* slot_gen = reinterpret_cast<volatile uint32_t*>(smem_raw + (slot - smem_u32(smem_raw)));
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    // the kernel behind (attention, tail pass) may set itself up while this one drains; this kernel itself is launched in plain
-    // stream order: started early behind the attention or row kernels it measured 15 us slower per launch
+    // the kernel behind may set itself up while this one drains, as this one does while the kernel in front of it drains
     pdl_launch_dependents();
     const int rank = (int)cluster_rank();                  // 0: the pair's even CTA (issues the MMAs, owns the full / acc_empty barriers)
     if (warp == 1) {
@@ -218,21 +218,37 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
             bool ok = true;
             Work w(pair, n_pairs, m_tiles, n_tiles, ksteps, g.groups);
             int mt, nt, k0, k1;
+            // A caller's W (not one that a kernel of this step has made) is complete before the step's first kernel lets anything start
+            // behind it.  So the first stages' W tiles are asked for while the kernel in front, which makes A, still drains.
+            bool first = true;
             while (ok && w.next(mt, nt, k0, k1)) {
                 const int m0 = mt * 2 * kGM + rank * kGM;
-                for (int k = k0; k < k1 && ok; ++k, ++it) {
-                    const int s = it % kGStages;
-                    if (it >= kGStages) ok = mbar_wait(empty(s), ((it / kGStages) - 1) & 1, kGWait);
-                    if (!ok) break;
-                    const uint32_t sA = base + s * kGStageBytes, sB = sA + kGABytes;
+                auto load_w = [&](int s, int k) {
                     if (rank == 0) mbar_arrive_expect_tx(full(s), 2 * kGStageBytes);     // both CTAs' bytes land on this barrier
-                    tma_load_2d_pair(sA, &mapA, full(s), k * kGK, m0);
 #pragma unroll
                     for (int c = 0; c < kGN / 2 / 64; ++c) {
                         // SWIGLU: columns 0-127 of the tile (the even CTA's half) are gate features nt * 128 .., columns 128-255 the same features of "up"
                         const int col = (EPI == GEMM_SWIGLU) ? (rank * g.e.m + nt * 128 + c * 64) : (nt * kGN + rank * (kGN / 2) + c * 64);
-                        tma_load_2d_pair(sB + c * (kGK * 128), &mapW, full(s), col, k * kGK);
+                        tma_load_2d_pair(base + s * kGStageBytes + kGABytes + c * (kGK * 128), &mapW, full(s), col, k * kGK);
                     }
+                };
+                auto load_a = [&](int s, int k) { tma_load_2d_pair(base + s * kGStageBytes, &mapA, full(s), k * kGK, m0); };
+                int k = k0;
+                if (first) {
+                    const int pre = min(kGStages, k1 - k0);
+                    if (!g.w_early) pdl_wait();
+                    for (int s = 0; s < pre; ++s) load_w(s, k0 + s);
+                    if (g.w_early) pdl_wait();
+                    for (int s = 0; s < pre; ++s) load_a(s, k0 + s);
+                    k += pre; it += pre;
+                    first = false;
+                }
+                for (; k < k1 && ok; ++k, ++it) {
+                    const int s = it % kGStages;
+                    if (it >= kGStages) ok = mbar_wait(empty(s), ((it / kGStages) - 1) & 1, kGWait);
+                    if (!ok) break;
+                    load_w(s, k);
+                    load_a(s, k);
                 }
             }
             if (!ok) atomicExch(g.status, DASH_ERR_TIMEOUT);
@@ -272,6 +288,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
         const int q = warp & 3, half = (warp - 2) >> 2;           // q: the TMEM lane quarter this warp may read
         const uint32_t lane_base = (uint32_t)(q * 32) << 16;
         const uint32_t stage = base + kGStages * kGStageBytes + (warp - 2) * kGEpiBytes;
+        pdl_wait();
         int n_true = g.n;
         if (g.n_dev) { const int nd = *g.n_dev; if (nd < n_true) n_true = nd; }
         const int r8 = lane >> 3, c8 = lane & 7;                  // eight lanes per row: row r8 + 4 i, chunk c8
@@ -651,8 +668,7 @@ static int launch_gemm(const CUtensorMap& ma, const CUtensorMap& mw, GemmArgs g,
     g.groups = gemm_groups(m_tiles, g.n_tiles, (g.K + kGK - 1) / kGK, pairs, g.part != nullptr);
     if (g.groups) pairs = g.groups * m_tiles;
     else if (pairs > tiles) pairs = tiles;
-    gemm_kernel<EPI><<<2 * pairs, kGThreads, smem, st>>>(ma, mw, g);
-    return cudaGetLastError() == cudaSuccess ? DASH_OK : DASH_ERR_CUDA;
+    return launch_pdl(gemm_kernel<EPI>, 2 * pairs, kGThreads, (size_t)smem, st, ma, mw, g) == cudaSuccess ? DASH_OK : DASH_ERR_CUDA;
 }
 
 bool gemm_shape_ok(GemmEpilogueKind kind, int64_t n, int64_t N, int64_t K, int64_t lda, int64_t ldw, const GemmEpilogue& e) {
@@ -680,6 +696,7 @@ int gemm_bf16(GemmEpilogueKind kind, const void* A, int64_t lda, const void* W, 
     g.n = (int)n; g.N = (int)N; g.K = (int)K;
     g.n_tiles = kind == GEMM_SWIGLU ? e.m / 128 : (int)((N + kGN - 1) / kGN);
     g.C = C; g.ldc = ldc; g.n_dev = n_dev; g.e = e; g.out_f32 = out_f32 ? 1 : 0;
+    g.w_early = out_f32 ? 0 : 1;         // (fp32 out: W is a bf16 copy made in this step)
     g.part = sc ? sc->part : nullptr; g.arrived = sc ? sc->arrived : nullptr; g.groups = 0;
     g.status = status_word_ptr();
     if (!g.status) return DASH_ERR_CUDA;

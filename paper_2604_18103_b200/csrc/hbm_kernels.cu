@@ -243,6 +243,8 @@ __global__ void __launch_bounds__(1024)
 select_keep_count_kernel(const float* __restrict__ r, const int32_t* __restrict__ cu, int S,
                          const int32_t* __restrict__ keep_counts, int keep_first, int keep_last,
                          uint8_t* __restrict__ mask, int halt_high) {
+    ptx::pdl_launch_dependents();
+    ptx::pdl_wait();
     const int s = blockIdx.x;
     const int a = cu[s], b = cu[s + 1], ns = b - a;
     if (ns <= 0) return;
@@ -836,7 +838,7 @@ extern "C" int dash_select(const float* r, int64_t n, const int32_t* cu_seqlens,
         select_threshold_kernel<<<grid, 256, 0, st>>>(r, n, cu_seqlens, S, tau, keep_first, keep_last, mask_out, halt_high);
     } else {
         if (!keep_counts) return DASH_ERR_INVALID_ARG;
-        select_keep_count_kernel<<<S, 1024, 0, st>>>(r, cu_seqlens, S, keep_counts, keep_first, keep_last, mask_out, halt_high);
+        DASH_CUDA_TRY(launch_pdl(select_keep_count_kernel, S, 1024, 0, st, r, cu_seqlens, S, keep_counts, keep_first, keep_last, mask_out, halt_high));
     }
     DASH_CUDA_TRY(cudaGetLastError());
     return DASH_OK;
@@ -1011,6 +1013,8 @@ namespace dash {
 __global__ void __launch_bounds__(256)
 sums_to_score_kernel(const float4* __restrict__ sums, int n_sum_tiles, int64_t n, int mode, float eps, float* __restrict__ r_out,
                      FusedThreshold ft, const int32_t* __restrict__ n_dev, float* __restrict__ inv_rms_out, float inv_d, float rms_eps) {
+    ptx::pdl_launch_dependents();
+    ptx::pdl_wait();
     if (n_dev) { int64_t nd = *n_dev; if (nd < n) n = nd; }
     // eight lanes per row: the row's partial sums lie next to each other
     const int sub = threadIdx.x & 7;
@@ -1043,8 +1047,8 @@ int launch_sums_to_score(const float4* sums, int n_sum_tiles, int64_t n, dash_no
     int64_t blocks = (n + 31) / 32, cap = (int64_t)sm_count() * 8;
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
-    sums_to_score_kernel<<<(int)blocks, 256, 0, st>>>(sums, n_sum_tiles, n, (int)mode, eps, r_out, ft, n_dev, inv_rms_out, 1.0f / d, rms_eps);
-    return cudaGetLastError() == cudaSuccess ? DASH_OK : DASH_ERR_CUDA;
+    return launch_pdl(sums_to_score_kernel, (int)blocks, 256, 0, st, sums, n_sum_tiles, n, (int)mode, eps, r_out, ft, n_dev, inv_rms_out, 1.0f / d,
+                      rms_eps) == cudaSuccess ? DASH_OK : DASH_ERR_CUDA;
 }
 
 // Fused tail of the block step (see delta_tail_kernel).  Preconditions checked by the caller: threshold rule, every row

@@ -175,6 +175,7 @@ struct PrologueArgs {
 __global__ void __launch_bounds__(256)
 prologue_kernel(const PrologueArgs a, const RopeFreqs fr) {
     ptx::pdl_wait();                         // launched to get onto the SMs while the kernel in front drains
+    ptx::pdl_launch_dependents();            // only now: the projection behind reads the caller's weights before it has waited for this kernel
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int cta = (int)blockIdx.x;
     if (cta == 0) {
