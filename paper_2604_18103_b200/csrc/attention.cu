@@ -97,6 +97,7 @@ __global__ void __launch_bounds__(1024)
 attention_plan_kernel(const int32_t* __restrict__ cu, int S, int Hq, int4* __restrict__ plan, int* __restrict__ n_items,
                       unsigned int* __restrict__ ticket, int64_t max_entries) {
     pdl_launch_dependents();
+    pdl_wait();
     attention_plan_items<1024>(cu, S, Hq, plan, n_items, ticket, max_entries);
 }
 
@@ -532,9 +533,8 @@ static int attention_plan(const int32_t* cu_seqlens, int S, int64_t n, int Hq, v
     if (n == 0) return DASH_OK;
     if (!ws || ((uintptr_t)ws % 256) || ws_bytes < 256 + plan_bytes(n, S)) return DASH_ERR_WORKSPACE;
     if ((int64_t)plan_entries(n, S) * Hq > 0x7fffffffLL) return DASH_ERR_UNSUPPORTED;
-    attention_plan_kernel<<<1, 1024, 0, st>>>(cu_seqlens, S, Hq, (int4*)((char*)ws + 256), (int*)((char*)ws + 4), (unsigned int*)ws,
-                                              (int64_t)plan_entries(n, S));
-    return cudaGetLastError() == cudaSuccess ? DASH_OK : DASH_ERR_CUDA;
+    return launch_pdl(attention_plan_kernel, 1, 1024, 0, st, cu_seqlens, S, Hq, (int4*)((char*)ws + 256), (int*)((char*)ws + 4), (unsigned int*)ws,
+                      (int64_t)plan_entries(n, S)) == cudaSuccess ? DASH_OK : DASH_ERR_CUDA;
 }
 
 static int attention_impl(const void* Q, const void* K, const void* V, void* O, float* lse,

@@ -56,6 +56,7 @@ delta_norm_kernel(const char* __restrict__ U, const char* __restrict__ H, int64_
                   FusedThreshold ft, const int32_t* __restrict__ n_dev, int aliased) {
     const int lane = threadIdx.x & 31;
     const int wpb = blockDim.x >> 5;
+    ptx::pdl_launch_dependents();
     if (n_dev) { int64_t nd = *n_dev; if (nd < n) n = nd; }
     const bool need_h = (mode == DASH_NORM_REL) || (Hres != nullptr);
     constexpr int CH = 4;
@@ -451,6 +452,137 @@ compact_kernel(const uint8_t* __restrict__ mask, int64_t n_upper, const int32_t*
                 warp_copy_row4(rs.src[q] + (int64_t)s_src[k] * rs.src_ld[q], rs.dst[q] + (int64_t)(base + k) * rs.dst_ld[q], rb, lane);
             first_warp = (first_warp + count) % NWARPS;
         }
+    }
+}
+
+// The same compaction as two kernels: the lists first, the rows behind them.  For inputs whose mask a CTA can count through from the
+// start (up to kCompactTwoMaxRows) and a caller that asks for the index list.  The rows are then dealt out evenly to all warps of the
+// machine: in compact_kernel a CTA goes through ticket, mask, look-back and only then its rows, 2.6 times over for 49 664 tokens, and
+// a row of 1 KB (a token's keys or values of four heads) is an item with two loads in flight per lane.
+// Both in us (in a graph, L2 flushed; rows of 7 KB, + two of 1 KB, + one of 7 KB): 1000 tokens 14.3 / 16.4 / 20.5 in one kernel and 14.3 / 14.3 / 14.3 in
+// two, 4000 tokens 14.4 / 16.4 / 18.5 and 16.4 / 16.4 / 18.4, 8192 22.5 / 26.7 / 39.9 and 24.6 / 28.7 / 38.9, 20 000 28.7 / 36.9 / 51.2 and 26.7 / 32.8 / 45.1,
+// 131 072 94 / 115 / 164 and 78 / 94 / 154: two kernels up to one tile of the lists and from the size on where compact_kernel takes more than
+// one wave of tiles.
+constexpr int64_t kCompactTwoMaxRows = 262144, kCompactOneMaxRows = 16384;
+constexpr int kListTile = 2048, kListThreads = 512;      // four tokens per thread
+__global__ void __launch_bounds__(kListThreads)
+compact_lists_kernel(const uint8_t* __restrict__ mask, int64_t n_upper, const int32_t* __restrict__ cu_in, int S, const int32_t* __restrict__ pos_in,
+                     int32_t* __restrict__ pos_out, const int32_t* __restrict__ tok_in, int32_t* __restrict__ tok_out, int32_t* __restrict__ idx_out,
+                     int32_t* __restrict__ cu_out, int32_t* __restrict__ n_out_dev, int aligned) {
+    __shared__ int s_warp[kListThreads / 32], s_part[kListThreads / 32], s_before[kListThreads];
+    __shared__ unsigned char s_bits[kListThreads];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    ptx::pdl_launch_dependents();
+    ptx::pdl_wait();
+    int64_t n = cu_in[S];
+    if (n > n_upper) n = n_upper;
+    const int64_t t0 = (int64_t)blockIdx.x * kListTile;
+    if (t0 >= n && blockIdx.x != 0) return;
+    const int64_t t_end = (t0 + kListTile < n) ? t0 + kListTile : n;
+    const bool last = t_end >= n;
+    // active tokens in front of this tile, from the mask itself
+    int front = 0;
+    if (aligned) {
+        const uint4* mv = reinterpret_cast<const uint4*>(mask);
+        const int nv = (int)(t0 >> 4);
+#pragma unroll 1
+        for (int v0 = tid; v0 < nv; v0 += 8 * kListThreads) {
+            uint4 w[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) w[k] = v0 + k * kListThreads < nv ? ld_nc_v4(mv + v0 + k * kListThreads) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) front += nonzero_bytes(w[k].x) + nonzero_bytes(w[k].y) + nonzero_bytes(w[k].z) + nonzero_bytes(w[k].w);
+        }
+    } else {
+        for (int64_t t = tid; t < t0; t += kListThreads) front += mask[t] != 0;
+    }
+    // own tokens
+    const int64_t t = t0 + 4 * tid;
+    unsigned int bits = 0;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) bits |= (t + e < n && mask[t + e] != 0) ? 1u << e : 0u;
+    const int mine = __popc(bits);
+    int inc = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) { const int x = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += x; }
+    front = __reduce_add_sync(0xffffffffu, front);
+    if (lane == 31) s_warp[warp] = inc;
+    if (lane == 0) s_part[warp] = front;
+    __syncthreads();
+    int base = 0, before = inc - mine, count = 0;
+#pragma unroll
+    for (int w = 0; w < kListThreads / 32; ++w) { base += s_part[w]; before += w < warp ? s_warp[w] : 0; count += s_warp[w]; }
+    s_before[tid] = before;
+    s_bits[tid] = (unsigned char)bits;
+    int k = base + before;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        if (bits >> e & 1) {
+            idx_out[k] = (int32_t)(t + e);
+            if (pos_out) pos_out[k] = pos_in[t + e];
+            if (tok_out) tok_out[k] = tok_in[t + e];
+            ++k;
+        }
+    }
+    __syncthreads();
+    // new sequence boundaries: cu_out[s] = number of active tokens before cu_in[s]
+    for (int s = tid; s <= S; s += kListThreads) {
+        int64_t c = cu_in[s];
+        if (c > n) c = n;
+        if ((c >= t0 && c < t_end) || (last && c == t_end)) {
+            const int p = (int)(c - t0);
+            const int v = base + (c >= t_end ? count : s_before[p >> 2] + __popc(s_bits[p >> 2] & ((1u << (p & 3)) - 1u)));
+            cu_out[s] = v;
+            if (s == S && n_out_dev) *n_out_dev = v;
+        }
+    }
+}
+
+// Row idx[k] of every source to row k of its destination, k < *n_out.  A warp's item: 4 KB of a row, or as many rows of up to 2 KB (a power of
+// two) as 2 KB hold: eight or four 16-byte loads per lane in flight.
+__global__ void __launch_bounds__(256, 3)
+move_rows_kernel(const RowStreams rs, const int32_t* __restrict__ idx, const int32_t* __restrict__ n_out) {
+    ptx::pdl_launch_dependents();
+    ptx::pdl_wait();
+    const int n = *n_out, lane = threadIdx.x & 31;
+    const int nw = (int)gridDim.x * 8;
+    int64_t it = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);      // next item of this warp, counted from the first of the current tensor
+#pragma unroll 1
+    for (int q = 0; q < rs.count; ++q) {
+        const int64_t rb = rs.row_bytes[q];
+        const int vpr = (int)(rb >> 4);
+        int64_t items;
+        if (rs.vec16[q] && rb <= 2048 && (vpr & (vpr - 1)) == 0) {
+            const int sh = 31 - __clz(vpr), rows = 128 >> sh;
+            items = (n + rows - 1) / rows;
+#pragma unroll 1
+            for (; it < items; it += nw) {
+                const int k0 = (int)it * rows;
+                uint4 r[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int v = i * 32 + lane, k = k0 + (v >> sh);
+                    if (k < n) r[i] = ld_nc_v4(rs.src[q] + (int64_t)idx[k] * rs.src_ld[q] + ((v & (vpr - 1)) << 4));
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int v = i * 32 + lane, k = k0 + (v >> sh);
+                    if (k < n) st_v4(rs.dst[q] + (int64_t)k * rs.dst_ld[q] + ((v & (vpr - 1)) << 4), r[i]);
+                }
+            }
+        } else if (rs.vec16[q]) {
+            const int64_t pieces = (rb + kPieceBytes - 1) / kPieceBytes;
+            items = n * pieces;
+#pragma unroll 1
+            for (; it < items; it += nw) {
+                const int64_t k = it / pieces, off = (it - k * pieces) * kPieceBytes;
+                warp_copy_row16(rs.src[q] + (int64_t)idx[k] * rs.src_ld[q] + off, rs.dst[q] + k * rs.dst_ld[q] + off, rb - off < kPieceBytes ? rb - off : kPieceBytes, lane);
+            }
+        } else {
+            items = n;
+            for (; it < items; it += nw) warp_copy_row4(rs.src[q] + (int64_t)idx[it] * rs.src_ld[q], rs.dst[q] + it * rs.dst_ld[q], rb, lane);
+        }
+        it -= items;
     }
 }
 
@@ -909,6 +1041,13 @@ static int compact_impl(const uint8_t* mask, int64_t n, const int32_t* cu_in, in
     }
     if (!ws || ((uintptr_t)ws % 256) || ws_bytes < compact_ws_bytes(n)) return DASH_ERR_WORKSPACE;
     cudaStream_t st = (cudaStream_t)stream;
+    if (idx_out && n_rows > 0 && n > 0 && (n <= kListTile || n > kCompactOneMaxRows) && n <= kCompactTwoMaxRows && !stall) {
+        const int grid = (int)((n + kListTile - 1) / kListTile);
+        DASH_CUDA_TRY(launch_pdl(compact_lists_kernel, grid, kListThreads, 0, st, mask, n, cu_in, S, pos_in, pos_out, tok_in, tok_out, idx_out, cu_out,
+                                 n_out_dev, aligned16(mask) ? 1 : 0));
+        DASH_CUDA_TRY(launch_pdl(move_rows_kernel, 3 * sm_count(), 256, 0, st, rs, (const int32_t*)idx_out, (const int32_t*)(cu_out + S)));
+        return DASH_OK;
+    }
     const int TILE = compact_tile_for(n);
     const int tiles = (int)((n + TILE - 1) / TILE) > 0 ? (int)((n + TILE - 1) / TILE) : 1;
     const bool direct = n <= kCompactDirectMaxRows && !stall;

@@ -499,3 +499,33 @@ def test_select_keep_count_at_the_edges_of_its_key_cache(n, kind):
             m = dash.dash_select(r.to(DEV), cu.to(DEV), mode, keep_counts=torch.tensor([k], dtype=torch.int32, device=DEV))
             ref = oc.select(r.numpy(), cu, oc.KEEP_COUNT, keep_counts=[k], halt_high=high)
             assert np.array_equal(m.cpu().numpy(), ref), (n, kind, k, high)
+
+
+@pytest.mark.parametrize("n", [1, 31, 2047, 2048, 2049, 16384, 16385, 33000, 262144, 262145])
+@pytest.mark.parametrize("keep", [0.0, 0.3, 1.0])
+def test_compact_lists_and_rows_at_the_edges_of_their_tiles(n, keep):
+    """Row widths that go by in pieces (7168 bytes), several to an item (16, 1024, 2048), alone (96: not a power of two vectors) and word by word
+    (20); a mask that starts on any byte; fewer valid rows than the buffers hold.  Everything equals the oracle's lists exactly."""
+    g = torch.Generator().manual_seed(n)
+    pad = 5 if n > 8 else 0
+    lens = [n // 3, 0, n - pad - n // 3]
+    cu = wl.cu_from_lengths(lens)
+    total = int(cu[-1])
+    mask = (torch.rand(n + 3, generator=g) < keep).to(torch.uint8) * 3                 # any non-zero byte keeps
+    widths = [1024, 20, 96, 16] if n > 60000 else ([7168, 1024, 20, 96] if keep != 0.3 else [7168, 16, 2048, 20])
+    rows = [torch.randint(0, 256, (n, w), generator=g, dtype=torch.uint8).to(DEV) for w in widths]
+    pos, tok = torch.randint(0, 1 << 20, (n,), generator=g, dtype=torch.int32), torch.randperm(n, generator=g).to(torch.int32)
+    for off in (0, 3):
+        m = mask.to(DEV)[off:off + n]
+        mh = m.cpu().numpy()[:total] != 0
+        idx = np.flatnonzero(mh)
+        out = [torch.full_like(r, 9) for r in rows]
+        c = dash.dash_compact(m, cu.to(DEV), rows=[r.view(torch.int32) for r in rows], rows_out=[r.view(torch.int32) for r in out],
+                              pos_in=pos.to(DEV), tok_in=tok.to(DEV))
+        k = idx.size
+        assert int(c["n_out"].item()) == k and np.array_equal(c["idx"][:k].cpu().numpy(), idx)
+        assert np.array_equal(c["pos_out"][:k].cpu().numpy(), pos.numpy()[idx]) and np.array_equal(c["tok_out"][:k].cpu().numpy(), tok.numpy()[idx])
+        assert c["cu_out"].tolist() == [int(mh[:int(x)].sum()) for x in cu]
+        sel = torch.from_numpy(idx).to(DEV)
+        for r, o in zip(rows, out):
+            assert torch.equal(o[:k], r[sel]) and (o[k:] == 9).all(), r.shape
