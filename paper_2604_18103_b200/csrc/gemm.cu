@@ -619,12 +619,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
     }
 }
 
+// (cos, sin) of every position 0 .. n - 1
 __global__ void __launch_bounds__(256)
-row_prep_kernel(const int32_t* __restrict__ pos, int64_t n, int half, RopeFreqs fr, float2* __restrict__ table, const char* __restrict__ H,
-                int64_t ldh_b, int nvec, float inv_d, float eps, float* __restrict__ inv_rms, const int32_t* __restrict__ n_dev) {
-    pdl_launch_dependents();
-    const int wpb = blockDim.x >> 5;
-    row_prep_rows(pos, n, half, fr, table, H, ldh_b, nvec, inv_d, eps, inv_rms, n_dev, (int64_t)blockIdx.x * wpb + (threadIdx.x >> 5), (int64_t)gridDim.x * wpb);
+rope_table_kernel(int64_t n, int half, RopeFreqs fr, float2* __restrict__ table) {
+    row_prep_rows(nullptr, n, half, fr, table, nullptr, 0, 0, 0.f, 0.f, nullptr, nullptr, (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5), (int64_t)gridDim.x * 8);
 }
 
 static int make_map_2d_bf16(CUtensorMap* map, const void* basep, uint64_t inner, uint64_t outer, uint64_t ld_elems, uint32_t box_inner,
@@ -708,14 +706,12 @@ int gemm_bf16(GemmEpilogueKind kind, const void* A, int64_t lda, const void* W, 
     }
 }
 
-int launch_row_prep(const int32_t* pos, int64_t n, int D, double rope_base, float2* table, const void* H, int64_t ldh, int d, float rms_eps,
-                    float* inv_rms, const int32_t* n_dev, cudaStream_t st) {
+int launch_rope_table(int64_t n, int D, double rope_base, float2* table, cudaStream_t st) {
     RopeFreqs fr;
     for (int i = 0; i < D / 2; ++i) fr.inv_freq[i] = pow(rope_base, -2.0 * i / D);
     int64_t blocks = (n + 7) / 8, cap = (int64_t)sm_count() * 8;
     if (blocks > cap) blocks = cap;
-    if (blocks < 1) blocks = 1;
-    row_prep_kernel<<<(int)blocks, 256, 0, st>>>(pos, n, D / 2, fr, table, (const char*)H, ldh * 2, d * 2 / 16, 1.0f / d, rms_eps, inv_rms, n_dev);
+    rope_table_kernel<<<(int)blocks, 256, 0, st>>>(n, D / 2, fr, table);
     return cudaGetLastError() == cudaSuccess ? DASH_OK : DASH_ERR_CUDA;
 }
 

@@ -322,7 +322,7 @@ extern "C" int dash_fold_norm_weight(const void* W, const void* rms_weight, int 
 
 extern "C" int dash_rope_table(double rope_base, int D, int64_t n_pos, void* table, void* stream) {
     if (!table || ((uintptr_t)table % 8) || n_pos < 1 || n_pos > 0x7fffffffLL || !(rope_base > 0.0) || (D != 64 && D != 128)) return DASH_ERR_INVALID_ARG;
-    return launch_row_prep(nullptr, n_pos, D, rope_base, (float2*)table, nullptr, 0, 0, 0.f, nullptr, nullptr, (cudaStream_t)stream);
+    return launch_rope_table(n_pos, D, rope_base, (float2*)table, (cudaStream_t)stream);
 }
 
 extern "C" int dash_layer_workspace(const dash_layer_cfg* cfg, int64_t n, int S, dash_layer_ws_layout* out) {
@@ -472,11 +472,12 @@ static int attention_to_O(const dash_layer_cfg* cfg, const void* H_in, const int
         }
         // rotary embedding on the Q and K heads
         const AttnCopies cp = {pa.ap.q, pa.ap.k, pa.ap.v, Hq, Hkv};
-        if (bf && D == 128) rope_kernel<true, 128><<<rows_grid8(n), 256, 0, st>>>(W.QKV, nq * es, pos_in, n, heads, fr, n_dev, cp);
-        else if (bf) rope_kernel<true, 64><<<rows_grid8(n), 256, 0, st>>>(W.QKV, nq * es, pos_in, n, heads, fr, n_dev, cp);
-        else if (D == 128) rope_kernel<false, 128><<<rows_grid8(n), 256, 0, st>>>(W.QKV, nq * es, pos_in, n, heads, fr, n_dev, cp);
-        else rope_kernel<false, 64><<<rows_grid8(n), 256, 0, st>>>(W.QKV, nq * es, pos_in, n, heads, fr, n_dev, cp);
-        DASH_CUDA_TRY(cudaGetLastError());
+        auto rope = [&](auto kernel) {       // in plain order: started early, with the attention kernel behind it, a small layer took 52.5 us instead of 48.3
+            kernel<<<rows_grid8(n), 256, 0, st>>>(W.QKV, nq * es, pos_in, n, heads, fr, n_dev, cp);
+            return cudaGetLastError();
+        };
+        DASH_CUDA_TRY(bf ? (D == 128 ? rope(rope_kernel<true, 128>) : rope(rope_kernel<true, 64>))
+                         : (D == 128 ? rope(rope_kernel<false, 128>) : rope(rope_kernel<false, 64>)));
     }
     if (cfg->k_cache && !cache_fused) {
         const int64_t kvb = (int64_t)Hkv * D * es;
