@@ -129,7 +129,6 @@ attention_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
     volatile uint32_t* abort_gen = reinterpret_cast<volatile uint32_t*>(smem_gen + L::kBars + 68);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    pdl_launch_dependents();                               // the kernel behind may set itself up while this one drains
     volatile int* item_gen = reinterpret_cast<volatile int*>(smem_gen + L::kBars + 72);
 
     if (warp == 4) {
@@ -148,6 +147,10 @@ attention_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    // The kernel behind may set itself up while this one drains, from here on and not before: this CTA holds its TMEM now.  Beside two
+    // CTAs for heads of 64 an SM has the registers and the shared memory for a CTA of the decode kernel, which takes 256 columns ahead
+    // of its wait for this grid; let in earlier it could take them in front of a CTA that it then waits for.
+    pdl_launch_dependents();
     pdl_wait();                                            // set-up done; from here on the kernel in front (plan, projection) has completed
     const uint32_t tmem = *tmem_slot_gen;
     const uint32_t tS = tmem, tP = tmem, tO = tmem + 128;

@@ -92,6 +92,31 @@ def test_decode_head_dim_64_no_grouping_and_wide_grouping():
     _decode_case([1500], 8, 1, 64, 5, pad=3)
 
 
+@pytest.mark.parametrize("D", [64, 128])
+def test_decode_right_behind_prefill_attention(D):
+    """Decoding enqueued directly behind a prefill attention on the same caches, several times over without a pause (for heads of 64 the decode
+    kernel's CTAs fit onto the SMs beside the attention kernel's): both results are the bits of calls made one at a time."""
+    Hq, Hkv, S, L = 8, 8, 12, 700
+    cu = wl.cu_from_lengths([L] * S)
+    g = torch.Generator().manual_seed(17)
+    Q, K, V = (torch.randn(S * L, h, D, generator=g).to(torch.bfloat16).to(DEV) for h in (Hq, Hkv, Hkv))
+    q, cu = Q[L - 1::L].contiguous(), cu.to(DEV)
+    ws_a = dash.workspace(dash.dash_workspace_bytes(dash.WS_ATTENTION, S * L, S, Hq, Hkv, D), DEV)
+    ws_d = dash.workspace(dash.dash_workspace_bytes(dash.WS_DECODE, S * L, S, Hq, Hkv, D), DEV)
+    O = dash.dash_varlen_attention(Q, K, V, cu, L, ws=ws_a)
+    torch.cuda.synchronize()
+    out = dash.dash_decode_attention(q, K, V, cu, ws=ws_d)
+    torch.cuda.synchronize()
+    assert_close_rms(out.float().cpu().numpy(), O[L - 1::L].float().cpu().numpy(), "the last row of every sequence")
+    runs = [(torch.empty_like(O), torch.empty_like(out)) for _ in range(8)]
+    for a, d in runs:
+        dash.dash_varlen_attention(Q, K, V, cu, L, O=a, ws=ws_a)
+        dash.dash_decode_attention(q, K, V, cu, out=d, ws=ws_d)
+    torch.cuda.synchronize()
+    for a, d in runs:
+        assert torch.equal(a, O) and torch.equal(d, out)
+
+
 def test_block_step_emits_the_kv_cache_rows_a_decode_step_reads():
     w = wl.config2(T=600, seed=41, shape=wl.MINI)
     w.cu = wl.cu_from_lengths([250, 350])
