@@ -59,32 +59,89 @@ def test_decode_few_long_sequences_one_item_per_cta():
     _decode_case([40000, 30001, 20000, 9000], 28, 4, 128, 7, pad=3)
 
 
-def test_decode_large_batch_takes_the_planned_path():
-    # more sequences than the CTAs plan for themselves: items come from the plan kernel, by ticket
-    g = torch.Generator().manual_seed(6)
-    lengths = torch.randint(0, 700, (45,), generator=g).tolist()
-    lengths[3] = 0
-    lengths[10] = 9000
-    _decode_case(lengths, 14, 2, 128, 6, pad=7)
+def _large_batch(S, seed, long_at=10):
+    """Lengths of S caches up to 700 rows, one of 9000; empty where the self-planning warp's lanes begin and end their groups of 32 sequences."""
+    lengths = torch.randint(1, 700, (S,), generator=torch.Generator().manual_seed(seed)).tolist()
+    for s in (3, 31, 32, 63, 64, 95, 96, 127, S - 1):
+        if s < S:
+            lengths[s] = 0
+    lengths[long_at] = 9000
+    return lengths
+
+
+@pytest.mark.parametrize("S", [33, 45, 64, 65, 96, 97, 127, 128])
+def test_decode_batch_that_the_ctas_plan_for_themselves(S):
+    # one to four sequences per lane of the planning warp; the last boundary is the warp's 129th at S = 128
+    _decode_case(_large_batch(S, S), 14, 2, 128, S, pad=7)
+    _decode_case(_large_batch(S, S + 1, long_at=S - 2), 8, 8, 64, S + 1)
+
+
+@pytest.mark.parametrize("S", [129, 200, 300])
+def test_decode_large_batch_takes_the_planned_path(S):
+    # more sequences than the CTAs plan for themselves (128): items come from the plan kernel, by ticket, and the merge finds them in its list
+    _decode_case(_large_batch(S, 6), 14, 2, 128, 6, pad=7)
+    _decode_case(_large_batch(S, 7, long_at=S - 2), 4, 4, 64, 7)
 
 
 def test_decode_random_batches_match_oracle():
-    """Seeded sweep over batch sizes on both sides of the self-planning limit, length mixes (many short, one long, equal,
+    """Seeded sweep over batch sizes on both sides of the self-planning limit (128), length mixes (many short, one long, equal,
     block-aligned), head groupings and head dims."""
     g = torch.Generator().manual_seed(2024)
-    for trial in range(16):
-        S = int(torch.randint(1, 41, (1,), generator=g))
+    for trial in range(24):
+        S = int(torch.randint(1, 41, (1,), generator=g)) if trial < 16 else int(torch.randint(41, 260, (1,), generator=g))
         kind = trial % 4
         if kind == 0:
-            lens = torch.randint(0, 3000, (S,), generator=g).tolist()
+            lens = torch.randint(0, 3000 if S <= 40 else 500, (S,), generator=g).tolist()
         elif kind == 1:
             lens = [int(torch.randint(1, 60000, (1,), generator=g))] + torch.randint(0, 300, (S - 1,), generator=g).tolist()
         elif kind == 2:
-            lens = [int(torch.randint(100, 9000, (1,), generator=g))] * S
+            lens = [int(torch.randint(100, 9000 if S <= 40 else 900, (1,), generator=g))] * S
         else:
-            lens = (torch.randint(0, 40, (S,), generator=g) * 128).tolist()
+            lens = (torch.randint(0, 40 if S <= 40 else 6, (S,), generator=g) * 128).tolist()
         Hkv, G, D = [1, 2, 4][trial % 3], [1, 4, 7, 8][trial % 4], [64, 128][trial % 2]
         _decode_case(lens, Hkv * G, Hkv, D, 100 + trial)
+
+
+@pytest.mark.parametrize("S", [1, 5, 40, 128])
+def test_decode_over_boundaries_that_the_call_in_front_writes(S):
+    """Decoding directly behind the compaction that shortens its caches: the decode kernel plans from the boundaries as they stand, while the
+    kernels that write them may still run, and has to make the plan again where they change.  Here they change in every round (other
+    masks into the same buffers), with rounds enqueued back to back; each result is the bits of a call made later on the same caches."""
+    Hq, Hkv, D, L = 8, 2, 128, 20000 // S
+    n = S * L
+    cu = wl.cu_from_lengths([L] * S).to(DEV)
+    g = torch.Generator(device=DEV).manual_seed(S)
+    K, V = (torch.randn(n, Hkv * D, generator=g, device=DEV).to(torch.bfloat16) for _ in range(2))
+    q = torch.randn(S, Hq, D, generator=g, device=DEV).to(torch.bfloat16)
+    masks = [(torch.rand(n, generator=g, device=DEV) < keep).to(torch.uint8) for keep in (0.9, 0.02, 0.5, 0.0, 1.0, 0.3)]
+    masks[2][:L] = 0                                       # the first sequence's cache is empty
+    Kc, Vc = torch.zeros_like(K), torch.zeros_like(V)
+    lists = {"idx": torch.zeros(n, dtype=torch.int32, device=DEV), "cu_out": torch.zeros(S + 1, dtype=torch.int32, device=DEV),
+             "n_out": torch.zeros(1, dtype=torch.int32, device=DEV)}
+    ws_c, ws_d = dash.workspace(dash.dash_workspace_bytes(dash.WS_COMPACT, n, S), DEV), dash.workspace(dash.dash_workspace_bytes(dash.WS_DECODE, n, S, Hq, Hkv, D), DEV)
+
+    def compact(m):
+        dash.dash_compact(m, cu, rows=[K, V], rows_out=[Kc, Vc], outputs=lists, ws=ws_c)
+
+    def decode(out):
+        return dash.dash_decode_attention(q, Kc.view(n, Hkv, D), Vc.view(n, Hkv, D), lists["cu_out"], out=out, ws=ws_d)
+
+    outs = [torch.empty_like(q) for _ in range(4 * len(masks))]
+    torch.cuda.synchronize()
+    for i, out in enumerate(outs):
+        compact(masks[i % len(masks)])
+        decode(out)
+    torch.cuda.synchronize()
+    for i, m in enumerate(masks):
+        compact(m)
+        torch.cuda.synchronize()
+        ref = decode(None)
+        torch.cuda.synchronize()
+        cu_m, k = lists["cu_out"].cpu(), int(lists["n_out"].item())
+        Oref, _ = oc.decode_attention(q.cpu(), Kc[:k].view(k, Hkv, D).cpu(), Vc[:k].view(k, Hkv, D).cpu(), cu_m)
+        assert_close_rms(ref.float().cpu().numpy(), Oref, f"mask {i}")
+        for out in outs[i::len(masks)]:
+            assert torch.equal(out, ref), i
 
 
 def test_decode_head_dim_64_no_grouping_and_wide_grouping():
