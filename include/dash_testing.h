@@ -28,6 +28,11 @@ int dash_testing_compact_stalled(const uint8_t* mask, int64_t n, const int32_t* 
                                  int32_t* idx_out, int32_t* cu_out, int32_t* n_out_dev,
                                  uint32_t spin_limit, void* ws, size_t ws_bytes, void* stream);
 
+/* Into how many shares a block step deals out the K steps (64 deep) of a bf16 projection C[n, N] = A[n, K] W[K, N] on the
+ * current device, 0: none, the projection runs in whole tiles (256 x 256).  A share runs through ceil(N / 256) * ceil(K / 64) /
+ * shares steps, tile after tile along N, for every row of tiles.  Pure host function. */
+int dash_testing_gemm_groups(int64_t n, int64_t N, int64_t K);
+
 #ifdef __cplusplus
 }
 #endif

@@ -24,6 +24,7 @@
 #include <math.h>
 
 #include "common.cuh"
+#include "dash_testing.h"
 #include "gemm.cuh"
 #include "prologue.cuh"
 #include "sm100_ptx.cuh"
@@ -716,3 +717,9 @@ int launch_rope_table(int64_t n, int D, double rope_base, float2* table, cudaStr
 }
 
 }  // namespace dash
+
+extern "C" int dash_testing_gemm_groups(int64_t n, int64_t N, int64_t K) {
+    using namespace dash;
+    if (n < 1 || N < 1 || K < 1) return 0;
+    return gemm_groups((int)((n + 2 * kGM - 1) / (2 * kGM)), (int)((N + kGN - 1) / kGN), (int)((K + kGK - 1) / kGK), sm_count() / 2, true);
+}

@@ -218,15 +218,41 @@ def test_block_step_shapes_without_whole_tiles(dtype):
     assert np.array_equal(b.tok_next[:k].cpu().numpy(), idx)
 
 
-@pytest.mark.parametrize("n", [100, 257, 523])
-@pytest.mark.parametrize("which", ["deep_output_and_down", "deep_qkv_and_gate_up"])
+def shares_of(n, N, K):
+    """(tiles along N, K steps of a tile, [(first, past the last)] step of every share) of a projection that is cut along K; no shares: it is not"""
+    tiles, steps, groups = -(-N // 256), -(-K // 64), dash.lib().dash_testing_gemm_groups(n, N, K)
+    return tiles, steps, [(i * tiles * steps // groups, (i + 1) * tiles * steps // groups) for i in range(groups)]
+
+
+def _straddling(n, N, K):
+    _, steps, shares = shares_of(n, N, K)
+    return sum(a // steps != (b - 1) // steps for a, b in shares)
+
+
+def _with_whole_tile_inside(n, N, K):
+    """shares that hold a whole tile between two parts of others"""
+    _, steps, shares = shares_of(n, N, K)
+    return sum(a % steps != 0 and b % steps != 0 and b // steps - -(-a // steps) >= 1 for a, b in shares)
+
+
+@pytest.mark.parametrize("which,n", [("deep_output_and_down", 100), ("deep_output_and_down", 257), ("deep_output_and_down", 523), ("deep_qkv_and_gate_up", 100),
+                                     ("deep_qkv_and_gate_up", 257), ("deep_qkv_and_gate_up", 523), ("uneven_output_and_down", 1400), ("uneven_qkv_and_gate_up", 1400)])
 def test_block_step_with_projections_cut_along_k(which, n):
     """Few column tiles over a deep K: the projections deal their K steps out to several pairs of CTAs, which add their partial tiles up (n: fewer
-    rows than half a tile, one row in a second row of tiles, three rows of tiles).  Two runs on the same workspace are bit-identical."""
+    rows than half a tile, one row in a second row of tiles, three rows of tiles; six rows of tiles over five column tiles, whose shares
+    begin in one tile and end in another).  Two runs on the same workspace are bit-identical."""
+    uneven = which.startswith("uneven")
     if which == "deep_output_and_down":
         sh = wl.LayerShape(d=512, Hq=64, Hkv=8, D=128, rope_base=1.0e6, dtype=torch.bfloat16, m=18944)
-    else:
+    elif which == "deep_qkv_and_gate_up":
         sh = wl.LayerShape(d=8192, Hq=4, Hkv=2, D=64, rope_base=1.0e6, dtype=torch.bfloat16, m=256)
+    elif which == "uneven_output_and_down":
+        sh = wl.LayerShape(d=1280, Hq=64, Hkv=8, D=128, rope_base=1.0e6, dtype=torch.bfloat16, m=8192)
+    else:
+        sh = wl.LayerShape(d=8192, Hq=12, Hkv=4, D=64, rope_base=1.0e6, dtype=torch.bfloat16, m=640)
+    deep = [((sh.Hq + 2 * sh.Hkv) * sh.D, sh.d), (2 * sh.m, sh.d)] if sh.d == 8192 else [(sh.d, sh.Hq * sh.D), (sh.d, sh.m)]
+    for N, K in deep:
+        assert shares_of(n, N, K)[2] and (_straddling(n, N, K) > 0) == uneven, (N, K)
     H, W, cu = wl.hidden_states(n, sh.d, 51, sh.dtype), _weights(sh, 51), wl.cu_from_lengths([n])
     if sh.d == 8192:
         # N(0, 0.02^2) entries over a depth of 8192 give queries and keys of standard deviation 1.8 and scores of 3.3, whose rounding
@@ -245,3 +271,36 @@ def test_block_step_with_projections_cut_along_k(which, n):
     assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
     assert np.max(np.abs(out[0][1].numpy() - ref["r"]) / ref["r"]) < 2e-2
     assert_close_h1(out[0][0].float().numpy(), ref["H1"], f"H' ({which}, n = {n})")
+
+
+@pytest.mark.parametrize("n", [1, 300, 701, 2100])
+def test_down_projection_cut_along_k_at_the_7b_shape(n):
+    """The FFN's down projection (depth 18944, 14 column tiles) against the same product in 64 bits of the activation that the step left in its
+    workspace: shares inside a tile, over a tile's end and (n = 2100) with a whole tile between two parts.  Every step on one workspace,
+    the largest first; two runs are bit-identical.  Bound: the result's rounding to bf16, 2^-8 of it, and 2^-24 of the products' absolute sum for each
+    of 18944 / 16 fp32 additions in a row (the MMA adds 16 products at a time), of which a random walk takes the square root."""
+    sh = wl.QWEN
+    assert {1: 0, 300: 1, 701: 1, 2100: 1}[n] == int(_straddling(n, sh.d, sh.m) > 0) and shares_of(n, sh.d, sh.m)[2]
+    assert n != 2100 or _with_whole_tile_inside(n, sh.d, sh.m) > 0
+    g = torch.Generator(device=DEV).manual_seed(n)
+    hd, kv = sh.Hq * sh.D, sh.Hkv * sh.D
+    W = {k: (torch.randn(*size, generator=g, device=DEV) * 0.02).to(sh.dtype) for k, size in
+         (("Wq", (sh.d, hd)), ("Wk", (sh.d, kv)), ("Wv", (sh.d, kv)), ("Wo", (hd, sh.d)), ("Wg", (sh.d, sh.m)), ("Wu", (sh.d, sh.m)), ("Wd", (sh.m, sh.d)))}
+    W["rms_w"] = W["rms2_w"] = torch.ones(sh.d, dtype=sh.dtype, device=DEV)
+    block = dash.Block(sh, W, DEV, tau=0.0)
+    b = BlockBuffers(block, 2100, 1)
+    out = []
+    for rows in (2100, n, n):
+        x_full = torch.zeros(rows, sh.d, dtype=sh.dtype, device=DEV)
+        H = torch.randn(rows, sh.d, generator=torch.Generator(device=DEV).manual_seed(1), device=DEV).to(sh.dtype)
+        tok = torch.arange(rows, dtype=torch.int32, device=DEV)
+        run_block(block, H, tok, tok, wl.cu_from_lengths([rows]).to(DEV), rows, x_full, b)
+        out.append(x_full)
+    assert torch.equal(out[1], out[2])
+    lay = dash.dash_block_workspace(block, n, 1)
+    view = lambda off, cols: b.ws[off:off + n * cols * 2].view(sh.dtype).view(n, cols)
+    act, F, Wd = view(lay.ACT, sh.m).double(), view(lay.F, sh.d).double(), W["Wd"].double()
+    ref, size = act @ Wd, act.abs() @ Wd.abs()
+    bound = 2.0 ** -8 * ref.abs() + 4 * 2.0 ** -24 * (sh.m / 16) ** 0.5 * size
+    worst = float(((F - ref).abs() / bound).max())
+    assert worst <= 1.0, worst
