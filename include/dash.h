@@ -299,6 +299,7 @@ int dash_rope_table(double rope_base, int D, int64_t n_pos, void* table, void* s
 typedef struct {
     size_t Hn, QKV, O, U, Ht, scratch, total;
 } dash_layer_ws_layout;
+/* `total` bytes serve a step of n rows and every step of fewer rows of the same shapes (whose offsets are those of their own n). */
 int dash_layer_workspace(const dash_layer_cfg* cfg, int64_t n, int S, dash_layer_ws_layout* out);
 
 /* H_in [n, d]: packed hidden states of the tokens entering the block, with
@@ -334,6 +335,7 @@ typedef struct {
     dash_layer_ws_layout attn;
     size_t GU, ACT, F, total;      /* gate | up [n, 2m], activation [n, m], FFN output [n, d] */
 } dash_block_ws_layout;
+/* As dash_layer_workspace (attn.total is where GU begins). */
 int dash_block_workspace(const dash_block_cfg* cfg, int64_t n, int S, dash_block_ws_layout* out);
 /* Arguments as dash_layer_step. */
 int dash_block_step(const dash_block_cfg* cfg, const void* H_in, const int32_t* tok_index_in,

@@ -639,8 +639,7 @@ static int make_map_2d_bf16(CUtensorMap* map, const void* basep, uint64_t inner,
                ? DASH_OK : DASH_ERR_CUDA;
 }
 
-// Scratch of tiles cut along K: two partial tiles per pair; a counter per tile, CTA and epilogue warp
-size_t gemm_split_part_bytes() { return (size_t)(sm_count() / 2) * 2 * (2 * kGM * kGN) * sizeof(float); }
+// Scratch of tiles cut along K: a counter per tile, CTA and epilogue warp; two partial tiles per pair (gemm_split_part_bytes)
 size_t gemm_split_count_bytes() { return align_up((size_t)(sm_count() / 2) * kGSplitMaxRounds * 2 * kGEpiWarps * sizeof(unsigned int), 256); }
 
 // Into how many groups of pairs the K steps are dealt out (0: whole tiles).  Whole tiles take ceil(tiles / P) rounds of `ksteps` steps, the last
@@ -656,6 +655,14 @@ static int gemm_groups(int m_tiles, int n_tiles, int ksteps, int P, bool can) {
     const long long whole = (tiles + P - 1) / P * ksteps, cut = ((long long)n_tiles * ksteps + groups - 1) / groups;
     return cut + kGSplitCost < whole ? groups : 0;
 }
+
+size_t gemm_split_part_bytes(int64_t n, int64_t N, int64_t K) {
+    if (n < 1 || N < 1 || K < 1 || n > 0x7fffffffLL || N > 0x7fffffffLL || K > 0x7fffffffLL) return 0;
+    const int m_tiles = (int)((n + 2 * kGM - 1) / (2 * kGM));
+    return (size_t)gemm_groups(m_tiles, (int)((N + kGN - 1) / kGN), (int)((K + kGK - 1) / kGK), sm_count() / 2, true) * m_tiles * 2 * (2 * kGM * kGN) * sizeof(float);
+}
+int gemm_tile_rows() { return 2 * kGM; }
+int64_t gemm_split_max_rows() { return (int64_t)(sm_count() / 2) * 2 * kGM; }
 
 template <int EPI>
 static int launch_gemm(const CUtensorMap& ma, const CUtensorMap& mw, GemmArgs g, cudaStream_t st) {

@@ -32,11 +32,14 @@ struct GemmEpilogue {
     int m = 0;
 };
 
-// Scratch of one GEMM at a time on one stream: part 16-byte aligned, gemm_split_part_bytes(); arrived gemm_split_count_bytes(), zero before the
-// first GEMM that uses it (every GEMM leaves it zero again).
+// Scratch of one GEMM at a time on one stream: part 16-byte aligned, gemm_split_part_bytes() of the GEMM (0: it runs in whole tiles); arrived
+// gemm_split_count_bytes(), zero before the first GEMM that uses it (every GEMM leaves it zero again).
 struct GemmSplit { float* part; unsigned int* arrived; };
-size_t gemm_split_part_bytes();
+size_t gemm_split_part_bytes(int64_t n, int64_t N, int64_t K);
 size_t gemm_split_count_bytes();
+// The scratch depends on n only through the number of rows of tiles, ceil(n / gemm_tile_rows()), and is 0 above gemm_split_max_rows()
+int gemm_tile_rows();
+int64_t gemm_split_max_rows();
 
 // true if the kernel takes this problem with this epilogue.  PLAIN: any N % 4 == 0, K % 8 == 0 (rows on 16-byte boundaries); the
 // fused epilogues: whole 256-column tiles (SWIGLU: m % 128 == 0) and K in steps of 64 -- otherwise the caller runs the projection

@@ -325,8 +325,20 @@ extern "C" int dash_rope_table(double rope_base, int D, int64_t n_pos, void* tab
     return launch_rope_table(n_pos, D, rope_base, (float2*)table, (cudaStream_t)stream);
 }
 
-extern "C" int dash_layer_workspace(const dash_layer_cfg* cfg, int64_t n, int S, dash_layer_ws_layout* out) {
-    if (!cfg_ok(cfg) || n < 0 || S < 1 || !out) return DASH_ERR_INVALID_ARG;
+namespace dash {
+
+// Scratch for the tiles that a step's projections cut along K: the most that one of them uses (m > 0: a block's, with its feed-forward)
+static size_t step_split_bytes(const dash_layer_cfg* cfg, int m, int64_t n) {
+    if (cfg->dt != DASH_BF16) return 0;
+    const int64_t d = cfg->d, hd = (int64_t)cfg->Hq * cfg->D, nq = (int64_t)(cfg->Hq + 2 * cfg->Hkv) * cfg->D;
+    size_t b = gemm_split_part_bytes(n, nq, d);
+    auto most = [&](size_t x) { if (x > b) b = x; };
+    most(gemm_split_part_bytes(n, d, hd));
+    if (m > 0) { most(gemm_split_part_bytes(n, 2 * (int64_t)m, d)); most(gemm_split_part_bytes(n, d, m)); }
+    return b;
+}
+
+static void layer_layout(const dash_layer_cfg* cfg, int64_t n, int S, size_t split, dash_layer_ws_layout* out) {
     const size_t es = cfg->dt == DASH_BF16 ? 2 : 4;
     const size_t nq = (size_t)(cfg->Hq + 2 * cfg->Hkv) * cfg->D;
     size_t off = 0;
@@ -341,13 +353,48 @@ extern "C" int dash_layer_workspace(const dash_layer_cfg* cfg, int64_t n, int S,
         off += conv_a_bytes(n, cfg->d > hd ? cfg->d : hd);
         off += conv_w_bytes(cfg->d, nq) + conv_w_bytes(hd, cfg->d);
     }
-    if (cfg->dt == DASH_BF16) off += gemm_split_part_bytes() + gemm_split_count_bytes();      // tiles of the projections cut along K
+    if (split) off += split + gemm_split_count_bytes();      // tiles of the projections cut along K
     off += step_compact_bytes(n, S, cfg->dt);
     off += align_up(dash_workspace_bytes(DASH_WS_ATTENTION, n, S, cfg->Hq, cfg->Hkv, cfg->D, cfg->dt), 256);
     off += align_up((size_t)n * (cfg->D / 2) * sizeof(float2), 256);              // (cos, sin) of every row for the QKV epilogue
     off += align_up((size_t)n * ((cfg->d + 127) / 128) * sizeof(float4), 256);    // per-row partial sums of the output-projection epilogue
     off += 2 * align_up((size_t)n * sizeof(float), 256);                          // row factors of the two folded norms
     out->total = off;
+}
+
+static void block_layout(const dash_block_cfg* cfg, int64_t n, int S, size_t split, dash_block_ws_layout* out) {
+    layer_layout(&cfg->attn, n, S, split, &out->attn);
+    const size_t es = cfg->attn.dt == DASH_BF16 ? 2 : 4;
+    size_t off = align_up(out->attn.total, 256);
+    out->GU = off;  off += align_up((size_t)n * 2 * cfg->m * es, 256);
+    out->ACT = off; off += align_up((size_t)n * cfg->m * es, 256);
+    out->F = off;   off += align_up((size_t)n * cfg->attn.d * es, 256);
+    if (cfg->attn.dt == DASH_F32) {        // bf16 copies of the operands of the feed-forward's projections
+        off += conv_a_bytes(n, cfg->m > cfg->attn.d ? cfg->m : cfg->attn.d);
+        off += conv_w_bytes(cfg->attn.d, 2 * (int64_t)cfg->m) > conv_w_bytes(cfg->m, cfg->attn.d) ? conv_w_bytes(cfg->attn.d, 2 * (int64_t)cfg->m) : conv_w_bytes(cfg->m, cfg->attn.d);
+    }
+    out->total = off;
+}
+
+// A workspace serves every step of at most n rows (a program sizes it once and goes on with the rows that stay), and the scratch of the cut
+// projections is not monotone in n: the most that total_of(rows) comes to for rows <= n.
+template <typename F>
+static size_t most_up_to(int64_t n, F total_of) {
+    size_t most = total_of(n);
+    int64_t rows = gemm_split_max_rows();
+    for (rows = rows < n ? rows : (n - 1) / gemm_tile_rows() * gemm_tile_rows(); rows > 0; rows -= gemm_tile_rows()) {
+        const size_t t = total_of(rows);
+        if (t > most) most = t;
+    }
+    return most;
+}
+
+}  // namespace dash
+
+extern "C" int dash_layer_workspace(const dash_layer_cfg* cfg, int64_t n, int S, dash_layer_ws_layout* out) {
+    if (!cfg_ok(cfg) || n < 0 || S < 1 || !out) return DASH_ERR_INVALID_ARG;
+    layer_layout(cfg, n, S, step_split_bytes(cfg, 0, n), out);
+    out->total = most_up_to(n, [&](int64_t rows) { dash_layer_ws_layout l; layer_layout(cfg, rows, S, step_split_bytes(cfg, 0, rows), &l); return l.total; });
     return DASH_OK;
 }
 
@@ -357,16 +404,15 @@ struct StepWs {
     dash_layer_ws_layout L;
     char *Hn, *QKV, *O, *U, *Ht, *compact_ws, *attn_ws;
     ConvScratch conv;
-    GemmSplit split;                 // part == null: fp32 tensors
+    GemmSplit split;                 // part == null: no projection of the step is cut
     size_t compact_bytes, attn_bytes;
     float2* rope_tab;
     float4* sums;
     float *inv_rms, *inv_rms2;
 };
 
-static int carve_ws(const dash_layer_cfg* cfg, int64_t n, int S, void* ws, StepWs* out) {
-    int rc = dash_layer_workspace(cfg, n, S, &out->L);
-    if (rc != DASH_OK) return rc;
+static void carve_ws(const dash_layer_cfg* cfg, int64_t n, int S, size_t split, void* ws, StepWs* out) {
+    layer_layout(cfg, n, S, split, &out->L);
     char* w = (char*)ws;
     out->Hn = w + out->L.Hn; out->QKV = w + out->L.QKV; out->O = w + out->L.O; out->U = w + out->L.U; out->Ht = w + out->L.Ht;
     out->conv = {nullptr, 0, nullptr, 0};
@@ -379,9 +425,9 @@ static int carve_ws(const dash_layer_cfg* cfg, int64_t n, int S, void* ws, StepW
         after += ab + w1 + w2;
     }
     out->split = {nullptr, nullptr};
-    if (cfg->dt == DASH_BF16) {
+    if (split) {
         out->split.part = (float*)after;
-        after += gemm_split_part_bytes();
+        after += split;
         out->split.arrived = (unsigned int*)after;         // directly in front of the look-back words: one clear takes both
         after += gemm_split_count_bytes();
     }
@@ -393,7 +439,6 @@ static int carve_ws(const dash_layer_cfg* cfg, int64_t n, int S, void* ws, StepW
     out->sums = (float4*)((char*)out->rope_tab + align_up((size_t)n * (cfg->D / 2) * sizeof(float2), 256));
     out->inv_rms = (float*)((char*)out->sums + align_up((size_t)n * ((cfg->d + 127) / 128) * sizeof(float4), 256));
     out->inv_rms2 = (float*)((char*)out->inv_rms + align_up((size_t)n * sizeof(float), 256));
-    return DASH_OK;
 }
 
 static int launch_rmsnorm(dash_dtype dt, const void* X, const void* weight, void* Y, int64_t n, int d, float eps, const int32_t* n_dev,
@@ -543,8 +588,8 @@ extern "C" int dash_layer_step(const dash_layer_cfg* cfg, const void* H_in, cons
     if (n > 0 && (!H_in || !pos_in || !tok_index_in || !x_full || !H_next || !tok_index_next || !pos_next || !r_out || !mask_out))
         return DASH_ERR_INVALID_ARG;
     StepWs W;
-    int rc = carve_ws(cfg, n, S, ws, &W);
-    if (rc != DASH_OK) return rc;
+    int rc;
+    carve_ws(cfg, n, S, step_split_bytes(cfg, 0, n), ws, &W);
     if (!ws || ((uintptr_t)ws % 256) || ws_bytes < W.L.total) return DASH_ERR_WORKSPACE;
     cudaStream_t st = (cudaStream_t)stream;
     const int es = cfg->dt == DASH_BF16 ? 2 : 4;
@@ -598,18 +643,8 @@ extern "C" int dash_layer_step(const dash_layer_cfg* cfg, const void* H_in, cons
 
 extern "C" int dash_block_workspace(const dash_block_cfg* cfg, int64_t n, int S, dash_block_ws_layout* out) {
     if (!block_cfg_ok(cfg) || n < 0 || S < 1 || !out) return DASH_ERR_INVALID_ARG;
-    int rc = dash_layer_workspace(&cfg->attn, n, S, &out->attn);
-    if (rc != DASH_OK) return rc;
-    const size_t es = cfg->attn.dt == DASH_BF16 ? 2 : 4;
-    size_t off = align_up(out->attn.total, 256);
-    out->GU = off;  off += align_up((size_t)n * 2 * cfg->m * es, 256);
-    out->ACT = off; off += align_up((size_t)n * cfg->m * es, 256);
-    out->F = off;   off += align_up((size_t)n * cfg->attn.d * es, 256);
-    if (cfg->attn.dt == DASH_F32) {        // bf16 copies of the operands of the feed-forward's projections
-        off += conv_a_bytes(n, cfg->m > cfg->attn.d ? cfg->m : cfg->attn.d);
-        off += conv_w_bytes(cfg->attn.d, 2 * (int64_t)cfg->m) > conv_w_bytes(cfg->m, cfg->attn.d) ? conv_w_bytes(cfg->attn.d, 2 * (int64_t)cfg->m) : conv_w_bytes(cfg->m, cfg->attn.d);
-    }
-    out->total = off;
+    block_layout(cfg, n, S, step_split_bytes(&cfg->attn, cfg->m, n), out);
+    out->total = most_up_to(n, [&](int64_t rows) { dash_block_ws_layout l; block_layout(cfg, rows, S, step_split_bytes(&cfg->attn, cfg->m, rows), &l); return l.total; });
     return DASH_OK;
 }
 
@@ -624,11 +659,12 @@ extern "C" int dash_block_step(const dash_block_cfg* cfg, const void* H_in, cons
         return DASH_ERR_INVALID_ARG;
     const dash_layer_cfg* a = &cfg->attn;
     dash_block_ws_layout BL;
-    int rc = dash_block_workspace(cfg, n, S, &BL);
-    if (rc != DASH_OK) return rc;
+    const size_t split = step_split_bytes(a, cfg->m, n);
+    int rc;
+    block_layout(cfg, n, S, split, &BL);
     if (!ws || ((uintptr_t)ws % 256) || ws_bytes < BL.total) return DASH_ERR_WORKSPACE;
     StepWs W;
-    if ((rc = carve_ws(a, n, S, ws, &W)) != DASH_OK) return rc;
+    carve_ws(a, n, S, split, ws, &W);
     cudaStream_t st = (cudaStream_t)stream;
     const int es = a->dt == DASH_BF16 ? 2 : 4;
     const int d = a->d, m = cfg->m;

@@ -75,3 +75,39 @@ def test_invalid_arguments_are_rejected_before_any_launch(lib):
     assert lib.dash_varlen_attention(*args(4, 3, 128, 1)) == 1
     assert lib.dash_status_string(3).decode().startswith("workspace")
     assert dash.dash_workspace_bytes(dash.WS_COMPACT, 131072) >= 131072 // 32 * 8
+
+
+def _cfgs(sh, dt):
+    c = dash.LayerCfg(d=sh[0], Hq=sh[1], Hkv=sh[2], D=sh[3], dt=dt, Wqkv=4096, Wo=4096, rms_weight=4096, rms_eps=1e-6, rope_base=1e4, scatter_which=2)
+    return c, dash.BlockCfg(attn=c, m=sh[4], Wgu=4096, Wd=4096, rms2_weight=4096)
+
+
+def _totals(lib, layer, block, n, S=1):
+    a, b = dash.LayerWsLayout(), dash.BlockWsLayout()
+    assert lib.dash_layer_workspace(ctypes.byref(layer), n, S, ctypes.byref(a)) == 0
+    assert lib.dash_block_workspace(ctypes.byref(block), n, S, ctypes.byref(b)) == 0
+    return a.total, b.total
+
+
+@pytest.mark.parametrize("dt", [dash.BF16, dash.F32], ids=["bf16", "fp32"])
+@pytest.mark.parametrize("shape", [(3584, 28, 4, 128, 18944), (512, 8, 2, 128, 1024), (8192, 4, 2, 64, 256)], ids=["7b", "mini", "deep"])
+def test_step_workspace_holds_what_the_step_can_use(lib, shape, dt):
+    """A step asks for its tensors and, where it cuts a projection along K, for the partial tiles (2 x 256 KB per pair of CTAs), else for none;
+    and a workspace of n rows serves every step of fewer rows."""
+    d, Hq, Hkv, D, m = shape
+    layer, block = _cfgs(shape, dt)
+    nq, hd, es = (Hq + 2 * Hkv) * D, Hq * D, 2 if dt == dash.BF16 else 4
+
+    def needs(n, ffn):
+        b = n * (3 * d + nq + hd) * es + n * (D // 2) * 8 + n * -(-d // 128) * 16 + 8 * n      # activations, rotary table, per-row sums and factors
+        b += n * (3 * m + d) * es if ffn else 0
+        if dt == dash.F32:                                                                     # bf16 copies of what is multiplied
+            b += (n * max(d, hd) + d * nq + hd * d + n * nq) * 2 + ((n * max(m, d) + d * 2 * m) * 2 if ffn else 0)
+            return b
+        projections = [(nq, d), (d, hd)] + ([(2 * m, d), (d, m)] if ffn else [])
+        return b + max(lib.dash_testing_gemm_groups(n, N, K) for N, K in projections) * -(-n // 256) * 2 * 256 * 1024
+
+    for n in (1, 2, 100, 256, 257, 701, 2368, 5376, 5377, 8192, 18944, 18945, 32768):
+        for ffn, total in enumerate(_totals(lib, layer, block, n)):
+            most = max(needs(r, ffn) for r in [n, *range(256, min(n, 75 * 256), 256)])
+            assert most <= total <= most + 80 * n + 40000, (n, ffn)                            # lists, look-back words, alignment
