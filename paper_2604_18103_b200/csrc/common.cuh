@@ -43,8 +43,8 @@ inline bool set_max_smem_once(K kernel, int smem_bytes, std::atomic<uint64_t>& d
     return true;
 }
 
-// Launch of a kernel that calls pdl_wait() before its first global access: it may start while the kernel in front of it in
-// the stream drains (programmatic dependent launch); behind anything else it is an ordinary launch.
+// Launch of a kernel that calls pdl_wait() before its global accesses (but for those that sm100_ptx.cuh allows ahead of it): it may
+// start while the kernel in front of it in the stream drains (programmatic dependent launch); behind anything else it is an ordinary launch.
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t st, Args&&... args) {
     cudaLaunchConfig_t cfg = {};

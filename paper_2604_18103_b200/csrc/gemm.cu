@@ -219,8 +219,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
             bool ok = true;
             Work w(pair, n_pairs, m_tiles, n_tiles, ksteps, g.groups);
             int mt, nt, k0, k1;
-            // A caller's W (not one that a kernel of this step has made) is complete before the step's first kernel lets anything start
-            // behind it.  So the first stages' W tiles are asked for while the kernel in front, which makes A, still drains.
+            // w_early: the first stages' W tiles are asked for while the kernel in front, which makes A, still drains (see gemm.cuh for when)
             bool first = true;
             while (ok && w.next(mt, nt, k0, k1)) {
                 const int m0 = mt * 2 * kGM + rank * kGM;
@@ -689,7 +688,7 @@ bool gemm_shape_ok(GemmEpilogueKind kind, int64_t n, int64_t N, int64_t K, int64
 }
 
 int gemm_bf16(GemmEpilogueKind kind, const void* A, int64_t lda, const void* W, int64_t ldw, void* C, int64_t ldc, int64_t n, int64_t N,
-              int64_t K, const GemmEpilogue& e, const int32_t* n_dev, cudaStream_t st, bool out_f32, const GemmSplit* sc) {
+              int64_t K, const GemmEpilogue& e, const int32_t* n_dev, cudaStream_t st, bool out_f32, const GemmSplit* sc, bool w_early) {
     if (!gemm_shape_ok(kind, n, N, K, lda, ldw, e)) return DASH_ERR_UNSUPPORTED;
     if (!aligned16(A) || !aligned16(W)) return DASH_ERR_INVALID_ARG;
     if (out_f32 && kind != GEMM_PLAIN) return DASH_ERR_UNSUPPORTED;
@@ -702,7 +701,7 @@ int gemm_bf16(GemmEpilogueKind kind, const void* A, int64_t lda, const void* W, 
     g.n = (int)n; g.N = (int)N; g.K = (int)K;
     g.n_tiles = kind == GEMM_SWIGLU ? e.m / 128 : (int)((N + kGN - 1) / kGN);
     g.C = C; g.ldc = ldc; g.n_dev = n_dev; g.e = e; g.out_f32 = out_f32 ? 1 : 0;
-    g.w_early = out_f32 ? 0 : 1;         // (fp32 out: W is a bf16 copy made in this step)
+    g.w_early = w_early ? 1 : 0;
     g.part = sc ? sc->part : nullptr; g.arrived = sc ? sc->arrived : nullptr; g.groups = 0;
     g.status = status_word_ptr();
     if (!g.status) return DASH_ERR_CUDA;

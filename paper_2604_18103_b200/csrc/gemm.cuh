@@ -46,9 +46,13 @@ int64_t gemm_split_max_rows();
 // PLAIN and the element-wise work as passes of their own.
 bool gemm_shape_ok(GemmEpilogueKind kind, int64_t n, int64_t N, int64_t K, int64_t lda, int64_t ldw, const GemmEpilogue& e);
 // C (or the epilogue's outputs) = A[n, K] W[K, N], A and W bf16; ld* in elements; n_dev: device true row count or null;
-// out_f32 (PLAIN only): C is fp32 instead of bf16; sc: scratch that lets the kernel cut tiles along K (null: whole tiles only)
+// out_f32 (PLAIN only): C is fp32 instead of bf16; sc: scratch that lets the kernel cut tiles along K (null: whole tiles only);
+// w_early: W may be read while the kernel in front of this one still runs.  Only for a W that no kernel of the step writes (a caller's weights),
+// behind a kernel of the step that has called pdl_wait() ahead of pdl_launch_dependents() (prologue_kernel): what made W is then
+// complete before anything of the step that is launched to start early can start.
 int gemm_bf16(GemmEpilogueKind kind, const void* A, int64_t lda, const void* W, int64_t ldw, void* C, int64_t ldc, int64_t n, int64_t N,
-              int64_t K, const GemmEpilogue& e, const int32_t* n_dev, cudaStream_t st, bool out_f32 = false, const GemmSplit* sc = nullptr);
+              int64_t K, const GemmEpilogue& e, const int32_t* n_dev, cudaStream_t st, bool out_f32 = false, const GemmSplit* sc = nullptr,
+              bool w_early = false);
 // dst (bf16, row stride ld_dst) = src (fp32, row stride ld_src) rounded to nearest even; cols % 4 == 0
 int launch_f32_to_bf16(const float* src, int64_t ld_src, void* dst, int64_t ld_dst, int64_t rows, int64_t cols, cudaStream_t st);
 // (cos, sin) of pos * base^(-2i/D) for the positions 0 .. n - 1 into table [n, D/2]

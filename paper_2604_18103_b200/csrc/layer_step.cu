@@ -141,12 +141,12 @@ struct ConvScratch { char* a; size_t a_bytes; char* w; size_t w_bytes; char* w2 
 static size_t conv_a_bytes(int64_t n, int64_t k_max) { return align_up((size_t)n * align_up((size_t)k_max, 8) * 2, 256); }
 static size_t conv_w_bytes(int64_t k, int64_t n_cols) { return align_up((size_t)k * align_up((size_t)n_cols, 8) * 2, 256); }
 
-// C = A W (plain).  bf16: the GEMM of gemm.cu as it is.  fp32: its operands are rounded to bf16 copies first (what the
+// C = A W (plain), W a matrix of the caller's.  bf16: the GEMM of gemm.cu as it is.  fp32: its operands are rounded to bf16 copies first (what the
 // attention kernel does with Q, K, V), the product accumulates in fp32 and is stored as fp32.
 static int project(dash_dtype dt, const void* A, int64_t lda, const void* W, int64_t ldw, void* C, int64_t ldc, int64_t n, int64_t N, int64_t K,
                    const int32_t* n_dev, const ConvScratch& cs, const GemmSplit& split, cudaStream_t st) {
     GemmEpilogue e;
-    if (dt == DASH_BF16) return gemm_bf16(GEMM_PLAIN, A, lda, W, ldw, C, ldc, n, N, K, e, n_dev, st, false, &split);
+    if (dt == DASH_BF16) return gemm_bf16(GEMM_PLAIN, A, lda, W, ldw, C, ldc, n, N, K, e, n_dev, st, false, &split, true);
     if ((K % 8) || (N % 4)) return DASH_ERR_UNSUPPORTED;
     const int64_t lda_b = K, ldw_b = (int64_t)align_up((size_t)N, 8);
     if ((size_t)n * lda_b * 2 > cs.a_bytes || (size_t)K * ldw_b * 2 > cs.w_bytes) return DASH_ERR_WORKSPACE;
@@ -174,8 +174,10 @@ struct PrologueArgs {
 };
 __global__ void __launch_bounds__(256)
 prologue_kernel(const PrologueArgs a, const RopeFreqs fr) {
+    // In this order: all in front of the step is complete before anything behind this kernel can start early, so that the step's projections
+    // may read the caller's weights (w_early, gemm.cuh) ahead of their own wait.
     ptx::pdl_wait();                         // launched to get onto the SMs while the kernel in front drains
-    ptx::pdl_launch_dependents();            // only now: the projection behind reads the caller's weights before it has waited for this kernel
+    ptx::pdl_launch_dependents();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int cta = (int)blockIdx.x;
     if (cta == 0) {
@@ -501,11 +503,11 @@ static int attention_to_O(const dash_layer_cfg* cfg, const void* H_in, const int
         // K rotated.
         if (cfg->rope_table) { e.rope_table = (const float2*)cfg->rope_table; e.rope_pos = pos_in; e.rope_len = cfg->rope_table_len; }
         e.row_scale = cfg->inv_rms_in ? cfg->inv_rms_in : W.inv_rms;
-        if ((rc = gemm_bf16(GEMM_ROPE, H_in, d, cfg->Wqkv, nq, W.QKV, nq, n, nq, d, e, n_dev, st, false, &W.split)) != DASH_OK) return rc;
+        if ((rc = gemm_bf16(GEMM_ROPE, H_in, d, cfg->Wqkv, nq, W.QKV, nq, n, nq, d, e, n_dev, st, false, &W.split, true)) != DASH_OK) return rc;
     } else if (fused) {
         // LN (read as RMSNorm), then Q | K | V = Hn Wqkv with the Q and K heads rotated on the accumulators
         if ((rc = launch_rmsnorm(cfg->dt, H_in, cfg->rms_weight, W.Hn, n, d, cfg->rms_eps, n_dev, st)) != DASH_OK) return rc;
-        if ((rc = gemm_bf16(GEMM_ROPE, W.Hn, d, cfg->Wqkv, nq, W.QKV, nq, n, nq, d, e, n_dev, st, false, &W.split)) != DASH_OK) return rc;
+        if ((rc = gemm_bf16(GEMM_ROPE, W.Hn, d, cfg->Wqkv, nq, W.QKV, nq, n, nq, d, e, n_dev, st, false, &W.split, true)) != DASH_OK) return rc;
     } else {
         const int heads = Hq + Hkv;
         if (bf) {
@@ -550,7 +552,7 @@ static int out_proj_residual(const dash_layer_cfg* cfg, const void* H_in, const 
     GemmEpilogue e;
     e.H = H_in; e.ldh = cfg->d; e.tok_index = idx; e.x_full = dst; e.ldx = cfg->d; e.sums = W.sums;
     if (cfg->dt != DASH_BF16 || !gemm_shape_ok(GEMM_RESID, n, cfg->d, hd, hd, cfg->d, e)) return DASH_ERR_UNSUPPORTED;
-    return gemm_bf16(GEMM_RESID, W.O, hd, cfg->Wo, cfg->d, nullptr, 0, n, cfg->d, hd, e, cu_in + S, st, false, &W.split);
+    return gemm_bf16(GEMM_RESID, W.O, hd, cfg->Wo, cfg->d, nullptr, 0, n, cfg->d, hd, e, cu_in + S, st, false, &W.split, true);
 }
 
 // r (and, threshold rule, the keep mask) from U and H, H~ = H + U into W.Ht; keep-count rule: the radix select on r
@@ -713,7 +715,7 @@ extern "C" int dash_block_step(const dash_block_cfg* cfg, const void* H_in, cons
         // gate | up projection with silu(gate) * up on the accumulators: the [n, 2m] intermediate is never stored; with the norm
         // folded in, the operand is H~ itself and the accumulators take the row factor 1 / rms first
         eg.row_scale = cfg->rms2_folded ? W.inv_rms2 : nullptr;
-        if ((rc = gemm_bf16(GEMM_SWIGLU, cfg->rms2_folded ? W.Ht : W.Hn, d, cfg->Wgu, 2 * (int64_t)m, ACT, m, n, 2 * (int64_t)m, d, eg, n_dev, st, false, &W.split)) != DASH_OK) return rc;
+        if ((rc = gemm_bf16(GEMM_SWIGLU, cfg->rms2_folded ? W.Ht : W.Hn, d, cfg->Wgu, 2 * (int64_t)m, ACT, m, n, 2 * (int64_t)m, d, eg, n_dev, st, false, &W.split, true)) != DASH_OK) return rc;
     } else {
         if ((rc = project(a->dt, W.Hn, d, cfg->Wgu, 2 * (int64_t)m, GU, 2 * (int64_t)m, n, 2 * (int64_t)m, d, n_dev, conv, W.split, st)) != DASH_OK) return rc;
         const int64_t total = n * (int64_t)(m / (16 / es));

@@ -218,8 +218,16 @@ __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.
 // Programmatic dependent launch.  A kernel launched with the stream-serialization attribute (launch_pdl) may be placed on an SM
 // while the kernel in front of it in the stream still runs: whatever it does before pdl_wait() -- barrier and TMEM set-up,
 // descriptor prefetch -- overlaps that kernel's tail; pdl_wait() returns once the kernel in front has completed and its writes
-// are visible (at once when there is none, or when the launch carried no attribute).  No global memory may be touched before it.
-// pdl_launch_dependents() lets the kernel behind start that early: once every CTA of this grid has executed it (or has exited).
+// are visible (at once when there is none, or when the launch carried no attribute).  pdl_launch_dependents() lets the kernel behind
+// start that early: once every CTA of this grid has executed it (or has exited).
+// Nothing global is written before pdl_wait(), and nothing read, but for
+//   - what is complete before any kernel that the reader could have overtaken was let in: a kernel that waits and only then lets the next
+//     one start (prologue_kernel, decode_kernel) has everything in front of itself behind it, for the kernels behind it too.  So
+//     the projections of a step read the caller's weights (w_early, gemm.cuh), the merge of the decoding the boundaries;
+//   - what is read again after the wait, with everything made from it thrown away if it was different: decode_kernel's boundaries
+//     (self_plan_confirm), and its prefetch into L2, which returns nothing.
+// A kernel that allocates TMEM lets the next one start only once it has its columns (the next one could take them in front of CTAs
+// that it then waits for), unless no CTA that allocates TMEM fits onto an SM beside its own (gemm_kernel: 225 KB of shared memory).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
