@@ -201,7 +201,7 @@ prologue_kernel(const PrologueArgs a, const RopeFreqs fr) {
             const float4* w = reinterpret_cast<const float4*>(a.rms_w);
             uint2* y = reinterpret_cast<uint2*>(a.Hn16) + t * a.nvec;
             float ss = 0.f;
-            for (int v = lane; v < a.nvec; v += 32) { const float4 c = x[v]; ss += c.x * c.x + c.y * c.y + c.z * c.z + c.w * c.w; }
+            for (int v = lane; v < a.nvec; v += 32) { const float4 c = x[v]; ss += c.x * c.x; ss += c.y * c.y; ss += c.z * c.z; ss += c.w * c.w; }      // as rmsnorm_kernel
             const float rs = rsqrtf(warp_sum(ss) * a.inv_d + a.eps);
             for (int v = lane; v < a.nvec; v += 32) {
                 const float4 c = x[v], g = w[v];

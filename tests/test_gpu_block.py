@@ -218,6 +218,26 @@ def test_block_step_shapes_without_whole_tiles(dtype):
     assert np.array_equal(b.tok_next[:k].cpu().numpy(), idx)
 
 
+def test_fp32_block_multiplies_the_same_normalised_rows_on_both_paths():
+    """fp32 tensors: the rows that the step's first kernel normalises and rounds to bf16 for the Q | K | V projection are to the bit what the norm in
+    front of the feed-forward, a pass of its own, gives for the same rows and weight.  (No update, Wo = 0, so that both norms see H; Wv the
+    identity, so that the value columns of the projection are its operand.)"""
+    sh = wl.LayerShape(d=256, Hq=2, Hkv=2, D=128, rope_base=1.0e4, dtype=torch.float32, m=128)
+    n = 16384
+    W = _weights(sh, 91)
+    W["Wv"], W["Wo"], W["rms2_w"] = torch.eye(sh.d), torch.zeros_like(W["Wo"]), W["rms_w"]
+    g = torch.Generator().manual_seed(91)
+    H = (torch.randn(n, sh.d, generator=g) * torch.exp(torch.randn(n, 1, generator=g))).to(DEV)
+    block = dash.Block(sh, W, DEV, tau=0.0)
+    b = BlockBuffers(block, n, 16)
+    tok = torch.arange(n, dtype=torch.int32, device=DEV)
+    cu = wl.cu_from_lengths([n // 16] * 16).to(DEV)
+    run_block(block, H, tok, tok % (n // 16), cu, n // 16, torch.zeros(n, sh.d, device=DEV), b)
+    view = lambda off, cols: b.ws[off:off + n * cols * 4].view(torch.float32).view(n, cols)
+    operand = view(b.lay.attn.QKV, 6 * 128)[:, 4 * 128:]
+    assert torch.equal(operand, view(b.lay.attn.Hn, sh.d).to(torch.bfloat16).float())
+
+
 def shares_of(n, N, K):
     """(tiles along N, K steps of a tile, [(first, past the last)] step of every share) of a projection that is cut along K; no shares: it is not"""
     tiles, steps, groups = -(-N // 256), -(-K // 64), dash.lib().dash_testing_gemm_groups(n, N, K)
