@@ -142,10 +142,15 @@ def _p(t: Optional[torch.Tensor]):
     return None if t is None else t.data_ptr()           # ctypes takes an int where the signature says c_void_p
 
 
+# The handle of torch.cuda.current_stream() without the Stream object around it, where this torch has the two (private) functions: a call on
+# a short cache is bound by the host, and half of its 15 us went into such wrappers
+_raw_stream, _device = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream():
-    # the handle of torch.cuda.current_stream() without the Stream object around it: a call on a short cache is bound by the host,
-    # and half of its 15 us went into such wrappers
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    if _raw_stream is None or _device is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(_device())
 
 
 def dtype_code(t: torch.Tensor) -> int:

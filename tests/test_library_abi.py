@@ -2,10 +2,13 @@
 the header declares, rejects bad arguments before touching a device, and its pure
 host helpers reproduce the paper's printed numbers."""
 import ctypes
+import importlib.util
 import os
 import re
+import types
 
 import pytest
+import torch
 
 from paper_2604_18103_b200 import build as dash_build
 from paper_2604_18103_b200 import dash
@@ -111,3 +114,14 @@ def test_step_workspace_holds_what_the_step_can_use(lib, shape, dt):
         for ffn, total in enumerate(_totals(lib, layer, block, n)):
             most = max(needs(r, ffn) for r in [n, *range(256, min(n, 75 * 256), 256)])
             assert most <= total <= most + 80 * n + 40000, (n, ffn)                            # lists, look-back words, alignment
+
+
+@pytest.mark.parametrize("missing", ["_cuda_getCurrentRawStream", "_cuda_getDevice"])
+def test_stream_handle_without_torchs_private_functions(monkeypatch, missing):
+    """A torch that lacks one of the two private functions behind the short way to the current stream's handle: the public way."""
+    monkeypatch.delattr(torch._C, missing, raising=False)
+    spec = importlib.util.spec_from_file_location("dash_on_another_torch", dash.__file__)
+    other = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(other)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=7))
+    assert other._stream() == 7
