@@ -138,8 +138,10 @@ typedef struct {
     int64_t     row_bytes, src_ld_bytes, dst_ld_bytes;
 } dash_rows;
 
-/* Exclusive prefix sum of mask (single pass, decoupled look-back) and stable
- * gather of the active rows.  Outputs (device): idx_out[k] = source row of
+/* Exclusive prefix sum of mask and stable gather of the active rows: in one pass (a
+ * tile's first output row counted from the mask in front of it or, longer inputs, found by
+ * decoupled look-back) or, for a caller that asks for idx_out and rows, up to 2048 and
+ * from 16385 to 262144 rows, in two (the lists, then the rows by idx_out).  Outputs (device): idx_out[k] = source row of
  * output row k (int32 [n]); cu_out int32 [S+1] = new packed boundaries;
  * n_out_dev int32 = number of active rows (= cu_out[S]).  pos / tok (int32 per
  * row: rotary position, row in the full-length buffer) are gathered when both
@@ -161,8 +163,9 @@ int dash_compact(const uint8_t* mask, int64_t n, const int32_t* cu_in, int S,
  * GPU that loads the library holds until the process exits (256 KiB + 512 B).
  *  - Limit: n <= DASH_COMPACT_STATIC_MAX_ROWS; larger inputs are rejected with
  *    DASH_ERR_TOO_LARGE before anything is enqueued.
- *  - Allocates nothing (no cudaMalloc / cudaFree, no allocating library routine); the
- *    part of the array a call uses is cleared on `stream` before its kernel runs.
+ *  - Allocates nothing (no cudaMalloc / cudaFree, no allocating library routine); what a
+ *    call uses of the array, if it looks back at all, is cleared on `stream` before its
+ *    kernel runs.
  *  - The first call on a device looks up the device address of the array (with that
  *    device current); make that first call before any stream capture begins.
  *  - All calls on one device share the array and it keeps the last call's contents:
@@ -271,9 +274,9 @@ typedef struct {
  * multiples of 64; the FFN width a multiple of 128) get the work that follows a projection on its accumulators: the rotary
  * embedding in the QKV projection; H~ and the score's row sums in the output projection; SwiGLU in the gate | up projection --
  * one rounding less per value, no U and no gate | up intermediate.  Other shapes (rows must still start on 16-byte boundaries:
- * d, Hq D, m multiples of 8) and fp32 tensors run the same GEMM kernel plain, with the norm, the rotary embedding, the residual
- * and the score as passes of their own; fp32 operands are rounded to bf16 copies in the workspace first (fp32 accumulation,
- * fp32 results), as the attention kernel does with Q, K, V. */
+ * d, Hq D, m multiples of 8) and fp32 tensors run the same GEMM kernel plain, with the rotary embedding, the residual and the
+ * score as passes of their own, and bf16 ones with the norm as one too; fp32 operands -- weights, normalised rows, the attention
+ * output -- are rounded to bf16 copies in the workspace (fp32 accumulation, fp32 results), as the attention kernel does with Q, K, V. */
 
 /* LN of Eq. 1 is read as RMSNorm, y = x / rms(x) * w.  Its weight w can be folded, once and ahead of time, into the
  * projection that follows the norm: W_out[i, j] = w[i] * W[i, j] for W, W_out [d, N] row-major of type dt (row strides ldw,
@@ -291,11 +294,20 @@ int dash_fold_norm_weight(const void* W, const void* rms_weight, int d, int64_t 
  * Asynchronous on `stream`.  DASH_ERR_INVALID_ARG for a null table, n_pos < 1, rope_base <= 0 or D not in {64, 128}. */
 int dash_rope_table(double rope_base, int D, int64_t n_pos, void* table, void* stream);
 
-/* Byte offsets of the intermediates inside the workspace of dash_layer_step
- * (for inspection by tests and tools).  Ht (H~ = H + U) is only written when the
- * halting rule is KEEP_COUNT or scatter_which is 0; with the threshold rule and
- * scatter_which = 2 the score, the residual, the scatter and the compaction run as
- * one pass that writes H~ straight to x_full and H_next. */
+/* Byte offsets of the intermediates inside the workspace of a step (for inspection by
+ * tests and tools).  QKV and O hold the rotated projections and the attention output after
+ * every step; the others only where the step has them in memory at all (what it does not
+ * write keeps whatever was there):
+ *  Hn  LN(H), of type dt: bf16 tensors with rms_folded = 0.  (fp32 tensors: the
+ *      normalised rows exist only as the projection's bf16 operand.)  After dash_block_step:
+ *      LN(H~), the feed-forward's operand, with rms2_folded = 0.
+ *  U   not where the output projection adds H itself: bf16 tensors, d a multiple of 256,
+ *      Hq D of 64, and, in dash_layer_step, scatter_which = 2 and x_full other than H_in
+ *      (THRESHOLD: also x_full = H_in); in dash_block_step, DASH_SIGNAL_ATTN.
+ *  Ht  H~ = H + U.  dash_block_step: always.  dash_layer_step: where U is written and
+ *      not (scatter_which = 2 and THRESHOLD), whose H~ goes straight to x_full and H_next;
+ *      where U is not written H~ goes straight to x_full, whatever the rule.
+ *  scratch  where what has no offset of its own begins. */
 typedef struct {
     size_t Hn, QKV, O, U, Ht, scratch, total;
 } dash_layer_ws_layout;

@@ -366,3 +366,32 @@ def test_kv_cache_rows_are_the_projections_for_every_head_size_and_alignment(sha
     q = shape.Hq * shape.D
     assert torch.equal(K[:n].reshape(n, width), QKV[:, q:q + width]) and torch.equal(V[:n].reshape(n, width), QKV[:, q + width:])
     assert (K[n:] == 7.0).all() and (V[n:] == 7.0).all()
+
+
+ODD = wl.LayerShape(d=520, Hq=3, Hkv=1, D=64, rope_base=1.0e4, dtype=torch.bfloat16)
+
+
+@pytest.mark.parametrize("in_place", [False, True], ids=["x_full", "x_full_is_H"])
+@pytest.mark.parametrize("scatter", [2, 0])
+@pytest.mark.parametrize("mode", [dash.SEL_THRESHOLD, dash.SEL_THRESHOLD_HALT_HIGH, dash.SEL_KEEP_COUNT])
+@pytest.mark.parametrize("shape,fold", [(wl.MINI, True), (wl.MINI, False), (ODD, False), (wl.TINY, False)], ids=["folded", "norm_as_a_pass", "odd", "fp32"])
+def test_layer_step_leaves_in_its_workspace_what_the_header_says(shape, fold, mode, scatter, in_place):
+    """Which of Hn, U and Ht a step writes, for every rule and path, and that Ht = H + U where both are there; the others keep what they held."""
+    n = 300
+    cu = wl.cu_from_lengths([n])
+    H = wl.hidden_states(n, shape.d, 95, shape.dtype).to(DEV)
+    H0 = H.clone()
+    layer = dash.Layer(shape, wl.layer_weights(shape, 95), DEV, sel_mode=mode, tau=0.3, scatter_which=scatter, fold_norms=fold,
+                       keep_counts=torch.tensor([n // 2], dtype=torch.int32, device=DEV))
+    bufs = StepBuffers(layer, n, 1, n, shape.dtype)
+    bufs.ws.fill_(0x3C)
+    tok = torch.arange(n, dtype=torch.int32, device=DEV)
+    run_step(layer, H, tok, tok, cu.to(DEV), n, H if in_place else torch.zeros_like(H), bufs)
+    got = {k: bufs.view(getattr(bufs.lay, k), n, shape.d, shape.dtype) for k in ("Hn", "U", "Ht")}
+    written = {k: not bool((v.view(torch.uint8) == 0x3C).all()) for k, v in got.items()}
+    bf, thr = shape.dtype == torch.bfloat16, mode == dash.SEL_THRESHOLD
+    fused_out = bf and shape.d % 256 == 0 and (shape.Hq * shape.D) % 64 == 0 and scatter == 2 and (thr or not in_place)
+    assert written == {"Hn": bf and not layer.rms_folded, "U": not fused_out, "Ht": not fused_out and not (scatter == 2 and thr)}
+    if written["Ht"]:
+        assert torch.equal(got["Ht"], (H0.float() + got["U"].float()).to(shape.dtype))
+    assert int(bufs.n_next.item()) == int(bufs.mask.sum())
