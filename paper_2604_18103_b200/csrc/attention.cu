@@ -570,15 +570,15 @@ static int attention_impl(const void* Q, const void* K, const void* V, void* O, 
         __nv_bfloat16* kb = qb + (size_t)n * Hq * D;
         __nv_bfloat16* vb = kb + (size_t)n * Hkv * D;
         if (!planned) {                          // (a planned call finds its copies there: the step's rotary pass wrote them)
-        const int cap = sm_count() * 8;
-        auto cvt = [&](const void* src, int64_t ld, __nv_bfloat16* dst, int cols) {
-            int64_t total = n * (cols / 4);
-            int grid = (int)((total + 255) / 256);
-            if (grid > cap) grid = cap;
-            f32_to_bf16_rows_kernel<<<grid, 256, 0, st>>>((const float*)src, ld, dst, cols, n, cols);
-        };
-        cvt(Q, ldq, qb, Hq * D); cvt(K, ldk, kb, Hkv * D); cvt(V, ldv, vb, Hkv * D);
-        DASH_CUDA_TRY(cudaGetLastError());
+            const int cap = sm_count() * 8;
+            auto cvt = [&](const void* src, int64_t ld, __nv_bfloat16* dst, int cols) {
+                int64_t total = n * (cols / 4);
+                int grid = (int)((total + 255) / 256);
+                if (grid > cap) grid = cap;
+                f32_to_bf16_rows_kernel<<<grid, 256, 0, st>>>((const float*)src, ld, dst, cols, n, cols);
+            };
+            cvt(Q, ldq, qb, Hq * D); cvt(K, ldk, kb, Hkv * D); cvt(V, ldv, vb, Hkv * D);
+            DASH_CUDA_TRY(cudaGetLastError());
         }
         q = qb; k = kb; v = vb;
         lq = (int64_t)Hq * D; lk = lv = (int64_t)Hkv * D;

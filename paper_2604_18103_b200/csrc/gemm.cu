@@ -20,7 +20,8 @@
 // 128 contiguous bytes, and what an epilogue reads is asked for a piece ahead.  With a lane per row in the loads and stores too (and
 // four warps) an epilogue took 23-30 thousand cycles (ROPE), 18-22 (RESID), 15 (SWIGLU), 7 (PLAIN) against 31 thousand of a
 // 3584-deep tile's MMAs: the QKV projection waited for it at every tile (41.9 thousand cycles per tile), and the last tile's showed
-// in every launch.  A tile's pieces come in loops: a launch with a tile per CTA runs their code once, and would wait for the instructions.
+// in every launch.  The fused epilogues' pieces of a tile come in loops: a launch with a tile per CTA runs their code once, and would
+// wait for the instructions (PLAIN, with little code per piece, is unrolled).
 #include <math.h>
 
 #include "common.cuh"

@@ -1062,12 +1062,8 @@ static int compact_impl(const uint8_t* mask, int64_t n, const int32_t* cu_in, in
     compact_kernel<T, DIRECT><<<tiles, kCompactThreads, 0, st>>>(mask, n, cu_in, S, rs, pos_in, pos_out, tok_in, tok_out, \
                                                                  idx_out, cu_out, n_out_dev, state, ticket, status, mask_vec16, spin_limit)
     if (direct) {
-        switch (TILE) {
-            case 256: DASH_LAUNCH_COMPACT(256, true); break;
-            case 128: DASH_LAUNCH_COMPACT(128, true); break;
-            case 64: DASH_LAUNCH_COMPACT(64, true); break;
-            default: DASH_LAUNCH_COMPACT(32, true); break;
-        }
+        if (TILE == 64) DASH_LAUNCH_COMPACT(64, true);          // (kCompactDirectMaxRows: tiles of 32 or 64)
+        else DASH_LAUNCH_COMPACT(32, true);
     } else {
         switch (TILE) {
             case 256: DASH_LAUNCH_COMPACT(256, false); break;
@@ -1190,20 +1186,17 @@ int launch_sums_to_score(const float4* sums, int n_sum_tiles, int64_t n, dash_no
                       rms_eps) == cudaSuccess ? DASH_OK : DASH_ERR_CUDA;
 }
 
-// Fused tail of the block step (see delta_tail_kernel).  Preconditions checked by the caller: threshold rule, every row
-// scattered, 16-byte aligned rows.  ws: the compaction workspace (ticket + one state word per 32-token tile); ws_is_clear: the
-// caller has already zeroed its first tail_ws_clear_bytes(n) on this stream (ahead of the kernels in front, so that this launch
-// follows a kernel directly and may start while that one drains).
+// Fused tail of the block step (see delta_tail_kernel).  Preconditions checked by the caller: every row scattered, 16-byte aligned
+// rows.  ws: the compaction workspace (ticket + one state word per tile), whose first tail_ws_clear_bytes(n) the caller has zeroed
+// on this stream (ahead of the kernels in front, so that this launch follows a kernel directly and may start while that one drains).
 // (tiles of kTailRows rows at the smallest)
 size_t tail_ws_clear_bytes(int64_t n) { return 256 + (size_t)((n + kTailRows - 1) / kTailRows > 0 ? (n + kTailRows - 1) / kTailRows : 1) * 8; }
 int launch_delta_tail(const void* U, const void* H, const uint8_t* mask_in, const float4* sums, int n_sum_tiles, int64_t n, int d, dash_dtype dt, dash_norm_mode mode, float eps, float tau,
                       int keep_first, int keep_last, const int32_t* cu_in, int S, const int32_t* tok_in, const int32_t* pos_in,
                       void* x_full, void* H_next, float* r_out, uint8_t* mask_out, int32_t* tok_next, int32_t* pos_next,
-                      int32_t* cu_next, int32_t* n_next, void* ws, size_t ws_bytes, bool ws_is_clear, cudaStream_t st, float* inv_next,
-                      float rms_eps) {
+                      int32_t* cu_next, int32_t* n_next, void* ws, size_t ws_bytes, cudaStream_t st, float* inv_next, float rms_eps) {
     const int es = dt == DASH_BF16 ? 2 : 4;
     if (!ws || ((uintptr_t)ws % 256) || ws_bytes < tail_ws_clear_bytes(n)) return DASH_ERR_WORKSPACE;
-    if (!ws_is_clear) DASH_CUDA_TRY(cudaMemsetAsync(ws, 0, tail_ws_clear_bytes(n), st));
     TailArgs a;
     a.mask_in = mask_in; a.sums = sums; a.n_sum_tiles = n_sum_tiles;
     a.U = (const char*)U; a.H = (const char*)H; a.ldU_b = a.ldH_b = (int64_t)d * es; a.nvec = d * es / 16; a.mode = (int)mode; a.eps = eps;

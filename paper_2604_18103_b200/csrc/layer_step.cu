@@ -129,8 +129,7 @@ int launch_sums_to_score(const float4* sums, int n_sum_tiles, int64_t n, dash_no
 int launch_delta_tail(const void* U, const void* H, const uint8_t* mask_in, const float4* sums, int n_sum_tiles, int64_t n, int d, dash_dtype dt, dash_norm_mode mode, float eps, float tau,
                       int keep_first, int keep_last, const int32_t* cu_in, int S, const int32_t* tok_in, const int32_t* pos_in,
                       void* x_full, void* H_next, float* r_out, uint8_t* mask_out, int32_t* tok_next, int32_t* pos_next,
-                      int32_t* cu_next, int32_t* n_next, void* ws, size_t ws_bytes, bool ws_is_clear, cudaStream_t st, float* inv_next,
-                      float rms_eps);
+                      int32_t* cu_next, int32_t* n_next, void* ws, size_t ws_bytes, cudaStream_t st, float* inv_next, float rms_eps);
 size_t tail_ws_clear_bytes(int64_t n);
 int attention_planned(const void* Q, const void* K, const void* V, void* O, float* lse, int64_t ldq, int64_t ldk, int64_t ldv, int64_t ldo,
                       const int32_t* cu_seqlens, int S, int64_t n, int64_t max_seqlen, int Hq, int Hkv, int D, float scale, dash_dtype dt,
@@ -609,14 +608,14 @@ extern "C" int dash_layer_step(const dash_layer_cfg* cfg, const void* H_in, cons
             if (rc == DASH_OK)
                 return launch_delta_tail(nullptr, nullptr, nullptr, W.sums, d / 128, n, d, cfg->dt, cfg->norm_mode, cfg->norm_eps, cfg->tau,
                                          cfg->keep_first, cfg->keep_last, cu_in, S, tok_index_in, pos_in, x_full, H_next, r_out, mask_out,
-                                         tok_index_next, pos_next, cu_next, n_next_dev, W.compact_ws, W.compact_bytes, true, st,
+                                         tok_index_next, pos_next, cu_next, n_next_dev, W.compact_ws, W.compact_bytes, st,
                                          cfg->inv_rms_next, cfg->rms_eps);
             if (rc != DASH_ERR_UNSUPPORTED) return rc;
             // fp32, or shapes without whole 256-column tiles: U through the plain GEMM, then r, H~, the rule, scatter and compaction in one pass
             if ((rc = out_proj_U(cfg, cu_in, S, n, W, st)) != DASH_OK) return rc;
             return launch_delta_tail(W.U, H_in, nullptr, nullptr, 0, n, d, cfg->dt, cfg->norm_mode, cfg->norm_eps, cfg->tau, cfg->keep_first,
                                      cfg->keep_last, cu_in, S, tok_index_in, pos_in, x_full, H_next, r_out, mask_out, tok_index_next,
-                                     pos_next, cu_next, n_next_dev, W.compact_ws, W.compact_bytes, true, st, nullptr, cfg->rms_eps);
+                                     pos_next, cu_next, n_next_dev, W.compact_ws, W.compact_bytes, st, nullptr, cfg->rms_eps);
         }
         if (cfg->inv_rms_next) return DASH_ERR_UNSUPPORTED;      // the row factors come out of the fused tail pass (threshold rule, every row scattered)
         if (every_row && x_full != H_in &&      // (H~ over H itself in another order: only once every row of H has been read)
@@ -629,7 +628,7 @@ extern "C" int dash_layer_step(const dash_layer_cfg* cfg, const void* H_in, cons
             if ((rc = dash_select(r_out, n, cu_in, S, cfg->sel_mode, cfg->tau, cfg->keep_counts, cfg->keep_first, cfg->keep_last, mask_out, st)) != DASH_OK) return rc;
             return launch_delta_tail(nullptr, nullptr, mask_out, nullptr, 0, n, d, cfg->dt, cfg->norm_mode, cfg->norm_eps, cfg->tau, cfg->keep_first,
                                      cfg->keep_last, cu_in, S, tok_index_in, pos_in, x_full, H_next, nullptr, nullptr, tok_index_next,
-                                     pos_next, cu_next, n_next_dev, W.compact_ws, W.compact_bytes, true, st, nullptr, cfg->rms_eps);
+                                     pos_next, cu_next, n_next_dev, W.compact_ws, W.compact_bytes, st, nullptr, cfg->rms_eps);
         }
         if ((rc = out_proj_U(cfg, cu_in, S, n, W, st)) != DASH_OK) return rc;
         if ((rc = score_and_select(cfg, H_in, cu_in, S, n, r_out, mask_out, W, st)) != DASH_OK) return rc;
@@ -741,5 +740,5 @@ extern "C" int dash_block_step(const dash_block_cfg* cfg, const void* H_in, cons
     // for the tokens that stay, to the next block's packed buffer -- one pass, keep decisions taken from mask_out
     return launch_delta_tail(F, W.Ht, mask_out, nullptr, 0, n, d, a->dt, a->norm_mode, a->norm_eps, a->tau, a->keep_first, a->keep_last, cu_in, S,
                              tok_index_in, pos_in, x_full, H_next, nullptr, nullptr, tok_index_next, pos_next, cu_next, n_next_dev,
-                             W.compact_ws, W.compact_bytes, true, st, a->inv_rms_next, a->rms_eps);
+                             W.compact_ws, W.compact_bytes, st, a->inv_rms_next, a->rms_eps);
 }
