@@ -33,6 +33,9 @@ int dash_testing_compact_stalled(const uint8_t* mask, int64_t n, const int32_t* 
  * shares steps, tile after tile along N, for every row of tiles.  Pure host function. */
 int dash_testing_gemm_groups(int64_t n, int64_t N, int64_t K);
 
+/* Shared memory of a CTA of the decoding kernel for heads of D (-1: no such kernel).  Pure host function. */
+int dash_testing_decode_smem_bytes(int D);
+
 #ifdef __cplusplus
 }
 #endif

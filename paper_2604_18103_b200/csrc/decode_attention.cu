@@ -10,6 +10,7 @@
 #include <math.h>
 
 #include "common.cuh"
+#include "dash_testing.h"
 #include "sm100_ptx.cuh"
 
 namespace dash {
@@ -160,6 +161,11 @@ struct DecSmem {
     static constexpr int kTileBytes = kDecBN * D * 2;
     static constexpr int kQ = 0, kK = kTileBytes, kV = 2 * kTileBytes, kBars = 3 * kTileBytes;
     static constexpr int kTotal = kBars + 128;
+    // What a launch asks for: so much that a third CTA does not fit onto an SM, whose TMEM holds two (kDecTmemCols each).  With heads of 64
+    // (50 KB) four fit.  Launched while the merge of the call in front still sits on some of the SMs, the CTAs stacked up on the others,
+    // where the third and fourth waited for columns with their share of the items, which nobody else takes: 8 heads of 64,
+    // in a graph, 33 caches of 1200 rows 36.7 us, 64 of 1000 72, 128 of 1000 112, one of 131 072 83; with two per SM 23.4, 45, 77, 52.
+    static constexpr int kLaunch = kTotal + 1024 > 80 * 1024 ? kTotal + 1024 : 80 * 1024;
 };
 
 template <int D>
@@ -548,8 +554,7 @@ static int make_map_heads_box(CUtensorMap* map, const void* base, int64_t rows, 
 template <int D>
 static int launch_decode(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const DecParams& p, int box_heads, int grid,
                          cudaStream_t st) {
-    using L = DecSmem<D>;
-    const int smem = L::kTotal + 1024;
+    const int smem = DecSmem<D>::kLaunch;
     static std::atomic<uint64_t> configured{0};
     if (!set_max_smem_once(decode_kernel<D>, smem, configured)) return DASH_ERR_CUDA;
     return launch_pdl(decode_kernel<D>, grid, kDecThreads, (size_t)smem, st, mq, mk, mv, p, box_heads) == cudaSuccess ? DASH_OK : DASH_ERR_CUDA;
@@ -630,4 +635,8 @@ extern "C" int dash_decode_attention(const void* q, const void* Kc, const void* 
     if (D == 128) DASH_CUDA_TRY(launch_pdl(decode_merge_kernel<128>, (int)mgrid, kMergeThreads, 0, st, mp));
     else DASH_CUDA_TRY(launch_pdl(decode_merge_kernel<64>, (int)mgrid, kMergeThreads, 0, st, mp));
     return DASH_OK;
+}
+
+extern "C" int dash_testing_decode_smem_bytes(int D) {
+    return D == 128 ? DecSmem<128>::kLaunch + (int)sizeof(SelfPlan) : D == 64 ? DecSmem<64>::kLaunch + (int)sizeof(SelfPlan) : -1;
 }

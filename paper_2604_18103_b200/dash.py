@@ -33,7 +33,7 @@ EXPORTS = [
     "dash_block_workspace", "dash_block_step", "dash_decode_attention", "dash_varlen_attention_indexed",
     "dash_keep_counts_device", "dash_fold_norm_weight", "dash_rope_table",
 ]
-TEST_HOOKS = ["dash_testing_compact_stalled", "dash_testing_gemm_groups"]        # include/dash_testing.h
+TEST_HOOKS = ["dash_testing_compact_stalled", "dash_testing_gemm_groups", "dash_testing_decode_smem_bytes"]        # include/dash_testing.h
 COMPACT_STATIC_MAX_ROWS = 1 << 20
 
 
@@ -121,6 +121,7 @@ def lib() -> ctypes.CDLL:
         L.dash_testing_compact_stalled.argtypes = [c_void_p, c_int64, c_void_p, c_int, c_void_p, c_void_p, c_void_p, ctypes.c_uint32,
                                                    c_void_p, c_size_t, c_void_p]
         L.dash_testing_gemm_groups.argtypes = [c_int64, c_int64, c_int64]
+        L.dash_testing_decode_smem_bytes.argtypes = [c_int]
         L.dash_workspace_bytes.restype = c_size_t
         L.dash_workspace_bytes.argtypes = [c_int, c_int64, c_int, c_int, c_int, c_int, c_int]
         _lib = L

@@ -125,3 +125,10 @@ def test_stream_handle_without_torchs_private_functions(monkeypatch, missing):
     spec.loader.exec_module(other)
     monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=7))
     assert other._stream() == 7
+
+
+@pytest.mark.parametrize("D", [64, 128])
+def test_an_sm_takes_as_many_decode_ctas_as_its_tensor_memory_holds(lib, D):
+    """Two, 256 of the SM's 512 columns each; a third CTA (228 KB of shared memory per SM, 1 KB of it the system's per CTA) would hold its share of the
+    caches' blocks back until one of the two has left."""
+    assert 228 * 1024 // (lib.dash_testing_decode_smem_bytes(D) + 1024) == 2
