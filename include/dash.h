@@ -140,8 +140,8 @@ typedef struct {
 
 /* Exclusive prefix sum of mask and stable gather of the active rows: in one pass (a
  * tile's first output row counted from the mask in front of it or, longer inputs, found by
- * decoupled look-back) or, for a caller that asks for idx_out and rows, up to 2048 and
- * from 16385 to 262144 rows, in two (the lists, then the rows by idx_out).  Outputs (device): idx_out[k] = source row of
+ * decoupled look-back) or, for a caller that asks for idx_out and rows, in two (the lists,
+ * then the rows by idx_out) at some sizes.  Outputs (device): idx_out[k] = source row of
  * output row k (int32 [n]); cu_out int32 [S+1] = new packed boundaries;
  * n_out_dev int32 = number of active rows (= cu_out[S]).  pos / tok (int32 per
  * row: rotary position, row in the full-length buffer) are gathered when both

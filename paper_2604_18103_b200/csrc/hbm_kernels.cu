@@ -459,11 +459,14 @@ compact_kernel(const uint8_t* __restrict__ mask, int64_t n_upper, const int32_t*
 // start (up to kCompactTwoMaxRows) and a caller that asks for the index list.  The rows are then dealt out evenly to all warps of the
 // machine: in compact_kernel a CTA goes through ticket, mask, look-back and only then its rows, 2.6 times over for 49 664 tokens, and
 // a row of 1 KB (a token's keys or values of four heads) is an item with two loads in flight per lane.
-// Both in us (in a graph, L2 flushed; rows of 7 KB, + two of 1 KB, + one of 7 KB): 1000 tokens 14.3 / 16.4 / 20.5 in one kernel and 14.3 / 14.3 / 14.3 in
-// two, 4000 tokens 14.4 / 16.4 / 18.5 and 16.4 / 16.4 / 18.4, 8192 22.5 / 26.7 / 39.9 and 24.6 / 28.7 / 38.9, 20 000 28.7 / 36.9 / 51.2 and 26.7 / 32.8 / 45.1,
-// 131 072 94 / 115 / 164 and 78 / 94 / 154: two kernels up to one tile of the lists and from the size on where compact_kernel takes more than
-// one wave of tiles.
-constexpr int64_t kCompactTwoMaxRows = 262144, kCompactOneMaxRows = 16384;
+// Both in us (in a graph, 30 % kept, L2 flushed; two rows of 1 KB / one of 7 KB / all three): 300 tokens 5.2 / 6.6 / 8.2 in one kernel and 5.6 / 6.9 /
+// 6.6 in two, 2048 tokens 5.9 / 7.2 / 8.8 and 6.2 / 7.5 / 8.3, 4000 5.7 / 8.6 / 9.7 and 7.1 / 8.8 / 10.6, 18 000 8.9 / 17.4 / 23.2 and 9.7 / 18.5 / 23.7,
+// 18 944 9.1 / 18.8 / 23.4 and 10.3 / 20.8 / 23.6, 19 500 13.0 / 22.7 / 27.4 and 10.4 / 20.7 / 24.2, 131 072 65 / 111 / 140 and 34 / 99 / 128, 262 144 122 / 216 /
+// 267 and 62 / 194 / 245, 524 288 175 / 378 / 474 and 115 / 380 / 484.  So two kernels where one would take more than a wave of its tiles
+// of 64 (two CTAs per SM: 18 944 rows), and up to one tile of the lists for more than a piece of bytes per row; the host's second launch,
+// 2 us, counts where nothing else is enqueued.
+constexpr int64_t kCompactTwoMaxRows = 262144;
+static int64_t compact_one_max_rows() { return 2LL * sm_count() * 64; }
 constexpr int kListTile = 2048, kListThreads = 512;      // four tokens per thread
 __global__ void __launch_bounds__(kListThreads)
 compact_lists_kernel(const uint8_t* __restrict__ mask, int64_t n_upper, const int32_t* __restrict__ cu_in, int S, const int32_t* __restrict__ pos_in,
@@ -1041,7 +1044,9 @@ static int compact_impl(const uint8_t* mask, int64_t n, const int32_t* cu_in, in
     }
     if (!ws || ((uintptr_t)ws % 256) || ws_bytes < compact_ws_bytes(n)) return DASH_ERR_WORKSPACE;
     cudaStream_t st = (cudaStream_t)stream;
-    if (idx_out && n_rows > 0 && n > 0 && (n <= kListTile || n > kCompactOneMaxRows) && n <= kCompactTwoMaxRows && !stall) {
+    int64_t all_bytes = 0;
+    for (int q = 0; q < n_rows; ++q) all_bytes += rs.row_bytes[q];
+    if (idx_out && n > 0 && ((n <= kListTile && all_bytes > kPieceBytes) || (n_rows > 0 && n > compact_one_max_rows() && n <= kCompactTwoMaxRows)) && !stall) {
         const int grid = (int)((n + kListTile - 1) / kListTile);
         DASH_CUDA_TRY(launch_pdl(compact_lists_kernel, grid, kListThreads, 0, st, mask, n, cu_in, S, pos_in, pos_out, tok_in, tok_out, idx_out, cu_out,
                                  n_out_dev, aligned16(mask) ? 1 : 0));

@@ -501,9 +501,18 @@ def test_select_keep_count_at_the_edges_of_its_key_cache(n, kind):
             assert np.array_equal(m.cpu().numpy(), ref), (n, kind, k, high)
 
 
-@pytest.mark.parametrize("n", [1, 31, 2047, 2048, 2049, 16384, 16385, 33000, 262144, 262145])
+@pytest.mark.parametrize("n", [1, 31, 2047, 2048, 2049, 16384, 16385, 18944, 18945, 33000, 262144, 262145])
 @pytest.mark.parametrize("keep", [0.0, 0.3, 1.0])
 def test_compact_lists_and_rows_at_the_edges_of_their_tiles(n, keep):
+    _compact_at_an_edge(n, keep, [1024, 20, 96, 16] if n > 60000 else ([7168, 1024, 20, 96] if keep != 0.3 else [7168, 16, 2048, 20]))
+
+
+@pytest.mark.parametrize("n,widths", [(n, w) for n in (1, 700, 2048) for w in ([1024, 1024], [4096], [4096, 16], [2048, 2052])])
+def test_compact_of_few_rows_on_both_sides_of_its_rule(n, widths):
+    _compact_at_an_edge(n, 0.3, widths)
+
+
+def _compact_at_an_edge(n, keep, widths):
     """Row widths that go by in pieces (7168 bytes), several to an item (16, 1024, 2048), alone (96: not a power of two vectors) and word by word
     (20); a mask that starts on any byte; fewer valid rows than the buffers hold.  Everything equals the oracle's lists exactly."""
     g = torch.Generator().manual_seed(n)
@@ -512,7 +521,6 @@ def test_compact_lists_and_rows_at_the_edges_of_their_tiles(n, keep):
     cu = wl.cu_from_lengths(lens)
     total = int(cu[-1])
     mask = (torch.rand(n + 3, generator=g) < keep).to(torch.uint8) * 3                 # any non-zero byte keeps
-    widths = [1024, 20, 96, 16] if n > 60000 else ([7168, 1024, 20, 96] if keep != 0.3 else [7168, 16, 2048, 20])
     rows = [torch.randint(0, 256, (n, w), generator=g, dtype=torch.uint8).to(DEV) for w in widths]
     pos, tok = torch.randint(0, 1 << 20, (n,), generator=g, dtype=torch.int32), torch.randperm(n, generator=g).to(torch.int32)
     for off in (0, 3):
