@@ -485,8 +485,11 @@ attention_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
                 const float2 sl2 = make_float2(p.scale_log2, p.scale_log2);
                 const float msl = m * p.scale_log2;
                 const float2 nm2 = make_float2(-msl, -msl);
-                float2 sumA = make_float2(0.f, 0.f), sumB = make_float2(0.f, 0.f);
-                // scale-subtract and row sums on packed fp32 pairs (two lanes per FMA-pipe instruction); P is packed in place
+                // scale-subtract and row sums on packed fp32 pairs (two lanes per FMA-pipe instruction); P is packed in place.  A row's sum is added
+                // up per 64 keys, in four chains of 16 (A, B: the first 64, C, D: the rest): a chain of 32 loses more of what lies below 2^-24 of a
+                // row's largest weight.  One loop over all of them: as two loops of 64 heads of 64 took 3 % longer (8192 tokens, 32 / 8: 350 us,
+                // 342 as it is, 339 with chains of 32), heads of 128 the same.
+                float2 sumA, sumB, sumC, sumD;
 #pragma unroll
                 for (int c = 0; c < 128; c += 4) {
                     const float2 xa = __ffma2_rn(make_float2(__uint_as_float(sreg[c]), __uint_as_float(sreg[c + 1])), sl2, nm2);
@@ -496,11 +499,14 @@ attention_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
                     pa.y = ex2(xa.y);
                     pb.x = ex2(xb.x);
                     pb.y = ex2(xb.y);
-                    sumA = __fadd2_rn(sumA, pa);
-                    sumB = __fadd2_rn(sumB, pb);
+                    float2 &s0 = c < 64 ? sumA : sumC, &s1 = c < 64 ? sumB : sumD;
+                    s0 = (c & 63) ? __fadd2_rn(s0, pa) : pa;
+                    s1 = (c & 63) ? __fadd2_rn(s1, pb) : pb;
                     sreg[c >> 1] = pack_bf16(pa.x, pa.y);
                     sreg[(c >> 1) + 1] = pack_bf16(pb.x, pb.y);
                 }
+                const float2 sum = __fadd2_rn(__fadd2_rn(make_float2(sumA.x, sumC.x), make_float2(sumA.y, sumC.y)),
+                                              __fadd2_rn(make_float2(sumB.x, sumD.x), make_float2(sumB.y, sumD.y)));
                 // (waited for and stored behind all exponentials: with the wait and the first store between the halves the loop was cut in two
                 // for the compiler, and a pair's block took 5 % longer: 8192 tokens 376 us instead of 357)
                 if (!o_waited) {                                  // PV_{j-1} has read the P that is overwritten now
@@ -510,7 +516,8 @@ attention_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
                 }
                 tmem_st32(tP(x) + lane_base, &sreg[0]);
                 tmem_st32(tP(x) + lane_base + 32, &sreg[32]);
-                l += (sumA.x + sumA.y) + (sumB.x + sumB.y);
+                l += sum.x;
+                l += sum.y;
                 if (diag && x == 1) {
                     // keys past the end of the sequence (only its last tile, which is a tile 1, meets them): their V rows may hold anything
                     // (another sequence, or never-written memory); zero them so 0 * garbage cannot make a NaN

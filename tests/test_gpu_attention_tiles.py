@@ -1,5 +1,7 @@
 """Prefill attention where its tiles begin and end: query tiles of 128 rows that go through the key blocks in pairs or alone, item lists from one
 item to several per SM, sequences on both sides of every tile boundary, rescaling in either tile of a pair."""
+import math
+
 import pytest
 import torch
 
@@ -44,3 +46,16 @@ def test_attention_of_a_sequence_is_the_same_alone_and_in_a_batch():
         one = dash.dash_varlen_attention(Q[a:b].contiguous(), K[a:b].contiguous(), V[a:b].contiguous(), wl.cu_from_lengths([b - a]).to(DEV), b - a)
         assert torch.equal(one, O[a:b])
     assert dash.dash_check_status() == dash.OK
+
+
+def test_attention_row_sums_keep_small_weights_beside_a_large_one():
+    """Row sums are formed per 64 keys, in four chains of 16: key 0 has weight 1, keys 64 to 127 have 2^-25 each, the others none.  In one chain
+    with key 0 a 2^-25 is lost (half a unit of 1 is 2^-24), in chains of their own all 64 count: l = 1 + 2^-19.  A chain of 32 over the whole block
+    would leave 16 of them out, 4.8e-7.  Sums that hold key 0 are rounded at most five times, 5 * 2^-24 = 3.0e-7; log and exp add 1e-12."""
+    K = torch.full((256, 1, 128), 0.0)
+    K[1:64, 0, 0], K[64:128, 0, 0], K[128:, 0, 0] = -1000.0, -25.0, -1000.0
+    Q = torch.zeros(256, 1, 128)
+    Q[:, 0, 0] = 1.0
+    Q, K, V = Q.to(torch.bfloat16).to(DEV), K.to(torch.bfloat16).to(DEV), torch.ones(256, 1, 128, dtype=torch.bfloat16, device=DEV)
+    _, lse = dash.dash_varlen_attention(Q, K, V, wl.cu_from_lengths([256]).to(DEV), 256, scale=math.log(2.0), want_lse=True)
+    assert float((lse[0, 127:].double() - math.log1p(2.0 ** -19)).abs().max()) < 3.0e-7
