@@ -117,20 +117,31 @@ attention_plan_kernel(const int32_t* __restrict__ cu, int S, int Hq, int pairs, 
     attention_plan_items<1024>(cu, S, Hq, pairs, plan, n_items, ticket, max_entries);
 }
 
+constexpr int kKSlots = 3, kVSlots = 2, kRecords = 4;      // rings of K tiles, V tiles and item records
 template <int D>
 struct AttnSmem {
     static constexpr int kTileBytes = kBM * D * 2;
-    static constexpr int kKSlots = 3, kVSlots = 2;
     static constexpr int kQ = 0, kK = 2 * kTileBytes, kV = kK + kKSlots * kTileBytes, kBars = kV + kVSlots * kTileBytes;
     static constexpr int kTotal = kBars + 512;
     // one CTA per SM, whose TMEM columns it takes all: with heads of 64 the tiles alone would let a second one in
     static constexpr int kLaunch = kTotal + 1024 > 120 * 1024 ? kTotal + 1024 : 120 * 1024;
 };
 
-// Barriers of a CTA (8 bytes each, in this order behind the tiles); [x]: per query tile x, [slot]: per ring slot
+// Barriers of a CTA (8 bytes each, in this order behind the tiles): two per query tile or one per slot of a ring
 enum AttnBar {
-    kBarQFull = 0, kBarQFree = 2, kBarKFull = 4, kBarKFree = 7, kBarVFull = 10, kBarVFree = 12, kBarSFull = 14, kBarSFree = 16,
-    kBarPFull = 18, kBarOFull = 20, kBarItemFull = 22, kBarItemFree = 24, kBarDrain = 26, kBarCount = 28
+    kBarQFull = 0, kBarQFree = kBarQFull + 2, kBarKFull = kBarQFree + 2, kBarKFree = kBarKFull + kKSlots, kBarVFull = kBarKFree + kKSlots,
+    kBarVFree = kBarVFull + kVSlots, kBarSFull = kBarVFree + kVSlots, kBarSFree = kBarSFull + 2, kBarPFull = kBarSFree + 2, kBarOFull = kBarPFull + 2,
+    kBarItemFull = kBarOFull + 2, kBarItemFree = kBarItemFull + kRecords, kBarDrain = kBarItemFree + kRecords, kBarCount = kBarDrain + 2
+};
+// behind them: TMEM address, the flag of a role that has given up, item records
+constexpr int kTmemSlot = 8 * kBarCount, kAbortFlag = kTmemSlot + 4, kRecordAt = kTmemSlot + 16;
+static_assert(kRecordAt % 16 == 0 && kRecordAt + kRecords * 16 <= 512, "what AttnSmem keeps behind the tiles");
+// An item: its sequence's first and end row, its highest query tile (-1: no more items), its head and the tiles 0 and 1 of the CTA that it takes, first .. last
+struct AttnItem {
+    int seq_a, seq_b, top, h, first, last;
+    __device__ int4 pack() const { return make_int4(seq_a, seq_b, top, h << 2 | first << 1 | last); }
+    __device__ explicit AttnItem(const int4& r) : seq_a(r.x), seq_b(r.y), top(r.z), h(r.w >> 2), first(r.w >> 1 & 1), last(r.w & 1) {}
+    __device__ AttnItem(int a, int b, int t, int head, int lo, int hi) : seq_a(a), seq_b(b), top(t), h(head), first(lo), last(hi) {}
 };
 
 // A wait of a single thread, bounded in time and given up as soon as another role of the CTA has given up.
@@ -151,13 +162,6 @@ __device__ __forceinline__ bool attn_wait_warp(uint32_t bar, uint32_t parity, vo
     }
 }
 
-// GATHER: Q, K and V are full-length [rows, heads * D] tensors and the packed active set is given by p.idx; tiles are fetched four
-// rows per instruction (TMA gather4, issued by all lanes of the loading warp: lane l brings rows 4l .. 4l+3 of the tile), so the active rows
-// of Q, K, V are never copied into packed buffers.  Everything else -- and the packed O -- is the same.
-//
-// Hand-overs.  Every barrier is waited for phase by phase by each of its waiters, and no phase can be overtaken: a tile buffer, the score
-// buffer, a P and an item record each come back through a "free" barrier before they are filled again; O of a tile is handed on by the P of
-// its next product.  Tile 1 is the upper one and visits every key block of the item, so what it has used of K and V nobody else waits for.
 // v[e] of lane i (of four neighbouring lanes) <-> v[i] of lane e
 __device__ __forceinline__ void quad_transpose(uint4 (&v)[4], int lane) {
     auto swap_halves = [](uint4& a, uint4& b, bool up, int d) {        // the lanes with `up` send a and keep b, the others the other way round
@@ -171,6 +175,17 @@ __device__ __forceinline__ void quad_transpose(uint4 (&v)[4], int lane) {
     swap_halves(v[0], v[2], b1, 2); swap_halves(v[1], v[3], b1, 2);
 }
 
+// GATHER: Q, K and V are full-length [rows, heads * D] tensors and the packed active set is given by p.idx; tiles are fetched four
+// rows per instruction (TMA gather4, issued by all lanes of the loading warp: lane l brings rows 4l .. 4l+3 of the tile), so the active rows
+// of Q, K, V are never copied into packed buffers.  Everything else -- and the packed O -- is the same.
+//
+// Hand-overs.  A tile buffer, the score buffer, a P and an item record each come back through a "free" barrier before they are filled again; O of
+// a tile is handed on by the P of its next product.  Loads, scores and products go through items, key blocks and tiles in one order.  Every waiter
+// sees the phases of a barrier one by one, so none can overtake it, with one exception: a softmax warp waits for a V tile only where it
+// has rows of it to clear, in the last block b of a sequence's last tile, and has to know that the tile before in that slot, of block b - 2, has
+// arrived.  If the item has more blocks the warp has seen the product of b - 1 done, so that of b - 2 was issued.  If not, the warp waits for b - 2 to
+// be given free, and can tell that phase from the one of b - 4: the load of b - 2 has waited for it, ahead of the item's record.
+// (tests/test_attention_handover.py runs these roles and barriers through a model of them.)
 template <int D, bool OUT_F32, bool GATHER>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 attention_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK,
@@ -184,10 +199,10 @@ attention_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
     const uint32_t bars = smem_base + L::kBars;
     auto bar = [&](int kind, uint32_t i) { return bars + 8u * ((uint32_t)kind + i); };
     uint8_t* smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
-    const uint32_t tmem_slot = bars + 256;
-    volatile uint32_t* tmem_slot_gen = reinterpret_cast<volatile uint32_t*>(smem_gen + L::kBars + 256);
-    volatile uint32_t* abort_gen = reinterpret_cast<volatile uint32_t*>(smem_gen + L::kBars + 260);
-    volatile int* rec_gen = reinterpret_cast<volatile int*>(smem_gen + L::kBars + 272);       // two item records of four words
+    const uint32_t tmem_slot = bars + kTmemSlot;
+    volatile uint32_t* tmem_slot_gen = reinterpret_cast<volatile uint32_t*>(smem_gen + L::kBars + kTmemSlot);
+    volatile uint32_t* abort_gen = reinterpret_cast<volatile uint32_t*>(smem_gen + L::kBars + kAbortFlag);
+    int4* const records = reinterpret_cast<int4*>(smem_gen + L::kBars + kRecordAt);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
@@ -195,11 +210,11 @@ attention_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
         if (lane == 0) {
             for (uint32_t x = 0; x < 2; ++x) {
                 mbar_init(bar(kBarQFull, x), 1); mbar_init(bar(kBarQFree, x), 1); mbar_init(bar(kBarSFull, x), 1); mbar_init(bar(kBarSFree, x), 4);
-                mbar_init(bar(kBarPFull, x), 4); mbar_init(bar(kBarOFull, x), 1); mbar_init(bar(kBarItemFull, x), 1);
-                mbar_init(bar(kBarItemFree, x), kSoftWarps + 2); mbar_init(bar(kBarDrain, x), 1);
+                mbar_init(bar(kBarPFull, x), 4); mbar_init(bar(kBarOFull, x), 1); mbar_init(bar(kBarDrain, x), 1);
             }
-            for (uint32_t i = 0; i < (uint32_t)L::kKSlots; ++i) { mbar_init(bar(kBarKFull, i), 1); mbar_init(bar(kBarKFree, i), 1); }
-            for (uint32_t i = 0; i < (uint32_t)L::kVSlots; ++i) { mbar_init(bar(kBarVFull, i), 1); mbar_init(bar(kBarVFree, i), 1); }
+            for (uint32_t i = 0; i < (uint32_t)kRecords; ++i) { mbar_init(bar(kBarItemFull, i), 1); mbar_init(bar(kBarItemFree, i), kSoftWarps + 2); }
+            for (uint32_t i = 0; i < (uint32_t)kKSlots; ++i) { mbar_init(bar(kBarKFull, i), 1); mbar_init(bar(kBarKFree, i), 1); }
+            for (uint32_t i = 0; i < (uint32_t)kVSlots; ++i) { mbar_init(bar(kBarVFull, i), 1); mbar_init(bar(kBarVFree, i), 1); }
             *abort_gen = 0;
             fence_barrier_init();
             fence_proxy_async_smem();
@@ -227,7 +242,7 @@ attention_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
     reg_dec<kOtherRegs>();
     if (warp == kLoadWarp) {
         // ---- loads, and the hand-out of items: all lanes go along (a fetch by index takes the whole warp) ----
-        uint32_t k_fills = 0, v_fills = 0, items = 0, q_any = 0, q_par = 0;      // q_any, q_par: bit x = tile x was ever loaded, parity of its count
+        uint32_t k_fills = 0, v_fills = 0, items = 0, turn = 0, q_any = 0, q_par = 0;      // q_any, q_par: bit x = tile x was ever loaded, parity of its count
         const int n_items = *p.n_items;
         auto wait = [&](uint32_t b, uint32_t parity) { return attn_wait_warp(b, parity, abort_gen); };
         int seq_a = 0, seq_b = 0;
@@ -257,62 +272,72 @@ attention_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
             return true;
         };
         auto load_k = [&](int kvh, int j) {
-            const uint32_t slot = k_fills % L::kKSlots;
-            if (!wait(bar(kBarKFree, slot), ((k_fills / L::kKSlots) & 1) ^ 1)) return false;
+            const uint32_t slot = k_fills % kKSlots;
+            if (!wait(bar(kBarKFree, slot), ((k_fills / kKSlots) & 1) ^ 1)) return false;
             load_tile(sK + slot * L::kTileBytes, &mapK, bar(kBarKFull, slot), kvh, seq_a + j * kBN, kv_by_index);
             ++k_fills;
             return true;
         };
         auto load_v = [&](int kvh, int j) {
-            const uint32_t slot = v_fills % L::kVSlots;
-            if (!wait(bar(kBarVFree, slot), ((v_fills / L::kVSlots) & 1) ^ 1)) return false;
+            const uint32_t slot = v_fills % kVSlots;
+            if (!wait(bar(kBarVFree, slot), ((v_fills / kVSlots) & 1) ^ 1)) return false;
             load_tile(sV + slot * L::kTileBytes, &mapV, bar(kBarVFull, slot), kvh, seq_a + j * kBN, kv_by_index);
             ++v_fills;
             return true;
         };
-        int item = 0;
+        // next item: its number, and then its plan entry (the sequence's bounds ride along); two round trips to L2, with loads in between
+        int item = 0, asked = 0;
         int4 e = make_int4(0, -1, 0, 0);
-        auto take = [&]() {                                       // next item: its number and plan entry (the sequence's bounds ride along)
-            if (lane == 0) item = (int)atomicAdd(p.ticket, 1u);
-            item = __shfl_sync(0xffffffffu, item, 0);
+        auto ask = [&]() { if (lane == 0) asked = (int)atomicAdd(p.ticket, 1u); };
+        auto take = [&]() {
+            item = __shfl_sync(0xffffffffu, asked, 0);
             e = item < n_items ? p.plan[item / p.Hq] : make_int4(0, -1, 0, 0);
         };
+        ask();
         take();
         bool ok = true;
         for (;;) {
-            const uint32_t slot = items & 1;
-            ok = wait(bar(kBarItemFree, slot), ((items >> 1) & 1) ^ 1);
+            const uint32_t slot = items % kRecords;
+            ok = wait(bar(kBarItemFree, slot), ((items / kRecords) & 1) ^ 1);
             if (!ok) break;
             const int h = item % p.Hq, qt = e.y, kvh = h / G, nb = qt + 1;
             seq_a = e.z; seq_b = e.w;
+            // An item of one tile takes tile 0 and tile 1 of the CTA in turn (0 behind a pair, whose tile 0 ends first): its start overlaps the
+            // end of the one before it, as it did with two CTAs per SM.  us a call, two CTAs of one tile / one CTA, every item in tile 1 / in
+            // turn: 200 sequences of 100 tokens, 28 / 4 heads of 128 157 / 163 / 116, 32 / 8 heads of 64 120 / 146 / 103; 64 of 300, 28 / 4 175 / 148 / 133.
+            const bool pair = p.pairs && qt > 0;
+            const int first = pair ? 0 : (int)turn, last = pair ? 1 : (int)turn;
+            turn = pair ? 0 : turn ^ 1;
             if (lane == 0) {
-                rec_gen[slot * 4] = seq_a; rec_gen[slot * 4 + 1] = seq_b; rec_gen[slot * 4 + 2] = qt; rec_gen[slot * 4 + 3] = h;
+                records[slot] = AttnItem(seq_a, seq_b, qt, h, first, last).pack();
                 mbar_arrive(bar(kBarItemFull, slot));
             }
             ++items;
             if (qt < 0) break;
-            // in the order of use; the next item is taken while this one's last tiles are waited for
-            if (p.pairs && qt > 0) ok = load_q(0, h, qt - 1);
-            ok = ok && load_k(kvh, 0) && load_q(1, h, qt);
+            // in the order of use; the next item is asked for while this one's last tiles are waited for
+            if (nb <= 2) ask();
+            if (pair) ok = load_q(0, h, qt - 1);
+            ok = ok && load_k(kvh, 0) && load_q(last, h, qt);
             for (int t = 1; t <= nb && ok; ++t) {
-                if (t == (nb > 2 ? nb - 2 : 1)) take();
+                if (nb > 2 && t == nb - 2) ask();
                 if (t < nb) ok = load_k(kvh, t);
                 ok = ok && load_v(kvh, t - 1);
             }
             if (!ok) break;
+            take();
         }
         if (!ok && lane == 0) give_up();
         __syncwarp();
         // Nothing is left in flight: every tile has arrived and, unless a wait ran out, been given free by the products that read it.
-        for (uint32_t i = 0; i < (uint32_t)L::kKSlots; ++i)
+        for (uint32_t i = 0; i < (uint32_t)kKSlots; ++i)
             if (k_fills > i) {
-                const uint32_t use = (k_fills - 1 - i) / L::kKSlots;
+                const uint32_t use = (k_fills - 1 - i) / kKSlots;
                 mbar_wait(bar(kBarKFull, i), use & 1, kWaitCycles);
                 if (ok) mbar_wait(bar(kBarKFree, i), use & 1, kWaitCycles);
             }
-        for (uint32_t i = 0; i < (uint32_t)L::kVSlots; ++i)
+        for (uint32_t i = 0; i < (uint32_t)kVSlots; ++i)
             if (v_fills > i) {
-                const uint32_t use = (v_fills - 1 - i) / L::kVSlots;
+                const uint32_t use = (v_fills - 1 - i) / kVSlots;
                 mbar_wait(bar(kBarVFull, i), use & 1, kWaitCycles);
                 if (ok) mbar_wait(bar(kBarVFree, i), use & 1, kWaitCycles);
             }
@@ -327,23 +352,23 @@ attention_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
         if (lane == 0) {
             constexpr uint32_t idesc_s = idesc_bf16_f32(kBM, kBN, false, false);
             uint32_t k_used = 0, items = 0, s_made = 0, q_used = 0;   // s_made, q_used: bit x = parity of tile x's count
-            int last = -1;                                        // tile whose scores the buffer holds
+            int holder = -1;                                      // tile whose scores the buffer holds
             bool ok = true;
             auto wait = [&](uint32_t b, uint32_t parity) { return attn_wait(b, parity, abort_gen); };
             while (ok) {
-                const uint32_t slot = items & 1;
-                if (!(ok = wait(bar(kBarItemFull, slot), (items >> 1) & 1))) break;
-                const int qt = rec_gen[slot * 4 + 2];
+                const uint32_t slot = items % kRecords;
+                if (!(ok = wait(bar(kBarItemFull, slot), (items / kRecords) & 1))) break;
+                const AttnItem it(records[slot]);
+                const int top = it.top, first = it.first, last = it.last;
                 mbar_arrive(bar(kBarItemFree, slot));
                 ++items;
-                if (qt < 0) break;
-                const int nb = qt + 1, first = (p.pairs && qt > 0) ? 0 : 1;
-                for (int j = 0; j < nb && ok; ++j) {
-                    const uint32_t ks = k_used % L::kKSlots;
-                    ok = wait(bar(kBarKFull, ks), (k_used / L::kKSlots) & 1);
-                    for (int x = j < qt ? first : 1; x < 2 && ok; ++x) {
+                if (top < 0) break;
+                for (int j = 0; j <= top && ok; ++j) {
+                    const uint32_t ks = k_used % kKSlots;
+                    ok = wait(bar(kBarKFull, ks), (k_used / kKSlots) & 1);
+                    for (int x = j < top ? first : last; x <= last && ok; ++x) {        // (a pair's tile 0 has a block less)
                         if (j == 0) ok = wait(bar(kBarQFull, x), (q_used >> x) & 1);
-                        if (ok && last >= 0) ok = wait(bar(kBarSFree, last), ((s_made >> last) & 1) ^ 1);
+                        if (ok && holder >= 0) ok = wait(bar(kBarSFree, holder), ((s_made >> holder) & 1) ^ 1);
                         if (!ok) break;
                         tc_fence_after();
                         const uint64_t dq = smem_desc_sw128(sQ + x * L::kTileBytes, 16, 1024), dk = smem_desc_sw128(sK + ks * L::kTileBytes, 16, 1024);
@@ -354,8 +379,8 @@ attention_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
                         }
                         tc_commit(bar(kBarSFull, x));
                         s_made ^= 1u << x;
-                        last = x;
-                        if (j == qt - 1 + x) { tc_commit(bar(kBarQFree, x)); q_used ^= 1u << x; }       // tile 0 ends a block ahead of tile 1
+                        holder = x;
+                        if (j == top - (last - x)) { tc_commit(bar(kBarQFree, x)); q_used ^= 1u << x; }
                     }
                     if (ok) tc_commit(bar(kBarKFree, ks));
                     ++k_used;
@@ -375,18 +400,18 @@ attention_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
             bool ok = true;
             auto wait = [&](uint32_t b, uint32_t parity) { return attn_wait(b, parity, abort_gen); };
             while (ok) {
-                const uint32_t slot = items & 1;
-                if (!(ok = wait(bar(kBarItemFull, slot), (items >> 1) & 1))) break;
-                const int qt = rec_gen[slot * 4 + 2];
+                const uint32_t slot = items % kRecords;
+                if (!(ok = wait(bar(kBarItemFull, slot), (items / kRecords) & 1))) break;
+                const AttnItem it(records[slot]);
+                const int top = it.top, first = it.first, last = it.last;
                 mbar_arrive(bar(kBarItemFree, slot));
                 ++items;
-                if (qt < 0) break;
-                const int nb = qt + 1, first = (p.pairs && qt > 0) ? 0 : 1;
-                for (int j = 0; j < nb && ok; ++j) {
-                    const uint32_t vs = v_used % L::kVSlots;
-                    ok = wait(bar(kBarVFull, vs), (v_used / L::kVSlots) & 1);
+                if (top < 0) break;
+                for (int j = 0; j <= top && ok; ++j) {
+                    const uint32_t vs = v_used % kVSlots;
+                    ok = wait(bar(kBarVFull, vs), (v_used / kVSlots) & 1);
                     const uint64_t dv = smem_desc_sw128(sV + vs * L::kTileBytes, kChunkBytes, 1024);
-                    for (int x = j < qt ? first : 1; x < 2 && ok; ++x) {
+                    for (int x = j < top ? first : last; x <= last && ok; ++x) {        // (a pair's tile 0 has a block less)
                         ok = wait(bar(kBarPFull, x), (p_used >> x) & 1);
                         if (!ok) break;
                         p_used ^= 1u << x;
@@ -416,15 +441,18 @@ attention_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
         bool ok = true;
         auto wait = [&](uint32_t b, uint32_t parity) { return attn_wait_warp(b, parity, abort_gen); };
         while (ok) {
-            const uint32_t slot = items & 1;
-            if (!(ok = wait(bar(kBarItemFull, slot), (items >> 1) & 1))) break;
-            const int seq_a = rec_gen[slot * 4], seq_b = rec_gen[slot * 4 + 1], top = rec_gen[slot * 4 + 2], h = rec_gen[slot * 4 + 3];
+            const uint32_t slot = items % kRecords;
+            if (!(ok = wait(bar(kBarItemFull, slot), (items / kRecords) & 1))) break;
+            const AttnItem it(records[slot]);
+            const int seq_a = it.seq_a, seq_b = it.seq_b, top = it.top, h = it.h, first = it.first, last = it.last;
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(kBarItemFree, slot));
             ++items;
             if (top < 0) break;
-            const int qt = top - 1 + x;                           // this tile; its key blocks are 0 .. qt
-            if (x == 0 && (!p.pairs || qt < 0)) continue;
+            const uint32_t v_first = v_blocks;
+            v_blocks += (uint32_t)top + 1;
+            if (x < first || x > last) continue;                  // the other tile's item
+            const int qt = top - (last - x);                      // this tile; its key blocks are 0 .. qt
             const int len = seq_b - seq_a, q0 = qt * kBM;
             const bool row_valid = (q0 + row) < len;
             float m = -INFINITY, l = 0.f;
@@ -518,11 +546,11 @@ attention_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
                 tmem_st32(tP(x) + lane_base + 32, &sreg[32]);
                 l += sum.x;
                 l += sum.y;
-                if (diag && x == 1) {
-                    // keys past the end of the sequence (only its last tile, which is a tile 1, meets them): their V rows may hold anything
-                    // (another sequence, or never-written memory); zero them so 0 * garbage cannot make a NaN
-                    const uint32_t vb = v_blocks + j, vs = vb % L::kVSlots;
-                    ok = wait(bar(kBarVFull, vs), (vb / L::kVSlots) & 1);
+                if (diag && x == last && q0 + (warp & 3) * 32 + 31 >= len) {
+                    // keys past the end of the sequence (only its last tile meets them): their V rows may hold anything (another sequence, or
+                    // never-written memory); zero them so 0 * garbage cannot make a NaN
+                    const uint32_t vb = v_first + j, vs = vb % kVSlots, use = vb / kVSlots;
+                    ok = (j > 0 || use == 0 || wait(bar(kBarVFree, vs), (use - 1) & 1)) && wait(bar(kBarVFull, vs), use & 1);
                     if (!ok) break;
                     if (j * kBN + row >= len) {
 #pragma unroll
@@ -539,7 +567,6 @@ attention_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar(kBarPFull, x));
             }
-            v_blocks += (uint32_t)top + 1;
             if (ok) ok = wait(bar(kBarOFull, x), (blocks - 1) & 1);
             if (!ok) break;
             tc_fence_after();

@@ -59,3 +59,21 @@ def test_attention_row_sums_keep_small_weights_beside_a_large_one():
     Q, K, V = Q.to(torch.bfloat16).to(DEV), K.to(torch.bfloat16).to(DEV), torch.ones(256, 1, 128, dtype=torch.bfloat16, device=DEV)
     _, lse = dash.dash_varlen_attention(Q, K, V, wl.cu_from_lengths([256]).to(DEV), 256, scale=math.log(2.0), want_lse=True)
     assert float((lse[0, 127:].double() - math.log1p(2.0 ** -19)).abs().max()) < 3.0e-7
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("lengths", [[100, 60, 1, 128, 90, 5] * 25, [100, 300, 5, 1, 257, 128, 40, 200, 129] * 8], ids=["one tile each", "pairs and single tiles"])
+def test_attention_of_short_sequences_keeps_their_rows_apart(lengths, D):
+    """Items of one tile take the two halves of a CTA in turn, and either half clears the value rows behind a sequence's end: NaN and infinities in every
+    second sequence leave the outputs of the others as they are without, bit for bit."""
+    g = torch.Generator().manual_seed(35)
+    cu = wl.cu_from_lengths(lengths)
+    n = int(cu[-1])
+    Q, K, V = (torch.randn(n, h, D, generator=g).to(torch.bfloat16).to(DEV) for h in (8, 4, 4))
+    odd = torch.cat([torch.full((x,), i % 2, dtype=torch.bool) for i, x in enumerate(lengths)]).to(DEV)
+    _attention_case(lengths, 8, 4, D, torch.bfloat16, 36, pad=3)
+    clean = dash.dash_varlen_attention(Q, K, V, cu.to(DEV), max(lengths))
+    K[odd], V[odd] = float("inf"), float("nan")
+    O = dash.dash_varlen_attention(Q, K, V, cu.to(DEV), max(lengths))
+    assert torch.equal(O[~odd], clean[~odd]) and bool(torch.isfinite(clean.float()).all())
+    assert dash.dash_check_status() == dash.OK
