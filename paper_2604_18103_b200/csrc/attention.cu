@@ -91,8 +91,7 @@ constexpr long long kWaitCycles = 4000000000LL;   // ~2 s: a wait that long is r
 constexpr uint32_t kTmemCols = 512;
 
 struct AttnParams {
-    const int32_t* cu;
-    int S, Hq, Hkv, pairs;
+    int Hq, Hkv;
     float scale_log2;       // softmax scale * log2(e)
     float scale;
     void* O;
@@ -101,7 +100,7 @@ struct AttnParams {
     float* lse;             // [Hq, n] or null
     int64_t n;
     int* status;
-    const int4* plan;           // (sequence, highest query tile, first row, end row of the sequence) of every item group, heaviest first; Hq items (heads) per entry
+    const int4* plan;           // (1: a pair of tiles, highest query tile, first row, end row of the sequence) of every item group, heaviest first; Hq items (heads) per entry
     const int* n_items;         // device: entries * Hq
     unsigned int* ticket;       // device: next item to hand out
     const int32_t* idx;         // GATHER: packed row i is row idx[i] of the full-length Q (and of K, V unless kv_packed)
@@ -109,12 +108,13 @@ struct AttnParams {
 };
 
 // ---- plan kernel of a call that is not part of a block step ----
-__global__ void __launch_bounds__(1024)
-attention_plan_kernel(const int32_t* __restrict__ cu, int S, int Hq, int pairs, int4* __restrict__ plan, int* __restrict__ n_items,
+constexpr int kPlanThreads = 256;
+__global__ void __launch_bounds__(kPlanThreads)
+attention_plan_kernel(const int32_t* __restrict__ cu, int S, int Hq, int sms, int4* __restrict__ plan, int* __restrict__ n_items,
                       unsigned int* __restrict__ ticket, int64_t max_entries) {
     pdl_launch_dependents();
     pdl_wait();
-    attention_plan_items<1024>(cu, S, Hq, pairs, plan, n_items, ticket, max_entries);
+    attention_plan_items<kPlanThreads>(cu, S, Hq, sms, plan, n_items, ticket, max_entries);
 }
 
 constexpr int kKSlots = 3, kVSlots = 2, kRecords = 4;      // rings of K tiles, V tiles and item records
@@ -305,7 +305,7 @@ attention_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
             // An item of one tile takes tile 0 and tile 1 of the CTA in turn (0 behind a pair, whose tile 0 ends first): its start overlaps the
             // end of the one before it, as it did with two CTAs per SM.  us a call, two CTAs of one tile / one CTA, every item in tile 1 / in
             // turn: 200 sequences of 100 tokens, 28 / 4 heads of 128 157 / 163 / 116, 32 / 8 heads of 64 120 / 146 / 103; 64 of 300, 28 / 4 175 / 148 / 133.
-            const bool pair = p.pairs && qt > 0;
+            const bool pair = e.x != 0;
             const int first = pair ? 0 : (int)turn, last = pair ? 1 : (int)turn;
             turn = pair ? 0 : turn ^ 1;
             if (lane == 0) {
@@ -669,23 +669,13 @@ static int launch_attention(const CUtensorMap& mq, const CUtensorMap& mk, const 
     return launch_pdl(attention_kernel<D, OUT_F32, GATHER>, grid, kAttnThreads, (size_t)smem, st, mq, mk, mv, p) == cudaSuccess ? DASH_OK : DASH_ERR_CUDA;
 }
 
-// Whether a call's items are pairs of tiles.  A pair takes 2700 cycles per key block, a tile alone about 1700: tiles go alone while the call ends with
-// its longest one, that is while the SMs have fewer key blocks each than the longest sequence has (the tiles counted as if all sequences
-// were as long).  us, alone / pairs, and blocks per SM over those of the longest sequence: 8192 rows of 4 heads of 64 79.3 / 105.0 (0.89), 1024
-// of 28 / 4 heads of 128 21.2 / 22.8 (0.96), two of 500 18.6 / 16.4 (1.06), 1300 30.4 / 27.0 (1.13), 1700 40.2 / 31.7 (1.4), 2728 76.9 / 58.7
-// (2.2), five of 267 22.9 / 19.5 (1.9), 40 of 200 81.3 / 65.1.
-static int attention_pairs(int64_t n, int S, int Hq, int64_t max_seqlen) {
-    const double tiles = (double)((max_seqlen + kBM - 1) / kBM), all = (double)Hq * (double)(n / kBM + S) * (tiles + 1) / 2;
-    return all > tiles * sm_count() ? 1 : 0;
-}
-
 // The item list of a call (see attention_plan_items) into the head of its workspace
-static int attention_plan(const int32_t* cu_seqlens, int S, int64_t n, int Hq, int pairs, void* ws, size_t ws_bytes, cudaStream_t st) {
+static int attention_plan(const int32_t* cu_seqlens, int S, int64_t n, int Hq, void* ws, size_t ws_bytes, cudaStream_t st) {
     if (!cu_seqlens || S < 1 || n < 0 || n > 0x7fffffffLL || Hq < 1) return DASH_ERR_INVALID_ARG;
     if (n == 0) return DASH_OK;
     if (!ws || ((uintptr_t)ws % 256) || ws_bytes < 256 + plan_bytes(n, S)) return DASH_ERR_WORKSPACE;
     if ((int64_t)plan_entries(n, S) * Hq > 0x7fffffffLL) return DASH_ERR_UNSUPPORTED;
-    return launch_pdl(attention_plan_kernel, 1, 1024, 0, st, cu_seqlens, S, Hq, pairs, (int4*)((char*)ws + 256), (int*)((char*)ws + 4), (unsigned int*)ws,
+    return launch_pdl(attention_plan_kernel, 1, kPlanThreads, 0, st, cu_seqlens, S, Hq, sm_count(), (int4*)((char*)ws + 256), (int*)((char*)ws + 4), (unsigned int*)ws,
                       (int64_t)plan_entries(n, S)) == cudaSuccess ? DASH_OK : DASH_ERR_CUDA;
 }
 
@@ -750,8 +740,7 @@ static int attention_impl(const void* Q, const void* K, const void* V, void* O, 
     }
 
     AttnParams p;
-    p.cu = cu_seqlens; p.S = S; p.Hq = Hq; p.Hkv = Hkv;
-    p.pairs = attention_pairs(n, S, Hq, max_seqlen);
+    p.Hq = Hq; p.Hkv = Hkv;
     p.scale = scale;
     p.scale_log2 = scale * 1.4426950408889634f;
     p.O = O; p.ldo = ldo; p.O16 = (__nv_bfloat16*)O16; p.lse = lse; p.n = n; p.idx = idx; p.kv_packed = kv_packed ? 1 : 0;
@@ -760,7 +749,7 @@ static int attention_impl(const void* Q, const void* K, const void* V, void* O, 
     p.ticket = (unsigned int*)ws;
     p.n_items = (const int*)((char*)ws + 4);
     p.plan = (const int4*)((char*)ws + 256);
-    if (!planned && (rc = attention_plan(cu_seqlens, S, n, Hq, p.pairs, ws, ws_bytes, st)) != DASH_OK) return rc;
+    if (!planned && (rc = attention_plan(cu_seqlens, S, n, Hq, ws, ws_bytes, st)) != DASH_OK) return rc;
     // persistent CTAs, one per SM, never more than there can be items
     int64_t grid64 = (max_seqlen + kBM - 1) / kBM * Hq * S;
     if (grid64 > sm_count()) grid64 = sm_count();
@@ -770,13 +759,13 @@ static int attention_impl(const void* Q, const void* K, const void* V, void* O, 
     return dt == DASH_F32 ? launch_attention<64, true, false>(mq, mk, mv, p, grid, st) : launch_attention<64, false, false>(mq, mk, mv, p, grid, st);
 }
 
-int attention_plan_ws(int S, int64_t n, int64_t max_seqlen, int Hq, int Hkv, int D, dash_dtype dt, void* ws, size_t ws_bytes, AttnPlanWs* out) {
+int attention_plan_ws(int S, int64_t n, int Hq, int Hkv, int D, dash_dtype dt, void* ws, size_t ws_bytes, AttnPlanWs* out) {
     if (!ws || ((uintptr_t)ws % 256) || ws_bytes < attention_ws_bytes(n, S, Hq, Hkv, D, dt)) return DASH_ERR_WORKSPACE;
     if ((int64_t)plan_entries(n, S) * Hq > 0x7fffffffLL) return DASH_ERR_UNSUPPORTED;
     char* w = (char*)ws;
     out->ticket = (unsigned int*)w; out->n_items = (int*)(w + 4); out->plan = (int4*)(w + 256);
     out->max_entries = (int64_t)plan_entries(n, S);
-    out->pairs = attention_pairs(n, S, Hq, max_seqlen);
+    out->sms = sm_count();
     out->q = out->k = out->v = nullptr;
     if (dt == DASH_F32) {
         out->q = (__nv_bfloat16*)(w + 256 + plan_bytes(n, S));

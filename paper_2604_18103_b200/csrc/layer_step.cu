@@ -180,7 +180,7 @@ prologue_kernel(const PrologueArgs a, const RopeFreqs fr) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int cta = (int)blockIdx.x;
     if (cta == 0) {
-        attention_plan_items<256>(a.cu, a.S, a.Hq, a.ap.pairs, a.ap.plan, a.ap.n_items, a.ap.ticket, a.ap.max_entries);
+        attention_plan_items<256>(a.cu, a.S, a.Hq, a.ap.sms, a.ap.plan, a.ap.n_items, a.ap.ticket, a.ap.max_entries);
         return;
     }
     if (cta == 1) {
@@ -475,7 +475,7 @@ static int attention_to_O(const dash_layer_cfg* cfg, const void* H_in, const int
     PrologueArgs pa = {};
     RopeFreqs fr;
     for (int i = 0; i < D / 2; ++i) fr.inv_freq[i] = pow(cfg->rope_base, -2.0 * i / D);
-    if ((rc = attention_plan_ws(S, n, max_seqlen, Hq, Hkv, D, cfg->dt, W.attn_ws, W.attn_bytes, &pa.ap)) != DASH_OK) return rc;
+    if ((rc = attention_plan_ws(S, n, Hq, Hkv, D, cfg->dt, W.attn_ws, W.attn_bytes, &pa.ap)) != DASH_OK) return rc;
     const size_t front = W.split.part ? gemm_split_count_bytes() : 0, tail = tail_words ? align_up(tail_ws_clear_bytes(n), 16) : 0;
     pa.cu = cu_in; pa.S = S; pa.Hq = Hq;
     pa.zero = (uint4*)(W.compact_ws - front); pa.n_zero = (int)((front + tail) / 16);

@@ -77,3 +77,22 @@ def test_attention_of_short_sequences_keeps_their_rows_apart(lengths, D):
     O = dash.dash_varlen_attention(Q, K, V, cu.to(DEV), max(lengths))
     assert torch.equal(O[~odd], clean[~odd]) and bool(torch.isfinite(clean.float()).all())
     assert dash.dash_check_status() == dash.OK
+
+
+def _entries(lengths, Hq, Hkv, D, n=None, max_seqlen=None):
+    """Entries of the item list that a call leaves in its workspace: tiles, where they go alone, pairs and odd tiles otherwise."""
+    cu = wl.cu_from_lengths(lengths).to(DEV)
+    n = n or int(cu[-1])
+    Q, K, V = (torch.zeros(n, h, D, dtype=torch.bfloat16, device=DEV) for h in (Hq, Hkv, Hkv))
+    ws = dash.workspace(dash.dash_workspace_bytes(dash.WS_ATTENTION, n, len(lengths), Hq, Hkv, D), DEV)
+    dash.dash_varlen_attention(Q, K, V, cu, max_seqlen or max(lengths), ws=ws)
+    return int(ws[4:8].view(torch.int32)) // Hq
+
+
+@pytest.mark.parametrize("lengths,Hq,Hkv,D,rows", [([1000], 16, 16, 64, 8192), ([1000], 28, 4, 128, 8192), ([2000], 4, 4, 64, 16000), ([300], 28, 4, 128, 131072),
+                                                   ([900] * 20, 14, 2, 128, 40000), ([200] * 40, 8, 2, 128, 8100)])
+def test_attention_items_follow_the_true_lengths(lengths, Hq, Hkv, D, rows):
+    """Behind a selection the caller knows bounds only; whether tiles go in pairs hangs on the lengths that are there (20 sequences of 900: pairs)."""
+    tiles = [(x + 127) // 128 for x in lengths]
+    expect = sum((t + 1) // 2 for t in tiles) if len(lengths) == 20 else sum(tiles)
+    assert _entries(lengths, Hq, Hkv, D) == expect and _entries(lengths, Hq, Hkv, D, rows, rows) == expect
