@@ -82,8 +82,8 @@ int make_map_rows_gather(CUtensorMap* map, const void* base, int64_t rows, int64
 constexpr int kBM = 128;                 // query rows per tile
 constexpr int kBN = 128;                 // keys per block
 constexpr int kSoftWarps = 8;            // warps 0-3: rows of tile 0, warps 4-7: rows of tile 1
-constexpr int kLoadWarp = 8, kScoreWarp = 9, kProductWarp = 10;
-constexpr int kAttnThreads = 384;         // three warpgroups: two of softmax, one of the rest (its fourth warp does nothing)
+constexpr int kLoadWarp = 8, kScoreWarp = 9, kProductWarp = 10, kHelpWarp = 11;
+constexpr int kAttnThreads = 384;         // three warpgroups: two of softmax, one of the rest
 // Registers: 384 threads x 168 at launch; the third warpgroup gives back what the softmax takes.
 constexpr int kSoftRegs = 208, kOtherRegs = 80;
 static_assert(2 * kSoftRegs + kOtherRegs <= 3 * 168, "a split above the launch's registers would wait for good");
@@ -212,7 +212,7 @@ attention_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
                 mbar_init(bar(kBarQFull, x), 1); mbar_init(bar(kBarQFree, x), 1); mbar_init(bar(kBarSFull, x), 1); mbar_init(bar(kBarSFree, x), 4);
                 mbar_init(bar(kBarPFull, x), 4); mbar_init(bar(kBarOFull, x), 1); mbar_init(bar(kBarDrain, x), 1);
             }
-            for (uint32_t i = 0; i < (uint32_t)kRecords; ++i) { mbar_init(bar(kBarItemFull, i), 1); mbar_init(bar(kBarItemFree, i), kSoftWarps + 2); }
+            for (uint32_t i = 0; i < (uint32_t)kRecords; ++i) { mbar_init(bar(kBarItemFull, i), 1); mbar_init(bar(kBarItemFree, i), kSoftWarps + 2 + GATHER); }
             for (uint32_t i = 0; i < (uint32_t)kKSlots; ++i) { mbar_init(bar(kBarKFull, i), 1); mbar_init(bar(kBarKFree, i), 1); }
             for (uint32_t i = 0; i < (uint32_t)kVSlots; ++i) { mbar_init(bar(kBarVFull, i), 1); mbar_init(bar(kBarVFree, i), 1); }
             *abort_gen = 0;
@@ -240,56 +240,66 @@ attention_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
 
     if (warp >= kSoftWarps) {
     reg_dec<kOtherRegs>();
-    if (warp == kLoadWarp) {
-        // ---- loads, and the hand-out of items: all lanes go along (a fetch by index takes the whole warp) ----
+    if (warp == kLoadWarp || (GATHER && warp == kHelpWarp)) {
+        // ---- loads, and the hand-out of items: all lanes go along.  A fetch by index is shared by two warps, the loading one and its helper, which
+        // go through the same tiles (the helper by the item records): a warp issues a gather4 of 512 bytes per 90 cycles, two of them twice that, as
+        // two CTAs per SM did.  K and V by index, 28 / 4 heads of 128, us a call, two CTAs per SM / one CTA, one warp /
+        // two warps: 8192 tokens 1231 / 1164 / 604, 100 sequences of 100 143 / 193 / 109; heads of 64, 8192 tokens 654 / 674 / 394. ----
+        const bool helper = GATHER && warp == kHelpWarp;
         uint32_t k_fills = 0, v_fills = 0, items = 0, turn = 0, q_any = 0, q_par = 0;      // q_any, q_par: bit x = tile x was ever loaded, parity of its count
         const int n_items = *p.n_items;
         auto wait = [&](uint32_t b, uint32_t parity) { return attn_wait_warp(b, parity, abort_gen); };
         int seq_a = 0, seq_b = 0;
-        // tile of 128 packed rows starting at row0; by index: lane l brings rows 4l .. 4l+3
-        auto load_tile = [&](uint32_t sT, const CUtensorMap* map, uint32_t b, int head, int row0, bool by_index) {
-            if (lane == 0) mbar_arrive_expect_tx(b, L::kTileBytes);
-            if (GATHER && by_index) {
-                __syncwarp();
-                int r[4];
+        // Tile of 128 packed rows starting at row0 into a buffer that has been given free.  By index: a lane brings rows 4 lane .. 4 lane + 3 of a
+        // 64-column chunk, of two chunks each warp one, of one chunk each every second lane.
+        auto load_tile = [&](uint32_t sT, const CUtensorMap* map, uint32_t full, uint32_t free, uint32_t parity, int head, int row0, bool by_index) {
+            int r[4];
+            const bool mine = KCH == 2 || (lane & 1) == (int)helper;
+            if (GATHER && by_index && mine) {
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     const int pr = row0 + 4 * lane + k;                  // rows past the sequence's end: its last row again (masked / zeroed later)
                     r[k] = p.idx[pr < seq_b ? pr : seq_b - 1];
                 }
-#pragma unroll
-                for (int c = 0; c < KCH; ++c) tma_gather4(sT + c * kChunkBytes + lane * 512, map, b, head * D + c * 64, r[0], r[1], r[2], r[3]);
+            }
+            if (!wait(free, parity)) return false;
+            if (lane == 0 && !helper) mbar_arrive_expect_tx(full, L::kTileBytes);
+            if (GATHER && by_index) {
+                __syncwarp();
+                const int c = KCH == 2 ? (int)helper : 0;
+                if (mine) tma_gather4(sT + c * kChunkBytes + lane * 512, map, full, head * D + c * 64, r[0], r[1], r[2], r[3]);
             } else if (lane == 0) {
 #pragma unroll
-                for (int c = 0; c < KCH; ++c) tma_load_3d(sT + c * kChunkBytes, map, b, c * 64, head, row0);
+                for (int c = 0; c < KCH; ++c) tma_load_3d(sT + c * kChunkBytes, map, full, c * 64, head, row0);
             }
+            return true;
         };
         const bool kv_by_index = GATHER && !p.kv_packed;
         auto load_q = [&](int x, int head, int tile) {
-            if (!wait(bar(kBarQFree, x), ((q_par >> x) & 1) ^ 1)) return false;
-            load_tile(sQ + x * L::kTileBytes, &mapQ, bar(kBarQFull, x), head, seq_a + tile * kBM, GATHER);
+            if (!load_tile(sQ + x * L::kTileBytes, &mapQ, bar(kBarQFull, x), bar(kBarQFree, x), ((q_par >> x) & 1) ^ 1, head, seq_a + tile * kBM, GATHER)) return false;
             q_any |= 1u << x; q_par ^= 1u << x;
             return true;
         };
         auto load_k = [&](int kvh, int j) {
+            if (helper && !kv_by_index) return true;
             const uint32_t slot = k_fills % kKSlots;
-            if (!wait(bar(kBarKFree, slot), ((k_fills / kKSlots) & 1) ^ 1)) return false;
-            load_tile(sK + slot * L::kTileBytes, &mapK, bar(kBarKFull, slot), kvh, seq_a + j * kBN, kv_by_index);
+            if (!load_tile(sK + slot * L::kTileBytes, &mapK, bar(kBarKFull, slot), bar(kBarKFree, slot), ((k_fills / kKSlots) & 1) ^ 1, kvh, seq_a + j * kBN, kv_by_index)) return false;
             ++k_fills;
             return true;
         };
         auto load_v = [&](int kvh, int j) {
+            if (helper && !kv_by_index) return true;
             const uint32_t slot = v_fills % kVSlots;
-            if (!wait(bar(kBarVFree, slot), ((v_fills / kVSlots) & 1) ^ 1)) return false;
-            load_tile(sV + slot * L::kTileBytes, &mapV, bar(kBarVFull, slot), kvh, seq_a + j * kBN, kv_by_index);
+            if (!load_tile(sV + slot * L::kTileBytes, &mapV, bar(kBarVFull, slot), bar(kBarVFree, slot), ((v_fills / kVSlots) & 1) ^ 1, kvh, seq_a + j * kBN, kv_by_index)) return false;
             ++v_fills;
             return true;
         };
         // next item: its number, and then its plan entry (the sequence's bounds ride along); two round trips to L2, with loads in between
         int item = 0, asked = 0;
         int4 e = make_int4(0, -1, 0, 0);
-        auto ask = [&]() { if (lane == 0) asked = (int)atomicAdd(p.ticket, 1u); };
+        auto ask = [&]() { if (lane == 0 && !helper) asked = (int)atomicAdd(p.ticket, 1u); };
         auto take = [&]() {
+            if (helper) return;
             item = __shfl_sync(0xffffffffu, asked, 0);
             e = item < n_items ? p.plan[item / p.Hq] : make_int4(0, -1, 0, 0);
         };
@@ -298,20 +308,30 @@ attention_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
         bool ok = true;
         for (;;) {
             const uint32_t slot = items % kRecords;
-            ok = wait(bar(kBarItemFree, slot), ((items / kRecords) & 1) ^ 1);
-            if (!ok) break;
-            const int h = item % p.Hq, qt = e.y, kvh = h / G, nb = qt + 1;
-            seq_a = e.z; seq_b = e.w;
-            // An item of one tile takes tile 0 and tile 1 of the CTA in turn (0 behind a pair, whose tile 0 ends first): its start overlaps the
-            // end of the one before it, as it did with two CTAs per SM.  us a call, two CTAs of one tile / one CTA, every item in tile 1 / in
-            // turn: 200 sequences of 100 tokens, 28 / 4 heads of 128 157 / 163 / 116, 32 / 8 heads of 64 120 / 146 / 103; 64 of 300, 28 / 4 175 / 148 / 133.
-            const bool pair = e.x != 0;
-            const int first = pair ? 0 : (int)turn, last = pair ? 1 : (int)turn;
-            turn = pair ? 0 : turn ^ 1;
-            if (lane == 0) {
-                records[slot] = AttnItem(seq_a, seq_b, qt, h, first, last).pack();
-                mbar_arrive(bar(kBarItemFull, slot));
+            if (!helper) {
+                // An item of one tile takes tile 0 and tile 1 of the CTA in turn (0 behind a pair, whose tile 0 ends first): its start overlaps the
+                // end of the one before it, as it did with two CTAs per SM.  us a call, two CTAs of one tile / one CTA, every item in tile 1 / in
+                // turn: 200 sequences of 100 tokens, 28 / 4 heads of 128 157 / 163 / 116, 32 / 8 heads of 64 120 / 146 / 103; 64 of 300, 28 / 4 175 / 148 / 133.
+                const bool pair = e.x != 0;
+                ok = wait(bar(kBarItemFree, slot), ((items / kRecords) & 1) ^ 1);
+                if (ok && lane == 0) {
+                    records[slot] = AttnItem(e.z, e.w, e.y, item % p.Hq, pair ? 0 : (int)turn, pair ? 1 : (int)turn).pack();
+                    mbar_arrive(bar(kBarItemFull, slot));
+                }
+                turn = pair ? 0 : turn ^ 1;
+                __syncwarp();
+            } else {
+                ok = wait(bar(kBarItemFull, slot), (items / kRecords) & 1);
             }
+            if (!ok) break;
+            const AttnItem it(records[slot]);
+            if (helper) {
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar(kBarItemFree, slot));
+            }
+            seq_a = it.seq_a; seq_b = it.seq_b;
+            const int h = it.h, qt = it.top, kvh = h / G, nb = qt + 1, last = it.last;
+            const bool pair = it.first < last;
             ++items;
             if (qt < 0) break;
             // in the order of use; the next item is asked for while this one's last tiles are waited for

@@ -1,5 +1,5 @@
 """The hand-overs of the prefill attention kernel (csrc/attention.cu), run through a model on the CPU: one generator per role (loads and items, scores,
-products, eight softmax warps), barriers that show one bit of their phase, loads that land in any order, products and commits that complete in the
+products, eight softmax warps, where rows are fetched by index a second loading warp), barriers that show one bit of their phase, loads that land in any order, products and commits that complete in the
 order in which their thread issued them, at any time.  Every buffer carries what was put into it and every reader checks it; a state in
 which nothing can move is an error."""
 import itertools
@@ -26,13 +26,14 @@ class Bar:
 class Model:
     """items: (pair, top), top the number of the highest query tile, key blocks 0 .. top; a pair has tile top - 1 as well."""
 
-    def __init__(self, items, rng, wait_free=True):
+    def __init__(self, items, rng, wait_free=True, helper=False):
+        self.helper, self.parts = helper, {}
         self.items, self.rng, self.wait_free, self.ragged = items, rng, wait_free, [rng.random() < 0.7 for _ in items]
         two = lambda c: [Bar(c), Bar(c)]
         self.q_full, self.q_free, self.s_full, self.s_free, self.p_full, self.o_full = two(1), two(1), two(1), two(4), two(4), two(1)
         self.k_full, self.k_free = [Bar(1) for _ in range(K_SLOTS)], [Bar(1) for _ in range(K_SLOTS)]
         self.v_full, self.v_free = [Bar(1) for _ in range(V_SLOTS)], [Bar(1) for _ in range(V_SLOTS)]
-        self.i_full, self.i_free = [Bar(1) for _ in range(RECORDS)], [Bar(10) for _ in range(RECORDS)]
+        self.i_full, self.i_free = [Bar(1) for _ in range(RECORDS)], [Bar(10 + helper) for _ in range(RECORDS)]
         self.rec, self.q, self.k, self.v = [None] * RECORDS, [None] * 2, [None] * K_SLOTS, [None] * V_SLOTS
         self.cleared = [0] * V_SLOTS
         self.s, self.s_readers, self.p, self.o = None, 0, [[None] * 4, [None] * 4], [None] * 2
@@ -48,13 +49,20 @@ class Model:
     def land(self):
         at = self.rng.choices(range(len(self.landing)), [self.haste[id(e[0])] for e in self.landing])[0]
         buf, slot, what, full = self.landing.pop(at)
+        if self.helper:                                 # a tile is there when both warps' halves are
+            parts = self.parts.setdefault((id(buf), slot), [])
+            parts.append(what)
+            assert parts.count(what) == len(parts)
+            if len(parts) < 2:
+                return
+            parts.clear()
         buf[slot] = what
         if buf is self.v:
             self.cleared[slot] = 0
         full.arrive()
 
     # -- roles --
-    def loader(self):
+    def loader(self, helps=False):
         kf = vf = turn = 0
         qn = [0, 0]
 
@@ -65,12 +73,16 @@ class Model:
 
         for n, (pair, top) in enumerate(self.items + [(False, -1)]):
             slot = n % RECORDS
-            yield self.i_free[slot], ((n // RECORDS) & 1) ^ 1
-            pair = pair and top > 0
-            first, last = (0, 1) if pair else (turn, turn)
-            turn = 0 if pair else turn ^ 1
-            self.rec[slot] = (n, top, first, last)
-            self.i_full[slot].arrive()
+            if helps:
+                _, top, first, last = yield from self.next_item(n)
+                pair = first < last
+            else:
+                yield self.i_free[slot], ((n // RECORDS) & 1) ^ 1
+                pair = pair and top > 0
+                first, last = (0, 1) if pair else (turn, turn)
+                turn = 0 if pair else turn ^ 1
+                self.rec[slot] = (n, top, first, last)
+                self.i_full[slot].arrive()
             if top < 0:
                 return
             if pair:
@@ -188,7 +200,7 @@ class Model:
                 self.done.append((n, qt))
 
     def run(self):
-        roles = [self.loader(), self.score(), self.product()] + [self.softmax(x, w) for x in range(2) for w in range(4)]
+        roles = [self.loader()] + [self.loader(True)] * self.helper + [self.score(), self.product()] + [self.softmax(x, w) for x in range(2) for w in range(4)]
         waits = {g: None for g in roles}
         # speeds drawn anew for every run: some roles and kinds of work are much slower than others
         speed = {k: self.rng.choice([1, 1, 4, 30]) for k in [*roles, "land", "score", "product"]}
@@ -221,10 +233,11 @@ def _mixes():
         yield [(rng.random() < 0.5, min(int(rng.expovariate(0.6)), 6)) for _ in range(rng.randint(4, 12))]
 
 
-def test_no_mix_of_items_gets_stuck_or_reads_a_buffer_out_of_turn():
+@pytest.mark.parametrize("helper", [False, True], ids=["tiles", "rows by index"])
+def test_no_mix_of_items_gets_stuck_or_reads_a_buffer_out_of_turn(helper):
     for n, items in enumerate(_mixes()):
         for s in range(3):
-            Model(items, random.Random(1000 * n + s)).run()
+            Model(items, random.Random(1000 * n + s), helper=helper).run()
 
 
 def test_the_model_sees_a_softmax_warp_that_takes_an_older_v_tile_for_its_own():

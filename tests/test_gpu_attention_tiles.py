@@ -7,7 +7,7 @@ import torch
 
 from paper_2604_18103_b200 import dash
 from paper_2604_18103_b200 import workloads as wl
-from test_gpu_kernels import _attention_case
+from test_gpu_kernels import _attention_case, _indexed_attention_case
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
@@ -96,3 +96,10 @@ def test_attention_items_follow_the_true_lengths(lengths, Hq, Hkv, D, rows):
     tiles = [(x + 127) // 128 for x in lengths]
     expect = sum((t + 1) // 2 for t in tiles) if len(lengths) == 20 else sum(tiles)
     assert _entries(lengths, Hq, Hkv, D) == expect and _entries(lengths, Hq, Hkv, D, rows, rows) == expect
+
+
+@pytest.mark.parametrize("lengths", [[150] * 60 + [1, 128, 40, 7], [700, 130, 1, 300, 900] * 4], ids=["one or two tiles", "pairs"])
+@pytest.mark.parametrize("D", [64, 128])
+def test_attention_by_index_of_many_sequences(lengths, D):
+    """Two warps share every fetch by index, items of one tile and pairs."""
+    _indexed_attention_case(lengths, 0.6, 12, 4, D, 37)
