@@ -102,7 +102,8 @@ struct AttnParams {
     int* status;
     const int4* plan;           // (1: a pair of tiles, highest query tile, first row, end row of the sequence) of every item group, heaviest first; Hq items (heads) per entry
     const int* n_items;         // device: entries * Hq
-    unsigned int* ticket;       // device: next item to hand out
+    int64_t max_entries;        // entries that the plan has room for
+    unsigned int* ticket;       // device: items handed out beyond the first one of every CTA
     const int32_t* idx;         // GATHER: packed row i is row idx[i] of the full-length Q (and of K, V unless kv_packed)
     int kv_packed;              // GATHER: K and V are packed already ([n, Hkv, D], tiled loads); only Q is fetched by index
 };
@@ -252,7 +253,7 @@ attention_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
         int seq_a = 0, seq_b = 0;
         // Tile of 128 packed rows starting at row0 into a buffer that has been given free.  By index: a lane brings rows 4 lane .. 4 lane + 3 of a
         // 64-column chunk, of two chunks each warp one, of one chunk each every second lane.
-        auto load_tile = [&](uint32_t sT, const CUtensorMap* map, uint32_t full, uint32_t free, uint32_t parity, int head, int row0, bool by_index) {
+        auto load_tile = [&](uint32_t sT, const CUtensorMap* map, uint32_t full, bool used, uint32_t free, uint32_t parity, int head, int row0, bool by_index) {
             int r[4];
             const bool mine = KCH == 2 || (lane & 1) == (int)helper;
             if (GATHER && by_index && mine) {
@@ -262,7 +263,7 @@ attention_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
                     r[k] = p.idx[pr < seq_b ? pr : seq_b - 1];
                 }
             }
-            if (!wait(free, parity)) return false;
+            if (used && !wait(free, parity)) return false;        // (a buffer's first load has nothing to wait for, and a wait takes its 60 to 100 cycles)
             if (lane == 0 && !helper) mbar_arrive_expect_tx(full, L::kTileBytes);
             if (GATHER && by_index) {
                 __syncwarp();
@@ -276,35 +277,37 @@ attention_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
         };
         const bool kv_by_index = GATHER && !p.kv_packed;
         auto load_q = [&](int x, int head, int tile) {
-            if (!load_tile(sQ + x * L::kTileBytes, &mapQ, bar(kBarQFull, x), bar(kBarQFree, x), ((q_par >> x) & 1) ^ 1, head, seq_a + tile * kBM, GATHER)) return false;
+            if (!load_tile(sQ + x * L::kTileBytes, &mapQ, bar(kBarQFull, x), (q_any >> x) & 1, bar(kBarQFree, x), ((q_par >> x) & 1) ^ 1, head, seq_a + tile * kBM, GATHER)) return false;
             q_any |= 1u << x; q_par ^= 1u << x;
             return true;
         };
         auto load_k = [&](int kvh, int j) {
             if (helper && !kv_by_index) return true;
             const uint32_t slot = k_fills % kKSlots;
-            if (!load_tile(sK + slot * L::kTileBytes, &mapK, bar(kBarKFull, slot), bar(kBarKFree, slot), ((k_fills / kKSlots) & 1) ^ 1, kvh, seq_a + j * kBN, kv_by_index)) return false;
+            if (!load_tile(sK + slot * L::kTileBytes, &mapK, bar(kBarKFull, slot), k_fills >= kKSlots, bar(kBarKFree, slot), ((k_fills / kKSlots) & 1) ^ 1, kvh, seq_a + j * kBN, kv_by_index)) return false;
             ++k_fills;
             return true;
         };
         auto load_v = [&](int kvh, int j) {
             if (helper && !kv_by_index) return true;
             const uint32_t slot = v_fills % kVSlots;
-            if (!load_tile(sV + slot * L::kTileBytes, &mapV, bar(kBarVFull, slot), bar(kBarVFree, slot), ((v_fills / kVSlots) & 1) ^ 1, kvh, seq_a + j * kBN, kv_by_index)) return false;
+            if (!load_tile(sV + slot * L::kTileBytes, &mapV, bar(kBarVFull, slot), v_fills >= kVSlots, bar(kBarVFree, slot), ((v_fills / kVSlots) & 1) ^ 1, kvh, seq_a + j * kBN, kv_by_index)) return false;
             ++v_fills;
             return true;
         };
-        // next item: its number, and then its plan entry (the sequence's bounds ride along); two round trips to L2, with loads in between
-        int item = 0, asked = 0;
-        int4 e = make_int4(0, -1, 0, 0);
-        auto ask = [&]() { if (lane == 0 && !helper) asked = (int)atomicAdd(p.ticket, 1u); };
+        // Next item: its number, and then its plan entry (the sequence's bounds ride along); two round trips to L2, with loads in between.  The first
+        // item is the CTA's own number, tickets count on from there, and its entry is fetched beside the number of items: one round trip instead of three
+        // ahead of the first load (one sequence of 64 tokens, 28 / 4 heads of 128, 10.1 -> 9.5 us a call, with two CTAs per SM 9.0; two of 500 14.0 -> 13.4, 16.6).
+        int item = (int)blockIdx.x, asked = 0;
+        const int64_t at = item / p.Hq;
+        int4 e = p.plan[at < p.max_entries ? at : 0];
+        auto ask = [&]() { if (lane == 0 && !helper) asked = (int)(gridDim.x + atomicAdd(p.ticket, 1u)); };
         auto take = [&]() {
             if (helper) return;
             item = __shfl_sync(0xffffffffu, asked, 0);
             e = item < n_items ? p.plan[item / p.Hq] : make_int4(0, -1, 0, 0);
         };
-        ask();
-        take();
+        if (item >= n_items) e = make_int4(0, -1, 0, 0);
         bool ok = true;
         for (;;) {
             const uint32_t slot = items % kRecords;
@@ -313,7 +316,7 @@ attention_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
                 // end of the one before it, as it did with two CTAs per SM.  us a call, two CTAs of one tile / one CTA, every item in tile 1 / in
                 // turn: 200 sequences of 100 tokens, 28 / 4 heads of 128 157 / 163 / 116, 32 / 8 heads of 64 120 / 146 / 103; 64 of 300, 28 / 4 175 / 148 / 133.
                 const bool pair = e.x != 0;
-                ok = wait(bar(kBarItemFree, slot), ((items / kRecords) & 1) ^ 1);
+                ok = items < kRecords || wait(bar(kBarItemFree, slot), ((items / kRecords) & 1) ^ 1);
                 if (ok && lane == 0) {
                     records[slot] = AttnItem(e.z, e.w, e.y, item % p.Hq, pair ? 0 : (int)turn, pair ? 1 : (int)turn).pack();
                     mbar_arrive(bar(kBarItemFull, slot));
@@ -769,6 +772,7 @@ static int attention_impl(const void* Q, const void* K, const void* V, void* O, 
     p.ticket = (unsigned int*)ws;
     p.n_items = (const int*)((char*)ws + 4);
     p.plan = (const int4*)((char*)ws + 256);
+    p.max_entries = (int64_t)plan_entries(n, S);
     if (!planned && (rc = attention_plan(cu_seqlens, S, n, Hq, ws, ws_bytes, st)) != DASH_OK) return rc;
     // persistent CTAs, one per SM, never more than there can be items
     int64_t grid64 = (max_seqlen + kBM - 1) / kBM * Hq * S;
