@@ -8,29 +8,69 @@ import torch
 from paper_2604_18103_b200 import dash
 from paper_2604_18103_b200 import workloads as wl
 from test_gpu_kernels import _attention_case, _indexed_attention_case
+from test_gpu_layer import StepBuffers, run_step
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
 
 
-# few items: tiles alone; the last two lists are long enough for pairs, with odd and even numbers of tiles and empty sequences
-EDGES = [[1], [127], [128], [129], [255, 256, 257], [385, 0, 1, 512, 640, 641], [1, 128, 129, 256, 257, 300, 383, 384, 385, 511, 513, 900] * 3]
+# few items: tiles alone; the last list is long enough for pairs, with odd and even numbers of tiles and empty sequences
+EDGES = [[1], [127], [128], [129], [255, 256, 257], [385, 0, 1, 512, 640, 641], [1, 128, 129, 256, 0, 257, 300, 383, 384, 385, 511, 513, 900] * 4]
 
 
 @pytest.mark.parametrize("lengths", EDGES, ids=lambda x: f"{len(x)}x{max(x)}")
 @pytest.mark.parametrize("D", [64, 128])
 def test_attention_at_the_edges_of_tiles(lengths, D):
+    pairs, tiles = len(lengths) > 6, [(x + 127) // 128 for x in lengths]
+    assert all(_entries(lengths, h, g, D) == sum((t + pairs) // (1 + pairs) for t in tiles) for h, g in ((4, 2), (7, 1)))
     _attention_case(lengths, 4, 2, D, torch.bfloat16, 31, pad=7)
     _attention_case(lengths, 7, 1, D, torch.bfloat16, 32)
 
 
+PAIRED = [900, 640, 513, 385] * 5                       # enough for pairs with 14 heads and up
+
+
+@pytest.mark.parametrize("D", [64, 128])
 @pytest.mark.parametrize("at", [100, 128, 255, 256, 700])
-def test_attention_rescales_in_either_tile_of_a_pair(at):
-    # scores grow at a key, 14 sequences so that the call has its tiles in pairs: the jump lies inside the first block, on block boundaries,
+def test_attention_rescales_in_either_tile_of_a_pair(at, D):
+    # scores grow at a key, the call has its tiles in pairs: the jump lies inside the first block, on block boundaries,
     # in the diagonal block of a pair's lower and of its upper tile.  One or two keys take all the weight of a row then, and the rounding of P and of
-    # O to bf16 is off by up to 2^-9 (sum p |v| + |o|) <= 2^-8 max |v|: 0.0207 for the largest of these 4e6 normal values, 5.3; the smallest
+    # O to bf16 is off by up to 2^-9 (sum p |v| + |o|) <= 2^-8 max |v|: 0.0207 for the largest of these 3e6 normal values, 5.3; the smallest
     # root mean square that a row is held against is 0.9, hence the 0.025.
-    _attention_case([900, 640, 513, 385] * 5, 14, 2, 128, torch.bfloat16, 33, pad=5, tol=2.5e-2, key_gain=[(at, 30.0), (at + 130, 3.0)])
+    _attention_case(PAIRED, 14, 2, D, torch.bfloat16, 33, pad=5, tol=2.5e-2, key_gain=[(at, 30.0), (at + 130, 3.0)])
+
+
+@pytest.mark.parametrize("D", [64, 128])
+def test_fp32_attention_in_pairs(D):
+    """fp32 results have a store path of their own.  Of values that bf16 holds exactly the two calls have the same operands, so the fp32 result rounded to
+    bf16 is the bf16 result, to the bit; that one is held against the oracle."""
+    assert _entries(PAIRED, 14, 2, D, dtype=torch.float32) == sum((x + 255) // 256 for x in PAIRED)
+    g = torch.Generator().manual_seed(38)
+    cu, n = wl.cu_from_lengths(PAIRED).to(DEV), sum(PAIRED)
+    Q, K, V = (torch.randn(n, h, D, generator=g).to(torch.bfloat16).to(DEV) for h in (14, 2, 2))
+    O, lse = dash.dash_varlen_attention(Q, K, V, cu, max(PAIRED), want_lse=True)
+    O32, lse32 = dash.dash_varlen_attention(Q.float(), K.float(), V.float(), cu, max(PAIRED), want_lse=True)
+    assert torch.equal(O32.to(torch.bfloat16), O) and torch.equal(lse32, lse)
+    _attention_case(PAIRED, 14, 2, D, torch.bfloat16, 38)
+
+
+@pytest.mark.parametrize("D", [64, 128])
+def test_fp32_step_multiplies_the_bf16_copy_of_its_attention_in_pairs(D):
+    """A step's attention leaves O in fp32 and, for the output projection, in bf16: O is what the plain call gives for the step's Q, K and V, to the bit,
+    and U is bf16(O) Wo up to fp32 sums of Hq D products, each sum off by at most Hq D 2^-24 of the sum of their absolute values."""
+    shape = wl.LayerShape(d=256, Hq=16, Hkv=4, D=D, rope_base=1.0e4, dtype=torch.float32)
+    cu = wl.cu_from_lengths(PAIRED)
+    n, nq, hd = int(cu[-1]), (shape.Hq + 2 * shape.Hkv) * D, shape.Hq * D
+    W = wl.layer_weights(shape, 39)
+    layer = dash.Layer(shape, W, DEV, sel_mode=dash.SEL_KEEP_COUNT, keep_counts=torch.tensor([x // 2 for x in PAIRED], dtype=torch.int32, device=DEV))
+    bufs = StepBuffers(layer, n, len(PAIRED), n, shape.dtype)
+    H, tok = wl.hidden_states(n, shape.d, 39, shape.dtype).to(DEV), torch.arange(n, dtype=torch.int32, device=DEV)
+    run_step(layer, H, tok, wl.positions(cu).to(DEV), cu.to(DEV), max(PAIRED), torch.zeros_like(H), bufs)
+    QKV, O = bufs.view(bufs.lay.QKV, n, nq, torch.float32), bufs.view(bufs.lay.O, n, hd, torch.float32)
+    q, k, v = (x.view(n, -1, D) for x in QKV.split([hd, shape.Hkv * D, shape.Hkv * D], dim=1))
+    assert torch.equal(O, dash.dash_varlen_attention(q, k, v, cu.to(DEV), max(PAIRED)).view(n, hd))
+    U, O16, Wo = bufs.view(bufs.lay.U, n, shape.d, torch.float32).double(), O.to(torch.bfloat16).double(), W["Wo"].to(DEV).to(torch.bfloat16).double()
+    assert bool(((U - O16 @ Wo).abs() <= hd * 2.0 ** -24 * (O16.abs() @ Wo.abs())).all())
 
 
 def test_attention_of_a_sequence_is_the_same_alone_and_in_a_batch():
@@ -79,12 +119,12 @@ def test_attention_of_short_sequences_keeps_their_rows_apart(lengths, D):
     assert dash.dash_check_status() == dash.OK
 
 
-def _entries(lengths, Hq, Hkv, D, n=None, max_seqlen=None):
+def _entries(lengths, Hq, Hkv, D, n=None, max_seqlen=None, dtype=torch.bfloat16):
     """Entries of the item list that a call leaves in its workspace: tiles, where they go alone, pairs and odd tiles otherwise."""
     cu = wl.cu_from_lengths(lengths).to(DEV)
     n = n or int(cu[-1])
-    Q, K, V = (torch.zeros(n, h, D, dtype=torch.bfloat16, device=DEV) for h in (Hq, Hkv, Hkv))
-    ws = dash.workspace(dash.dash_workspace_bytes(dash.WS_ATTENTION, n, len(lengths), Hq, Hkv, D), DEV)
+    Q, K, V = (torch.zeros(n, h, D, dtype=dtype, device=DEV) for h in (Hq, Hkv, Hkv))
+    ws = dash.workspace(dash.dash_workspace_bytes(dash.WS_ATTENTION, n, len(lengths), Hq, Hkv, D, dash.dtype_code(Q)), DEV)
     dash.dash_varlen_attention(Q, K, V, cu, max_seqlen or max(lengths), ws=ws)
     return int(ws[4:8].view(torch.int32)) // Hq
 

@@ -151,8 +151,8 @@ def test_decode_head_dim_64_no_grouping_and_wide_grouping():
 
 @pytest.mark.parametrize("D", [64, 128])
 def test_decode_right_behind_prefill_attention(D):
-    """Decoding enqueued directly behind a prefill attention on the same caches, several times over without a pause (for heads of 64 the decode
-    kernel's CTAs fit onto the SMs beside the attention kernel's): both results are the bits of calls made one at a time."""
+    """Decoding enqueued directly behind a prefill attention on the same caches, several times over without a pause (the decode kernel
+    is let in while the last CTAs of the attention kernel drain): both results are the bits of calls made one at a time."""
     Hq, Hkv, S, L = 8, 8, 12, 700
     cu = wl.cu_from_lengths([L] * S)
     g = torch.Generator().manual_seed(17)

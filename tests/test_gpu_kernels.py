@@ -371,8 +371,8 @@ def test_attention_varlen_with_empty_and_short_sequences_and_poisoned_tail():
 
 
 def test_attention_scores_that_tower_over_the_first_key_block():
-    # The kernel keeps the first key block's row maximum as the reference of the exponentials and only moves it when a block's
-    # sum says it must.  Here later keys are 40, then 100 times longer: scores tens of units above everything before them, the
+    # The kernel keeps the first key block's row maximum as the reference of the exponentials and moves it where a block's maximum is more than
+    # 2^8 above it.  Here later keys are 40, then 100 times longer: scores tens of units above everything before them, the
     # jumps falling into the second half of a block (position 200), the first half (position 650) and a block's first key (1024).
     _attention_case([1500, 700], 4, 2, 128, torch.bfloat16, 21, key_gain=[(200, 40.0), (650, 2.5), (1024, 3.0)])
     _attention_case([900], 2, 1, 64, torch.bfloat16, 22, key_gain=[(130, 60.0)], pad=4)
