@@ -1,11 +1,12 @@
 // Causal grouped-query attention over a packed (varlen) batch of active tokens,
 // on tcgen05 tensor cores with TMEM accumulators, operands staged by TMA.
 //
-// Work item: two neighbouring tiles of 128 query rows (or one, where a call has few) of one head of one sequence.  A plan lists the items
-// that exist (from cu_seqlens, on the device), heaviest first; persistent CTAs, one per SM, take them by ticket, so that no CTA is
-// spent on query tiles that a shorter sequence does not have.
+// Work item: two neighbouring tiles of 128 query rows, or one (a sequence's odd tile; every tile of a call with few: attention_in_pairs), of one head of
+// one sequence.  A plan lists the items that exist (from cu_seqlens, on the device), heaviest first; persistent CTAs, one per SM, take them
+// by ticket, so that no CTA is spent on query tiles that a shorter sequence does not have.
 // Thread roles: warps 0-3 and 4-7 are the softmax of tile 0 and of tile 1 (thread <-> query row <-> TMEM lane), warp 8 takes the items and
-// loads their tiles, a thread of warp 9 issues the scores, one of warp 10 the products.
+// loads their tiles (with warp 11, where rows are fetched by index), a thread of warp 9 issues the scores, one of warp 10 the products.
+// Items of one tile take tile 0 and tile 1 in turn, so that one item's start overlaps the end of the one before it.
 //
 // Per key block j (128 keys) and tile x, with K_j and V_j in shared memory for both tiles:
 //   S = Q_x K_j^T  (SS MMA, fp32 in TMEM)  ->  softmax warps of x: scores into registers, buffer handed back, mask, maximum, exp2, row
@@ -13,17 +14,12 @@
 // TMEM holds O of both tiles, P of both tiles and ONE score buffer (128 + 128 + 64 + 64 + 128 columns).  The scores are in it only until
 // a tile's threads have loaded them, so the tiles take turns with it, and the next block's scores of a tile are made while its
 // exponentials of this block are still being formed: neither the score nor the product is on the softmax's chain.  Where S and P
-// share columns (one tile per CTA, two CTAs per SM, each a chain score -> softmax -> product -> next score: the kernel that this one
-// replaces) a key block of a tile took 1714 to 1800 cycles of an SM, here 1350; K and V come through shared memory once for two tiles.
-// Heads of 128, 28 / 4, one B200, that kernel and this one: 8192 tokens 411 -> 357 us alone, 472 -> 407 under a steady load (the power
-// cap: 1.65 GHz; 1020 -> 1181 TFLOP/s), 26 214 tokens 3934 -> 3420 and 4472 -> 3900 (1263 TFLOP/s), 5 sequences of 1337 103 -> 87.  What bounds it: per pair
-// of tiles and block 2700 cycles, of which a softmax warp waits 200 for its scores, loads 130, looks for the maximum 385, forms exponentials
-// 1660 (2 x 1024 cycles of the MUFU are the floor of a sub-partition, 2048 cycles that of the tensor pipe).
-// Tried on this kernel and slower: no maximum, the scores kept in registers until the row sum has shown that none was needed (exponentials 2000
-// instead of 1600 cycles, 8192 tokens 382 us where this kernel stood at 376); a warpgroup of its own for the results (402); 16 softmax warps of
-// 16 rows each (their turn takes 2100 cycles, but with four of them on a sub-partition the issuing threads come too late: 427); one thread for
-// scores and products (507 to 640); the maximum of the second half beside the exponentials of the first (402); P rounded by integer
-// instructions (382); one exponential pair in eight by a polynomial of degree 5 on the FMA pipe (374, and 366 where this kernel takes 357), in four (409).
+// share columns (one tile per CTA, two CTAs per SM, each a chain score -> softmax -> product -> next score) a key block of a tile took
+// 1714 to 1800 cycles of an SM, here 1350; K and V come through shared memory once for two tiles.
+// Heads of 128, 28 / 4, one B200, that form and this one, us a call: 8192 tokens 411 / 351 alone, 450 / 390 in a loop at the power cap (1.65 GHz), 26 214 tokens 4400 / 3920
+// (1256 TFLOP/s), 5 sequences of 1337 94 / 72, 200 of 100 157 / 90.  What bounds it: per pair of tiles and block 2700 cycles, of which a softmax warp
+// waits 200 for its scores, loads 130, looks for the maximum 385, forms exponentials 1660 (2 x 1024 cycles of the MUFU are the floor of a
+// sub-partition, 2048 cycles that of the tensor pipe).
 // Causal tile skipping: a query tile only visits key blocks 0..its own index.
 //
 // The kernel is launched to start while the kernel in front of it in the stream drains (barriers, TMEM and descriptor prefetch are
@@ -228,8 +224,8 @@ attention_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    // The kernel behind may set itself up while this one drains, from here on and not before: this CTA holds its TMEM now.  Let in
-    // earlier, a CTA of the kernel behind could take columns in front of a CTA of this grid that it then waits for.
+    // The kernel behind may set itself up from here on, when every CTA of this grid is on its SM and holds its TMEM: on SMs without one, as the register
+    // file is full beside it, and on the others while this kernel drains.
     pdl_launch_dependents();
     pdl_wait();                                            // set-up done; from here on the kernel in front (plan, projection) has completed
     const uint32_t tmem = *tmem_slot_gen;
@@ -507,7 +503,8 @@ attention_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
                 }
                 const float mx = fmaxf(fmaxf(mx0, mx1), fmaxf(mx2, mx3));
                 // The reference m of a row (exponentials are taken of s - m) moves only when a block's maximum is more than 2^8 above it: P up to
-                // 2^8 has the same relative precision in bf16 and is harmless in the fp32 sums.
+                // 2^8 has the same relative precision in bf16 and is harmless in the fp32 sums.  (Not much later either: of a row that one key dominates
+                // P is 1, without rounding, once the reference has moved.)
                 bool o_waited = (j == 0);
                 if (j == 0) {
                     m = mx;                                       // finite: key 0 is visible to every query row
@@ -558,8 +555,8 @@ attention_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
                 }
                 const float2 sum = __fadd2_rn(__fadd2_rn(make_float2(sumA.x, sumC.x), make_float2(sumA.y, sumC.y)),
                                               __fadd2_rn(make_float2(sumB.x, sumD.x), make_float2(sumB.y, sumD.y)));
-                // (waited for and stored behind all exponentials: with the wait and the first store between the halves the loop was cut in two
-                // for the compiler, and a pair's block took 5 % longer: 8192 tokens 376 us instead of 357)
+                // (waited for and stored behind all exponentials: a wait and a store between their halves cut the loop in two for the compiler, and a
+                // pair's block took 5 % longer)
                 if (!o_waited) {                                  // PV_{j-1} has read the P that is overwritten now
                     ok = wait(bar(kBarOFull, x), (blocks - 1) & 1);
                     if (!ok) break;
