@@ -49,7 +49,7 @@ UNIT = "tokens/s"
 L2_FLUSH_BYTES = 256 << 20
 # dram__bytes_read.sum + dram__bytes_write.sum of one attention launch (from the committed ncu summary of this kernel and
 # workload); null where no capture of the current kernel exists
-ATTN_TRAFFIC = {"cfg2": 90.3e6}
+ATTN_TRAFFIC = {"cfg2": 94.8e6}
 
 
 def rank_seed(base: int, rank: int) -> int:
