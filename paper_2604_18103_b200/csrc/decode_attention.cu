@@ -96,11 +96,11 @@ __device__ __forceinline__ void self_plan_build(SelfPlan& sp, const int32_t* cu,
     }
     __syncthreads();
 }
-// Made ahead of its time, from boundaries that may still change: made again if they did
-__device__ __forceinline__ void self_plan_confirm(SelfPlan& sp, const int32_t* cu, int S, int Hkv, int target) {
+// Whether the boundaries have become others since the plan was made from them (called by all threads of the CTA)
+__device__ __forceinline__ bool self_plan_outdated(const SelfPlan& sp, const int32_t* cu, int S) {
     int changed = 0;
     for (int s = threadIdx.x; s <= S; s += blockDim.x) changed |= __ldcg(cu + s) != sp.cu[s];
-    if (__syncthreads_or(changed)) self_plan_build(sp, cu, S, Hkv, target);
+    return __syncthreads_or(changed) != 0;
 }
 __device__ __forceinline__ DecItem self_plan_item(const SelfPlan& sp, int S, int item) {
     int lo = 0, hi = S;               // first[lo] <= item < first[hi]: the last such lo owns the item (sequences without keys own none)
@@ -226,9 +226,40 @@ decode_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
     const uint32_t tS = tmem, tP = tmem, tO = tmem + 128;
     constexpr uint32_t idesc_s = idesc_bf16_f32(128, kDecBN, false, false);
     constexpr uint32_t idesc_o = idesc_bf16_f32(128, D, false, true);
-    if (SELF) self_plan_confirm(sp, p.cu, p.S, p.Hkv, p.target);
-    const int n_items = SELF ? sp.n_items : *p.n_items;
+    // Q and the first key block of an item (one thread)
+    auto load_first = [&](const DecItem& it, int seq_a) {
+        mbar_arrive_expect_tx(bar_q, (uint32_t)(KCH * q_box_heads * 128));
+        for (int c = 0; c < KCH; ++c) tma_load_3d(sQ + c * kChunkBytes, &mapQ, bar_q, c * 64, it.kvh * p.G, it.s);
+        mbar_arrive_expect_tx(bar_k, L::kTileBytes);
+        for (int c = 0; c < KCH; ++c) tma_load_3d(sK + c * kChunkBytes, &mapK, bar_k, c * 64, it.kvh, seq_a + it.b0 * kDecBN);
+        mbar_arrive_expect_tx(bar_v, L::kTileBytes);
+        for (int c = 0; c < KCH; ++c) tma_load_3d(sV + c * kChunkBytes, &mapV, bar_v, c * 64, it.kvh, seq_a + it.b0 * kDecBN);
+    };
     uint32_t blk0 = 0, items_done = 0;       // barrier phases run on across the items of this CTA
+    uint32_t again = 0;                      // loads of Q, K and V that were thrown away: their barriers are that many phases ahead
+    bool loaded = false;                     // the first item's first loads are out
+    if (SELF) {
+        // The loads of the plan made ahead of the wait go out before its boundaries have been compared with those that stand now (0.7 us, and as
+        // much again when the loads read the boundaries from memory once more: Q and the first K were in 2.4 us after the wait, now 1.2).  If they
+        // differ, what was loaded (rows of the maps, or zeros where a coordinate lies outside) is waited for and loaded again by a new plan.
+        loaded = (int)blockIdx.x < sp.n_items;
+        if (tid == 32 && loaded) {
+            const DecItem it = self_plan_item(sp, p.S, (int)blockIdx.x);
+            load_first(it, sp.cu[it.s]);
+        }
+        if (self_plan_outdated(sp, p.cu, p.S)) {
+            if (loaded) {
+                if (tid == 32 && !(mbar_wait(bar_q, 0, kDecWaitCycles) && mbar_wait(bar_k, 0, kDecWaitCycles) && mbar_wait(bar_v, 0, kDecWaitCycles))) {
+                    *abort_gen = 1;
+                    atomicExch(p.status, DASH_ERR_TIMEOUT);
+                }
+                again = 1;
+                loaded = false;
+            }
+            self_plan_build(sp, p.cu, p.S, p.Hkv, p.target);
+        }
+    }
+    const int n_items = SELF ? sp.n_items : *p.n_items;
 
     for (;;) {
         int item;
@@ -242,18 +273,14 @@ decode_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
         if (item >= n_items || *abort_gen) break;
         tc_fence_after();
         const DecItem it = SELF ? self_plan_item(sp, p.S, item) : p.plan[item];
-        const int seq_a = p.cu[it.s], len = p.cu[it.s + 1] - seq_a;
+        const int32_t* cu = SELF ? sp.cu : p.cu;
+        const int seq_a = cu[it.s], len = cu[it.s + 1] - seq_a;
         const int nblk = it.b1 - it.b0;
         const int last_blk = (len + kDecBN - 1) / kDecBN - 1;       // the block of the sequence with a ragged end
         if (warp == 1) {
             if (lane == 0) {
                 bool ok = true;
-                mbar_arrive_expect_tx(bar_q, (uint32_t)(KCH * q_box_heads * 128));
-                for (int c = 0; c < KCH; ++c) tma_load_3d(sQ + c * kChunkBytes, &mapQ, bar_q, c * 64, it.kvh * p.G, it.s);
-                mbar_arrive_expect_tx(bar_k, L::kTileBytes);
-                for (int c = 0; c < KCH; ++c) tma_load_3d(sK + c * kChunkBytes, &mapK, bar_k, c * 64, it.kvh, seq_a + it.b0 * kDecBN);
-                mbar_arrive_expect_tx(bar_v, L::kTileBytes);
-                for (int c = 0; c < KCH; ++c) tma_load_3d(sV + c * kChunkBytes, &mapV, bar_v, c * 64, it.kvh, seq_a + it.b0 * kDecBN);
+                if (!loaded) load_first(it, seq_a);
                 auto issue_s = [&]() {
                     tc_fence_after();
 #pragma unroll
@@ -263,7 +290,7 @@ decode_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
                     }
                     tc_commit(bar_s);
                 };
-                ok = mbar_wait(bar_q, items_done & 1, kDecWaitCycles) && mbar_wait(bar_k, blk0 & 1, kDecWaitCycles);
+                ok = mbar_wait(bar_q, (items_done + again) & 1, kDecWaitCycles) && mbar_wait(bar_k, (blk0 + again) & 1, kDecWaitCycles);
                 if (ok) issue_s();
                 for (int j = 0; j < nblk && ok; ++j) {
                     const uint32_t ph = (blk0 + j) & 1;
@@ -273,7 +300,7 @@ decode_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
                         mbar_arrive_expect_tx(bar_k, L::kTileBytes);
                         for (int c = 0; c < KCH; ++c) tma_load_3d(sK + c * kChunkBytes, &mapK, bar_k, c * 64, it.kvh, seq_a + (it.b0 + j + 1) * kDecBN);
                     }
-                    ok = mbar_wait(bar_p0, ph, kDecWaitCycles) && mbar_wait(bar_v, ph, kDecWaitCycles);
+                    ok = mbar_wait(bar_p0, ph, kDecWaitCycles) && mbar_wait(bar_v, ph ^ again, kDecWaitCycles);
                     if (!ok) break;
                     tc_fence_after();
 #pragma unroll
@@ -287,7 +314,7 @@ decode_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
                         mma_ts(tO, tP + kk * 8, smem_desc_sw128(sV + kk * 2048, kChunkBytes, 1024), idesc_o, 1);
                     tc_commit(bar_o);
                     if (j + 1 < nblk) {
-                        ok = mbar_wait(bar_k, (blk0 + j + 1) & 1, kDecWaitCycles);
+                        ok = mbar_wait(bar_k, (blk0 + j + 1 + again) & 1, kDecWaitCycles);
                         if (!ok) break;
                         issue_s();                                         // in issue order behind PV_j, which reads P_j from the same columns
                     }
@@ -362,7 +389,7 @@ decode_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
                 }
                 if (ragged) {
                     // cached rows past the end of the sequence may hold anything: zero them (0 * garbage must not make a NaN)
-                    ok = mbar_wait(bar_v, ph, kDecWaitCycles);
+                    ok = mbar_wait(bar_v, ph ^ again, kDecWaitCycles);
                     if (!ok) break;
                     for (int r = lane; r < kDecBN; r += 32) {
                         if (r >= valid) {
@@ -400,26 +427,23 @@ decode_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
                 m = m_new;
             }
             if (ok) ok = mbar_wait(bar_o, (blk0 + nblk - 1) & 1, kDecWaitCycles);
-            // row sum: the four threads' shares; then lane r < G writes row r (its m and l sit in thread 4 r)
+            // row sum: the four threads' shares; the row leaves as it is read, four threads to 32 contiguous bytes (a lane per row wrote 8 bytes
+            // of seven rows at a time: 64 store instructions, now 32 of whole sectors)
             l += __shfl_xor_sync(0xffffffffu, l, 1);
             l += __shfl_xor_sync(0xffffffffu, l, 2);
-            const float m_row = __shfl_sync(0xffffffffu, m, (lane * 4) & 31), l_row = __shfl_sync(0xffffffffu, l, (lane * 4) & 31);
-            (void)hrow;
             if (ok && !*abort_gen) {
                 tc_fence_after();
-                float* dst = p.partial + ((size_t)item * kDecRows + lane) * D;
+                float* dst = p.partial + ((size_t)item * kDecRows + hrow) * D + 2 * sub;
+                uint32_t o[D / 2];
 #pragma unroll
-                for (int c = 0; c < D / 32; ++c) {
-                    uint32_t o[32];
-                    tmem_ld32(tO + c * 32, o);
-                    tmem_wait_ld();
-                    if (lane < p.G) {
+                for (int c = 0; c < KCH; ++c) tmem_ld16x256_x8(tO + c * 64, &o[c * 32]);
+                tmem_wait_ld();
+                if (hrow < p.G) {
 #pragma unroll
-                        for (int e = 0; e < 32; e += 2)
-                            *reinterpret_cast<float2*>(dst + c * 32 + e) = make_float2(__uint_as_float(o[e]), __uint_as_float(o[e + 1]));
-                    }
+                    for (int u = 0; u < D / 8; ++u)
+                        *reinterpret_cast<float2*>(dst + 8 * u) = make_float2(__uint_as_float(o[4 * u]), __uint_as_float(o[4 * u + 1]));
+                    if (sub == 0) p.ml[(size_t)(it.kvh * p.G + hrow) * p.max_items + item] = make_float2(m, l);
                 }
-                if (lane < p.G) p.ml[(size_t)(it.kvh * p.G + lane) * p.max_items + item] = make_float2(m_row, l_row);
             } else if (!ok && lane == 0) {
                 *abort_gen = 1;
                 atomicExch(p.status, DASH_ERR_TIMEOUT);
@@ -429,6 +453,7 @@ decode_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
         __syncthreads();                      // end of the item: O read out, every tile buffer free
         blk0 += (uint32_t)nblk;
         ++items_done;
+        loaded = false;
     }
     tc_fence_before();
     __syncthreads();
@@ -512,6 +537,70 @@ __device__ __forceinline__ void decode_merge_units(const MergeParams& p, const S
     }
 }
 
+// The same where there are more units than warps, that is few splits to a sequence and head: a warp takes the whole head, a lane D / 32 neighbouring
+// columns, so that each warp goes through its loads once instead of two or three times.
+template <int D>
+__device__ __forceinline__ void decode_merge_heads(const MergeParams& p, const SelfPlan& sp) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int NW = kMergeThreads / 32, W = D / 32, B = 8;           // B: splits whose loads are in flight at a time
+    const size_t stride = (size_t)kDecRows * D;
+    struct alignas(4 * W) Cols { float v[W]; };
+    for (int u = (int)blockIdx.x * NW + warp; u < p.S * p.Hq; u += (int)gridDim.x * NW) {
+        const int hd = u % p.Hq, s = u / p.Hq, kvh = hd / p.G, row = hd % p.G;
+        int first, cnt;
+        if (!p.seg) { cnt = sp.per[s]; first = sp.first[s] + kvh * cnt; }
+        else { const int2 sg = p.seg[s * p.Hkv + kvh]; first = sg.x; cnt = sg.y; }
+        const float* base = p.partial + ((size_t)first * kDecRows + row) * D + lane * W;
+        const float2* mlb = p.ml + (size_t)hd * p.max_items + first;
+        auto fetch = [&](int i) {
+            Cols c;
+            if (W == 4) { const float4 t = __ldcg(reinterpret_cast<const float4*>(base + i * stride)); c.v[0] = t.x; c.v[1] = t.y; c.v[W - 2] = t.z; c.v[W - 1] = t.w; }
+            else { const float2 t = __ldcg(reinterpret_cast<const float2*>(base + i * stride)); c.v[0] = t.x; c.v[1] = t.y; }
+            return c;
+        };
+        Cols dv[B];
+#pragma unroll
+        for (int b = 0; b < B; ++b)
+            if (b < cnt) dv[b] = fetch(b);
+        float2 ml = lane < cnt ? __ldcg(mlb + lane) : make_float2(-INFINITY, 0.f);
+        float mx = ml.x;
+        for (int i = lane + 32; i < cnt; i += 32) mx = fmaxf(mx, __ldcg(mlb + i).x);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        float ls = 0.f, acc[W];
+#pragma unroll
+        for (int e = 0; e < W; ++e) acc[e] = 0.f;
+        for (int i0 = 0; i0 < cnt; i0 += 32) {                          // 32 splits' weights at a time, lane = split
+            if (i0 > 0) ml = i0 + lane < cnt ? __ldcg(mlb + i0 + lane) : make_float2(-INFINITY, 0.f);
+            const float wgt = exp2f((ml.x - mx) * p.scale_log2);        // 0 where there is no split
+            ls = fmaf(wgt, ml.y, ls);
+            for (int j0 = 0; j0 < min(32, cnt - i0); j0 += B) {
+                if (i0 + j0 > 0) {
+#pragma unroll
+                    for (int b = 0; b < B; ++b)
+                        if (i0 + j0 + b < cnt) dv[b] = fetch(i0 + j0 + b);
+                }
+#pragma unroll
+                for (int b = 0; b < B; ++b) {
+                    const float w = __shfl_sync(0xffffffffu, wgt, j0 + b);
+                    if (i0 + j0 + b < cnt) {
+#pragma unroll
+                        for (int e = 0; e < W; ++e) acc[e] = fmaf(w, dv[b].v[e], acc[e]);
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) ls += __shfl_xor_sync(0xffffffffu, ls, o);
+#pragma unroll
+        for (int e = 0; e < W; ++e) acc[e] = cnt > 0 ? acc[e] / ls : 0.f;
+        __nv_bfloat16* dst = p.out + (int64_t)s * p.ldo + (int64_t)hd * D + lane * W;
+        if (W == 4) *reinterpret_cast<uint2*>(dst) = make_uint2(pack_bf16(acc[0], acc[1]), pack_bf16(acc[W - 2], acc[W - 1]));
+        else *reinterpret_cast<uint32_t*>(dst) = pack_bf16(acc[0], acc[1]);
+        if (p.lse && lane == 0) p.lse[(int64_t)s * p.Hq + hd] = cnt > 0 ? mx * p.scale + logf(ls) : -INFINITY;
+    }
+}
+
 template <int D>
 __global__ void __launch_bounds__(kMergeThreads)
 decode_merge_kernel(const MergeParams p) {
@@ -526,7 +615,8 @@ decode_merge_kernel(const MergeParams p) {
     if (n_units * 16 <= warps) decode_merge_units<D, 8>(p, sp, s_acc);
     else if (n_units * 8 <= warps) decode_merge_units<D, 4>(p, sp, s_acc);
     else if (n_units * 4 <= warps) decode_merge_units<D, 2>(p, sp, s_acc);
-    else decode_merge_units<D, 1>(p, sp, s_acc);
+    else if (n_units <= warps) decode_merge_units<D, 1>(p, sp, s_acc);
+    else decode_merge_heads<D>(p, sp);
 }
 
 static int decode_max_items(int S, int Hkv) { return 4 * sm_count() + S * Hkv; }
