@@ -9,9 +9,9 @@
 //            u^2, h^2 and (h+u)^2 of this tile's columns go to a small buffer (the score of Eq. 2 and the next norm's row factor are
 //            finished from them)
 //   SWIGLU : one tile holds 128 gate and the matching 128 up columns: act = silu(g) * u      (FFN of Alg. 1)
-// One CTA per SM, in clusters of two: a pair computes a 256 x 256 tile with tcgen05.mma.cta_group::2 -- CTA r holds rows
-// 128 r .. of the A tile and columns 128 r .. of the W tile, so every SM loads only half of the W operand.  K in steps of 64
-// through a 6-stage TMA ring; warp 0 of each CTA issues its loads (their bytes are counted on the pair's even CTA), warp 1 of
+// One CTA per SM, in clusters of two: a pair computes a 256 x 256 tile (256 x 128 where there are few, see gemm_narrow) with tcgen05.mma.cta_group::2 -- CTA r holds
+// rows 128 r .. of the A tile and half r of the W tile's columns, so every SM loads only half of the W operand.  K in steps of 64
+// through a TMA ring of 6 (8) stages; warp 0 of each CTA issues its loads (their bytes are counted on the pair's even CTA), warp 1 of
 // the even CTA issues the MMAs and releases stages / hands over accumulators in both CTAs with multicast commits, warps 2-9
 // of each CTA read their 128 accumulator rows (two TMEM buffers, so a tile's epilogue overlaps the next tile's MMAs).
 //
@@ -34,8 +34,12 @@ namespace dash {
 
 using namespace ptx;
 
-constexpr int kGM = 128, kGN = 256, kGK = 64, kGStages = 6;      // kGM: rows per CTA (256 per pair)
-constexpr int kGABytes = kGM * kGK * 2, kGBBytes = kGK * (kGN / 2) * 2, kGStageBytes = kGABytes + kGBBytes;   // per CTA
+constexpr int kGM = 128, kGN = 256, kGNarrow = 128, kGK = 64;    // kGM: rows per CTA (256 per pair); columns of a pair's tile
+constexpr int kGABytes = kGM * kGK * 2;      // per CTA and stage
+// tiles BN columns wide: bytes of a stage per CTA, stages of the ring (192 KB either way)
+template <int BN> struct Ring { static constexpr int kStage = kGABytes + kGK * (BN / 2) * 2, kStages = BN == kGN ? 6 : 8; };
+constexpr int kGRingBytes = Ring<kGN>::kStage * Ring<kGN>::kStages;
+static_assert(kGRingBytes == Ring<kGNarrow>::kStage * Ring<kGNarrow>::kStages, "one size of shared memory");
 constexpr int kGEpiWarps = 8;                // two per TMEM lane quarter, each with one half of the tile's columns
 constexpr int kGThreads = 64 + 32 * kGEpiWarps;
 constexpr int kGEpiBytes = 4096;             // staging per epilogue warp: 32 rows of 128 bytes
@@ -131,7 +135,6 @@ struct GemmArgs {
     int n, N, K;                 // rows (upper bound), columns of W that one tile row of the output spans, depth
     int n_tiles;                 // tiles along the output columns
     void* C; int64_t ldc;        // PLAIN / ROPE / SWIGLU output (elements)
-    int out_f32;                 // PLAIN: C is fp32 (else bf16)
     int w_early;                 // W may be read before the kernel in front is complete
     const int32_t* n_dev;        // device: true number of rows (<= n), or null
     int* status;
@@ -174,9 +177,12 @@ __device__ __forceinline__ void reduce_rows8(float (&v)[8], int lane) {
     }
 }
 
-template <int EPI>
+// F32 (PLAIN, ROPE): C is fp32
+template <int EPI, int BN, bool F32>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGThreads, 1)
 gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapW, const GemmArgs g) {
+    static_assert(BN == kGN || (BN == kGNarrow && EPI != GEMM_SWIGLU), "tile widths");
+    constexpr int kGStages = Ring<BN>::kStages, kGStageBytes = Ring<BN>::kStage;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t bars = base + kGStages * kGStageBytes + kGEpiWarps * kGEpiBytes;
@@ -210,11 +216,11 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
     const uint32_t tmem = *slot_gen;
     const int m_tiles = (g.n + 2 * kGM - 1) / (2 * kGM), n_tiles = g.n_tiles, ksteps = (g.K + kGK - 1) / kGK;
     const int n_pairs = (int)gridDim.x / 2, pair = (int)blockIdx.x / 2;
-    constexpr uint32_t idesc = idesc_bf16_f32(2 * kGM, kGN, false, true);
+    constexpr uint32_t idesc = idesc_bf16_f32(2 * kGM, BN, false, true);
     constexpr uint32_t hi = smem_desc_hi_sw128(1024);
 
     if (warp == 0) {
-        // ---- loads of this CTA: its 128 x 64 half of the A tile (K-major), its 64 x 128 half of the W tile as two 64-column chunks ----
+        // ---- loads of this CTA: its 128 x 64 half of the A tile (K-major), its half of the W tile as one or two chunks of 64 columns ----
         if (lane == 0) {
             uint32_t it = 0;
             bool ok = true;
@@ -227,9 +233,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                 auto load_w = [&](int s, int k) {
                     if (rank == 0) mbar_arrive_expect_tx(full(s), 2 * kGStageBytes);     // both CTAs' bytes land on this barrier
 #pragma unroll
-                    for (int c = 0; c < kGN / 2 / 64; ++c) {
+                    for (int c = 0; c < BN / 2 / 64; ++c) {
                         // SWIGLU: columns 0-127 of the tile (the even CTA's half) are gate features nt * 128 .., columns 128-255 the same features of "up"
-                        const int col = (EPI == GEMM_SWIGLU) ? (rank * g.e.m + nt * 128 + c * 64) : (nt * kGN + rank * (kGN / 2) + c * 64);
+                        const int col = (EPI == GEMM_SWIGLU) ? (rank * g.e.m + nt * 128 + c * 64) : (nt * BN + rank * (BN / 2) + c * 64);
                         tma_load_2d_pair(base + s * kGStageBytes + kGABytes + c * (kGK * 128), &mapW, full(s), col, k * kGK);
                     }
                 };
@@ -255,7 +261,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
             if (!ok) atomicExch(g.status, DASH_ERR_TIMEOUT);
         }
     } else if (warp == 1) {
-        // ---- MMAs (even CTA only): four 256 x 256 x 16 steps per stage into the tile's TMEM buffer of both CTAs ----
+        // ---- MMAs (even CTA only): four 256 x BN x 16 steps per stage into the tile's TMEM buffer of both CTAs ----
         if (lane == 0 && rank == 0) {
             uint32_t it = 0, tl = 0;
             bool ok = true;
@@ -266,7 +272,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                 if (tl >= 2) ok = mbar_wait(acc_empty(b), ((tl >> 1) - 1) & 1, kGWait);
                 if (!ok) break;
                 tc_fence_after();
-                const uint32_t tD = tmem + b * kGN;
+                const uint32_t tD = tmem + b * BN;
                 for (int k = k0; k < k1 && ok; ++k, ++it) {
                     const int s = it % kGStages;
                     ok = mbar_wait(full(s), (it / kGStages) & 1, kGWait);
@@ -284,9 +290,12 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
             if (!ok) atomicExch(g.status, DASH_ERR_TIMEOUT);
         }
     } else {
-        // ---- epilogue: warp (q, half) holds rows 32 q .. of this CTA's 128 and columns 128 half .. of the tile's 256 (SWIGLU: gate and
-        // up columns of features 64 half ..) ----
+        // ---- epilogue: warp (q, half) holds rows 32 q .. of this CTA's 128 and half of the tile's columns (SWIGLU: gate and up columns of
+        // features 64 half ..).  A tile of 256 columns: the four pieces of 128 columns; of 128: two of its four pieces ----
         const int q = warp & 3, half = (warp - 2) >> 2;           // q: the TMEM lane quarter this warp may read
+        const int wcol = BN == kGN ? half * 128 : 0;              // the 128 columns of the tile that this warp's pieces are counted in
+        constexpr int kPieces = BN == kGN ? 4 : 2;                // of 32 columns
+        const int p0 = BN == kGN ? 0 : 2 * half;                  // the first of them
         const uint32_t lane_base = (uint32_t)(q * 32) << 16;
         const uint32_t stage = base + kGStages * kGStageBytes + (warp - 2) * kGEpiBytes;
         pdl_wait();
@@ -300,7 +309,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
         for (; w.next(mt, nt, k0, k1); ++tl) {
             const int b = tl & 1;
             const int row0 = mt * 2 * kGM + rank * kGM + q * 32;  // first row of this warp's 32
-            const uint32_t tD = tmem + b * kGN + lane_base;
+            const uint32_t tD = tmem + b * BN + lane_base;
             auto wait_acc = [&]() { ok = __all_sync(0xffffffffu, mbar_wait(acc_full(b), (tl >> 1) & 1, kGWait)); tc_fence_after(); };
             // every TMEM read of this warp for the tile has completed: the buffer goes back to the MMA thread
             auto release_acc = [&]() {
@@ -319,6 +328,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                        rank * kGM + q * 32 + lane;
             };
             auto leave_part = [&]() -> bool {                     // true: the tile is left to another pair
+                if constexpr (BN != kGN) return false;            // narrow tiles are never cut
                 const long long U = (long long)n_tiles * ksteps, u0 = (long long)nt * ksteps;
                 first_grp = (int)(((u0 + 1) * g.groups - 1) / U);
                 n_parts = (int)(((u0 + ksteps) * g.groups - 1) / U) - first_grp + 1;
@@ -392,21 +402,22 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
             };
             if (EPI == GEMM_PLAIN) {
                 // columns at or past N (a last, partial tile) are not stored; N is a multiple of 8 (bf16) / 4 (fp32)
-                const int col0 = nt * kGN + half * 128;
+                const int col0 = nt * BN + wcol;
                 wait_acc();
                 if (!ok) break;
                 if (k1 - k0 != ksteps && leave_part()) { release_acc(); continue; }
-                if (g.out_f32) {
+                if (F32) {
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
+                    for (int i = 0; i < kPieces; ++i) {
+                        const int k = p0 + i;
                         uint32_t o[32];
-                        load_acc(w16, half * 128 + k * 32, half * 128 + k * 32 + 16, o);
-                        if (k == 3) release_acc();
+                        load_acc(w16, wcol + k * 32, wcol + k * 32 + 16, o);
+                        if (i == kPieces - 1) release_acc();
                         stage_f32(o);
                         const int col = col0 + k * 32 + c8 * 4;
 #pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            const int r = r8 + 4 * i, row = row0 + r;
+                        for (int i2 = 0; i2 < 8; ++i2) {
+                            const int r = r8 + 4 * i2, row = row0 + r;
                             const uint4 v = lds_v4(stage_addr(stage, r, c8));
                             if (row < n_true && col < g.N) st_v4(reinterpret_cast<float*>(g.C) + (int64_t)row * g.ldc + col, v);
                         }
@@ -414,18 +425,19 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                     }
                 } else {
 #pragma unroll
-                    for (int k = 0; k < 2; ++k) {
+                    for (int i = 0; i < kPieces / 2; ++i) {
+                        const int k = p0 / 2 + i;
                         uint32_t o[64];
-                        load_acc(w32, half * 128 + k * 64, half * 128 + k * 64 + 32, o);
-                        if (k == 1) release_acc();
+                        load_acc(w32, wcol + k * 64, wcol + k * 64 + 32, o);
+                        if (i == kPieces / 2 - 1) release_acc();
                         auto pk = [&](int e) { return pack_bf16(__uint_as_float(o[e]), __uint_as_float(o[e + 1])); };
 #pragma unroll
                         for (int c = 0; c < 8; ++c) sts_v4(stage_addr(stage, lane, c), pk(8 * c), pk(8 * c + 2), pk(8 * c + 4), pk(8 * c + 6));
                         __syncwarp();
                         const int col = col0 + k * 64 + c8 * 8;
 #pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            const int r = r8 + 4 * i, row = row0 + r;
+                        for (int i2 = 0; i2 < 8; ++i2) {
+                            const int r = r8 + 4 * i2, row = row0 + r;
                             const uint4 v = lds_v4(stage_addr(stage, r, c8));
                             if (row < n_true && col < g.N) st_v4(reinterpret_cast<__nv_bfloat16*>(g.C) + (int64_t)row * g.ldc + col, v);
                         }
@@ -448,7 +460,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                     tab[i] = (int)trow;
                     rsc[i] = (g.e.row_scale && live) ? g.e.row_scale[row] : 1.0f;
                 }
-                const int colw = nt * kGN + half * 128;           // first column of this warp
+                const int colw = nt * BN + wcol;                  // first column of this warp's 128
                 auto head_of = [&](int k) { return D == 128 ? 0 : (k >> 1) * 64; };
                 auto pair_of = [&](int k) { return D == 128 ? k * 16 : (k & 1) * 16; };
                 const bool tab16 = (reinterpret_cast<uint64_t>(g.e.rope_table) & 15u) == 0;
@@ -470,22 +482,24 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                         }
                     }
                 };
-                fetch_cs(0);
+                fetch_cs(p0);
                 wait_acc();
                 if (!ok) break;
                 if (k1 - k0 != ksteps && leave_part()) { release_acc(); continue; }
 #pragma unroll 1
-                for (int k = 0; k < 4; ++k) {
+                for (int k = p0; k < p0 + kPieces; ++k) {
                     const int h0 = head_of(k), c = pair_of(k), colh = colw + h0;
                     uint32_t o[32];
-                    load_acc(w16, half * 128 + h0 + c, half * 128 + h0 + hd2 + c, o);
-                    if (k == 3) release_acc();
+                    load_acc(w16, wcol + h0 + c, wcol + h0 + hd2 + c, o);
+                    if (k == p0 + kPieces - 1) release_acc();
                     stage_f32(o);
-                    const bool rotate = colh < g.e.n_rot_cols;
-                    // a head of K or V goes to the caller's cache as well
+                    const bool rotate = colh < g.e.n_rot_cols, is_q = colh < g.e.q_cols;
+                    // a head of K or V goes to the caller's cache as well; fp32: every head to the bf16 copies that the attention kernel reads
                     __nv_bfloat16* cache = nullptr;
-                    if (g.e.k_cache && colh >= g.e.q_cols)
+                    int64_t ld_cache = g.e.ld_cache;
+                    if (g.e.k_cache && !is_q)
                         cache = reinterpret_cast<__nv_bfloat16*>(rotate ? g.e.k_cache : g.e.v_cache) + (colh - (rotate ? g.e.q_cols : g.e.n_rot_cols));
+                    if (F32 && is_q) { cache = reinterpret_cast<__nv_bfloat16*>(g.e.q_copy) + colh; ld_cache = g.e.q_cols; }
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
                         const int r = rr + 8 * i, row = row0 + r;
@@ -507,22 +521,29 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                         }
                         if (row < n_true) {
                             const uint32_t a0 = pack_bf16(y1[0], y1[1]), a1 = pack_bf16(y1[2], y1[3]), b0 = pack_bf16(y2[0], y2[1]), b1 = pack_bf16(y2[2], y2[3]);
-                            __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(g.C) + (int64_t)row * g.ldc + colh + c + c4 * 4;
-                            st_v2(dst, a0, a1);
-                            st_v2(dst + hd2, b0, b1);
+                            const int64_t at = (int64_t)row * g.ldc + colh + c + c4 * 4;
+                            if (F32) {
+                                float* dst = reinterpret_cast<float*>(g.C) + at;
+                                st_v4(dst, make_uint4(__float_as_uint(y1[0]), __float_as_uint(y1[1]), __float_as_uint(y1[2]), __float_as_uint(y1[3])));
+                                st_v4(dst + hd2, make_uint4(__float_as_uint(y2[0]), __float_as_uint(y2[1]), __float_as_uint(y2[2]), __float_as_uint(y2[3])));
+                            } else {
+                                __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(g.C) + at;
+                                st_v2(dst, a0, a1);
+                                st_v2(dst + hd2, b0, b1);
+                            }
                             if (cache) {
-                                __nv_bfloat16* kv = cache + (int64_t)row * g.e.ld_cache + c + c4 * 4;
+                                __nv_bfloat16* kv = cache + (int64_t)row * ld_cache + c + c4 * 4;
                                 st_v2(kv, a0, a1);
                                 st_v2(kv + hd2, b0, b1);
                             }
                         }
                     }
-                    if (k < 3) fetch_cs(k + 1);
+                    if (k < p0 + kPieces - 1) fetch_cs(k + 1);
                     __syncwarp();
                 }
             } else if (EPI == GEMM_RESID) {
-                // H~ = H + U (U in fp32, one rounding) to x_full[tok[row]]; sums of u^2, h^2 and (h+u)^2 over this warp's 128 columns
-                const int col0 = nt * kGN + half * 128 + c8 * 4;
+                // H~ = H + U (U in fp32, one rounding) to x_full[tok[row]]; sums of u^2, h^2 and (h+u)^2 over 128 columns
+                const int col0 = nt * BN + wcol + c8 * 4;
                 const __nv_bfloat16* hsrc = reinterpret_cast<const __nv_bfloat16*>(g.e.H) + col0;
                 __nv_bfloat16* xdst = reinterpret_cast<__nv_bfloat16*>(g.e.x_full) + col0;
                 int tok[8];
@@ -539,18 +560,19 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                         if (row < n_true) hv[i] = ld_v2(hsrc + (int64_t)row * g.e.ldh + k * 32);
                     }
                 };
-                fetch_h(0);
+                fetch_h(p0);
                 float su[8], sh[8], st2[8];
 #pragma unroll
                 for (int i = 0; i < 8; ++i) su[i] = sh[i] = st2[i] = 0.f;
                 wait_acc();
-                if (!ok) break;
+                if (BN == kGN && !ok) break;
+                if (!ok) n_true = 0;                              // a narrow tile's two warps meet below, come what may: nothing is stored
                 if (k1 - k0 != ksteps && leave_part()) { release_acc(); continue; }
 #pragma unroll 1
-                for (int k = 0; k < 4; ++k) {
+                for (int k = p0; k < p0 + kPieces; ++k) {
                     uint32_t o[32];
-                    load_acc(w16, half * 128 + k * 32, half * 128 + k * 32 + 16, o);
-                    if (k == 3) release_acc();
+                    load_acc(w16, wcol + k * 32, wcol + k * 32 + 16, o);
+                    if (k == p0 + kPieces - 1) release_acc();
                     stage_f32(o);
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
@@ -570,12 +592,24 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                             st_v2(xdst + (int64_t)tok[i] * g.e.ldx + k * 32, pack_bf16(y[0], y[1]), pack_bf16(y[2], y[3]));
                         }
                     }
-                    if (k < 3) fetch_h(k + 1);
+                    if (k < p0 + kPieces - 1) fetch_h(k + 1);
                     __syncwarp();
                 }
                 reduce_rows8(su, lane); reduce_rows8(sh, lane); reduce_rows8(st2, lane);
                 const int row = row0 + r8 + 4 * c8;               // this lane holds the sums of row r8 + 4 c8
-                if (row < n_true) g.e.sums[(int64_t)row * (2 * n_tiles) + 2 * nt + half] = make_float4(su[0], sh[0], st2[0], 0.f);
+                if (BN == kGN) {
+                    if (row < n_true) g.e.sums[(int64_t)row * (2 * n_tiles) + 2 * nt + half] = make_float4(su[0], sh[0], st2[0], 0.f);
+                } else {
+                    // of 64 columns: the quarter's two warps add theirs up, the second one's through its staging block
+                    if (half == 1) sts_v4(stage + lane * 16, __float_as_uint(su[0]), __float_as_uint(sh[0]), __float_as_uint(st2[0]), 0u);
+                    asm volatile("bar.sync %0, 64;" ::"r"(1 + q) : "memory");
+                    if (half == 0) {
+                        const uint4 o = lds_v4(stage + 4 * kGEpiBytes + lane * 16);
+                        if (row < n_true)
+                            g.e.sums[(int64_t)row * n_tiles + nt] = make_float4(su[0] + __uint_as_float(o.x), sh[0] + __uint_as_float(o.y), st2[0] + __uint_as_float(o.z), 0.f);
+                    }
+                    asm volatile("bar.sync %0, 64;" ::"r"(1 + q) : "memory");
+                }
             } else {
                 // SWIGLU: columns 0-127 gate, 128-255 up of the same 128 features
                 const float rsc = (g.e.row_scale && row0 + lane < n_true) ? g.e.row_scale[row0 + lane] : 1.0f;
@@ -668,17 +702,33 @@ size_t gemm_split_part_bytes(int64_t n, int64_t N, int64_t K) {
 int gemm_tile_rows() { return 2 * kGM; }
 int64_t gemm_split_max_rows() { return (int64_t)(sm_count() / 2) * 2 * kGM; }
 
-template <int EPI>
-static int launch_gemm(const CUtensorMap& ma, const CUtensorMap& mw, GemmArgs g, cudaStream_t st) {
-    const int smem = kGStages * kGStageBytes + kGEpiWarps * kGEpiBytes + 1024 + 256;
+template <int EPI, int BN, bool F32>
+static int launch_tiles(const CUtensorMap& ma, const CUtensorMap& mw, const GemmArgs& g, int pairs, cudaStream_t st) {
+    const int smem = kGRingBytes + kGEpiWarps * kGEpiBytes + 1024 + 256;
     static std::atomic<uint64_t> configured{0};
-    if (!set_max_smem_once(gemm_kernel<EPI>, smem, configured)) return DASH_ERR_CUDA;
-    const int m_tiles = (g.n + 2 * kGM - 1) / (2 * kGM), tiles = m_tiles * g.n_tiles;
+    if (!set_max_smem_once(gemm_kernel<EPI, BN, F32>, smem, configured)) return DASH_ERR_CUDA;
+    return launch_pdl(gemm_kernel<EPI, BN, F32>, 2 * pairs, kGThreads, (size_t)smem, st, ma, mw, g) == cudaSuccess ? DASH_OK : DASH_ERR_CUDA;
+}
+
+// Tiles of 128 columns instead of 256 where every one of them still has a pair of SMs to itself.  What that saves is epilogue: an epilogue warp
+// has half the columns (a 256 x 128 x 16 MMA takes the 134 cycles of a 256 x 256 x 16, so a tile's products take as long).  First
+// tile in to the last result out, us, 256 / 128 columns: Q | K | V of the 7B shape at 233 rows 27 / 21, at 375 27 / 24, output projection at 233 28 / 23, at 375 28 / 24;
+// fp32, 1024 rows of d = 256, Q | K | V 4.0 / 3.6, output projection 4.2 / 2.4.
+static bool gemm_narrow(int m_tiles, int n_tiles, int P) { return 2LL * m_tiles * n_tiles <= P; }
+
+template <int EPI, bool F32>
+static int launch_gemm(const CUtensorMap& ma, const CUtensorMap& mw, GemmArgs g, cudaStream_t st) {
+    const int m_tiles = (g.n + 2 * kGM - 1) / (2 * kGM);
     int pairs = sm_count() / 2;
     g.groups = gemm_groups(m_tiles, g.n_tiles, (g.K + kGK - 1) / kGK, pairs, g.part != nullptr);
+    if (EPI != GEMM_SWIGLU && !g.groups && gemm_narrow(m_tiles, g.n_tiles, pairs)) {
+        g.n_tiles = (g.N + kGNarrow - 1) / kGNarrow;
+        return launch_tiles<EPI, EPI == GEMM_SWIGLU ? kGN : kGNarrow, F32>(ma, mw, g, m_tiles * g.n_tiles, st);
+    }
+    const int tiles = m_tiles * g.n_tiles;
     if (g.groups) pairs = g.groups * m_tiles;
     else if (pairs > tiles) pairs = tiles;
-    return launch_pdl(gemm_kernel<EPI>, 2 * pairs, kGThreads, (size_t)smem, st, ma, mw, g) == cudaSuccess ? DASH_OK : DASH_ERR_CUDA;
+    return launch_tiles<EPI, kGN, F32>(ma, mw, g, pairs, st);
 }
 
 bool gemm_shape_ok(GemmEpilogueKind kind, int64_t n, int64_t N, int64_t K, int64_t lda, int64_t ldw, const GemmEpilogue& e) {
@@ -696,7 +746,8 @@ int gemm_bf16(GemmEpilogueKind kind, const void* A, int64_t lda, const void* W, 
               int64_t K, const GemmEpilogue& e, const int32_t* n_dev, cudaStream_t st, bool out_f32, const GemmSplit* sc, bool w_early) {
     if (!gemm_shape_ok(kind, n, N, K, lda, ldw, e)) return DASH_ERR_UNSUPPORTED;
     if (!aligned16(A) || !aligned16(W)) return DASH_ERR_INVALID_ARG;
-    if (out_f32 && kind != GEMM_PLAIN) return DASH_ERR_UNSUPPORTED;
+    if (out_f32 && kind != GEMM_PLAIN && kind != GEMM_ROPE) return DASH_ERR_UNSUPPORTED;
+    if (out_f32 && kind == GEMM_ROPE && (!e.q_copy || !e.k_cache || !aligned16(C) || (ldc % 4))) return DASH_ERR_INVALID_ARG;
     if (kind == GEMM_PLAIN && (!aligned16(C) || (ldc * (out_f32 ? 4 : 2)) % 16 || (!out_f32 && (N % 8)))) return DASH_ERR_UNSUPPORTED;
     CUtensorMap ma, mw;
     int rc;
@@ -705,16 +756,16 @@ int gemm_bf16(GemmEpilogueKind kind, const void* A, int64_t lda, const void* W, 
     GemmArgs g;
     g.n = (int)n; g.N = (int)N; g.K = (int)K;
     g.n_tiles = kind == GEMM_SWIGLU ? e.m / 128 : (int)((N + kGN - 1) / kGN);
-    g.C = C; g.ldc = ldc; g.n_dev = n_dev; g.e = e; g.out_f32 = out_f32 ? 1 : 0;
+    g.C = C; g.ldc = ldc; g.n_dev = n_dev; g.e = e;
     g.w_early = w_early ? 1 : 0;
     g.part = sc ? sc->part : nullptr; g.arrived = sc ? sc->arrived : nullptr; g.groups = 0;
     g.status = status_word_ptr();
     if (!g.status) return DASH_ERR_CUDA;
     switch (kind) {
-        case GEMM_PLAIN: return launch_gemm<GEMM_PLAIN>(ma, mw, g, st);
-        case GEMM_ROPE: return launch_gemm<GEMM_ROPE>(ma, mw, g, st);
-        case GEMM_RESID: return launch_gemm<GEMM_RESID>(ma, mw, g, st);
-        default: return launch_gemm<GEMM_SWIGLU>(ma, mw, g, st);
+        case GEMM_PLAIN: return out_f32 ? launch_gemm<GEMM_PLAIN, true>(ma, mw, g, st) : launch_gemm<GEMM_PLAIN, false>(ma, mw, g, st);
+        case GEMM_ROPE: return out_f32 ? launch_gemm<GEMM_ROPE, true>(ma, mw, g, st) : launch_gemm<GEMM_ROPE, false>(ma, mw, g, st);
+        case GEMM_RESID: return launch_gemm<GEMM_RESID, false>(ma, mw, g, st);
+        default: return launch_gemm<GEMM_SWIGLU, false>(ma, mw, g, st);
     }
 }
 

@@ -17,8 +17,9 @@ struct GemmEpilogue {
     // rope_pos null: the table holds one entry per row; else one per position and row t uses entry min(rope_pos[t], rope_len - 1)
     const int32_t* rope_pos = nullptr; int64_t rope_len = 0;
     // ROPE: k_cache / v_cache (null: none): the K and V heads' columns (behind q_cols of Q) once more, rows of ld_cache elements, 8-byte aligned
+    // fp32 C: the bf16 copies of the heads, q_copy [n, q_cols] and k_cache / v_cache
     int q_cols = 0;
-    void *k_cache = nullptr, *v_cache = nullptr; int64_t ld_cache = 0;
+    void *k_cache = nullptr, *v_cache = nullptr, *q_copy = nullptr; int64_t ld_cache = 0;
     // ROPE, SWIGLU: row_scale (null: none) multiplies the accumulators of a row first -- 1 / rms(row) when the RMSNorm in front of the
     // projection is folded into it (its weight into W, its row factor here)
     const float* row_scale = nullptr;
@@ -46,7 +47,7 @@ int64_t gemm_split_max_rows();
 // PLAIN and the element-wise work as passes of their own.
 bool gemm_shape_ok(GemmEpilogueKind kind, int64_t n, int64_t N, int64_t K, int64_t lda, int64_t ldw, const GemmEpilogue& e);
 // C (or the epilogue's outputs) = A[n, K] W[K, N], A and W bf16; ld* in elements; n_dev: device true row count or null;
-// out_f32 (PLAIN only): C is fp32 instead of bf16; sc: scratch that lets the kernel cut tiles along K (null: whole tiles only);
+// out_f32 (PLAIN, ROPE): C is fp32 instead of bf16; sc: scratch that lets the kernel cut tiles along K (null: whole tiles only);
 // w_early: W may be read while the kernel in front of this one still runs.  Only for a W that no kernel of the step writes (a caller's weights),
 // behind a kernel of the step that has called pdl_wait() ahead of pdl_launch_dependents() (prologue_kernel): what made W is then
 // complete before anything of the step that is launched to start early can start.

@@ -167,7 +167,7 @@ struct PrologueArgs {
     int row_ctas;
     // bf16: see row_prep_rows (table and inv_rms null: no rows)
     const int32_t* pos; int half; float2* table; float* inv_rms;
-    // fp32: Hn16 [n, d] = bf16 of the RMSNorm of H
+    // fp32: Hn16 [n, d] = bf16 of the RMSNorm of H; the rotary table (null: none) with angle, sine and cosine in fp64
     const float* rms_w; __nv_bfloat16* Hn16;
     const float4 *w0, *w1; uint2 *w0_16, *w1_16; int64_t n_w0, n_w1;      // contiguous matrices, in vectors of four
 };
@@ -205,6 +205,14 @@ prologue_kernel(const PrologueArgs a, const RopeFreqs fr) {
             for (int v = lane; v < a.nvec; v += 32) {
                 const float4 c = x[v], g = w[v];
                 y[v] = make_uint2(pack_bf16(c.x * rs * g.x, c.y * rs * g.y), pack_bf16(c.z * rs * g.z, c.w * rs * g.w));
+            }
+            if (a.table) {
+                const double ps = (double)a.pos[t];
+                for (int i = lane; i < a.half; i += 32) {
+                    double sn, cs;
+                    sincos(ps * fr.inv_freq[i], &sn, &cs);
+                    a.table[t * a.half + i] = make_float2((float)cs, (float)sn);
+                }
             }
         }
         return;
@@ -464,7 +472,8 @@ static int attention_to_O(const dash_layer_cfg* cfg, const void* H_in, const int
     int rc;
     GemmEpilogue e;
     e.D = D; e.n_rot_cols = (Hq + Hkv) * D; e.rope_table = W.rope_tab;
-    const bool fused = bf && gemm_shape_ok(GEMM_ROPE, n, nq, d, d, nq, e);
+    const bool fits = gemm_shape_ok(GEMM_ROPE, n, nq, d, d, nq, e), fused = bf && fits;
+    const bool fused32 = !bf && fits;
     if ((cfg->rope_table || cfg->inv_rms_in || cfg->inv_rms_next) && !(fused && cfg->rms_folded)) return DASH_ERR_UNSUPPORTED;
     // this depth's KV cache rows: keys (rotary applied) and values of the entering tokens, packed [n, Hkv, D].  From the fused projection's
     // epilogue where the buffers allow its 8-byte stores, else copied out of QKV (two launches, 3.5 us each for 701 tokens)
@@ -487,7 +496,7 @@ static int attention_to_O(const dash_layer_cfg* cfg, const void* H_in, const int
         pa.table = cfg->rope_table ? nullptr : W.rope_tab;
         pa.inv_rms = cfg->rms_folded && !cfg->inv_rms_in ? W.inv_rms : nullptr;
     } else if (!bf) {
-        pa.rms_w = (const float*)cfg->rms_weight; pa.Hn16 = (__nv_bfloat16*)W.conv.a;
+        pa.rms_w = (const float*)cfg->rms_weight; pa.Hn16 = (__nv_bfloat16*)W.conv.a; pa.table = fused32 ? W.rope_tab : nullptr;
         pa.w0 = (const float4*)cfg->Wqkv; pa.w0_16 = (uint2*)W.conv.w; pa.n_w0 = (int64_t)d * nq / 4;
         pa.w1 = (const float4*)cfg->Wo; pa.w1_16 = (uint2*)W.conv.w2; pa.n_w1 = (int64_t)Hq * D * d / 4;
         w_ctas = (pa.n_w0 + pa.n_w1 + 1023) / 1024;
@@ -507,6 +516,11 @@ static int attention_to_O(const dash_layer_cfg* cfg, const void* H_in, const int
         // LN (read as RMSNorm), then Q | K | V = Hn Wqkv with the Q and K heads rotated on the accumulators
         if ((rc = launch_rmsnorm(cfg->dt, H_in, cfg->rms_weight, W.Hn, n, d, cfg->rms_eps, n_dev, st)) != DASH_OK) return rc;
         if ((rc = gemm_bf16(GEMM_ROPE, W.Hn, d, cfg->Wqkv, nq, W.QKV, nq, n, nq, d, e, n_dev, st, false, &W.split, true)) != DASH_OK) return rc;
+    } else if (fused32) {
+        // operands as the prologue left them: bf16 copies, products accumulated, rotated and stored in fp32, the attention kernel's bf16 copies
+        // beside them.  (With the rotary embedding and the copies as a kernel of their own a layer of 1024 rows, d = 256, took 5 us more.)
+        e.q_cols = Hq * D; e.q_copy = pa.ap.q; e.k_cache = pa.ap.k; e.v_cache = pa.ap.v; e.ld_cache = (int64_t)Hkv * D;
+        if ((rc = gemm_bf16(GEMM_ROPE, W.conv.a, d, W.conv.w, nq, W.QKV, nq, n, nq, d, e, n_dev, st, true)) != DASH_OK) return rc;
     } else {
         const int heads = Hq + Hkv;
         if (bf) {

@@ -368,6 +368,27 @@ def test_kv_cache_rows_are_the_projections_for_every_head_size_and_alignment(sha
     assert (K[n:] == 7.0).all() and (V[n:] == 7.0).all()
 
 
+@pytest.mark.parametrize("shape,n", [(wl.MINI, 1), (wl.MINI, 255), (wl.MINI, 257), (wl.MINI, 1536), (wl.MINI, 1537), (wl.TINY, 1), (wl.TINY, 257), (wl.TINY, 3072),
+                                     (wl.TINY, 3073)], ids=lambda x: x if isinstance(x, int) else ("fp32" if x.dtype == torch.float32 else "bf16"))
+def test_layer_step_over_projection_tiles_of_both_widths(shape, n):
+    """Projections of few tiles take 128 columns per tile, others 256 (Q | K | V of MINI: up to 1536 rows, of the fp32 shape: up to 3072): one row, an
+    incomplete and a second row of tiles, both sides of the line."""
+    cu = wl.cu_from_lengths([n])
+    H, W = wl.hidden_states(n, shape.d, 61, shape.dtype), wl.layer_weights(shape, 61)
+    pos = wl.positions(cu)
+    ref = oc.layer_step(H, W, cu, pos, shape, tau=0.0)
+    layer = dash.Layer(shape, W, DEV, tau=0.0)
+    bufs = StepBuffers(layer, n, 1, n, shape.dtype)
+    x_full = torch.full((n, shape.d), 9.0, dtype=shape.dtype, device=DEV)
+    run_step(layer, H.to(DEV), torch.arange(n, dtype=torch.int32, device=DEV), pos.to(DEV), cu.to(DEV), n, x_full, bufs)
+    q, k = shape.Hq * shape.D, shape.Hkv * shape.D
+    QKV = bufs.view(bufs.lay.QKV, n, q + 2 * k, shape.dtype).float().cpu().numpy()
+    for name, got in (("Q", QKV[:, :q]), ("K", QKV[:, q:q + k]), ("V", QKV[:, q + k:])):
+        assert_close_rms(got, ref[name].reshape(n, -1), name)
+    assert_close_rms(x_full.float().cpu().numpy(), ref["Ht"], "H~")
+    assert np.max(np.abs(bufs.r.cpu().numpy() - ref["r"]) / ref["r"]) < 2e-2
+
+
 ODD = wl.LayerShape(d=520, Hq=3, Hkv=1, D=64, rope_base=1.0e4, dtype=torch.bfloat16)
 
 
