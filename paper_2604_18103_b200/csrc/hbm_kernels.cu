@@ -677,9 +677,12 @@ __device__ __forceinline__ int tail_decide(const TailArgs& a, int64_t row, float
     return keep;
 }
 
-// The same pass with a warp per row and tiles of eight rows, so that 700 rows are 88 CTAs and not 22.  Bound by the chain ticket -> rows ->
-// look-back -> copy; for inputs whose tiles are all resident.  Loops of seven vectors per lane (two for a row of 3584 bf16), not
-// unrolled: with the whole row in registers and straight-line code the warps waited 14 us for instructions they run once.
+// The same pass with a warp per row and tiles of eight rows, so that 700 rows are 88 CTAs and not 22 (threshold rule: with the decisions given see
+// delta_given_kernel).  Bound by the chain ticket -> rows -> look-back -> copy; for inputs whose tiles are all resident.  So the number of rows is
+// asked for beside the ticket, every tile in front is asked for its count at once, a thread to each, and a row's vectors stay in registers for the
+// copy, or are loaded for it, before the base is known (from the end of the kernel in front, us: fp32 layer of 1024 rows 6.6, 8.3 with these one behind
+// the other, 1500 rows of the 7B shape 10.3, was 12.4).  Loops of seven vectors per lane (two for a row of 3584 bf16), not unrolled: with the whole row in registers and straight-line
+// code the warps waited 14 us for instructions they run once.
 constexpr int kTailRows = 8;
 constexpr int kTailSmallTiles = 2;          // per SM: with more tiles than fit at once, a tile waits for the look-back chain of up to a
                                             // thousand others (behind the projection in front, 6683 rows: 64 us against 40 of the general kernel, 8192: 80 against 42).
@@ -688,16 +691,15 @@ constexpr int kTailSmallTiles = 2;          // per SM: with more tiles than fit 
 template <bool BF16>
 __global__ void __launch_bounds__(32 * kTailRows)
 delta_tail_rows_kernel(const TailArgs a, int64_t n_upper) {
-    constexpr int CH = 7;
-    __shared__ int s_keep[kTailRows];
-    __shared__ int s_base, s_count;
-    __shared__ unsigned int s_tile, s_ballot;
+    constexpr int CH = 7, THREADS = 32 * kTailRows;
+    __shared__ int s_keep[kTailRows], s_part[kTailRows];
+    __shared__ unsigned int s_tile;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     ptx::pdl_wait();                                       // launched to start early: nothing global is touched before the kernel in front is done
+    int64_t n = a.cu_in[a.S];
     if (threadIdx.x == 0) s_tile = atomicAdd(a.ticket, 1u);
     __syncthreads();
     const int tile = (int)s_tile;
-    int64_t n = a.cu_in[a.S];
     if (n > n_upper) n = n_upper;
     const int64_t t_start = (int64_t)tile * kTailRows;
     if (t_start >= n && tile != 0) return;
@@ -705,66 +707,90 @@ delta_tail_rows_kernel(const TailArgs a, int64_t n_upper) {
     const bool last_tile = (t_end >= n);
     const int64_t row = t_start + warp;
     int keep = 0, tok = 0, pos = 0;
-    float ss = 0.f, su = 0.f, sh = 0.f;                    // ss: sum of squares of the row as it goes on (H~ or H')
+    float ss = 0.f, su = 0.f, sh = 0.f;                    // ss: sum of squares of the row as it goes on
     char* x = a.x_full;
+    uint4 p[CH];
+    int have = lane;                                       // p: the row's vectors have + 32 k
     if (row < n) {
         tok = a.tok_in[row];
         pos = a.pos_in[row];
-        x += (int64_t)tok * a.ldx_b;
-        if (a.mask_in) keep = a.mask_in[row] != 0;
         if (a.U) {
             const char* u = a.U + row * a.ldU_b;
             const char* h = a.H + row * a.ldH_b;
 #pragma unroll 1
             for (int v0 = lane; v0 < a.nvec; v0 += 32 * CH) {
-                uint4 p[CH], q[CH];
+                uint4 q[CH];
+                have = v0;
 #pragma unroll
                 for (int k = 0; k < CH; ++k) {
                     const int64_t v = v0 + k * 32;
                     if (v < a.nvec) { p[k] = ld_nc_v4(u + (v << 4)); q[k] = ld_nc_v4(h + (v << 4)); }
                     else p[k] = q[k] = make_uint4(0, 0, 0, 0);
                 }
-                if (!a.mask_in) {
 #pragma unroll
-                    for (int k = 0; k < CH; ++k) { su += sumsq_vec<BF16>(p[k]); sh += sumsq_vec<BF16>(q[k]); }
-                }
+                for (int k = 0; k < CH; ++k) { su += sumsq_vec<BF16>(p[k]); sh += sumsq_vec<BF16>(q[k]); }
+                char* o = x + (int64_t)tok * a.ldx_b;
 #pragma unroll
                 for (int k = 0; k < CH; ++k) {
                     const int64_t v = v0 + k * 32;
                     p[k] = add_vec<BF16>(p[k], q[k]);
-                    if (v < a.nvec) st_v4(x + (v << 4), p[k]);
+                    if (v < a.nvec) st_v4(o + (v << 4), p[k]);
                 }
                 if (a.inv_next) {
 #pragma unroll
                     for (int k = 0; k < CH; ++k) ss += sumsq_vec<BF16>(p[k]);
                 }
             }
-        } else if (a.sums) {
+        } else {
             for (int i = lane; i < a.n_sum_tiles; i += 32) { const float4 p2 = a.sums[row * a.n_sum_tiles + i]; su += p2.x; sh += p2.y; ss += p2.z; }
         }
-        if (!a.mask_in) keep = tail_decide(a, row, warp_sum(su), warp_sum(sh), lane);
+        x += (int64_t)tok * a.ldx_b;
+        keep = tail_decide(a, row, warp_sum(su), warp_sum(sh), lane);
     }
     if (a.inv_next) ss = warp_sum(ss);
     if (lane == 0) s_keep[warp] = keep;
+    auto load_chunk = [&](int v0) {
+#pragma unroll
+        for (int k = 0; k < CH; ++k) { const int64_t v = v0 + k * 32; if (v < a.nvec) p[k] = ld_cg_v4(x + (v << 4)); }
+    };
+    if (keep && !a.U) load_chunk(have);                    // in flight while the base is looked for
     __syncthreads();
-    if (warp == 0) {
-        const unsigned int bal = __ballot_sync(0xffffffffu, lane < kTailRows && s_keep[lane < kTailRows ? lane : 0]);
-        const int agg = __popc(bal), base = tail_look_back(a.tile_state, tile, agg, a.status, lane);
-        if (lane == 0) { s_base = base; s_count = agg; s_ballot = bal; }
+    const unsigned int bal = __ballot_sync(0xffffffffu, lane < kTailRows && s_keep[lane < kTailRows ? lane : 0]);
+    const int count = __popc(bal);
+    if (threadIdx.x == 0) st_state(&a.tile_state[tile], kFlagAgg | (unsigned int)count);
+    int front = 0;
+    bool timed_out = false;
+    for (int j = threadIdx.x; j < tile && !timed_out; j += THREADS) {
+        unsigned long long st = ld_state(&a.tile_state[j]);
+        for (uint32_t spins = 0; (st >> 32) == 0 && !timed_out; timed_out = ++spins > kSpinLimit) {
+            __nanosleep(32);
+            st = ld_state(&a.tile_state[j]);
+        }
+        front += (int)(unsigned int)(st & 0xffffffffu);
     }
-    __syncthreads();
-    const int base = s_base, count = s_count;
-    const unsigned int bal = s_ballot;
+    front = __reduce_add_sync(0xffffffffu, front);
+    if (lane == 0) s_part[warp] = front;
+    timed_out = __syncthreads_or(timed_out);
+    int base = 0;
+    if (!timed_out) {
+#pragma unroll
+        for (int w = 0; w < kTailRows; ++w) base += s_part[w];
+    } else if (threadIdx.x == 0) {
+        atomicExch(a.status, DASH_ERR_TIMEOUT);
+    }
     if (keep) {
         const int64_t k = base + __popc(bal & ((1u << warp) - 1u));
         char* dst = a.H_next + k * a.ldn_b;
-#pragma unroll 1
-        for (int v0 = lane; v0 < a.nvec; v0 += 32 * CH) {
-            uint4 p[CH];
-#pragma unroll
-            for (int i = 0; i < CH; ++i) { const int64_t v = v0 + i * 32; if (v < a.nvec) p[i] = ld_cg_v4(x + (v << 4)); }
+        auto store_chunk = [&](int v0) {
 #pragma unroll
             for (int i = 0; i < CH; ++i) { const int64_t v = v0 + i * 32; if (v < a.nvec) st_v4(dst + (v << 4), p[i]); }
+        };
+        store_chunk(have);
+#pragma unroll 1
+        for (int v0 = lane; v0 < a.nvec; v0 += 32 * CH) {
+            if (v0 == have) continue;
+            load_chunk(v0);
+            store_chunk(v0);
         }
         if (lane == 0) {
             a.tok_next[k] = tok;
@@ -772,13 +798,121 @@ delta_tail_rows_kernel(const TailArgs a, int64_t n_upper) {
             if (a.inv_next) a.inv_next[k] = rsqrtf(ss * a.inv_d + a.rms_eps);
         }
     }
-    for (int s = threadIdx.x; s <= a.S; s += 32 * kTailRows) {
+    for (int s = threadIdx.x; s <= a.S; s += THREADS) {
         int64_t c = a.cu_in[s];
         if (c > n) c = n;
         bool mine = (c >= t_start && c < t_end) || (last_tile && c == t_end);
         if (tile == 0 && n == 0) mine = true;
         if (mine) {
             const int v = base + (c >= t_end ? count : __popc(bal & ((1u << (int)(c - t_start)) - 1u)));
+            a.cu_next[s] = v;
+            if (s == a.S && a.n_next) *a.n_next = v;
+        }
+    }
+}
+
+// The tail pass where the decisions are given (mask_in): the output base of a tile is counted from the mask itself, as dash_compact does it, so that
+// a row needs no ticket, no look-back and no second visit -- U and H are read once, their sum goes to x_full[tok] and, where the row
+// stays, to H_next (U null: the rows are in x_full, those that stay are copied).  A warp per row, RPW rows one behind the other.  Bound by HBM, for few
+// rows by the chain mask -> rows.  From the end of the kernel in front to its own, us, kernels with look-back / this one: blocks of the 7B shape of 701
+// rows that all stay 15.2 / 9.8, 1500 17.8 / 11.1, 3000 47.8 / 22.9, 6683 53 / 38.5, 8192 61.6 / 51.1 (235 MB), 32 768 245 / 203, of 2728 51 / 23;
+// count rule, 12 345 rows 40.5 / 29.9.  (As many rows to every CTA, all resident at once: 701 11.7, 8192 55.7, 32 768 210.)  Up to kGivenMaxRows:
+// further up the mask in front is too long to be counted by every tile.
+constexpr int kGivenMaxRows = 32768, kGivenThreads = 256, kGivenPerSm = 2;
+template <bool BF16, int RPW>
+__global__ void __launch_bounds__(kGivenThreads)
+delta_given_kernel(const TailArgs a, int64_t n_upper) {
+    constexpr int CH = 7, NW = kGivenThreads / 32, TILE = NW * RPW;
+    static_assert(TILE <= 32 && (TILE == 8 || TILE % 16 == 0), "a lane per row of a tile; whole vectors of the mask in front of it");
+    __shared__ int s_part[NW];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    ptx::pdl_wait();                                       // launched to start early: nothing global is touched before the kernel in front is done
+    int64_t n = a.cu_in[a.S];
+    const int64_t t_start = (int64_t)blockIdx.x * TILE;
+    int front = 0;
+    if ((reinterpret_cast<uintptr_t>(a.mask_in) & (TILE == 8 ? 7 : 15)) == 0) {
+        if (TILE == 8) {
+            const uint2* mv = reinterpret_cast<const uint2*>(a.mask_in);
+#pragma unroll 2
+            for (int v = threadIdx.x; v < (int)(t_start >> 3); v += kGivenThreads) { const uint2 w = mv[v]; front += nonzero_bytes(w.x) + nonzero_bytes(w.y); }
+        } else {
+            const uint4* mv = reinterpret_cast<const uint4*>(a.mask_in);
+#pragma unroll 4
+            for (int v = threadIdx.x; v < (int)(t_start >> 4); v += kGivenThreads) {
+                const uint4 w = mv[v];
+                front += nonzero_bytes(w.x) + nonzero_bytes(w.y) + nonzero_bytes(w.z) + nonzero_bytes(w.w);
+            }
+        }
+    } else {
+        for (int64_t t = threadIdx.x; t < t_start; t += kGivenThreads) front += a.mask_in[t] != 0;
+    }
+    if (n > n_upper) n = n_upper;
+    const int64_t t_end = (t_start + TILE < n) ? t_start + TILE : n;
+    if (t_start >= n && blockIdx.x != 0) return;
+    const unsigned int bal = __ballot_sync(0xffffffffu, lane < TILE && t_start + lane < n && a.mask_in[t_start + lane] != 0);
+    front = __reduce_add_sync(0xffffffffu, front);
+    if (lane == 0) s_part[warp] = front;
+    __syncthreads();
+    int base = 0;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) base += s_part[w];
+#pragma unroll 1
+    for (int rr = 0; rr < RPW; ++rr) {
+        const int local = rr * NW + warp;
+        const int64_t row = t_start + local;
+        if (row >= n) break;
+        const bool keep = bal >> local & 1;
+        if (!keep && !a.U) continue;
+        const int64_t k = base + __popc(bal & ((1u << local) - 1u));
+        const int tok = a.tok_in[row], pos = a.pos_in[row];
+        char* x = a.x_full + (int64_t)tok * a.ldx_b;
+        char* dst = a.H_next + k * a.ldn_b;
+        float ss = 0.f;
+#pragma unroll 1
+        for (int v0 = lane; v0 < a.nvec; v0 += 32 * CH) {
+            uint4 p[CH];
+            if (a.U) {
+                const char* u = a.U + row * a.ldU_b;
+                const char* h = a.H + row * a.ldH_b;
+                uint4 q[CH];
+#pragma unroll
+                for (int i = 0; i < CH; ++i) {
+                    const int64_t v = v0 + i * 32;
+                    if (v < a.nvec) { p[i] = ld_nc_v4(u + (v << 4)); q[i] = ld_nc_v4(h + (v << 4)); }
+                    else p[i] = q[i] = make_uint4(0, 0, 0, 0);
+                }
+#pragma unroll
+                for (int i = 0; i < CH; ++i) {
+                    const int64_t v = v0 + i * 32;
+                    p[i] = add_vec<BF16>(p[i], q[i]);
+                    if (v < a.nvec) st_v4(x + (v << 4), p[i]);
+                    if (a.inv_next) ss += sumsq_vec<BF16>(p[i]);
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < CH; ++i) { const int64_t v = v0 + i * 32; if (v < a.nvec) p[i] = ld_cg_v4(x + (v << 4)); }
+            }
+            if (keep) {
+#pragma unroll
+                for (int i = 0; i < CH; ++i) { const int64_t v = v0 + i * 32; if (v < a.nvec) st_v4(dst + (v << 4), p[i]); }
+            }
+        }
+        if (keep) {
+            if (a.inv_next) ss = warp_sum(ss);
+            if (lane == 0) {
+                a.tok_next[k] = tok;
+                a.pos_next[k] = pos;
+                if (a.inv_next) a.inv_next[k] = rsqrtf(ss * a.inv_d + a.rms_eps);
+            }
+        }
+    }
+    const bool last_tile = t_end >= n;
+    for (int s = threadIdx.x; s <= a.S; s += kGivenThreads) {
+        int64_t c = a.cu_in[s];
+        if (c > n) c = n;
+        if ((c >= t_start && c < t_end) || (last_tile && c == t_end) || (blockIdx.x == 0 && n == 0)) {
+            const int at = (int)(c - t_start);
+            const int v = base + __popc(at >= 32 ? bal : bal & ((1u << at) - 1u));
             a.cu_next[s] = v;
             if (s == a.S && a.n_next) *a.n_next = v;
         }
@@ -1214,8 +1348,20 @@ int launch_delta_tail(const void* U, const void* H, const uint8_t* mask_in, cons
     a.inv_next = inv_next; a.inv_d = 1.0f / (float)d; a.rms_eps = rms_eps;
     a.status = status_word_ptr();
     if (!a.status) return DASH_ERR_CUDA;
+    if (mask_in && n <= kGivenMaxRows && (U || !inv_next)) {
+        // tiles of eight rows where they fill their waves better than tiles of sixteen (us from the end of the kernel in front, 8 / 16: 6683 rows 38.5 /
+        // 46.5; as well filled: 8192 rows 54.6 / 51.1, 12 345 rows, count rule 31.6 / 29.9, 3000 rows 23.1 / 22.9)
+        auto tiles = [&](int rows) { return n > 0 ? (n + rows - 1) / rows : 1; };
+        auto waves = [&](int64_t t) { return (t + kGivenPerSm * sm_count() - 1) / (kGivenPerSm * sm_count()); };
+        constexpr int NW = kGivenThreads / 32;
+        const bool one = waves(tiles(NW)) < 2 * waves(tiles(2 * NW));
+        auto go = [&](auto kernel) { return launch_pdl(kernel, (int)tiles(one ? NW : 2 * NW), kGivenThreads, 0, st, a, n); };
+        DASH_CUDA_TRY(dt == DASH_BF16 ? (one ? go(delta_given_kernel<true, 1>) : go(delta_given_kernel<true, 2>))
+                                      : (one ? go(delta_given_kernel<false, 1>) : go(delta_given_kernel<false, 2>)));
+        return DASH_OK;
+    }
     const int small = (int)((n + kTailRows - 1) / kTailRows) > 0 ? (int)((n + kTailRows - 1) / kTailRows) : 1;
-    if (small <= kTailSmallTiles * sm_count()) {
+    if (!mask_in && small <= kTailSmallTiles * sm_count()) {
         if (dt == DASH_BF16) DASH_CUDA_TRY(launch_pdl(delta_tail_rows_kernel<true>, small, 32 * kTailRows, 0, st, a, n));
         else DASH_CUDA_TRY(launch_pdl(delta_tail_rows_kernel<false>, small, 32 * kTailRows, 0, st, a, n));
         return DASH_OK;

@@ -324,3 +324,41 @@ def test_down_projection_cut_along_k_at_the_7b_shape(n):
     bound = 2.0 ** -8 * ref.abs() + 4 * 2.0 ** -24 * (sh.m / 16) ** 0.5 * size
     worst = float(((F - ref).abs() / bound).max())
     assert worst <= 1.0, worst
+
+
+@pytest.mark.parametrize("n,offset", [(1, 0), (9, 3), (2368, 8), (2369, 1), (4740, 0), (7000, 4), (32768, 0), (32769, 0)])
+def test_block_step_tail_with_given_decisions_at_the_edges_of_its_tiles(n, offset):
+    """The tail pass of a block, whose decisions are in the mask: row counts at which it takes other tiles or the form with look-back, masks that
+    start anywhere, fewer rows than there is room for.  x_full gets H~ + F of every row, what goes on is exactly the kept rows of it in order,
+    with token and position indices, boundaries and row factors; nothing behind them is written."""
+    sh = wl.MINI
+    live = n - n // 9
+    lens = [live // 3, 0, live - live // 3]
+    cu = wl.cu_from_lengths(lens)
+    H = wl.hidden_states(n, sh.d, 93, sh.dtype).to(DEV)
+    pos = torch.cat([wl.positions(cu), torch.zeros(n - live, dtype=torch.int32)]).to(DEV)
+    block = dash.Block(sh, _weights(sh, 93), DEV, tau=0.0, keep_first=2, keep_last=1)
+    b = BlockBuffers(block, n, 3)
+    b.mask = torch.zeros(n + offset, dtype=torch.uint8, device=DEV)[offset:]
+    tok = torch.randperm(n, generator=torch.Generator().manual_seed(n)).to(torch.int32).to(DEV)
+    inv = torch.zeros(n, dtype=torch.float32, device=DEV)
+    block.set_handover(dash.dash_rope_table(sh.rope_base, sh.D, n, DEV), None, inv)
+    for tau in (0.0, None):
+        if tau is None:
+            tau = float(b.r[:live].median())
+        block.set_tau(tau)
+        x_full = torch.full((n, sh.d), 9.0, dtype=sh.dtype, device=DEV)
+        b.H_next.fill_(7.0)
+        run_block(block, H, tok, pos, cu.to(DEV), max(lens), x_full, b)
+        view = lambda off: b.ws[off:off + n * sh.d * 2].view(sh.dtype).view(n, sh.d)
+        rows = (view(b.lay.attn.Ht)[:live].float() + view(b.lay.F)[:live].float()).to(sh.dtype)
+        assert torch.equal(x_full[tok[:live].long()], rows) and (x_full[tok[live:].long()] == 9.0).all()
+        mask = b.mask[:live].bool()
+        k = int(b.n_next.item())
+        assert k == int(mask.sum()) and (tau > 0.0 or k == live)
+        assert torch.equal(b.H_next[:k], rows[mask]) and (b.H_next[k:] == 7.0).all()
+        assert torch.equal(b.tok_next[:k], tok[:live][mask]) and torch.equal(b.pos_next[:k], pos[:live][mask])
+        a = int(mask[:lens[0]].sum())
+        assert b.cu_next.tolist() == [0, a, a, k]
+        ref = torch.rsqrt(rows[mask].double().square().mean(1) + sh.rms_eps)
+        assert k == 0 or ((inv[:k].double() - ref).abs() / ref).max() < 1e-5
