@@ -43,7 +43,7 @@ static_assert(kGRingBytes == Ring<kGNarrow>::kStage * Ring<kGNarrow>::kStages, "
 constexpr int kGEpiWarps = 8;                // two per TMEM lane quarter, each with one half of the tile's columns
 constexpr int kGThreads = 64 + 32 * kGEpiWarps;
 constexpr int kGEpiBytes = 4096;             // staging per epilogue warp: 32 rows of 128 bytes
-constexpr int kGGroupN = 16;                 // n tiles per group of the tile order
+constexpr int kGGroup = 16;                  // tiles per group of the tile order
 constexpr int kGSplitMaxRounds = 4;          // tiles may be cut along K where whole tiles take up to so many rounds
 constexpr int kGSplitMaxParts = 4;           // parts of a tile, on the average
 constexpr int kGSplitMinShare = 6;           // K steps of a pair's share, at least
@@ -86,14 +86,16 @@ __device__ __forceinline__ void mma_ss_lh(uint32_t d_tmem, uint32_t a_lo, uint32
         ::"r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate), "r"(0u) : "memory");
 }
 
-// tile t -> (m tile of 256 rows, n tile): the n tiles come in groups of kGGroupN; within a group the m tiles run one after the other and
-// each visits the group's n tiles, so that the CTAs of a wave share a few A row-blocks and a few W column-blocks in L2
-__device__ __forceinline__ void tile_coords(int t, int m_tiles, int n_tiles, int& mt, int& nt) {
-    const int per_group = m_tiles * kGGroupN;
+// tile t -> (m tile of 256 rows, n tile): the n tiles come in groups of kGGroup; within a group the m tiles run one after the other and
+// each visits the group's n tiles, so that the CTAs of a wave share a few A row-blocks and a few W column-blocks in L2.  by_m: the same with
+// rows and columns exchanged
+__device__ __forceinline__ void tile_coords(int t, int m_tiles, int n_tiles, bool by_m, int& mt, int& nt) {
+    const int grouped = by_m ? m_tiles : n_tiles, swept = by_m ? n_tiles : m_tiles, per_group = swept * kGGroup;
     const int g = t / per_group, r = t - g * per_group;
-    const int gw = min(kGGroupN, n_tiles - g * kGGroupN);        // the last group may be narrower
-    mt = r / gw;
-    nt = g * kGGroupN + r % gw;
+    const int gw = min(kGGroup, grouped - g * kGGroup);          // the last group may be narrower
+    const int in = g * kGGroup + r % gw, along = r / gw;
+    mt = by_m ? in : along;
+    nt = by_m ? along : in;
 }
 
 template <int N> struct Width { static constexpr int value = N; };
@@ -105,9 +107,9 @@ template <int N> struct Width { static constexpr int value = N; };
 struct Work {
     int t, tiles, P, m_tiles, n_tiles, ksteps, mt;
     long long u, u1;
-    bool cut;
-    __device__ __forceinline__ Work(int pair, int P_, int m_tiles_, int n_tiles_, int ksteps_, int groups)
-        : t(pair), tiles(m_tiles_ * n_tiles_), P(P_), m_tiles(m_tiles_), n_tiles(n_tiles_), ksteps(ksteps_), mt(0), u(0), u1(0), cut(groups > 0) {
+    bool cut, by_m;
+    __device__ __forceinline__ Work(int pair, int P_, int m_tiles_, int n_tiles_, int ksteps_, int groups, int by_m_)
+        : t(pair), tiles(m_tiles_ * n_tiles_), P(P_), m_tiles(m_tiles_), n_tiles(n_tiles_), ksteps(ksteps_), mt(0), u(0), u1(0), cut(groups > 0), by_m(by_m_ != 0) {
         if (cut) {
             const int grp = pair / m_tiles;
             const long long U = (long long)n_tiles * ksteps;
@@ -118,7 +120,7 @@ struct Work {
     __device__ __forceinline__ bool next(int& m, int& n, int& k0, int& k1) {
         if (!cut) {
             if (t >= tiles) return false;
-            tile_coords(t, m_tiles, n_tiles, m, n);
+            tile_coords(t, m_tiles, n_tiles, by_m, m, n);
             k0 = 0; k1 = ksteps; t += P;
             return true;
         }
@@ -138,6 +140,7 @@ struct GemmArgs {
     int w_early;                 // W may be read before the kernel in front is complete
     const int32_t* n_dev;        // device: true number of rows (<= n), or null
     int* status;
+    int by_m;                    // order of the tiles (see tile_coords)
     int groups;                  // > 0: tiles are cut along K (see Work)
     float* part;                 // partial tiles of the pairs: two of 256 x 256 fp32 each
     unsigned int* arrived;       // per tile, CTA of the pair and epilogue warp: parts that are in `part`
@@ -224,7 +227,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
         if (lane == 0) {
             uint32_t it = 0;
             bool ok = true;
-            Work w(pair, n_pairs, m_tiles, n_tiles, ksteps, g.groups);
+            Work w(pair, n_pairs, m_tiles, n_tiles, ksteps, g.groups, g.by_m);
             int mt, nt, k0, k1;
             // w_early: the first stages' W tiles are asked for while the kernel in front, which makes A, still drains (see gemm.cuh for when)
             bool first = true;
@@ -265,7 +268,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
         if (lane == 0 && rank == 0) {
             uint32_t it = 0, tl = 0;
             bool ok = true;
-            Work w(pair, n_pairs, m_tiles, n_tiles, ksteps, g.groups);
+            Work w(pair, n_pairs, m_tiles, n_tiles, ksteps, g.groups, g.by_m);
             int mt, nt, k0, k1;
             for (; ok && w.next(mt, nt, k0, k1); ++tl) {
                 const int b = tl & 1;
@@ -304,7 +307,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
         const int r8 = lane >> 3, c8 = lane & 7;                  // eight lanes per row: row r8 + 4 i, chunk c8
         uint32_t tl = 0;
         bool ok = true;
-        Work w(pair, n_pairs, m_tiles, n_tiles, ksteps, g.groups);
+        Work w(pair, n_pairs, m_tiles, n_tiles, ksteps, g.groups, g.by_m);
         int mt, nt, k0, k1;
         for (; w.next(mt, nt, k0, k1); ++tl) {
             const int b = tl & 1;
@@ -716,6 +719,16 @@ static int launch_tiles(const CUtensorMap& ma, const CUtensorMap& mw, const Gemm
 // fp32, 1024 rows of d = 256, Q | K | V 4.0 / 3.6, output projection 4.2 / 2.4.
 static bool gemm_narrow(int m_tiles, int n_tiles, int P) { return 2LL * m_tiles * n_tiles <= P; }
 
+// Groups of rows of tiles or of columns: the group's operand (16 tiles of 256 x 3584, 29 MB) stays in L2 while the other one streams past it, once
+// per group.  So of the two orders the one that reads less: (groups - 1) times the other operand more than both once.  The gate | up projection of
+// 8192 rows, 32 x 148 tiles, read 1.01 GB from HBM in groups of columns (its operands are 0.33 GB; 0.60 expected in groups of rows); the
+// step runs at the power cap, where bytes are time: three blocks of 701, 6683, 8192 rows in a loop, columns / rows, us 883 / 877, 5772 / 5737,
+// 7817 / 7768.  Groups of 8, 11 and 32: 8192 rows 7812, 7828, 7910.
+static bool gemm_by_m(int m_tiles, int n_tiles) {
+    auto more = [](int grouped, int swept) { return (int64_t)((grouped + kGGroup - 1) / kGGroup - 1) * swept; };
+    return more(m_tiles, n_tiles) < more(n_tiles, m_tiles);
+}
+
 template <int EPI, bool F32>
 static int launch_gemm(const CUtensorMap& ma, const CUtensorMap& mw, GemmArgs g, cudaStream_t st) {
     const int m_tiles = (g.n + 2 * kGM - 1) / (2 * kGM);
@@ -725,6 +738,7 @@ static int launch_gemm(const CUtensorMap& ma, const CUtensorMap& mw, GemmArgs g,
         g.n_tiles = (g.N + kGNarrow - 1) / kGNarrow;
         return launch_tiles<EPI, EPI == GEMM_SWIGLU ? kGN : kGNarrow, F32>(ma, mw, g, m_tiles * g.n_tiles, st);
     }
+    g.by_m = gemm_by_m(m_tiles, g.n_tiles);
     const int tiles = m_tiles * g.n_tiles;
     if (g.groups) pairs = g.groups * m_tiles;
     else if (pairs > tiles) pairs = tiles;
@@ -758,7 +772,7 @@ int gemm_bf16(GemmEpilogueKind kind, const void* A, int64_t lda, const void* W, 
     g.n_tiles = kind == GEMM_SWIGLU ? e.m / 128 : (int)((N + kGN - 1) / kGN);
     g.C = C; g.ldc = ldc; g.n_dev = n_dev; g.e = e;
     g.w_early = w_early ? 1 : 0;
-    g.part = sc ? sc->part : nullptr; g.arrived = sc ? sc->arrived : nullptr; g.groups = 0;
+    g.part = sc ? sc->part : nullptr; g.arrived = sc ? sc->arrived : nullptr; g.groups = 0; g.by_m = 0;
     g.status = status_word_ptr();
     if (!g.status) return DASH_ERR_CUDA;
     switch (kind) {
