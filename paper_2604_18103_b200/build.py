@@ -1,14 +1,16 @@
-"""Builds the C-ABI CUDA library in-tree: paper_2604_18103_b200/libdash.so (sm_100a only)."""
+"""Builds in-tree the C-ABI CUDA library, paper_2604_18103_b200/libdash.so (sm_100a only), and the binding's C part, _pycall.so."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libdash.so")
+PYCALL = os.path.join(HERE, "_pycall.so")
 SOURCES = ["api.cu", "hbm_kernels.cu", "attention.cu", "decode_attention.cu", "gemm.cu", "layer_step.cu"]
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -16,9 +18,9 @@ FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(PYCALL):
         return True
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(PYCALL))
     inc = os.path.join(ROOT, "include")
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(inc, f) for f in os.listdir(inc)]
     return any(os.path.getmtime(d) > t for d in deps)
@@ -43,6 +45,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
             raise RuntimeError(f"nvcc failed on {src}")
     link = [NVCC, "-shared", "-o", LIB, *objs]          # the CUDA runtime is linked statically: no library dependency beyond libc / libstdc++
     subprocess.check_call(link)
+    subprocess.check_call(["gcc", "-O2", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], os.path.join(CSRC, "pycall.c"), "-o", PYCALL, "-lm"])
     return LIB
 
 

@@ -9,6 +9,8 @@ loaded the import of a symbol raises -- there is no CPU fallback.
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
 from ctypes import (POINTER, Structure, c_char_p, c_double, c_float, c_int, c_int32, c_int64,
                     c_size_t, c_uint8, c_void_p)
@@ -25,6 +27,7 @@ OK = 0
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libdash.so")
+PYCALL_PATH = os.path.join(_HERE, "_pycall.so")
 
 EXPORTS = [
     "dash_status_string", "dash_check_status", "dash_keep_count", "dash_flops_per_layer", "dash_flops_speedup",
@@ -70,15 +73,17 @@ class BlockWsLayout(Structure):
 
 
 _lib = None
+_pycall = None          # the binding's C part (csrc/pycall.c), loaded with the library
 
 
 def lib() -> ctypes.CDLL:
     """Loads libdash.so (raises if it has not been built)."""
-    global _lib
+    global _lib, _pycall
     if _lib is None:
-        if not os.path.exists(LIB_PATH):
-            raise RuntimeError(f"{LIB_PATH} is missing: run `python -m paper_2604_18103_b200.build` "
-                               "(there is no fallback path)")
+        for path in (LIB_PATH, PYCALL_PATH):
+            if not os.path.exists(path):
+                raise RuntimeError(f"{path} is missing: run `python -m paper_2604_18103_b200.build` "
+                                   "(there is no fallback path)")
         L = ctypes.CDLL(LIB_PATH)
         L.dash_status_string.restype = c_char_p
         L.dash_status_string.argtypes = [c_int]
@@ -124,7 +129,11 @@ def lib() -> ctypes.CDLL:
         L.dash_testing_decode_smem_bytes.argtypes = [c_int]
         L.dash_workspace_bytes.restype = c_size_t
         L.dash_workspace_bytes.argtypes = [c_int, c_int64, c_int, c_int, c_int, c_int, c_int]
-        _lib = L
+        loader = importlib.machinery.ExtensionFileLoader("_pycall", PYCALL_PATH)
+        C = importlib.util.module_from_spec(importlib.util.spec_from_file_location("_pycall", PYCALL_PATH, loader=loader))
+        loader.exec_module(C)
+        C.setup(ctypes.cast(L.dash_decode_attention, c_void_p).value, torch.bfloat16, torch.float32)
+        _lib, _pycall = L, C
     return _lib
 
 
@@ -359,19 +368,20 @@ def dash_varlen_attention_indexed(Q: torch.Tensor, K: torch.Tensor, V: torch.Ten
 def dash_decode_attention(q: torch.Tensor, Kc: torch.Tensor, Vc: torch.Tensor, cu_seqlens: torch.Tensor, scale: Optional[float] = None,
                           out: Optional[torch.Tensor] = None, want_lse: bool = False, ws: Optional[torch.Tensor] = None):
     """q [S,Hq,D] (one new token per sequence), Kc, Vc [n,Hkv,D] packed caches.  Returns out [S,Hq,D] (and lse [S,Hq])."""
-    _dev(q, Kc, Vc, cu_seqlens)
-    S, Hq, D = q.shape
-    n, Hkv = Kc.shape[:2]
-    if scale is None:
-        scale = 1.0 / (D ** 0.5)
-    if out is None:
-        out = torch.empty(S, Hq, D, dtype=q.dtype, device=q.device)
-    lse = torch.empty(S, Hq, dtype=torch.float32, device=q.device) if want_lse else None
-    if ws is None:
-        ws = workspace(dash_workspace_bytes(WS_DECODE, n, S, Hq, Hkv, D, dtype_code(q)), q.device)
-    st = lib().dash_decode_attention(_p(q), _p(Kc), _p(Vc), _p(out), _p(lse), q.stride(0), Kc.stride(0) if n else Hkv * D,
-                                     Vc.stride(0) if n else Hkv * D, out.stride(0), _p(cu_seqlens), S, n, Hq, Hkv, D, float(scale),
-                                     dtype_code(q), _p(ws), ws.numel(), _stream())
+    if _pycall is None:
+        lib()
+    lse = None
+    if out is None or ws is None or want_lse:
+        _dev(q, Kc, Vc, cu_seqlens)
+        S, Hq, D = q.shape
+        n, Hkv = Kc.shape[:2]
+        if out is None:
+            out = torch.empty(S, Hq, D, dtype=q.dtype, device=q.device)
+        if want_lse:
+            lse = torch.empty(S, Hq, dtype=torch.float32, device=q.device)
+        if ws is None:
+            ws = workspace(dash_workspace_bytes(WS_DECODE, n, S, Hq, Hkv, D, dtype_code(q)), q.device)
+    st = _pycall.decode(q, Kc, Vc, cu_seqlens, scale, out, lse, ws, _stream())
     _check(st, "dash_decode_attention")
     return (out, lse) if want_lse else out
 

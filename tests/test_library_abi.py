@@ -132,3 +132,48 @@ def test_an_sm_takes_as_many_decode_ctas_as_its_tensor_memory_holds(lib, D):
     """Two, 256 of the SM's 512 columns each; a third CTA (228 KB of shared memory per SM, 1 KB of it the system's per CTA) would hold its share of the
     caches' blocks back until one of the two has left."""
     assert 228 * 1024 // (lib.dash_testing_decode_smem_bytes(D) + 1024) == 2
+
+
+class _Tensor:
+    """What the binding's C part asks of a tensor."""
+
+    def __init__(self, shape, ptr=4096, dtype=torch.bfloat16, is_cuda=True):
+        self.shape, self.ptr, self.dtype, self.is_cuda = shape, ptr, dtype, is_cuda
+
+    def data_ptr(self):
+        if self.ptr is None:
+            raise RuntimeError("no storage")
+        return self.ptr
+
+    def stride(self, dim):
+        return 96 if len(self.shape) < 3 else self.shape[1] * self.shape[2]
+
+    def numel(self):
+        return 256
+
+
+def test_the_bindings_c_part_checks_and_raises_as_the_python_one(lib):
+    """Decoding goes through csrc/pycall.c: host tensors, wrong dimensions and types and a tensor without storage raise what the checks in Python
+    raise; what is left is refused by the library (head dimension 96: unsupported, misaligned cache: invalid, no room: workspace)."""
+    t, k = _Tensor((1, 28, 128)), _Tensor((10, 4, 128))
+
+    def call(q=t, K=k, V=k, cu=t, scale=None, out=t, ws=t):
+        return dash._pycall.decode(q, K, V, cu, scale, out, None, ws, 0)
+
+    with pytest.raises(ValueError, match="device tensor expected"):
+        call(V=_Tensor((10, 4, 128), is_cuda=False))
+    with pytest.raises(ValueError):
+        call(q=_Tensor((28, 128)))
+    with pytest.raises(TypeError, match="unsupported dtype"):
+        call(q=_Tensor((1, 28, 128), dtype=torch.float16))
+    with pytest.raises(TypeError):
+        call(scale="large")
+    with pytest.raises(RuntimeError, match="no storage"):
+        call(K=_Tensor((10, 4, 128), ptr=None))
+    with pytest.raises(AttributeError):
+        call(ws=3)
+    with pytest.raises(ValueError, match="device tensor expected"):
+        dash.dash_decode_attention(torch.zeros(1, 28, 128).bfloat16(), torch.zeros(10, 4, 128).bfloat16(), torch.zeros(10, 4, 128).bfloat16(), torch.zeros(2, dtype=torch.int32))
+    assert call(q=_Tensor((1, 28, 96)), K=_Tensor((10, 4, 96)), V=_Tensor((10, 4, 96))) == 2
+    assert call(q=_Tensor((1, 28, 128), dtype=torch.float32)) == 2
+    assert call(K=_Tensor((10, 4, 128), ptr=4100)) == 1 and call(scale=-1.0) == 1 and call(scale=0.1) == 3
