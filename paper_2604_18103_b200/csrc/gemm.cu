@@ -313,6 +313,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
             const int b = tl & 1;
             const int row0 = mt * 2 * kGM + rank * kGM + q * 32;  // first row of this warp's 32
             const uint32_t tD = tmem + b * BN + lane_base;
+            const bool cut = BN == kGN && k1 - k0 != ksteps;      // (what an epilogue reads ahead it then reads behind leave_part, for the registers)
             auto wait_acc = [&]() { ok = __all_sync(0xffffffffu, mbar_wait(acc_full(b), (tl >> 1) & 1, kGWait)); tc_fence_after(); };
             // every TMEM read of this warp for the tile has completed: the buffer goes back to the MMA thread
             auto release_acc = [&]() {
@@ -320,10 +321,13 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                 __syncwarp();
                 if (lane == 0) arrive_on_leader(acc_empty(b));
             };
-            // A tile that was cut along K: every pair leaves its partial sums in `part` (a lane's row in 16-byte pieces, so that a warp's
-            // piece is 512 contiguous bytes), the last one to do so adds them up in the order of K and goes on as with a whole tile.
-            // Nobody waits for anybody.  Warp by warp: the same warp of every pair holds the same rows and columns.
-            int n_parts = 1, first_grp = 0;
+            // A tile that was cut along K.  Every pair says that it is done; all but the last to say so leave their partial sums in `part` (a lane's
+            // row in 16-byte pieces, so that a warp's piece is 512 contiguous bytes) and say that too.  The last one waits for what the others are
+            // writing at that moment -- they wait for nothing -- adds the parts up in the order of K, its own from TMEM, and goes on as with a whole
+            // tile.  Warp by warp: the same warp of every pair holds the same rows and columns.  Bound by that one SM's loads from L2, a few at a time.  (With its
+            // own part written and read back as well the last pair of the down projection was done 14 us after its last product at 701 rows, 13 at
+            // 1500, now 12 and 10.)
+            auto part_col = [&](int k) { return EPI == GEMM_SWIGLU ? (k >> 1) * 128 + half * 64 + (k & 1) * 32 : half * 128 + k * 32; };   // of piece k
             auto part_of = [&](int grp, int col) {
                 const long long U = (long long)n_tiles * ksteps;
                 const int seg = (int)((grp * U / g.groups) / ksteps) == nt ? 0 : 1;      // the tile its share begins in, or the one it ends in
@@ -333,69 +337,89 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
             auto leave_part = [&]() -> bool {                     // true: the tile is left to another pair
                 if constexpr (BN != kGN) return false;            // narrow tiles are never cut
                 const long long U = (long long)n_tiles * ksteps, u0 = (long long)nt * ksteps;
-                first_grp = (int)(((u0 + 1) * g.groups - 1) / U);
-                n_parts = (int)(((u0 + ksteps) * g.groups - 1) / U) - first_grp + 1;
+                const int first_grp = (int)(((u0 + 1) * g.groups - 1) / U), n_parts = (int)(((u0 + ksteps) * g.groups - 1) / U) - first_grp + 1;
                 unsigned int* cnt = g.arrived + (size_t)((nt * m_tiles + mt) * 2 + rank) * kGEpiWarps + (warp - 2);
                 if (row0 >= g.n) return true;                     // no rows here: nothing to add up, nothing to store
-                float4* dst0 = part_of(pair / m_tiles, 0);
+                const int own = pair / m_tiles - first_grp;
+                constexpr unsigned int kLeft = 1u << 16;          // low half of the counter: pairs that are done, high half: parts that are in `part`
+                unsigned int in = 0;
+                if (lane == 0) in = atomicAdd(cnt, 1u) & (kLeft - 1u);
+                in = __shfl_sync(0xffffffffu, in, 0);
+                if (in == (unsigned int)(n_parts - 1)) {
+                    bool all = true;
+                    if (lane == 0) {
+                        const unsigned int want = (unsigned int)(n_parts - 1) * kLeft + (unsigned int)n_parts;
+                        uint32_t spins = 0;
+                        while (*reinterpret_cast<volatile unsigned int*>(cnt) != want && all) {
+                            __nanosleep(32);
+                            all = ++spins <= kSpinLimit;
+                        }
+                        *cnt = 0u;                                // for the next launch
+                    }
+                    __threadfence();
+                    ok = __all_sync(0xffffffffu, all) && ok;
+                    if (!ok) return true;
+                    // into this warp's accumulators, 32 columns at a time, the loads of up to two of the other parts in flight (where registers are left)
+                    constexpr bool kTwo = EPI == GEMM_PLAIN || EPI == GEMM_SWIGLU;
+#pragma unroll 1
+                    for (int k = 0; k < 4; ++k) {
+                        const int col = part_col(k);
+                        uint32_t o[32];
+#pragma unroll
+                        for (int e = 0; e < 32; ++e) o[e] = 0u;
+#pragma unroll 1
+                        for (int p = 0; p < n_parts;) {
+                            uint32_t v[kTwo ? 64 : 32];
+                            const bool mine = p == own, two = kTwo && !mine && p + 1 < n_parts && p + 1 != own;
+                            if (mine) {
+                                tmem_ld32(tD + col, v);
+                                tmem_wait_ld();
+                            } else {
+                                const float4 *s0 = part_of(first_grp + p, col), *s1 = two ? part_of(first_grp + p + 1, col) : s0;
+#pragma unroll
+                                for (int c = 0; c < (kTwo ? 16 : 8); ++c) {
+                                    if (c < 8 || two) {
+                                        const float4 x = __ldcg((c < 8 ? s0 : s1) + (c & 7) * (2 * kGM));
+                                        v[4 * c] = __float_as_uint(x.x); v[4 * c + 1] = __float_as_uint(x.y); v[4 * c + 2] = __float_as_uint(x.z); v[4 * c + 3] = __float_as_uint(x.w);
+                                    }
+                                }
+                            }
+#pragma unroll
+                            for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) + __uint_as_float(v[e]));
+                            if constexpr (kTwo) {
+                                if (two) {
+#pragma unroll
+                                    for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) + __uint_as_float(v[32 + e]));
+                                }
+                            }
+                            p += two ? 2 : 1;
+                        }
+                        tmem_st32(tD + col, o);
+                    }
+                    tmem_wait_st();
+                    return false;
+                }
 #pragma unroll 1
                 for (int k = 0; k < 4; ++k) {
-                    const int col = EPI == GEMM_SWIGLU ? (k >> 1) * 128 + half * 64 + (k & 1) * 32 : half * 128 + k * 32;
+                    const int col = part_col(k);
                     uint32_t o[32];
                     tmem_ld32(tD + col, o);
                     tmem_wait_ld();
-                    float4* dst = dst0 + (size_t)(col >> 2) * (2 * kGM);
+                    float4* dst = part_of(pair / m_tiles, col);
 #pragma unroll
                     for (int c = 0; c < 8; ++c) st_v4(dst + c * (2 * kGM), make_uint4(o[4 * c], o[4 * c + 1], o[4 * c + 2], o[4 * c + 3]));
                 }
                 __threadfence();
                 __syncwarp();
-                unsigned int in = 0;
-                if (lane == 0) in = atomicAdd(cnt, 1u);
-                in = __shfl_sync(0xffffffffu, in, 0);
-                if (in != (unsigned int)(n_parts - 1)) return true;
-                __threadfence();
-                if (lane == 0) *cnt = 0u;                         // for the next launch
-                return false;
+                if (lane == 0) atomicAdd(cnt, kLeft);
+                return true;
             };
             // o[0 .. N) and o[N .. 2N): N columns of this lane's row from columns col0 and col1 of the tile
             auto load_acc = [&](auto width, int col0, int col1, uint32_t* o) {
                 constexpr int N = decltype(width)::value;
-                if (n_parts == 1) {
-                    if constexpr (N == 32) { tmem_ld32(tD + col0, o); tmem_ld32(tD + col1, o + 32); }
-                    else { tmem_ld16(tD + col0, o); tmem_ld16(tD + col1, o + 16); }
-                    tmem_wait_ld();
-                } else {
-#pragma unroll
-                    for (int e = 0; e < 2 * N; ++e) o[e] = 0u;
-#pragma unroll 1
-                    for (int p = 0; p < n_parts; p += 2) {        // two parts' loads in flight
-                        const bool two = p + 1 < n_parts;
-                        const float4* s0 = part_of(first_grp + p, 0);
-                        const float4* s1 = two ? part_of(first_grp + p + 1, 0) : s0;
-#pragma unroll
-                        for (int h = 0; h < N / 16; ++h) {
-                            float4 v[16];
-#pragma unroll
-                            for (int c = 0; c < 16; ++c) {
-                                const int cc = h * 8 + (c & 7);
-                                const int col = (cc < N / 4 ? col0 + 4 * cc : col1 + 4 * (cc - N / 4));
-                                v[c] = __ldcg((c < 8 ? s0 : s1) + (size_t)(col >> 2) * (2 * kGM));
-                            }
-#pragma unroll
-                            for (int c = 0; c < 16; ++c) {
-                                if (c < 8 || two) {
-                                    const float add[4] = {v[c].x, v[c].y, v[c].z, v[c].w};
-#pragma unroll
-                                    for (int e = 0; e < 4; ++e) {
-                                        uint32_t& x = o[(h * 8 + (c & 7)) * 4 + e];
-                                        x = __float_as_uint(__uint_as_float(x) + add[e]);
-                                    }
-                                }
-                            }
-                        }
-                    }
-                }
+                if constexpr (N == 32) { tmem_ld32(tD + col0, o); tmem_ld32(tD + col1, o + 32); }
+                else { tmem_ld16(tD + col0, o); tmem_ld16(tD + col1, o + 16); }
+                tmem_wait_ld();
             };
             const Width<16> w16; const Width<32> w32;
             auto stage_f32 = [&](const uint32_t* o) {             // 32 columns of this lane's row
@@ -408,7 +432,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                 const int col0 = nt * BN + wcol;
                 wait_acc();
                 if (!ok) break;
-                if (k1 - k0 != ksteps && leave_part()) { release_acc(); continue; }
+                if (cut && leave_part()) { release_acc(); continue; }
                 if (F32) {
 #pragma unroll
                     for (int i = 0; i < kPieces; ++i) {
@@ -485,10 +509,13 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                         }
                     }
                 };
-                fetch_cs(p0);
+                if (!cut) fetch_cs(p0);
                 wait_acc();
                 if (!ok) break;
-                if (k1 - k0 != ksteps && leave_part()) { release_acc(); continue; }
+                if (cut) {
+                    if (leave_part()) { release_acc(); continue; }
+                    fetch_cs(p0);
+                }
 #pragma unroll 1
                 for (int k = p0; k < p0 + kPieces; ++k) {
                     const int h0 = head_of(k), c = pair_of(k), colh = colw + h0;
@@ -563,14 +590,17 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                         if (row < n_true) hv[i] = ld_v2(hsrc + (int64_t)row * g.e.ldh + k * 32);
                     }
                 };
-                fetch_h(p0);
+                if (!cut) fetch_h(p0);
                 float su[8], sh[8], st2[8];
 #pragma unroll
                 for (int i = 0; i < 8; ++i) su[i] = sh[i] = st2[i] = 0.f;
                 wait_acc();
                 if (BN == kGN && !ok) break;
                 if (!ok) n_true = 0;                              // a narrow tile's two warps meet below, come what may: nothing is stored
-                if (k1 - k0 != ksteps && leave_part()) { release_acc(); continue; }
+                if (cut) {
+                    if (leave_part()) { release_acc(); continue; }
+                    fetch_h(p0);
+                }
 #pragma unroll 1
                 for (int k = p0; k < p0 + kPieces; ++k) {
                     uint32_t o[32];
@@ -618,7 +648,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                 const float rsc = (g.e.row_scale && row0 + lane < n_true) ? g.e.row_scale[row0 + lane] : 1.0f;
                 wait_acc();
                 if (!ok) break;
-                if (k1 - k0 != ksteps && leave_part()) { release_acc(); continue; }
+                if (cut && leave_part()) { release_acc(); continue; }
 #pragma unroll 1
                 for (int k = 0; k < 4; ++k) {
                     uint32_t gu[32];                              // 16 gate, 16 up columns of this lane's row
@@ -685,7 +715,8 @@ size_t gemm_split_count_bytes() { return align_up((size_t)(sm_count() / 2) * kGS
 // and 24 steps (233 rows, d = 2048) 71 / 53, of 42 and 42 (233 rows, 7B) 76 / 68, of 64 to 74 (down projections) about even: 701 rows of
 // d = 2048 151 / 146, in a graph 143 / 160, 1024 and 2100 rows of 7B 384 / 385 and 793 / 781; 72 at 233 rows of d = 2048 114 / 122, 123 at
 // 701 rows of 7B 304 / 320, 184 at 300 233 / 268, 197 at 2728 1009 / 1047.  (Two rounds of tiles of which the second is half empty, 1500 rows of 7B,
-// gain 11 us of 149 by cuts that save 28 and 46 steps: the rule leaves those.)
+// gain 11 us of 149 by cuts that save 28 and 46 steps: the rule leaves those.  In a loop at the power cap, three blocks, a cost of
+// 60 / 45 / 25: 600 rows 863 / 865 / 873 us, 1500 1567 / 1570 / 1590, 2000 2005 / 2015 / 2010.)
 static int gemm_groups(int m_tiles, int n_tiles, int ksteps, int P, bool can) {
     const long long tiles = (long long)m_tiles * n_tiles;
     if (!can || m_tiles > P || tiles > (long long)kGSplitMaxRounds * P) return 0;
