@@ -199,15 +199,32 @@ prologue_kernel(const PrologueArgs a, const RopeFreqs fr) {
             const float4* x = reinterpret_cast<const float4*>(a.H + t * a.ldh_b);
             const float4* w = reinterpret_cast<const float4*>(a.rms_w);
             uint2* y = reinterpret_cast<uint2*>(a.Hn16) + t * a.nvec;
+            const int32_t pos = a.table ? a.pos[t] : 0;
             float ss = 0.f;
-            for (int v = lane; v < a.nvec; v += 32) { const float4 c = x[v]; ss += c.x * c.x; ss += c.y * c.y; ss += c.z * c.z; ss += c.w * c.w; }      // as rmsnorm_kernel
-            const float rs = rsqrtf(warp_sum(ss) * a.inv_d + a.eps);
-            for (int v = lane; v < a.nvec; v += 32) {
-                const float4 c = x[v], g = w[v];
-                y[v] = make_uint2(pack_bf16(c.x * rs * g.x, c.y * rs * g.y), pack_bf16(c.z * rs * g.z, c.w * rs * g.w));
+            auto add = [&](float4 c) { ss += c.x * c.x; ss += c.y * c.y; ss += c.z * c.z; ss += c.w * c.w; };      // as rmsnorm_kernel
+            auto normalised = [&](float4 c, float4 g, float rs) { return make_uint2(pack_bf16(c.x * rs * g.x, c.y * rs * g.y), pack_bf16(c.z * rs * g.z, c.w * rs * g.w)); };
+            constexpr int KEEP = 4;              // rows of up to 512 columns stay in registers, their weights asked for beside them
+            if (a.nvec <= 32 * KEEP) {
+                float4 c[KEEP], g[KEEP];
+#pragma unroll
+                for (int k = 0; k < KEEP; ++k) {
+                    const int v = lane + 32 * k;
+                    if (v < a.nvec) { c[k] = x[v]; g[k] = w[v]; }
+                }
+#pragma unroll
+                for (int k = 0; k < KEEP; ++k)
+                    if (lane + 32 * k < a.nvec) add(c[k]);
+                const float rs = rsqrtf(warp_sum(ss) * a.inv_d + a.eps);
+#pragma unroll
+                for (int k = 0; k < KEEP; ++k)
+                    if (lane + 32 * k < a.nvec) y[lane + 32 * k] = normalised(c[k], g[k], rs);
+            } else {
+                for (int v = lane; v < a.nvec; v += 32) add(x[v]);
+                const float rs = rsqrtf(warp_sum(ss) * a.inv_d + a.eps);
+                for (int v = lane; v < a.nvec; v += 32) y[v] = normalised(x[v], w[v], rs);
             }
             if (a.table) {
-                const double ps = (double)a.pos[t];
+                const double ps = (double)pos;
                 for (int i = lane; i < a.half; i += 32) {
                     double sn, cs;
                     sincos(ps * fr.inv_freq[i], &sn, &cs);
@@ -219,10 +236,19 @@ prologue_kernel(const PrologueArgs a, const RopeFreqs fr) {
     }
     cta -= a.row_ctas;
     const int64_t step = (int64_t)((int)gridDim.x - 2 - a.row_ctas) * 256;
-    for (int64_t i = (int64_t)cta * 256 + threadIdx.x; i < a.n_w0 + a.n_w1; i += step) {
-        const bool second = i >= a.n_w0;
-        const float4 c = second ? a.w1[i - a.n_w0] : a.w0[i];
-        (second ? a.w1_16[i - a.n_w0] : a.w0_16[i]) = make_uint2(pack_bf16(c.x, c.y), pack_bf16(c.z, c.w));
+    const int64_t all = a.n_w0 + a.n_w1;
+    for (int64_t i0 = (int64_t)cta * 256 + threadIdx.x; i0 < all; i0 += 4 * step) {      // four loads in flight per thread
+        float4 c[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int64_t i = i0 + k * step;
+            if (i < all) c[k] = i >= a.n_w0 ? a.w1[i - a.n_w0] : a.w0[i];
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int64_t i = i0 + k * step;
+            if (i < all) (i >= a.n_w0 ? a.w1_16[i - a.n_w0] : a.w0_16[i]) = make_uint2(pack_bf16(c[k].x, c[k].y), pack_bf16(c[k].z, c[k].w));
+        }
     }
 }
 
