@@ -53,10 +53,14 @@ struct SelfPlan {
     int cu[kSelfPlanSeqs + 1];        // the boundaries it was made from
     int chunk, n_items;
 };
-// Called by all threads of the CTA (it synchronises).  `target` is twice the number of CTAs.  Chunk length (key blocks per item):
-// preferred is one item per CTA -- the shortest chunk with at most target / 2 items (the last chunk of every sequence and head is an
-// item of its own, so the first guess can overshoot, and a CTA with a second item would double the kernel's time); half the pipeline
-// ramps and half the partial results to merge.  Taken when it keeps at least 17 of 20 CTAs busy; otherwise about `target` items.
+// Called by all threads of the CTA (it synchronises).  `target` is twice the number of CTAs; the items at a chunk length of ceil(all blocks / target) and more are
+// never more than target + sequences x heads, which the workspace has room for.  Chunk length (key blocks per item): an even share per CTA, if
+// that makes no more items than CTAs (the last chunk of every sequence and head is an item of its own, so it can overshoot); else, of that, the next one, and three
+// from two items per CTA on, the one with the fewest rounds x (chunk + 1.5): a CTA goes through an item in about 2 us a block and 3 us beside.  us a call in
+// a graph, 28 / 4 heads of 128: this rule / one item per CTA where that kept 17 of 20 CTAs busy, else about two / the best of all lengths: one cache
+// of 8192 rows 7.7 / 7.7 / 7.6, of 20 000 12.5 / 14.9 / 12.5, 4 of 7500 on the average 16.4 / 18.3 / 16.4, 8 of 2500 13.3 / 16.4 / 13.3, 16 of 750 11.6 / 14.1 / 11.6, 24 of
+// 3125 31.3 / 31.3 / 31.3, 33 of 485 14.3 / 15.4 / 14.3, 40 of 750 19.3 / 18.6 / 18.4, 80 of 625 28.8 / 31.7 / 28.8, 96 of 1250 54.1 / 60.3 / 53.8.  (Little
+// code on purpose: with every length up to the first that fits tried, in two loops, a call took 0.4 to 1.7 us longer.)
 __device__ __forceinline__ void self_plan_build(SelfPlan& sp, const int32_t* cu, int S, int Hkv, int target) {
     if (threadIdx.x < 32) {
         constexpr int PL = kSelfPlanSeqs / 32;
@@ -75,12 +79,18 @@ __device__ __forceinline__ void self_plan_build(SelfPlan& sp, const int32_t* cu,
                 if (32 * j < S) k += (nb[j] + chunk - 1) / chunk;
             return (int)(__reduce_add_sync(0xffffffffu, k) * (unsigned int)Hkv);
         };
-        unsigned int chunk = max(1u, (all + (unsigned int)target - 1) / (unsigned int)target);
-        const int ctas = target / 2;
-        unsigned int c1 = max(1u, (all + (unsigned int)ctas - 1) / (unsigned int)ctas);
-        int cnt = count(c1);
-        for (int tries = 0; tries < 8 && cnt > ctas; ++tries) cnt = count(++c1);
-        if (cnt <= ctas && cnt * 20 >= ctas * 17) chunk = c1;
+        const unsigned int ctas = (unsigned int)target / 2, even = max(1u, (all + ctas - 1) / ctas), half = max(1u, (all + (unsigned int)target - 1) / (unsigned int)target);
+        unsigned int chunk = even;
+        if ((unsigned int)count(even) > ctas) {
+            unsigned int least = 0xffffffffu;
+#pragma unroll 1
+            for (unsigned int i = 0; i < 5; ++i) {
+                const unsigned int c = i < 2 ? even + i : half + i - 2;
+                unsigned int rounds = 0;
+                for (unsigned int left = (unsigned int)count(c); rounds < 1 || left > 0; ++rounds) left -= min(left, ctas);
+                if (rounds * (2 * c + 3) < least) { least = rounds * (2 * c + 3); chunk = c; }
+            }
+        }
         int k = 0;                    // items in front of the current group of 32 sequences
 #pragma unroll
         for (int j = 0; j < PL; ++j) {

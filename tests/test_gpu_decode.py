@@ -102,6 +102,14 @@ def test_decode_random_batches_match_oracle():
         _decode_case(lens, Hkv * G, Hkv, D, 100 + trial)
 
 
+@pytest.mark.parametrize("lens", [[37888], [37889], [20000], [2500, 1700, 3300, 2900, 2100, 2600, 1900, 3000], [128 * 37] * 8, [128 * 37] * 7 + [128 * 38],
+                                  [485 + 31 * (i % 7) for i in range(33)], [128 * 9] * 74, [1250 + 11 * i for i in range(96)]], ids=lambda x: f"{len(x)}x{x[0]}")
+def test_decode_chunk_lengths_on_both_sides_of_the_plans_rule(lens):
+    """One KV head per sequence: as many items as CTAs at an even share, one more than that, and batches in which the plan takes a longer chunk or two
+    items per CTA."""
+    _decode_case(lens, 4, 1, 64, len(lens))
+
+
 @pytest.mark.parametrize("S", [1, 5, 40, 128])
 def test_decode_over_boundaries_that_the_call_in_front_writes(S):
     """Decoding directly behind the compaction that shortens its caches: the decode kernel plans from the boundaries as they stand, while the
