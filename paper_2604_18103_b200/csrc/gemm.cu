@@ -752,7 +752,7 @@ static bool gemm_narrow(int m_tiles, int n_tiles, int P) { return 2LL * m_tiles 
 
 // Groups of rows of tiles or of columns: the group's operand (16 tiles of 256 x 3584, 29 MB) stays in L2 while the other one streams past it, once
 // per group.  So of the two orders the one that reads less: (groups - 1) times the other operand more than both once.  The gate | up projection of
-// 8192 rows, 32 x 148 tiles, read 1.01 GB from HBM in groups of columns (its operands are 0.33 GB; 0.60 expected in groups of rows); the
+// 8192 rows, 32 x 148 tiles, reads 1.01 GB from HBM in groups of columns, 0.83 in groups of rows (its operands are 0.33 GB); the
 // step runs at the power cap, where bytes are time: three blocks of 701, 6683, 8192 rows in a loop, columns / rows, us 883 / 877, 5772 / 5737,
 // 7817 / 7768.  Groups of 8, 11 and 32: 8192 rows 7812, 7828, 7910.
 static bool gemm_by_m(int m_tiles, int n_tiles) {

@@ -677,17 +677,15 @@ __device__ __forceinline__ int tail_decide(const TailArgs& a, int64_t row, float
     return keep;
 }
 
-// The same pass with a warp per row and tiles of eight rows, so that 700 rows are 88 CTAs and not 22 (threshold rule: with the decisions given see
-// delta_given_kernel).  Bound by the chain ticket -> rows -> look-back -> copy; for inputs whose tiles are all resident.  So the number of rows is
-// asked for beside the ticket, every tile in front is asked for its count at once, a thread to each, and a row's vectors stay in registers for the
-// copy, or are loaded for it, before the base is known (from the end of the kernel in front, us: fp32 layer of 1024 rows 6.6, 8.3 with these one behind
-// the other, 1500 rows of the 7B shape 10.3, was 12.4).  Loops of seven vectors per lane (two for a row of 3584 bf16), not unrolled: with the whole row in registers and straight-line
-// code the warps waited 14 us for instructions they run once.
+// The same pass with a warp per row and tiles of eight rows, so that 700 rows are 88 CTAs and not 22: threshold rule on U and H (fp32 tensors, shapes whose
+// projections run plain; the others decide in sums_to_score_kernel, tail_in_two).  Bound by the chain ticket -> rows -> look-back -> copy; for inputs
+// whose tiles are all resident.  So the number of rows is asked for beside the ticket, every tile in front is asked for its count at once, a thread
+// to each, and a row's last vectors stay in registers for the copy (from the end of the kernel in front, us: fp32 layer of 1024 rows 6.6, 8.3 with these
+// one behind the other).  Loops of seven vectors per lane (two for a row of 3584 bf16), not unrolled: with the whole row in registers and
+// straight-line code the warps waited 14 us for instructions they run once.
 constexpr int kTailRows = 8;
-constexpr int kTailSmallTiles = 2;          // per SM: with more tiles than fit at once, a tile waits for the look-back chain of up to a
-                                            // thousand others (behind the projection in front, 6683 rows: 64 us against 40 of the general kernel, 8192: 80 against 42).
-                                            // Whole layers of the 7B shape, this kernel / the general one: 1185 rows 107 / 116, 2000 144 / 152, 2368
-                                            // 170 / 180, 2700 203 / 208, 3500 267 / 271, 4000 334 / 323, 4736 381 / 369: the line could lie as high as 3
+constexpr int kTailSmallTiles = 3;          // per SM.  fp32 layers (d = 256) in a graph, this kernel / the general one, us: 1200 rows 35.7 / 38.2, 2300 42.2 / 45.6, 3000 45.3 /
+                                            // 48.2, 3500 52.6 / 52.9, 5000 63.6 / 63.8.  (Rows of 7 KB, while they came here too: 2368 170 / 180, 3500 267 / 271, 4000 334 / 323)
 template <bool BF16>
 __global__ void __launch_bounds__(32 * kTailRows)
 delta_tail_rows_kernel(const TailArgs a, int64_t n_upper) {
@@ -714,46 +712,37 @@ delta_tail_rows_kernel(const TailArgs a, int64_t n_upper) {
     if (row < n) {
         tok = a.tok_in[row];
         pos = a.pos_in[row];
-        if (a.U) {
-            const char* u = a.U + row * a.ldU_b;
-            const char* h = a.H + row * a.ldH_b;
+        const char* u = a.U + row * a.ldU_b;
+        const char* h = a.H + row * a.ldH_b;
 #pragma unroll 1
-            for (int v0 = lane; v0 < a.nvec; v0 += 32 * CH) {
-                uint4 q[CH];
-                have = v0;
+        for (int v0 = lane; v0 < a.nvec; v0 += 32 * CH) {
+            uint4 q[CH];
+            have = v0;
 #pragma unroll
-                for (int k = 0; k < CH; ++k) {
-                    const int64_t v = v0 + k * 32;
-                    if (v < a.nvec) { p[k] = ld_nc_v4(u + (v << 4)); q[k] = ld_nc_v4(h + (v << 4)); }
-                    else p[k] = q[k] = make_uint4(0, 0, 0, 0);
-                }
-#pragma unroll
-                for (int k = 0; k < CH; ++k) { su += sumsq_vec<BF16>(p[k]); sh += sumsq_vec<BF16>(q[k]); }
-                char* o = x + (int64_t)tok * a.ldx_b;
-#pragma unroll
-                for (int k = 0; k < CH; ++k) {
-                    const int64_t v = v0 + k * 32;
-                    p[k] = add_vec<BF16>(p[k], q[k]);
-                    if (v < a.nvec) st_v4(o + (v << 4), p[k]);
-                }
-                if (a.inv_next) {
-#pragma unroll
-                    for (int k = 0; k < CH; ++k) ss += sumsq_vec<BF16>(p[k]);
-                }
+            for (int k = 0; k < CH; ++k) {
+                const int64_t v = v0 + k * 32;
+                if (v < a.nvec) { p[k] = ld_nc_v4(u + (v << 4)); q[k] = ld_nc_v4(h + (v << 4)); }
+                else p[k] = q[k] = make_uint4(0, 0, 0, 0);
             }
-        } else {
-            for (int i = lane; i < a.n_sum_tiles; i += 32) { const float4 p2 = a.sums[row * a.n_sum_tiles + i]; su += p2.x; sh += p2.y; ss += p2.z; }
+#pragma unroll
+            for (int k = 0; k < CH; ++k) { su += sumsq_vec<BF16>(p[k]); sh += sumsq_vec<BF16>(q[k]); }
+            char* o = x + (int64_t)tok * a.ldx_b;
+#pragma unroll
+            for (int k = 0; k < CH; ++k) {
+                const int64_t v = v0 + k * 32;
+                p[k] = add_vec<BF16>(p[k], q[k]);
+                if (v < a.nvec) st_v4(o + (v << 4), p[k]);
+            }
+            if (a.inv_next) {
+#pragma unroll
+                for (int k = 0; k < CH; ++k) ss += sumsq_vec<BF16>(p[k]);
+            }
         }
         x += (int64_t)tok * a.ldx_b;
         keep = tail_decide(a, row, warp_sum(su), warp_sum(sh), lane);
     }
     if (a.inv_next) ss = warp_sum(ss);
     if (lane == 0) s_keep[warp] = keep;
-    auto load_chunk = [&](int v0) {
-#pragma unroll
-        for (int k = 0; k < CH; ++k) { const int64_t v = v0 + k * 32; if (v < a.nvec) p[k] = ld_cg_v4(x + (v << 4)); }
-    };
-    if (keep && !a.U) load_chunk(have);                    // in flight while the base is looked for
     __syncthreads();
     const unsigned int bal = __ballot_sync(0xffffffffu, lane < kTailRows && s_keep[lane < kTailRows ? lane : 0]);
     const int count = __popc(bal);
@@ -789,7 +778,8 @@ delta_tail_rows_kernel(const TailArgs a, int64_t n_upper) {
 #pragma unroll 1
         for (int v0 = lane; v0 < a.nvec; v0 += 32 * CH) {
             if (v0 == have) continue;
-            load_chunk(v0);
+#pragma unroll
+            for (int k = 0; k < CH; ++k) { const int64_t v = v0 + k * 32; if (v < a.nvec) p[k] = ld_cg_v4(x + (v << 4)); }
             store_chunk(v0);
         }
         if (lane == 0) {
@@ -813,7 +803,7 @@ delta_tail_rows_kernel(const TailArgs a, int64_t n_upper) {
 
 // The tail pass where the decisions are given (mask_in): the output base of a tile is counted from the mask itself, as dash_compact does it, so that
 // a row needs no ticket, no look-back and no second visit -- U and H are read once, their sum goes to x_full[tok] and, where the row
-// stays, to H_next (U null: the rows are in x_full, those that stay are copied).  A warp per row, RPW rows one behind the other.  Bound by HBM, for few
+// stays, to H_next (U null: the rows are in x_full, those that stay are copied, and inv_next comes from sums).  A warp per row, RPW rows one behind the other.  Bound by HBM, for few
 // rows by the chain mask -> rows.  From the end of the kernel in front to its own, us, kernels with look-back / this one: blocks of the 7B shape of 701
 // rows that all stay 15.2 / 9.8, 1500 17.8 / 11.1, 3000 47.8 / 22.9, 6683 53 / 38.5, 8192 61.6 / 51.1 (235 MB), 32 768 245 / 203, of 2728 51 / 23;
 // count rule, 12 345 rows 40.5 / 29.9.  (As many rows to every CTA, all resident at once: 701 11.7, 8192 55.7, 32 768 210.)  Up to kGivenMaxRows:
@@ -868,6 +858,8 @@ delta_given_kernel(const TailArgs a, int64_t n_upper) {
         char* x = a.x_full + (int64_t)tok * a.ldx_b;
         char* dst = a.H_next + k * a.ldn_b;
         float ss = 0.f;
+        if (!a.U && a.inv_next)
+            for (int i = lane; i < a.n_sum_tiles; i += 32) ss += a.sums[row * a.n_sum_tiles + i].z;
 #pragma unroll 1
         for (int v0 = lane; v0 < a.nvec; v0 += 32 * CH) {
             uint4 p[CH];
@@ -1331,6 +1323,10 @@ int launch_sums_to_score(const float4* sums, int n_sum_tiles, int64_t n, dash_no
 // rows.  ws: the compaction workspace (ticket + one state word per tile), whose first tail_ws_clear_bytes(n) the caller has zeroed
 // on this stream (ahead of the kernels in front, so that this launch follows a kernel directly and may start while that one drains).
 // (tiles of kTailRows rows at the smallest)
+// Whether a threshold step of n rows whose H~ and row sums the output projection has written decides in a launch of its own (sums_to_score_kernel)
+// and then moves the rows (delta_given_kernel).  Layers of the 7B shape in a loop, 60 % stay, one launch for both / two, us: 700 rows 78.1 / 78.0, 1500
+// 126.2 / 125.0, 2300 171.2 / 170.7, 3000 218 / 212, 5000 364 / 359.5, 8192 827 / 819, 15 000 1494 / 1490, 24 000 3015 / 3017.
+bool tail_in_two(int64_t n) { return n <= kGivenMaxRows; }
 size_t tail_ws_clear_bytes(int64_t n) { return 256 + (size_t)((n + kTailRows - 1) / kTailRows > 0 ? (n + kTailRows - 1) / kTailRows : 1) * 8; }
 int launch_delta_tail(const void* U, const void* H, const uint8_t* mask_in, const float4* sums, int n_sum_tiles, int64_t n, int d, dash_dtype dt, dash_norm_mode mode, float eps, float tau,
                       int keep_first, int keep_last, const int32_t* cu_in, int S, const int32_t* tok_in, const int32_t* pos_in,
@@ -1348,7 +1344,7 @@ int launch_delta_tail(const void* U, const void* H, const uint8_t* mask_in, cons
     a.inv_next = inv_next; a.inv_d = 1.0f / (float)d; a.rms_eps = rms_eps;
     a.status = status_word_ptr();
     if (!a.status) return DASH_ERR_CUDA;
-    if (mask_in && n <= kGivenMaxRows && (U || !inv_next)) {
+    if (mask_in && n <= kGivenMaxRows) {
         // tiles of eight rows where they fill their waves better than tiles of sixteen (us from the end of the kernel in front, 8 / 16: 6683 rows 38.5 /
         // 46.5; as well filled: 8192 rows 54.6 / 51.1, 12 345 rows, count rule 31.6 / 29.9, 3000 rows 23.1 / 22.9)
         auto tiles = [&](int rows) { return n > 0 ? (n + rows - 1) / rows : 1; };
@@ -1361,7 +1357,7 @@ int launch_delta_tail(const void* U, const void* H, const uint8_t* mask_in, cons
         return DASH_OK;
     }
     const int small = (int)((n + kTailRows - 1) / kTailRows) > 0 ? (int)((n + kTailRows - 1) / kTailRows) : 1;
-    if (!mask_in && small <= kTailSmallTiles * sm_count()) {
+    if (U && !mask_in && small <= kTailSmallTiles * sm_count()) {
         if (dt == DASH_BF16) DASH_CUDA_TRY(launch_pdl(delta_tail_rows_kernel<true>, small, 32 * kTailRows, 0, st, a, n));
         else DASH_CUDA_TRY(launch_pdl(delta_tail_rows_kernel<false>, small, 32 * kTailRows, 0, st, a, n));
         return DASH_OK;

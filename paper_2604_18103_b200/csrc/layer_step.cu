@@ -131,6 +131,7 @@ int launch_delta_tail(const void* U, const void* H, const uint8_t* mask_in, cons
                       void* x_full, void* H_next, float* r_out, uint8_t* mask_out, int32_t* tok_next, int32_t* pos_next,
                       int32_t* cu_next, int32_t* n_next, void* ws, size_t ws_bytes, cudaStream_t st, float* inv_next, float rms_eps);
 size_t tail_ws_clear_bytes(int64_t n);
+bool tail_in_two(int64_t n);
 int attention_planned(const void* Q, const void* K, const void* V, void* O, float* lse, int64_t ldq, int64_t ldk, int64_t ldv, int64_t ldo,
                       const int32_t* cu_seqlens, int S, int64_t n, int64_t max_seqlen, int Hq, int Hkv, int D, float scale, dash_dtype dt,
                       void* ws, size_t ws_bytes, cudaStream_t st, void* O16 = nullptr);
@@ -645,8 +646,14 @@ extern "C" int dash_layer_step(const dash_layer_cfg* cfg, const void* H_in, cons
             // output projection with H~ = H + U written straight to x_full and the row sums of u^2, h^2 beside it; then the score, the
             // halting rule and the compaction of the rows that stay (from x_full) in one pass
             rc = out_proj_residual(cfg, H_in, tok_index_in, x_full, cu_in, S, n, W, st);
+            const uint8_t* decided = nullptr;
+            if (rc == DASH_OK && tail_in_two(n)) {
+                dash_threshold ft = {cfg->tau, cfg->keep_first, cfg->keep_last, cu_in, S, mask_out};
+                if ((rc = launch_sums_to_score(W.sums, d / 128, n, cfg->norm_mode, cfg->norm_eps, r_out, &ft, cu_in + S, nullptr, d, cfg->rms_eps, st)) != DASH_OK) return rc;
+                decided = mask_out;
+            }
             if (rc == DASH_OK)
-                return launch_delta_tail(nullptr, nullptr, nullptr, W.sums, d / 128, n, d, cfg->dt, cfg->norm_mode, cfg->norm_eps, cfg->tau,
+                return launch_delta_tail(nullptr, nullptr, decided, W.sums, d / 128, n, d, cfg->dt, cfg->norm_mode, cfg->norm_eps, cfg->tau,
                                          cfg->keep_first, cfg->keep_last, cu_in, S, tok_index_in, pos_in, x_full, H_next, r_out, mask_out,
                                          tok_index_next, pos_next, cu_next, n_next_dev, W.compact_ws, W.compact_bytes, st,
                                          cfg->inv_rms_next, cfg->rms_eps);

@@ -369,10 +369,10 @@ def test_kv_cache_rows_are_the_projections_for_every_head_size_and_alignment(sha
 
 
 @pytest.mark.parametrize("shape,n", [(wl.MINI, 1), (wl.MINI, 255), (wl.MINI, 257), (wl.MINI, 1536), (wl.MINI, 1537), (wl.TINY, 1), (wl.TINY, 257), (wl.TINY, 3072),
-                                     (wl.TINY, 3073)], ids=lambda x: x if isinstance(x, int) else ("fp32" if x.dtype == torch.float32 else "bf16"))
+                                     (wl.TINY, 3073), (wl.TINY, 3553)], ids=lambda x: x if isinstance(x, int) else ("fp32" if x.dtype == torch.float32 else "bf16"))
 def test_layer_step_over_projection_tiles_of_both_widths(shape, n):
     """Projections of few tiles take 128 columns per tile, others 256 (Q | K | V of MINI: up to 1536 rows, of the fp32 shape: up to 3072): one row, an
-    incomplete and a second row of tiles, both sides of the line."""
+    incomplete and a second row of tiles, both sides of the line (3553 rows: the general tail pass, too)."""
     cu = wl.cu_from_lengths([n])
     H, W = wl.hidden_states(n, shape.d, 61, shape.dtype), wl.layer_weights(shape, 61)
     pos = wl.positions(cu)
