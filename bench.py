@@ -301,10 +301,10 @@ def setup_block_step(args, dash, dev, rank):
     name = "configs[0]: single fp32 layer, hidden 256, 4 heads of 64" if args.workload == "cfg1" else "configs[1]: Qwen2.5-7B-shaped single layer, bf16"
     return {
         "workload": f"{name}, batch 1, seq {T}, threshold at the {int(w.rho * 100)}th percentile ({n_active} of {T} tokens stay active)",
-        "dtype": "f32" if sh.dtype == torch.float32 else "bf16", "step": step, "h2d": h2d, "d2h": d2h, "tokens": T, "launches": 6 if sh.dtype == torch.float32 else 5,
+        "dtype": "f32" if sh.dtype == torch.float32 else "bf16", "step": step, "h2d": h2d, "d2h": d2h, "tokens": T, "launches": 5 if sh.dtype == torch.float32 else 6,
         "launch_note": "per step: prologue (attention item list, zeroed words, row factors of the norm; the rotary angles come from a table made once "
-                       "per prefill; fp32: normalised rows and weights in bf16), QKV GEMM (norm factor + rotary on the accumulators; fp32: plain, "
-                       "the rotary embedding a kernel of its own), attention, output GEMM (+ residual, score sums), tail (score + threshold + compaction)",
+                       "per prefill; fp32: normalised rows and weights in bf16, rotary angles), QKV GEMM (norm factor + rotary on the accumulators), attention, "
+                       "output GEMM (+ residual, score sums), score + threshold, tail (compaction; fp32: score and threshold too)",
         "h2d_bytes": _bytes(H_host, pos_host, tok_host, cu_host), "d2h_bytes": _bytes(*host_out),
         "extra": {"n_active_after": n_active, "tau": tau}, "e2e_pipeline": e2e_pipeline,
         "attn": (lambda: dash.dash_varlen_attention(Q, Kt, V, cu, T, O=Obuf, ws=attn_ws)), "attn_flops": attention_flops(w.cu.tolist(), sh.Hq, sh.D),
@@ -388,8 +388,8 @@ def setup_cascade(args, dash, dev, rank):
     fl_all = sum(attention_flops([0, n], sh.Hq, sh.D) for n in n_in)
     return {
         "workload": f"configs[2]: cascade of {Lr} Qwen2.5-7B-shaped layers, bf16, batch 1, seq {T}, tokens entering the layers {n_in}, "
-                    f"{got} active after the last", "dtype": "bf16", "step": step, "h2d": h2d, "d2h": d2h, "tokens": sum(n_in), "launches": 5 * Lr,
-        "launch_note": f"{Lr} block steps of 5 kernels each (prologue, QKV GEMM, attention, output GEMM, tail; the first prologue also forms its row factors; "
+                    f"{got} active after the last", "dtype": "bf16", "step": step, "h2d": h2d, "d2h": d2h, "tokens": sum(n_in), "launches": sum(6 if n <= 32768 else 5 for n in n_in),
+        "launch_note": f"{Lr} block steps of 6 kernels each (prologue, QKV GEMM, attention, output GEMM, score, tail; the first prologue also forms its row factors; "
                        "rotary table made once per prefill, row factors handed from block to block)",
         "h2d_bytes": _bytes(H_host, pos_host, tok_host, cu_host), "d2h_bytes": _bytes(x_full_h, tok_h, cu_h),
         "extra": {"tokens_entering_layers": n_in, "active_after_last": got, "attention_flops_per_step": fl_all,

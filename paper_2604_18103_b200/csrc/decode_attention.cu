@@ -86,9 +86,8 @@ __device__ __forceinline__ void self_plan_build(SelfPlan& sp, const int32_t* cu,
 #pragma unroll 1
             for (unsigned int i = 0; i < 5; ++i) {
                 const unsigned int c = i < 2 ? even + i : half + i - 2;
-                unsigned int rounds = 0;
-                for (unsigned int left = (unsigned int)count(c); rounds < 1 || left > 0; ++rounds) left -= min(left, ctas);
-                if (rounds * (2 * c + 3) < least) { least = rounds * (2 * c + 3); chunk = c; }
+                const unsigned int cost = ((unsigned int)count(c) + ctas - 1) / ctas * (2 * c + 3);
+                if (cost < least) { least = cost; chunk = c; }
             }
         }
         int k = 0;                    // items in front of the current group of 32 sequences

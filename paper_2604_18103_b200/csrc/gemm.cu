@@ -355,10 +355,11 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                             all = ++spins <= kSpinLimit;
                         }
                         *cnt = 0u;                                // for the next launch
+                        if (!all) atomicExch(g.status, DASH_ERR_TIMEOUT);
                     }
+                    __syncwarp();
                     __threadfence();
-                    ok = __all_sync(0xffffffffu, all) && ok;
-                    if (!ok) return true;
+                    if (__any_sync(0xffffffffu, !all)) return true;
                     // into this warp's accumulators, 32 columns at a time, the loads of up to two of the other parts in flight (where registers are left)
                     constexpr bool kTwo = EPI == GEMM_PLAIN || EPI == GEMM_SWIGLU;
 #pragma unroll 1
