@@ -104,13 +104,14 @@ template <int N> struct Width { static constexpr int value = N; };
 // `groups` groups with one pair per row of tiles; the K steps of all column tiles are dealt out evenly to the groups, in order, so that
 // a group's share begins and ends anywhere inside a tile, and its pairs go through the same part of W at the same time (W comes from
 // HBM once: with the tiles' K steps simply dealt out to the pairs, a 136 MB weight matrix was read 3.6 times for three rows of tiles).
+template <bool CUT>
 struct Work {
     int t, tiles, P, m_tiles, n_tiles, ksteps, mt;
     long long u, u1;
-    bool cut, by_m;
+    bool by_m;
     __device__ __forceinline__ Work(int pair, int P_, int m_tiles_, int n_tiles_, int ksteps_, int groups, int by_m_)
-        : t(pair), tiles(m_tiles_ * n_tiles_), P(P_), m_tiles(m_tiles_), n_tiles(n_tiles_), ksteps(ksteps_), mt(0), u(0), u1(0), cut(groups > 0), by_m(by_m_ != 0) {
-        if (cut) {
+        : t(pair), tiles(m_tiles_ * n_tiles_), P(P_), m_tiles(m_tiles_), n_tiles(n_tiles_), ksteps(ksteps_), mt(0), u(0), u1(0), by_m(by_m_ != 0) {
+        if constexpr (CUT) {
             const int grp = pair / m_tiles;
             const long long U = (long long)n_tiles * ksteps;
             mt = pair % m_tiles;
@@ -118,7 +119,7 @@ struct Work {
         }
     }
     __device__ __forceinline__ bool next(int& m, int& n, int& k0, int& k1) {
-        if (!cut) {
+        if constexpr (!CUT) {
             if (t >= tiles) return false;
             tile_coords(t, m_tiles, n_tiles, by_m, m, n);
             k0 = 0; k1 = ksteps; t += P;
@@ -180,11 +181,13 @@ __device__ __forceinline__ void reduce_rows8(float (&v)[8], int lane) {
     }
 }
 
-// F32 (PLAIN, ROPE): C is fp32
-template <int EPI, int BN, bool F32>
+// F32 (PLAIN, ROPE): C is fp32.  CUT: tiles may be cut along K; kernels of their own, because the adding up of parts beside their epilogue's code cost those of
+// whole tiles registers (gate | up projection 544 cycles per K step without, 550 with it; in one kernel / apart, in a loop, us: layer of 5000 rows 368 / 360, of 8192 834 / 826, three blocks of 701
+// rows 875 / 869, of 8192 7815 / 7755)
+template <int EPI, int BN, bool F32, bool CUT>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGThreads, 1)
 gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapW, const GemmArgs g) {
-    static_assert(BN == kGN || (BN == kGNarrow && EPI != GEMM_SWIGLU), "tile widths");
+    static_assert(BN == kGN || (BN == kGNarrow && EPI != GEMM_SWIGLU && !CUT), "tile widths");
     constexpr int kGStages = Ring<BN>::kStages, kGStageBytes = Ring<BN>::kStage;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -227,7 +230,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
         if (lane == 0) {
             uint32_t it = 0;
             bool ok = true;
-            Work w(pair, n_pairs, m_tiles, n_tiles, ksteps, g.groups, g.by_m);
+            Work<CUT> w(pair, n_pairs, m_tiles, n_tiles, ksteps, g.groups, g.by_m);
             int mt, nt, k0, k1;
             // w_early: the first stages' W tiles are asked for while the kernel in front, which makes A, still drains (see gemm.cuh for when)
             bool first = true;
@@ -268,7 +271,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
         if (lane == 0 && rank == 0) {
             uint32_t it = 0, tl = 0;
             bool ok = true;
-            Work w(pair, n_pairs, m_tiles, n_tiles, ksteps, g.groups, g.by_m);
+            Work<CUT> w(pair, n_pairs, m_tiles, n_tiles, ksteps, g.groups, g.by_m);
             int mt, nt, k0, k1;
             for (; ok && w.next(mt, nt, k0, k1); ++tl) {
                 const int b = tl & 1;
@@ -307,13 +310,13 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
         const int r8 = lane >> 3, c8 = lane & 7;                  // eight lanes per row: row r8 + 4 i, chunk c8
         uint32_t tl = 0;
         bool ok = true;
-        Work w(pair, n_pairs, m_tiles, n_tiles, ksteps, g.groups, g.by_m);
+        Work<CUT> w(pair, n_pairs, m_tiles, n_tiles, ksteps, g.groups, g.by_m);
         int mt, nt, k0, k1;
         for (; w.next(mt, nt, k0, k1); ++tl) {
             const int b = tl & 1;
             const int row0 = mt * 2 * kGM + rank * kGM + q * 32;  // first row of this warp's 32
             const uint32_t tD = tmem + b * BN + lane_base;
-            const bool cut = BN == kGN && k1 - k0 != ksteps;      // (what an epilogue reads ahead it then reads behind leave_part, for the registers)
+            const bool cut = CUT && k1 - k0 != ksteps;      // (what an epilogue reads ahead it then reads behind leave_part, for the registers)
             auto wait_acc = [&]() { ok = __all_sync(0xffffffffu, mbar_wait(acc_full(b), (tl >> 1) & 1, kGWait)); tc_fence_after(); };
             // every TMEM read of this warp for the tile has completed: the buffer goes back to the MMA thread
             auto release_acc = [&]() {
@@ -335,7 +338,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                        rank * kGM + q * 32 + lane;
             };
             auto leave_part = [&]() -> bool {                     // true: the tile is left to another pair
-                if constexpr (BN != kGN) return false;            // narrow tiles are never cut
+                if constexpr (!CUT) return false;
                 const long long U = (long long)n_tiles * ksteps, u0 = (long long)nt * ksteps;
                 const int first_grp = (int)(((u0 + 1) * g.groups - 1) / U), n_parts = (int)(((u0 + ksteps) * g.groups - 1) / U) - first_grp + 1;
                 unsigned int* cnt = g.arrived + (size_t)((nt * m_tiles + mt) * 2 + rank) * kGEpiWarps + (warp - 2);
@@ -737,12 +740,12 @@ size_t gemm_split_part_bytes(int64_t n, int64_t N, int64_t K) {
 int gemm_tile_rows() { return 2 * kGM; }
 int64_t gemm_split_max_rows() { return (int64_t)(sm_count() / 2) * 2 * kGM; }
 
-template <int EPI, int BN, bool F32>
+template <int EPI, int BN, bool F32, bool CUT>
 static int launch_tiles(const CUtensorMap& ma, const CUtensorMap& mw, const GemmArgs& g, int pairs, cudaStream_t st) {
     const int smem = kGRingBytes + kGEpiWarps * kGEpiBytes + 1024 + 256;
     static std::atomic<uint64_t> configured{0};
-    if (!set_max_smem_once(gemm_kernel<EPI, BN, F32>, smem, configured)) return DASH_ERR_CUDA;
-    return launch_pdl(gemm_kernel<EPI, BN, F32>, 2 * pairs, kGThreads, (size_t)smem, st, ma, mw, g) == cudaSuccess ? DASH_OK : DASH_ERR_CUDA;
+    if (!set_max_smem_once(gemm_kernel<EPI, BN, F32, CUT>, smem, configured)) return DASH_ERR_CUDA;
+    return launch_pdl(gemm_kernel<EPI, BN, F32, CUT>, 2 * pairs, kGThreads, (size_t)smem, st, ma, mw, g) == cudaSuccess ? DASH_OK : DASH_ERR_CUDA;
 }
 
 // Tiles of 128 columns instead of 256 where every one of them still has a pair of SMs to itself.  What that saves is epilogue: an epilogue warp
@@ -768,13 +771,15 @@ static int launch_gemm(const CUtensorMap& ma, const CUtensorMap& mw, GemmArgs g,
     g.groups = gemm_groups(m_tiles, g.n_tiles, (g.K + kGK - 1) / kGK, pairs, g.part != nullptr);
     if (EPI != GEMM_SWIGLU && !g.groups && gemm_narrow(m_tiles, g.n_tiles, pairs)) {
         g.n_tiles = (g.N + kGNarrow - 1) / kGNarrow;
-        return launch_tiles<EPI, EPI == GEMM_SWIGLU ? kGN : kGNarrow, F32>(ma, mw, g, m_tiles * g.n_tiles, st);
+        return launch_tiles<EPI, EPI == GEMM_SWIGLU ? kGN : kGNarrow, F32, false>(ma, mw, g, m_tiles * g.n_tiles, st);
     }
+    if constexpr (!F32) {                                     // (fp32 results come with no scratch for parts)
+        if (g.groups) return launch_tiles<EPI, kGN, F32, true>(ma, mw, g, g.groups * m_tiles, st);
+    }
+    g.groups = 0;
     g.by_m = gemm_by_m(m_tiles, g.n_tiles);
     const int tiles = m_tiles * g.n_tiles;
-    if (g.groups) pairs = g.groups * m_tiles;
-    else if (pairs > tiles) pairs = tiles;
-    return launch_tiles<EPI, kGN, F32>(ma, mw, g, pairs, st);
+    return launch_tiles<EPI, kGN, F32, false>(ma, mw, g, pairs > tiles ? tiles : pairs, st);
 }
 
 bool gemm_shape_ok(GemmEpilogueKind kind, int64_t n, int64_t N, int64_t K, int64_t lda, int64_t ldw, const GemmEpilogue& e) {
