@@ -25,8 +25,8 @@
  *    the device) and rows at or beyond it are neither read nor written.
  *  - Row-major tensors; `ld*` are row strides in ELEMENTS, `*_ld_bytes` in
  *    bytes.  Data pointers and row strides must be multiples of 16 bytes.
- *  - Kernels that wait (tile look-back, TMA/MMA barriers) give up after a
- *    bounded number of polls and set DASH_ERR_TIMEOUT in a device status word
+ *  - Kernels that wait (tile look-back, parts of a projection's tile, TMA/MMA
+ *    barriers) give up after a bounded number of polls and set DASH_ERR_TIMEOUT in a device status word
  *    that dash_check_status returns.
  */
 #ifndef DASH_H_

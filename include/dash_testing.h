@@ -33,6 +33,15 @@ int dash_testing_compact_stalled(const uint8_t* mask, int64_t n, const int32_t* 
  * shares steps, tile after tile along N, for every row of tiles.  Pure host function. */
 int dash_testing_gemm_groups(int64_t n, int64_t N, int64_t K);
 
+/* C [n, N] = A [n, K] W [K, N], bf16, contiguous, in tiles cut along K as a block step cuts them (DASH_ERR_UNSUPPORTED where dash_testing_gemm_groups is 0).
+ * ws: the arrival counters -- 32-bit words, one per tile, CTA of the pair and epilogue warp, tile 0 first, 74 x 4 x 16 of them on 148 SMs --, then the
+ * partial tiles, 512 KB per share and row of tiles.  The counters are cleared on `stream` first, as a step does.
+ * stall = 1: the first counter then starts at 1, so that the pair that takes itself for the last one of rows 64 .. 95, columns 0 .. 127 waits for parts that
+ * do not add up: after `spin_limit` polls (1 .. 2^22) it gives up, sets DASH_ERR_TIMEOUT in the device status word, leaves these rows and columns
+ * of C unwritten and the counter as it is, and the kernel returns. */
+int dash_testing_gemm_cut(const void* A, const void* W, void* C, int64_t n, int64_t N, int64_t K, int stall, uint32_t spin_limit,
+                          void* ws, size_t ws_bytes, void* stream);
+
 /* Shared memory of a CTA of the decoding kernel for heads of D (-1: no such kernel).  Pure host function. */
 int dash_testing_decode_smem_bytes(int D);
 

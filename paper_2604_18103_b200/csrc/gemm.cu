@@ -145,6 +145,7 @@ struct GemmArgs {
     int groups;                  // > 0: tiles are cut along K (see Work)
     float* part;                 // partial tiles of the pairs: two of 256 x 256 fp32 each
     unsigned int* arrived;       // per tile, CTA of the pair and epilogue warp: parts that are in `part`
+    uint32_t spin_limit;         // polls for parts that others are writing before a pair gives up
     GemmEpilogue e;
 };
 
@@ -355,10 +356,12 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                         uint32_t spins = 0;
                         while (*reinterpret_cast<volatile unsigned int*>(cnt) != want && all) {
                             __nanosleep(32);
-                            all = ++spins <= kSpinLimit;
+                            all = ++spins <= g.spin_limit;
                         }
-                        *cnt = 0u;                                // for the next launch
-                        if (!all) atomicExch(g.status, DASH_ERR_TIMEOUT);
+                        // Zero for the next launch, but not where the wait ran out: a pair that is late would still add its part, and what is neither
+                        // zero nor told by the status would look like a count.  Every step clears its counters ahead of its projections.
+                        if (all) *cnt = 0u;
+                        else atomicExch(g.status, DASH_ERR_TIMEOUT);
                     }
                     __syncwarp();
                     __threadfence();
@@ -810,6 +813,7 @@ int gemm_bf16(GemmEpilogueKind kind, const void* A, int64_t lda, const void* W, 
     g.C = C; g.ldc = ldc; g.n_dev = n_dev; g.e = e;
     g.w_early = w_early ? 1 : 0;
     g.part = sc ? sc->part : nullptr; g.arrived = sc ? sc->arrived : nullptr; g.groups = 0; g.by_m = 0;
+    g.spin_limit = sc ? sc->spin_limit : kSpinLimit;
     g.status = status_word_ptr();
     if (!g.status) return DASH_ERR_CUDA;
     switch (kind) {
@@ -835,4 +839,18 @@ extern "C" int dash_testing_gemm_groups(int64_t n, int64_t N, int64_t K) {
     using namespace dash;
     if (n < 1 || N < 1 || K < 1) return 0;
     return gemm_groups((int)((n + 2 * kGM - 1) / (2 * kGM)), (int)((N + kGN - 1) / kGN), (int)((K + kGK - 1) / kGK), sm_count() / 2, true);
+}
+
+extern "C" int dash_testing_gemm_cut(const void* A, const void* W, void* C, int64_t n, int64_t N, int64_t K, int stall, uint32_t spin_limit, void* ws, size_t ws_bytes,
+                                     void* stream) {
+    using namespace dash;
+    if (!A || !W || !C || n < 1 || N < 1 || K < 1 || spin_limit < 1 || spin_limit > kSpinLimit) return DASH_ERR_INVALID_ARG;
+    const size_t count = gemm_split_count_bytes(), part = gemm_split_part_bytes(n, N, K);
+    if (!part) return DASH_ERR_UNSUPPORTED;
+    if (!ws || ((uintptr_t)ws % 256) || ws_bytes < count + part) return DASH_ERR_WORKSPACE;
+    cudaStream_t st = (cudaStream_t)stream;
+    DASH_CUDA_TRY(cudaMemsetAsync(ws, 0, count, st));
+    if (stall) DASH_CUDA_TRY(cudaMemsetAsync(ws, 1, 1, st));      // the first counter says 1: one pair too many will have said that it is done
+    const GemmSplit sc = {(float*)((char*)ws + count), (unsigned int*)ws, spin_limit};
+    return gemm_bf16(GEMM_PLAIN, A, K, W, N, C, N, n, N, K, GemmEpilogue(), nullptr, st, false, &sc);
 }

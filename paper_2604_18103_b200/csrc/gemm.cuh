@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "common.cuh"
 #include "dash.h"
 
 namespace dash {
@@ -34,8 +35,9 @@ struct GemmEpilogue {
 };
 
 // Scratch of one GEMM at a time on one stream: part 16-byte aligned, gemm_split_part_bytes() of the GEMM (0: it runs in whole tiles); arrived
-// gemm_split_count_bytes(), zero before the first GEMM that uses it (every GEMM leaves it zero again).
-struct GemmSplit { float* part; unsigned int* arrived; };
+// gemm_split_count_bytes(), zero before the first GEMM that uses it (every GEMM leaves it zero again, but for a tile whose parts it waited for in
+// vain: DASH_ERR_TIMEOUT); spin_limit: polls of that wait.
+struct GemmSplit { float* part = nullptr; unsigned int* arrived = nullptr; uint32_t spin_limit = kSpinLimit; };
 size_t gemm_split_part_bytes(int64_t n, int64_t N, int64_t K);
 size_t gemm_split_count_bytes();
 // The scratch depends on n only through the number of rows of tiles, ceil(n / gemm_tile_rows()), and is 0 above gemm_split_max_rows()

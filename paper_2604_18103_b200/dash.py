@@ -36,7 +36,7 @@ EXPORTS = [
     "dash_block_workspace", "dash_block_step", "dash_decode_attention", "dash_varlen_attention_indexed",
     "dash_keep_counts_device", "dash_fold_norm_weight", "dash_rope_table",
 ]
-TEST_HOOKS = ["dash_testing_compact_stalled", "dash_testing_gemm_groups", "dash_testing_decode_smem_bytes"]        # include/dash_testing.h
+TEST_HOOKS = ["dash_testing_compact_stalled", "dash_testing_gemm_groups", "dash_testing_gemm_cut", "dash_testing_decode_smem_bytes"]        # include/dash_testing.h
 COMPACT_STATIC_MAX_ROWS = 1 << 20
 
 
@@ -126,6 +126,7 @@ def lib() -> ctypes.CDLL:
         L.dash_testing_compact_stalled.argtypes = [c_void_p, c_int64, c_void_p, c_int, c_void_p, c_void_p, c_void_p, ctypes.c_uint32,
                                                    c_void_p, c_size_t, c_void_p]
         L.dash_testing_gemm_groups.argtypes = [c_int64, c_int64, c_int64]
+        L.dash_testing_gemm_cut.argtypes = [c_void_p] * 3 + [c_int64] * 3 + [c_int, ctypes.c_uint32, c_void_p, c_size_t, c_void_p]
         L.dash_testing_decode_smem_bytes.argtypes = [c_int]
         L.dash_workspace_bytes.restype = c_size_t
         L.dash_workspace_bytes.argtypes = [c_int, c_int64, c_int, c_int, c_int, c_int, c_int]
@@ -301,6 +302,18 @@ def dash_testing_compact_stalled(mask: torch.Tensor, cu_in: torch.Tensor, spin_l
     st = lib().dash_testing_compact_stalled(_p(mask), n, _p(cu_in), S, _p(idx), _p(cu_out), _p(n_out), int(spin_limit), _p(ws), ws.numel(), _stream())
     _check(st, "dash_testing_compact_stalled")
     return {"idx": idx, "cu_out": cu_out, "n_out": n_out}
+
+
+def dash_testing_gemm_cut(A: torch.Tensor, W: torch.Tensor, out: torch.Tensor, stall: bool = False, spin_limit: int = 1000) -> torch.Tensor:
+    """Test hook (include/dash_testing.h): out = A W in tiles cut along K; stall: a bounded device-side wait runs out, and the device status word
+    then holds DASH_ERR_TIMEOUT.  Returns the arrival counters."""
+    _dev(A, W, out)
+    n, K, N = A.shape[0], A.shape[1], W.shape[1]
+    counters = torch.cuda.get_device_properties(A.device).multi_processor_count // 2 * 4 * 16
+    ws = workspace((counters * 4 + 255) // 256 * 256 + lib().dash_testing_gemm_groups(n, N, K) * ((n + 255) // 256) * (512 << 10), A.device)
+    st = lib().dash_testing_gemm_cut(_p(A), _p(W), _p(out), n, N, K, int(stall), int(spin_limit), _p(ws), ws.numel(), _stream())
+    _check(st, "dash_testing_gemm_cut")
+    return ws[:counters * 4].view(torch.int32)
 
 
 def dash_scatter(src: torch.Tensor, dst_full: torch.Tensor, tok_index: Optional[torch.Tensor] = None,

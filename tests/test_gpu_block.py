@@ -362,3 +362,26 @@ def test_block_step_tail_with_given_decisions_at_the_edges_of_its_tiles(n, offse
         assert b.cu_next.tolist() == [0, a, a, k]
         ref = torch.rsqrt(rows[mask].double().square().mean(1) + sh.rms_eps)
         assert k == 0 or ((inv[:k].double() - ref).abs() / ref).max() < 1e-5
+
+
+def test_a_cut_tile_whose_parts_never_come_gives_up_and_the_next_projection_is_right():
+    """A projection of two column tiles in eight shares, four parts to a tile.  The hook lets the first counter begin at 1, so that of one warp's rows and columns
+    (64 .. 95, 0 .. 127) the third pair to be done takes itself for the last and waits for parts that do not add up.  It gives up after its polls and
+    reports DASH_ERR_TIMEOUT; nothing else is missing; the counter still says what came (five arrivals, three parts left: the fourth pair may have added its
+    part before or after), and the next projection, whose counters are cleared first, is whole again, to the bit."""
+    n, N, K = 200, 512, 8192
+    assert dash.lib().dash_testing_gemm_groups(n, N, K) == 8
+    g = torch.Generator(device=DEV).manual_seed(8)
+    A, W = (torch.randn(*size, generator=g, device=DEV).to(torch.bfloat16) for size in ((n, K), (K, N)))
+    C = [torch.full((n, N), 7.0, dtype=torch.bfloat16, device=DEV) for _ in range(3)]
+    assert (dash.dash_testing_gemm_cut(A, W, C[0]) == 0).all() and dash.dash_check_status() == dash.OK
+    counters = dash.dash_testing_gemm_cut(A, W, C[1], stall=True, spin_limit=1000)
+    assert dash.dash_check_status() == 5                       # the kernel returned
+    assert int(counters[0]) == (3 << 16) + 5 and (counters[1:] == 0).all()
+    assert (dash.dash_testing_gemm_cut(A, W, C[2]) == 0).all() and dash.dash_check_status() == dash.OK
+    # rounding to bf16 and 2^-24 of the products' absolute sum for the square root of 8192 / 16 additions in a row (the MMA adds 16 products at a time)
+    ref, size = A.double() @ W.double(), A.double().abs() @ W.double().abs()
+    assert ((C[0] - ref).abs() <= 2.0 ** -8 * ref.abs() + 4 * 2.0 ** -24 * (K / 16) ** 0.5 * size).all()
+    assert torch.equal(C[2], C[0])
+    C[0][64:96, :128] = 7.0
+    assert torch.equal(C[1], C[0])
