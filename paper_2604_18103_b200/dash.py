@@ -134,7 +134,8 @@ def lib() -> ctypes.CDLL:
         C = importlib.util.module_from_spec(importlib.util.spec_from_file_location("_pycall", PYCALL_PATH, loader=loader))
         loader.exec_module(C)
         C.setup(ctypes.cast(L.dash_decode_attention, c_void_p).value, torch.bfloat16, torch.float32)
-        _lib, _pycall = L, C
+        _pycall = C             # ahead of _lib: a thread that finds the library loaded decodes
+        _lib = L
     return _lib
 
 

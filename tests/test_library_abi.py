@@ -5,6 +5,7 @@ import ctypes
 import importlib.util
 import os
 import re
+import sys
 import types
 
 import pytest
@@ -177,3 +178,34 @@ def test_the_bindings_c_part_checks_and_raises_as_the_python_one(lib):
     assert call(q=_Tensor((1, 28, 96)), K=_Tensor((10, 4, 96)), V=_Tensor((10, 4, 96))) == 2
     assert call(q=_Tensor((1, 28, 128), dtype=torch.float32)) == 2
     assert call(K=_Tensor((10, 4, 128), ptr=4100)) == 1 and call(scale=-1.0) == 1 and call(scale=0.1) == 3
+
+
+def test_a_thread_that_finds_the_library_loaded_can_decode(lib):
+    """Between any two bytecodes of the first lib() another thread may run: as soon as that one would find the library loaded, a decoding call reaches its
+    checks."""
+    spec = importlib.util.spec_from_file_location("paper_2604_18103_b200.dash_again", dash.__file__)
+    again = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(again)
+    host = [torch.zeros(1, 28, 128).bfloat16(), torch.zeros(10, 4, 128).bfloat16()]
+    seen, busy = [], []
+
+    def other_thread(code, offset):
+        if again._lib is not None and not busy:
+            busy.append(True)
+            try:
+                again.dash_decode_attention(host[0], host[1], host[1], torch.zeros(2, dtype=torch.int32), out=host[0], ws=torch.zeros(256, dtype=torch.uint8))
+            except Exception as e:
+                seen.append(type(e))
+            busy.pop()
+
+    again._stream = lambda: 0
+    m = sys.monitoring
+    m.use_tool_id(m.DEBUGGER_ID, "every bytecode")
+    m.register_callback(m.DEBUGGER_ID, m.events.INSTRUCTION, other_thread)
+    m.set_local_events(m.DEBUGGER_ID, again.lib.__code__, m.events.INSTRUCTION)
+    try:
+        again.lib()
+    finally:
+        m.set_local_events(m.DEBUGGER_ID, again.lib.__code__, 0)
+        m.free_tool_id(m.DEBUGGER_ID)
+    assert seen and set(seen) == {ValueError}, seen
