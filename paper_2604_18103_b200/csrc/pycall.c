@@ -2,7 +2,7 @@
  * with this): what dash.py does with ctypes for the other entry points --
  * pointers, strides and sizes read from the tensors, one call of the C ABI without the interpreter's lock -- in C.  Per call: 2.9 us of attribute reads
  * in bytecode and 1.8 us of argument conversion in ctypes, 2.0 together here.  Tensors are asked through their Python methods (no torch header: nothing here depends
- * on a version of it, and subclasses and tracing tensors answer, or raise, as they do in Python). */
+ * on a version of it, and subclasses and tracing tensors answer, or raise, as they do in Python).  Not needed: where it is not built for the running interpreter dash.py takes ctypes here too. */
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 #include <math.h>

@@ -12,6 +12,7 @@ import ctypes
 import importlib.machinery
 import importlib.util
 import os
+import sysconfig
 from ctypes import (POINTER, Structure, c_char_p, c_double, c_float, c_int, c_int32, c_int64,
                     c_size_t, c_uint8, c_void_p)
 from typing import Optional, Sequence
@@ -27,7 +28,7 @@ OK = 0
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libdash.so")
-PYCALL_PATH = os.path.join(_HERE, "_pycall.so")
+PYCALL_PATH = os.path.join(_HERE, "_pycall" + sysconfig.get_config_var("EXT_SUFFIX"))      # of this interpreter
 
 EXPORTS = [
     "dash_status_string", "dash_check_status", "dash_keep_count", "dash_flops_per_layer", "dash_flops_speedup",
@@ -73,17 +74,16 @@ class BlockWsLayout(Structure):
 
 
 _lib = None
-_pycall = None          # the binding's C part (csrc/pycall.c), loaded with the library
+_pycall = None          # the binding's C part (csrc/pycall.c), loaded with the library; False: not built for this interpreter, decoding calls go through ctypes
 
 
 def lib() -> ctypes.CDLL:
     """Loads libdash.so (raises if it has not been built)."""
     global _lib, _pycall
     if _lib is None:
-        for path in (LIB_PATH, PYCALL_PATH):
-            if not os.path.exists(path):
-                raise RuntimeError(f"{path} is missing: run `python -m paper_2604_18103_b200.build` "
-                                   "(there is no fallback path)")
+        if not os.path.exists(LIB_PATH):
+            raise RuntimeError(f"{LIB_PATH} is missing: run `python -m paper_2604_18103_b200.build` "
+                               "(there is no fallback path)")
         L = ctypes.CDLL(LIB_PATH)
         L.dash_status_string.restype = c_char_p
         L.dash_status_string.argtypes = [c_int]
@@ -130,10 +130,12 @@ def lib() -> ctypes.CDLL:
         L.dash_testing_decode_smem_bytes.argtypes = [c_int]
         L.dash_workspace_bytes.restype = c_size_t
         L.dash_workspace_bytes.argtypes = [c_int, c_int64, c_int, c_int, c_int, c_int, c_int]
-        loader = importlib.machinery.ExtensionFileLoader("_pycall", PYCALL_PATH)
-        C = importlib.util.module_from_spec(importlib.util.spec_from_file_location("_pycall", PYCALL_PATH, loader=loader))
-        loader.exec_module(C)
-        C.setup(ctypes.cast(L.dash_decode_attention, c_void_p).value, torch.bfloat16, torch.float32)
+        C = False
+        if os.path.exists(PYCALL_PATH):
+            loader = importlib.machinery.ExtensionFileLoader("_pycall", PYCALL_PATH)
+            C = importlib.util.module_from_spec(importlib.util.spec_from_file_location("_pycall", PYCALL_PATH, loader=loader))
+            loader.exec_module(C)
+            C.setup(ctypes.cast(L.dash_decode_attention, c_void_p).value, torch.bfloat16, torch.float32)
         _pycall = C             # ahead of _lib: a thread that finds the library loaded decodes
         _lib = L
     return _lib
@@ -385,7 +387,7 @@ def dash_decode_attention(q: torch.Tensor, Kc: torch.Tensor, Vc: torch.Tensor, c
     if _pycall is None:
         lib()
     lse = None
-    if out is None or ws is None or want_lse:
+    if out is None or ws is None or want_lse or not _pycall:
         _dev(q, Kc, Vc, cu_seqlens)
         S, Hq, D = q.shape
         n, Hkv = Kc.shape[:2]
@@ -395,7 +397,12 @@ def dash_decode_attention(q: torch.Tensor, Kc: torch.Tensor, Vc: torch.Tensor, c
             lse = torch.empty(S, Hq, dtype=torch.float32, device=q.device)
         if ws is None:
             ws = workspace(dash_workspace_bytes(WS_DECODE, n, S, Hq, Hkv, D, dtype_code(q)), q.device)
-    st = _pycall.decode(q, Kc, Vc, cu_seqlens, scale, out, lse, ws, _stream())
+    if _pycall:
+        st = _pycall.decode(q, Kc, Vc, cu_seqlens, scale, out, lse, ws, _stream())
+    else:
+        st = lib().dash_decode_attention(_p(q), _p(Kc), _p(Vc), _p(out), _p(lse), q.stride(0), Kc.stride(0) if n else Hkv * D, Vc.stride(0) if n else Hkv * D,
+                                         out.stride(0), _p(cu_seqlens), S, n, Hq, Hkv, D, 1.0 / (D ** 0.5) if scale is None else float(scale),
+                                         dtype_code(q), _p(ws), ws.numel(), _stream())
     _check(st, "dash_decode_attention")
     return (out, lse) if want_lse else out
 

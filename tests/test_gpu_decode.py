@@ -217,3 +217,24 @@ def test_block_step_emits_the_kv_cache_rows_a_decode_step_reads():
     O = ws[lay.attn.O:lay.attn.O + T * sh.Hq * sh.D * 2].view(sh.dtype).view(T, sh.Hq, sh.D)[last]
     assert_close_rms(out.float().cpu().numpy(), O.float().cpu().numpy(), "decode over the emitted cache vs prefill row")
     assert_close_rms(out.float().cpu().numpy(), ref["O"][last.cpu().numpy()], "decode over the emitted cache vs oracle", atol=2.0 ** -8)
+
+
+def test_decode_through_ctypes_is_the_same_call(monkeypatch):
+    """Where the binding's C part is not built: with and without the caller's buffers, strided caches, an empty one, the caller's scale."""
+    cu = wl.cu_from_lengths([129, 0, 700]).to(DEV)
+    g = torch.Generator(device=DEV).manual_seed(5)
+    q = torch.randn(3, 14, 128, generator=g, device=DEV).to(torch.bfloat16)
+    K, V = torch.randn(2, 829, 4, 128, generator=g, device=DEV).to(torch.bfloat16)[:, :, :2]
+    ws = dash.workspace(dash.dash_workspace_bytes(dash.WS_DECODE, 829, 3, 14, 2, 128), DEV)
+
+    def both(scale):
+        out = torch.zeros_like(q)
+        return [dash.dash_decode_attention(q, K, V, cu, scale=scale, out=out, ws=ws), *dash.dash_decode_attention(q, K, V, cu, scale=scale, want_lse=True)]
+
+    assert dash._pycall
+    want = both(None) + both(0.05)
+    monkeypatch.setattr(dash, "_pycall", False)
+    got = both(None) + both(0.05)
+    assert all(torch.equal(a, b) for a, b in zip(got, want)) and not torch.equal(want[0], want[3])
+    empty = dash.dash_decode_attention(q[:1], K[:0], V[:0], torch.zeros(2, dtype=torch.int32, device=DEV))
+    assert (empty == 0).all()

@@ -209,3 +209,36 @@ def test_a_thread_that_finds_the_library_loaded_can_decode(lib):
         m.set_local_events(m.DEBUGGER_ID, again.lib.__code__, 0)
         m.free_tool_id(m.DEBUGGER_ID)
     assert seen and set(seen) == {ValueError}, seen
+
+
+def test_without_its_c_part_the_library_builds_loads_and_decodes_through_ctypes(lib, monkeypatch, tmp_path, capfd):
+    """No C compiler, or a tree built under another Python (the C part's name carries the interpreter's tag): every entry point is there, a decoding
+    call raises and is refused as with it."""
+    monkeypatch.setattr(dash_build, "PYCALL", str(tmp_path / os.path.basename(dash_build.PYCALL)))
+    with open(dash_build.PYCALL, "w") as f:
+        f.write("of an older source")
+    with monkeypatch.context() as m:
+        m.setenv("PATH", str(tmp_path))
+        assert dash_build.build_pycall(force=True) is None and not os.path.exists(dash_build.PYCALL) and "ctypes" in capfd.readouterr().err
+    assert dash_build.build_pycall() == dash_build.PYCALL and os.path.exists(dash_build.PYCALL)
+    spec = importlib.util.spec_from_file_location("paper_2604_18103_b200.dash_without", dash.__file__)
+    without = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(without)
+    without.PYCALL_PATH, without._stream = str(tmp_path / "none.so"), lambda: 0
+    assert without.lib().dash_keep_count(8192, 0.4, 0, 0, 0) == 4915 and without._pycall is False
+    t, k = _Tensor((1, 28, 128)), _Tensor((10, 4, 128))
+
+    def refused(error, q=t, K=k, V=k, scale=None, out=t, ws=t):
+        for module in (dash, without):
+            with monkeypatch.context() as m:
+                m.setattr(module, "_stream", lambda: 0)
+                with pytest.raises(error) as e:
+                    module.dash_decode_attention(q, K, V, t, scale=scale, out=out, ws=ws)
+            yield getattr(e.value, "status", None)
+
+    assert list(refused(ValueError, V=_Tensor((10, 4, 128), is_cuda=False))) == [None] * 2
+    assert list(refused(ValueError, q=_Tensor((28, 128)))) == [None] * 2
+    assert list(refused(TypeError, q=_Tensor((1, 28, 128), dtype=torch.float16))) == [None] * 2
+    for want, kw in ((2, dict(q=_Tensor((1, 28, 96)), K=_Tensor((10, 4, 96)), V=_Tensor((10, 4, 96)))), (1, dict(K=_Tensor((10, 4, 128), ptr=4100))),
+                     (1, dict(scale=-1.0)), (3, dict(scale=0.1))):
+        assert list(refused(RuntimeError, **kw)) == [want] * 2
