@@ -398,7 +398,7 @@ def dash_decode_attention(q: torch.Tensor, Kc: torch.Tensor, Vc: torch.Tensor, c
         if ws is None:
             ws = workspace(dash_workspace_bytes(WS_DECODE, n, S, Hq, Hkv, D, dtype_code(q)), q.device)
     if _pycall:
-        st = _pycall.decode(q, Kc, Vc, cu_seqlens, scale, out, lse, ws, _stream())
+        st = _pycall.decode(q, Kc, Vc, cu_seqlens, None if scale is None else float(scale), out, lse, ws, _stream())
     else:
         st = lib().dash_decode_attention(_p(q), _p(Kc), _p(Vc), _p(out), _p(lse), q.stride(0), Kc.stride(0) if n else Hkv * D, Vc.stride(0) if n else Hkv * D,
                                          out.stride(0), _p(cu_seqlens), S, n, Hq, Hkv, D, 1.0 / (D ** 0.5) if scale is None else float(scale),

@@ -242,3 +242,15 @@ def test_without_its_c_part_the_library_builds_loads_and_decodes_through_ctypes(
     for want, kw in ((2, dict(q=_Tensor((1, 28, 96)), K=_Tensor((10, 4, 96)), V=_Tensor((10, 4, 96)))), (1, dict(K=_Tensor((10, 4, 128), ptr=4100))),
                      (1, dict(scale=-1.0)), (3, dict(scale=0.1))):
         assert list(refused(RuntimeError, **kw)) == [want] * 2
+
+
+def test_decode_takes_for_a_scale_what_float_takes(lib, monkeypatch):
+    """As the other attention entry points do: -1 in any form is read and refused by the library, text that is no number is a ValueError."""
+    monkeypatch.setattr(dash, "_stream", lambda: 0)
+    t, k = _Tensor((1, 28, 128)), _Tensor((10, 4, 128))
+    for scale in (-1, -1.0, "-1.0", torch.tensor(-1.0)):
+        with pytest.raises(dash.DashError) as e:
+            dash.dash_decode_attention(t, k, k, t, scale=scale, out=t, ws=t)
+        assert e.value.status == 1
+    with pytest.raises(ValueError):
+        dash.dash_decode_attention(t, k, k, t, scale="large", out=t, ws=t)
