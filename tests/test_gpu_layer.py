@@ -277,10 +277,11 @@ def test_layer_step_rows_beyond_the_packed_end_and_protected_tokens():
 
 
 @pytest.mark.parametrize("handover", [False, True], ids=["own_factors", "factors_handed_on"])
-@pytest.mark.parametrize("n", [1, 7, 8, 9, 255, 2368, 2369, 4801])
+@pytest.mark.parametrize("n", [1, 7, 8, 9, 255, 2368, 2369, 4801, 32768, 32769])
 def test_layer_step_tail_at_the_edges_of_its_tiles(n, handover):
-    """Row counts around the tail pass's tiles of 8 rows and around the count from which its general form (tiles of 32) takes over: what goes on
-    is exactly the kept rows of x_full in order, with their token and position indices, boundaries and row factors."""
+    """Row counts around the tiles of 8 and 16 rows of the pass that moves the rows by the mask (8 up to 2368 rows, 16 from there, 8 again from 4737) and around
+    the count from which one pass decides from the row sums and looks back (tiles of 32, above 32 768 rows): what goes on is exactly the kept rows of x_full in
+    order, with their token and position indices, boundaries and row factors.  The workspace holds anything when a step begins."""
     sh = wl.MINI
     lens = [n // 3, 0, n - n // 3]
     cu = wl.cu_from_lengths(lens)
@@ -294,6 +295,7 @@ def test_layer_step_tail_at_the_edges_of_its_tiles(n, handover):
     if handover:
         layer.set_handover(table, None, inv)
     x_full = torch.zeros(n, sh.d, dtype=sh.dtype, device=DEV)
+    bufs.ws.fill_(0x5A)
     run_step(layer, H, tok, pos, cu.to(DEV), max(lens), x_full, bufs)
     assert int(bufs.n_next.item()) == n and bufs.mask.all() and torch.equal(bufs.H_next, x_full[tok.long()])
     r = bufs.r.cpu().numpy()
@@ -341,6 +343,39 @@ def test_layer_step_other_rules_with_every_row_written(mode, n):
     assert np.array_equal(bufs.tok_next[:k].cpu().numpy(), tok.numpy()[idx]) and np.array_equal(bufs.pos_next[:k].cpu().numpy(), pos.numpy()[idx])
     a = int(mask[:lens[0]].sum())
     assert bufs.cu_next.tolist() == [0, a, a, k]
+
+
+@pytest.mark.parametrize("mode", [dash.SEL_KEEP_COUNT, dash.SEL_KEEP_COUNT_HALT_HIGH, dash.SEL_THRESHOLD_HALT_HIGH])
+@pytest.mark.parametrize("n", [32768, 32769])
+def test_layer_step_other_rules_where_the_tail_begins_to_look_back(mode, n):
+    """The rules beside the threshold on both sides of the count up to which rows are moved by the mask alone (above it: tiles of 32 with look-back, decisions
+    given, the rows already in x_full).  Decisions follow the step's own scores; rows and indices are exact; H~ is what a threshold step writes."""
+    sh = wl.MINI
+    lens = [n // 4, 0, n - n // 4]
+    cu = wl.cu_from_lengths(lens)
+    H, W, pos = wl.hidden_states(n, sh.d, 71, sh.dtype).to(DEV), wl.layer_weights(sh, 71), wl.positions(cu).to(DEV)
+    Ks = [oc.keep_count(x, 0.5, 16, 8, mode=1) for x in lens]
+    tok = torch.randperm(n, generator=torch.Generator().manual_seed(n)).to(torch.int32).to(DEV)
+    out = []
+    for m in (dash.SEL_THRESHOLD, mode):
+        layer = dash.Layer(sh, W, DEV, sel_mode=m, keep_counts=torch.tensor(Ks, dtype=torch.int32, device=DEV), keep_first=16, keep_last=8, tau=0.3)
+        bufs = StepBuffers(layer, n, 3, n, sh.dtype)
+        bufs.ws.fill_(0x5A)
+        bufs.H_next.fill_(7.0)
+        x_full = torch.zeros(n, sh.d, dtype=sh.dtype, device=DEV)
+        run_step(layer, H, tok, pos, cu.to(DEV), max(lens), x_full, bufs)
+        out.append((x_full, bufs.r))
+    assert torch.equal(out[0][0], out[1][0])
+    # sums of four partial sums of squares in another order: a few units in the last place of 32 bits
+    assert ((out[0][1] - out[1][1]).abs() / out[0][1]).max() < 2e-6
+    r, mask = bufs.r.cpu().numpy(), bufs.mask.cpu().numpy()
+    base = oc.THRESHOLD if mode == dash.SEL_THRESHOLD_HALT_HIGH else oc.KEEP_COUNT
+    assert np.array_equal(mask, oc.select(r, cu, base, tau=0.3, keep_counts=Ks, keep_first=16, keep_last=8, halt_high=mode != dash.SEL_KEEP_COUNT))
+    idx = torch.from_numpy(np.flatnonzero(mask)).to(DEV)
+    k, a = idx.numel(), int(mask[:lens[0]].sum())
+    assert int(bufs.n_next.item()) == k and bufs.cu_next.tolist() == [0, a, a, k]
+    assert torch.equal(bufs.H_next[:k], x_full[tok.long()][idx]) and (bufs.H_next[k:] == 7.0).all()
+    assert torch.equal(bufs.tok_next[:k], tok[idx]) and torch.equal(bufs.pos_next[:k], pos[idx])
 
 
 @pytest.mark.parametrize("offset", [0, 4, 2], ids=["aligned", "8_bytes", "4_bytes"])
