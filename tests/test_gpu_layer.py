@@ -380,10 +380,13 @@ def test_layer_step_other_rules_where_the_tail_begins_to_look_back(mode, n):
 
 @pytest.mark.parametrize("offset", [0, 4, 2], ids=["aligned", "8_bytes", "4_bytes"])
 @pytest.mark.parametrize("shape", [wl.LayerShape(d=512, Hq=4, Hkv=4, D=64, rope_base=1.0e4, dtype=torch.bfloat16, m=512),
-                                   wl.LayerShape(d=512, Hq=8, Hkv=2, D=128, rope_base=1.0e6, dtype=torch.bfloat16, m=512)], ids=["heads_of_64", "heads_of_128"])
+                                   wl.LayerShape(d=512, Hq=8, Hkv=2, D=128, rope_base=1.0e6, dtype=torch.bfloat16, m=512),
+                                   wl.LayerShape(d=512, Hq=4, Hkv=4, D=64, rope_base=1.0e4, dtype=torch.float32, m=512),
+                                   wl.LayerShape(d=512, Hq=8, Hkv=2, D=128, rope_base=1.0e6, dtype=torch.float32, m=512)],
+                         ids=["heads_of_64", "heads_of_128", "fp32_heads_of_64", "fp32_heads_of_128"])
 def test_kv_cache_rows_are_the_projections_for_every_head_size_and_alignment(shape, offset):
     """The K and V columns that a step leaves in its workspace and the cache rows are the same bits, whether the projection's epilogue writes
-    them (8-byte aligned buffers) or a copy does; rows past the batch stay untouched."""
+    them (bf16, 8-byte aligned buffers) or a copy does (fp32, whose epilogue writes the attention kernel's bf16 copies as well); rows past the batch stay untouched."""
     n, pad = 300, 20
     cu = wl.cu_from_lengths([n])
     layer = dash.Layer(shape, wl.layer_weights(shape, 81), DEV, tau=0.0)
@@ -403,11 +406,15 @@ def test_kv_cache_rows_are_the_projections_for_every_head_size_and_alignment(sha
     assert (K[n:] == 7.0).all() and (V[n:] == 7.0).all()
 
 
-@pytest.mark.parametrize("shape,n", [(wl.MINI, 1), (wl.MINI, 255), (wl.MINI, 257), (wl.MINI, 1536), (wl.MINI, 1537), (wl.TINY, 1), (wl.TINY, 257), (wl.TINY, 3072),
-                                     (wl.TINY, 3073), (wl.TINY, 3553)], ids=lambda x: x if isinstance(x, int) else ("fp32" if x.dtype == torch.float32 else "bf16"))
+FP32_128 = wl.LayerShape(d=256, Hq=4, Hkv=2, D=128, rope_base=1.0e6, dtype=torch.float32, m=512)
+
+
+@pytest.mark.parametrize("shape,n", [(FP32_128, 1), (FP32_128, 257), (FP32_128, 2304), (FP32_128, 2305), (wl.MINI, 1), (wl.MINI, 255), (wl.MINI, 257), (wl.MINI, 1536), (wl.MINI, 1537), (wl.TINY, 1), (wl.TINY, 257), (wl.TINY, 3072),
+                                     (wl.TINY, 3073), (wl.TINY, 3553)],
+                         ids=lambda x: x if isinstance(x, int) else ("fp32_128" if x is FP32_128 else "fp32" if x.dtype == torch.float32 else "bf16"))
 def test_layer_step_over_projection_tiles_of_both_widths(shape, n):
-    """Projections of few tiles take 128 columns per tile, others 256 (Q | K | V of MINI: up to 1536 rows, of the fp32 shape: up to 3072): one row, an
-    incomplete and a second row of tiles, both sides of the line (3553 rows: the general tail pass, too)."""
+    """Projections of few tiles take 128 columns per tile, others 256 (Q | K | V of MINI: up to 1536 rows, of the fp32 shape with heads of 64: up to 3072, of 128: up to
+    2304): one row, an incomplete and a second row of tiles, both sides of the line (3553 rows: the general tail pass, too)."""
     cu = wl.cu_from_lengths([n])
     H, W = wl.hidden_states(n, shape.d, 61, shape.dtype), wl.layer_weights(shape, 61)
     pos = wl.positions(cu)
