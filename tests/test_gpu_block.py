@@ -364,6 +364,80 @@ def test_block_step_tail_with_given_decisions_at_the_edges_of_its_tiles(n, offse
         assert k == 0 or ((inv[:k].double() - ref).abs() / ref).max() < 1e-5
 
 
+@pytest.mark.parametrize("n,offset", [(1, 0), (9, 3), (2368, 8), (2369, 1), (4740, 4), (32768, 0), (32769, 0)])
+def test_fp32_block_step_tail_with_given_decisions_at_the_edges_of_its_tiles(n, offset):
+    """The same of fp32 rows, whose sum H~ + F is one rounding in 32 bits: x_full and what goes on are that to the bit."""
+    sh = wl.TINY
+    live = n - n // 9
+    lens = [live // 3, 0, live - live // 3]
+    cu = wl.cu_from_lengths(lens)
+    H = wl.hidden_states(n, sh.d, 94, sh.dtype).to(DEV)
+    pos = torch.cat([wl.positions(cu), torch.zeros(n - live, dtype=torch.int32)]).to(DEV)
+    block = dash.Block(sh, _weights(sh, 94), DEV, tau=0.0, keep_first=2, keep_last=1)
+    b = BlockBuffers(block, n, 3)
+    b.ws.fill_(0x5A)
+    b.mask = torch.zeros(n + offset, dtype=torch.uint8, device=DEV)[offset:]
+    tok = torch.randperm(n, generator=torch.Generator().manual_seed(n)).to(torch.int32).to(DEV)
+    for tau in (0.0, None):
+        block.set_tau(float(b.r[:live].median()) if tau is None else tau)
+        x_full = torch.full((n, sh.d), 9.0, device=DEV)
+        b.H_next.fill_(7.0)
+        run_block(block, H, tok, pos, cu.to(DEV), max(lens), x_full, b)
+        view = lambda off: b.ws[off:off + n * sh.d * 4].view(torch.float32).view(n, sh.d)
+        rows = view(b.lay.attn.Ht)[:live] + view(b.lay.F)[:live]
+        assert torch.equal(x_full[tok[:live].long()], rows) and (x_full[tok[live:].long()] == 9.0).all()
+        mask = b.mask[:live].bool()
+        k, a = int(b.n_next.item()), int(mask[:lens[0]].sum())
+        assert k == int(mask.sum()) and (tau is None or k == live) and b.cu_next.tolist() == [0, a, a, k]
+        assert torch.equal(b.H_next[:k], rows[mask]) and (b.H_next[k:] == 7.0).all()
+        assert torch.equal(b.tok_next[:k], tok[:live][mask]) and torch.equal(b.pos_next[:k], pos[:live][mask])
+
+
+@pytest.mark.parametrize("n", [4100, 4700])
+def test_projections_with_their_tiles_in_groups_of_rows(n):
+    """Projections of more than 16 rows of tiles at the 7B shape, where the tiles come in groups of 16 rows of tiles, the last group incomplete: gate | up of 17 and
+    19 rows of tiles, Q | K | V of 19 (of 17 in groups of columns).  Every row and column against the same product in 64 bits of the operand that the
+    step was given or left in its workspace.  Bound: a projection is rounded to bf16 once, 2^-8 of the value; its fp32 sums are off by 2^-24 of the products'
+    absolute sum for each of 3584 / 16 additions in a row (the MMA adds 16 products at a time), of which a random walk takes the square root; the row
+    factors come from H~ before its rounding to bf16, 2^-9 an element; silu's slope is at most 1.1."""
+    sh = wl.QWEN
+    g = torch.Generator(device=DEV).manual_seed(n)
+    hd, kv = sh.Hq * sh.D, sh.Hkv * sh.D
+    W = {k: (torch.randn(*size, generator=g, device=DEV) * 0.02).to(sh.dtype) for k, size in
+         (("Wq", (sh.d, hd)), ("Wk", (sh.d, kv)), ("Wv", (sh.d, kv)), ("Wo", (hd, sh.d)), ("Wg", (sh.d, sh.m)), ("Wu", (sh.d, sh.m)), ("Wd", (sh.m, sh.d)))}
+    W["rms_w"] = W["rms2_w"] = torch.ones(sh.d, dtype=sh.dtype, device=DEV)
+    block = dash.Block(sh, W, DEV, tau=0.0)
+    b = BlockBuffers(block, n, 1)
+    H = torch.randn(n, sh.d, generator=g, device=DEV).to(sh.dtype)
+    tok = torch.arange(n, dtype=torch.int32, device=DEV)
+    run_block(block, H, tok, tok, wl.cu_from_lengths([n]).to(DEV), n, torch.zeros_like(H), b)
+    view = lambda off, cols: b.ws[off:off + n * cols * 2].view(sh.dtype).view(n, cols)
+
+    def product(X, Wm):
+        """X / rms(X) Wm in 64 bits and the bound of what 32-bit sums and the row factor lose"""
+        Xd, Wd = X.double(), Wm.double()
+        inv = torch.rsqrt(Xd.square().mean(1, keepdim=True) + sh.rms_eps)
+        y = inv * (Xd @ Wd)
+        return y, inv * (Xd.abs() @ Wd.abs()) * 4 * 2.0 ** -24 * (sh.d / 16) ** 0.5 + 2.0 ** -9 * y.abs()
+
+    QKV = view(b.lay.attn.QKV, hd + 2 * kv)
+    for at, name, heads in ((0, "Wq", sh.Hq), (hd, "Wk", sh.Hkv), (hd + kv, "Wv", sh.Hkv)):
+        y, e = (x.view(n, heads, 2, sh.D // 2) for x in product(H, W[name]))
+        if name != "Wv":
+            ang = tok.double()[:, None] * sh.rope_base ** (-2.0 * torch.arange(sh.D // 2, dtype=torch.float64, device=DEV) / sh.D)
+            c, s = ang.cos()[:, None], ang.sin()[:, None]
+            # (the angles' cosines and sines are held in 32 bits)
+            y, e = torch.stack([y[:, :, 0] * c - y[:, :, 1] * s, y[:, :, 1] * c + y[:, :, 0] * s], 2), \
+                e.sum(2, keepdim=True) + 2.0 ** -22 * y.abs().sum(2, keepdim=True)
+        got = QKV[:, at:at + heads * sh.D].double().view(n, heads, 2, sh.D // 2)
+        assert ((got - y).abs() <= 2.0 ** -8 * y.abs() + e).all(), name
+    Ht = view(b.lay.attn.Ht, sh.d)
+    (gate, eg), (up, eu) = product(Ht, W["Wg"]), product(Ht, W["Wu"])
+    silu = gate * torch.sigmoid(gate)
+    act = view(b.lay.ACT, sh.m).double()
+    assert ((act - silu * up).abs() <= (2.0 ** -8 + 2.0 ** -18) * (silu * up).abs() + 1.1 * eg * up.abs() + silu.abs() * eu + 1.1 * eg * eu).all()
+
+
 def test_a_cut_tile_whose_parts_never_come_gives_up_and_the_next_projection_is_right():
     """A projection of two column tiles in eight shares, four parts to a tile.  The hook lets the first counter begin at 1, so that of one warp's rows and columns
     (64 .. 95, 0 .. 127) the third pair to be done takes itself for the last and waits for parts that do not add up.  It gives up after its polls and
