@@ -43,6 +43,17 @@ inline bool set_max_smem_once(K kernel, int smem_bytes, std::atomic<uint64_t>& d
     return true;
 }
 
+// CTAs of `threads` threads and no dynamic shared memory that an SM holds of `kernel`; asked for once per device (two threads that race here store the same)
+template <typename K>
+inline int ctas_per_sm(K kernel, int threads, std::atomic<int> (&known)[64]) {
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 1;
+    if ((n = known[dev].load(std::memory_order_acquire)) > 0) return n;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, threads, 0) != cudaSuccess || n < 1) return 1;
+    known[dev].store(n, std::memory_order_release);
+    return n;
+}
+
 // Launch of a kernel that calls pdl_wait() before its global accesses (but for those that sm100_ptx.cuh allows ahead of it): it may
 // start while the kernel in front of it in the stream drains (programmatic dependent launch); behind anything else it is an ordinary launch.
 template <typename... KArgs, typename... Args>

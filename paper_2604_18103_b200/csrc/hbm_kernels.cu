@@ -1,5 +1,7 @@
 // HBM-bound kernels of the halted-prefill path: delta-attention score (+ fused
 // residual and threshold), halting rule, single-pass compaction, scatter.
+#include <type_traits>
+
 #include "common.cuh"
 #include "dash_testing.h"
 #include "sm100_ptx.cuh"
@@ -808,7 +810,7 @@ delta_tail_rows_kernel(const TailArgs a, int64_t n_upper) {
 // rows that all stay 15.2 / 9.8, 1500 17.8 / 11.1, 3000 47.8 / 22.9, 6683 53 / 38.5, 8192 61.6 / 51.1 (235 MB), 32 768 245 / 203, of 2728 51 / 23;
 // count rule, 12 345 rows 40.5 / 29.9.  (As many rows to every CTA, all resident at once: 701 11.7, 8192 55.7, 32 768 210.)  Up to kGivenMaxRows:
 // further up the mask in front is too long to be counted by every tile.
-constexpr int kGivenMaxRows = 32768, kGivenThreads = 256, kGivenPerSm = 2;
+constexpr int kGivenMaxRows = 32768, kGivenThreads = 256;
 template <bool BF16, int RPW>
 __global__ void __launch_bounds__(kGivenThreads)
 delta_given_kernel(const TailArgs a, int64_t n_upper) {
@@ -1345,15 +1347,21 @@ int launch_delta_tail(const void* U, const void* H, const uint8_t* mask_in, cons
     a.status = status_word_ptr();
     if (!a.status) return DASH_ERR_CUDA;
     if (mask_in && n <= kGivenMaxRows) {
-        // tiles of eight rows where they fill their waves better than tiles of sixteen (us from the end of the kernel in front, 8 / 16: 6683 rows 38.5 /
-        // 46.5; as well filled: 8192 rows 54.6 / 51.1, 12 345 rows, count rule 31.6 / 29.9, 3000 rows 23.1 / 22.9)
-        auto tiles = [&](int rows) { return n > 0 ? (n + rows - 1) / rows : 1; };
-        auto waves = [&](int64_t t) { return (t + kGivenPerSm * sm_count() - 1) / (kGivenPerSm * sm_count()); };
+        // tiles of eight rows where they fill their waves better than tiles of sixteen.  us, 8 / 16, bf16 rows of 7 KB from the end of the kernel in front: 6683
+        // rows 38.5 / 46.5; as well filled: 8192 rows 54.6 / 51.1, 12 345 rows, count rule 31.6 / 29.9, 3000 rows 23.1 / 22.9.  fp32 rows of 14 KB, the pass
+        // alone: 2500 rows 30.8 / 38.9, 5000 61.4 / 53.3, 8192 76.6 / 92.3, 32 768 276 / 285; of 4 KB: 2500 15.2 / 18.4, 5000 24.6 / 22.6, 8192 29.5 / 34.8.
+        // (Counted with the two CTAs per SM of bf16 the fp32 rows took the slower of the two at each of these.)
         constexpr int NW = kGivenThreads / 32;
-        const bool one = waves(tiles(NW)) < 2 * waves(tiles(2 * NW));
-        auto go = [&](auto kernel) { return launch_pdl(kernel, (int)tiles(one ? NW : 2 * NW), kGivenThreads, 0, st, a, n); };
-        DASH_CUDA_TRY(dt == DASH_BF16 ? (one ? go(delta_given_kernel<true, 1>) : go(delta_given_kernel<true, 2>))
-                                      : (one ? go(delta_given_kernel<false, 1>) : go(delta_given_kernel<false, 2>)));
+        auto tiles = [&](int rows) { return n > 0 ? (n + rows - 1) / rows : 1; };
+        auto waves = [&](int64_t t, int per_sm) { const int64_t at_once = (int64_t)per_sm * sm_count(); return (t + at_once - 1) / at_once; };
+        auto go = [&](auto bf16) {
+            constexpr bool B = decltype(bf16)::value;
+            static std::atomic<int> eight[64], sixteen[64];      // CTAs per SM
+            const bool one = waves(tiles(NW), ctas_per_sm(delta_given_kernel<B, 1>, kGivenThreads, eight)) <
+                             2 * waves(tiles(2 * NW), ctas_per_sm(delta_given_kernel<B, 2>, kGivenThreads, sixteen));
+            return launch_pdl(one ? delta_given_kernel<B, 1> : delta_given_kernel<B, 2>, (int)tiles(one ? NW : 2 * NW), kGivenThreads, 0, st, a, n);
+        };
+        DASH_CUDA_TRY(dt == DASH_BF16 ? go(std::true_type()) : go(std::false_type()));
         return DASH_OK;
     }
     const int small = (int)((n + kTailRows - 1) / kTailRows) > 0 ? (int)((n + kTailRows - 1) / kTailRows) : 1;

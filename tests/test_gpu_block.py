@@ -364,7 +364,7 @@ def test_block_step_tail_with_given_decisions_at_the_edges_of_its_tiles(n, offse
         assert k == 0 or ((inv[:k].double() - ref).abs() / ref).max() < 1e-5
 
 
-@pytest.mark.parametrize("n,offset", [(1, 0), (9, 3), (2368, 8), (2369, 1), (4740, 4), (32768, 0), (32769, 0)])
+@pytest.mark.parametrize("n,offset", [(1, 0), (9, 3), (2368, 8), (2369, 1), (4736, 8), (4737, 4), (7104, 0), (7105, 1), (32768, 0), (32769, 0)])
 def test_fp32_block_step_tail_with_given_decisions_at_the_edges_of_its_tiles(n, offset):
     """The same of fp32 rows, whose sum H~ + F is one rounding in 32 bits: x_full and what goes on are that to the bit."""
     sh = wl.TINY
