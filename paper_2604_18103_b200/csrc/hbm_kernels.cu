@@ -1321,15 +1321,18 @@ int launch_sums_to_score(const float4* sums, int n_sum_tiles, int64_t n, dash_no
                       rms_eps) == cudaSuccess ? DASH_OK : DASH_ERR_CUDA;
 }
 
-// Fused tail of the block step (see delta_tail_kernel).  Preconditions checked by the caller: every row scattered, 16-byte aligned
-// rows.  ws: the compaction workspace (ticket + one state word per tile), whose first tail_ws_clear_bytes(n) the caller has zeroed
-// on this stream (ahead of the kernels in front, so that this launch follows a kernel directly and may start while that one drains).
-// (tiles of kTailRows rows at the smallest)
 // Whether a threshold step of n rows whose H~ and row sums the output projection has written decides in a launch of its own (sums_to_score_kernel)
 // and then moves the rows (delta_given_kernel).  Layers of the 7B shape in a loop, 60 % stay, one launch for both / two, us: 700 rows 78.1 / 78.0, 1500
 // 126.2 / 125.0, 2300 171.2 / 170.7, 3000 218 / 212, 5000 364 / 359.5, 8192 827 / 819, 15 000 1494 / 1490, 24 000 3015 / 3017.
 bool tail_in_two(int64_t n) { return n <= kGivenMaxRows; }
+// Whether launch_delta_tail takes one of the kernels with look-back
+bool tail_looks_back(bool decided, int64_t n) { return !(decided && n <= kGivenMaxRows); }
+// (tiles of kTailRows rows at the smallest)
 size_t tail_ws_clear_bytes(int64_t n) { return 256 + (size_t)((n + kTailRows - 1) / kTailRows > 0 ? (n + kTailRows - 1) / kTailRows : 1) * 8; }
+// Tail of a step: by the mask where the decisions are given (mask_in; delta_given_kernel), else, or for more rows, the fused passes with look-back
+// (delta_tail_rows_kernel, delta_tail_kernel).  Preconditions checked by the caller: every row scattered, 16-byte aligned rows.  ws: the compaction workspace
+// (ticket + one state word per tile), whose first tail_ws_clear_bytes(n) the caller has zeroed on this stream where tail_looks_back() (ahead of the
+// kernels in front, so that this launch follows a kernel directly and may start while that one drains).
 int launch_delta_tail(const void* U, const void* H, const uint8_t* mask_in, const float4* sums, int n_sum_tiles, int64_t n, int d, dash_dtype dt, dash_norm_mode mode, float eps, float tau,
                       int keep_first, int keep_last, const int32_t* cu_in, int S, const int32_t* tok_in, const int32_t* pos_in,
                       void* x_full, void* H_next, float* r_out, uint8_t* mask_out, int32_t* tok_next, int32_t* pos_next,
@@ -1346,7 +1349,7 @@ int launch_delta_tail(const void* U, const void* H, const uint8_t* mask_in, cons
     a.inv_next = inv_next; a.inv_d = 1.0f / (float)d; a.rms_eps = rms_eps;
     a.status = status_word_ptr();
     if (!a.status) return DASH_ERR_CUDA;
-    if (mask_in && n <= kGivenMaxRows) {
+    if (!tail_looks_back(mask_in != nullptr, n)) {
         // tiles of eight rows where they fill their waves better than tiles of sixteen.  us, 8 / 16, bf16 rows of 7 KB from the end of the kernel in front: 6683
         // rows 38.5 / 46.5; as well filled: 8192 rows 54.6 / 51.1, 12 345 rows, count rule 31.6 / 29.9, 3000 rows 23.1 / 22.9.  fp32 rows of 14 KB, the pass
         // alone: 2500 rows 30.8 / 38.9, 5000 61.4 / 53.3, 8192 76.6 / 92.3, 32 768 276 / 285; of 4 KB: 2500 15.2 / 18.4, 5000 24.6 / 22.6, 8192 29.5 / 34.8.

@@ -132,6 +132,7 @@ int launch_delta_tail(const void* U, const void* H, const uint8_t* mask_in, cons
                       int32_t* cu_next, int32_t* n_next, void* ws, size_t ws_bytes, cudaStream_t st, float* inv_next, float rms_eps);
 size_t tail_ws_clear_bytes(int64_t n);
 bool tail_in_two(int64_t n);
+bool tail_looks_back(bool decided, int64_t n);
 int attention_planned(const void* Q, const void* K, const void* V, void* O, float* lse, int64_t ldq, int64_t ldk, int64_t ldv, int64_t ldo,
                       const int32_t* cu_seqlens, int S, int64_t n, int64_t max_seqlen, int Hq, int Hkv, int D, float scale, dash_dtype dt,
                       void* ws, size_t ws_bytes, cudaStream_t st, void* O16 = nullptr);
@@ -584,14 +585,18 @@ static int out_proj_U(const dash_layer_cfg* cfg, const int32_t* cu_in, int S, in
     return project(cfg->dt, W.O, hd, cfg->Wo, cfg->d, W.U, cfg->d, n, cfg->d, hd, cu_in + S, W.conv, W.split, st);
 }
 
+static bool residual_fits(const dash_layer_cfg* cfg, int64_t n) {
+    const int64_t hd = (int64_t)cfg->Hq * cfg->D;
+    return cfg->dt == DASH_BF16 && gemm_shape_ok(GEMM_RESID, n, cfg->d, hd, hd, cfg->d, GemmEpilogue());
+}
 // Output projection with the residual in its epilogue: dst[idx[row]] = H + O Wo (idx null: row), per-row sums of u^2, h^2 into W.sums.
 // Returns DASH_ERR_UNSUPPORTED when this library's GEMM does not take the shape (the caller then goes through U).
 static int out_proj_residual(const dash_layer_cfg* cfg, const void* H_in, const int32_t* idx, void* dst, const int32_t* cu_in, int S, int64_t n,
                              const StepWs& W, cudaStream_t st) {
+    if (!residual_fits(cfg, n)) return DASH_ERR_UNSUPPORTED;
     const int64_t hd = (int64_t)cfg->Hq * cfg->D;
     GemmEpilogue e;
     e.H = H_in; e.ldh = cfg->d; e.tok_index = idx; e.x_full = dst; e.ldx = cfg->d; e.sums = W.sums;
-    if (cfg->dt != DASH_BF16 || !gemm_shape_ok(GEMM_RESID, n, cfg->d, hd, hd, cfg->d, e)) return DASH_ERR_UNSUPPORTED;
     return gemm_bf16(GEMM_RESID, W.O, hd, cfg->Wo, cfg->d, nullptr, 0, n, cfg->d, hd, e, cu_in + S, st, false, &W.split, true);
 }
 
@@ -641,13 +646,14 @@ extern "C" int dash_layer_step(const dash_layer_cfg* cfg, const void* H_in, cons
             (cfg->rms_weight && !aligned16(cfg->rms_weight)))
             return DASH_ERR_INVALID_ARG;
         const bool every_row = cfg->scatter_which == 2, tail_pass = cfg->sel_mode == DASH_SEL_THRESHOLD && every_row;
-        if ((rc = attention_to_O(cfg, H_in, pos_in, cu_in, S, n, max_seqlen, every_row, W, st)) != DASH_OK) return rc;
+        const bool in_two = tail_pass && residual_fits(cfg, n) && tail_in_two(n), decided_first = in_two || !tail_pass;
+        if ((rc = attention_to_O(cfg, H_in, pos_in, cu_in, S, n, max_seqlen, every_row && tail_looks_back(decided_first, n), W, st)) != DASH_OK) return rc;
         if (tail_pass) {
-            // output projection with H~ = H + U written straight to x_full and the row sums of u^2, h^2 beside it; then the score, the
-            // halting rule and the compaction of the rows that stay (from x_full) in one pass
+            // output projection with H~ = H + U written straight to x_full and the row sums of u^2, h^2 beside it; then the score and the halting
+            // rule in a launch of their own and the compaction of the rows that stay (from x_full) by the mask, or, for more rows, all of it in one pass
             rc = out_proj_residual(cfg, H_in, tok_index_in, x_full, cu_in, S, n, W, st);
             const uint8_t* decided = nullptr;
-            if (rc == DASH_OK && tail_in_two(n)) {
+            if (rc == DASH_OK && in_two) {
                 dash_threshold ft = {cfg->tau, cfg->keep_first, cfg->keep_last, cu_in, S, mask_out};
                 if ((rc = launch_sums_to_score(W.sums, d / 128, n, cfg->norm_mode, cfg->norm_eps, r_out, &ft, cu_in + S, nullptr, d, cfg->rms_eps, st)) != DASH_OK) return rc;
                 decided = mask_out;
@@ -733,7 +739,7 @@ extern "C" int dash_block_step(const dash_block_cfg* cfg, const void* H_in, cons
         return DASH_ERR_INVALID_ARG;
     const int32_t* n_dev = cu_in + S;
     // U = Attn(LN(H)); score and selection from U; H~ = H + U
-    if ((rc = attention_to_O(a, H_in, pos_in, cu_in, S, n, max_seqlen, true, W, st)) != DASH_OK) return rc;
+    if ((rc = attention_to_O(a, H_in, pos_in, cu_in, S, n, max_seqlen, tail_looks_back(true, n), W, st)) != DASH_OK) return rc;
     bool have_inv_rms2 = false;
     rc = cfg->signal == DASH_SIGNAL_ATTN ? out_proj_residual(a, H_in, nullptr, W.Ht, cu_in, S, n, W, st) : DASH_ERR_UNSUPPORTED;
     if (rc == DASH_OK) {

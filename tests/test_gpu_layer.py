@@ -345,6 +345,28 @@ def test_layer_step_other_rules_with_every_row_written(mode, n):
     assert bufs.cu_next.tolist() == [0, a, a, k]
 
 
+@pytest.mark.parametrize("rule,n,looks_back", [(dash.SEL_THRESHOLD, 700, False), (dash.SEL_KEEP_COUNT, 700, False), (dash.SEL_THRESHOLD, 32769, True)])
+def test_layer_step_clears_look_back_words_only_where_its_tail_looks_back(rule, n, looks_back):
+    """The words behind `scratch` (no projection of these steps is cut along K, whose scratch would come first): left as they were where rows are moved by
+    the mask, ticket drawn where the tail pass looks back."""
+    sh = wl.MINI
+    for N, K in (((sh.Hq + 2 * sh.Hkv) * sh.D, sh.d), (sh.d, sh.Hq * sh.D)):
+        assert dash.lib().dash_testing_gemm_groups(n, N, K) == 0
+    cu = wl.cu_from_lengths([n])
+    layer = dash.Layer(sh, wl.layer_weights(sh, 71), DEV, sel_mode=rule, tau=0.3, keep_counts=torch.tensor([n // 2], dtype=torch.int32, device=DEV))
+    bufs = StepBuffers(layer, n, 1, n, sh.dtype)
+    bufs.ws.fill_(0x5A)
+    tok = torch.arange(n, dtype=torch.int32, device=DEV)
+    H = wl.hidden_states(n, sh.d, 71, sh.dtype).to(DEV)
+    run_step(layer, H, tok, tok, cu.to(DEV), n, torch.zeros_like(H), bufs)
+    words = bufs.ws[bufs.lay.scratch:bufs.lay.scratch + 256 + (n + 31) // 32 * 8]
+    if looks_back:
+        assert int(words[:4].view(torch.int32)) == (n + 31) // 32 and (words[256:].view(torch.int64) != 0x5A5A5A5A5A5A5A5A).all()
+    else:
+        assert (words == 0x5A).all()
+    assert int(bufs.n_next.item()) == int(bufs.mask.sum())
+
+
 @pytest.mark.parametrize("mode", [dash.SEL_KEEP_COUNT, dash.SEL_KEEP_COUNT_HALT_HIGH, dash.SEL_THRESHOLD_HALT_HIGH])
 @pytest.mark.parametrize("n", [32768, 32769])
 def test_layer_step_other_rules_where_the_tail_begins_to_look_back(mode, n):
