@@ -4,7 +4,9 @@
 // head form the (mostly empty) 128-row operand of the tcgen05 MMAs, so K and V tiles stream through
 // shared memory once per KV head; the keys of a sequence are split over persistent CTAs (flash-decoding),
 // whose partial (max, sum, O) results a merge kernel spread over all SMs combines.
-//   plan kernel   : items (sequence, KV head, key-block range), sized so that one item exists per CTA (batches of up to 128 sequences: the CTAs plan for themselves) or four per SM (handed out by ticket)
+//   plan          : items (sequence, KV head, key-block range).  Batches of up to 128 sequences: every CTA makes it for itself, an even share of the key blocks per CTA
+//                   or, where that makes more items than CTAs, the length that takes the fewest rounds (self_plan_build); more sequences: a plan kernel, about four
+//                   items per SM, handed out by ticket
 //   decode kernel : per item  S = Q K_j^T -> masked online softmax (one warp: the rows that exist) -> O += P V_j
 //   merge kernel  : O = sum_i 2^((m_i - m) c) O_i / sum_i 2^((m_i - m) c) l_i
 #include <math.h>
@@ -35,7 +37,7 @@ struct DecParams {
     const DecItem* plan;        // not where the CTAs plan for themselves (S <= kSelfPlanSeqs)
     const int* n_items;
     unsigned int* ticket;
-    int target;                 // items aimed at (self-planning)
+    int target;                 // twice the number of CTAs (see self_plan_build)
     int* status;
 };
 
@@ -493,56 +495,54 @@ __device__ __forceinline__ void decode_merge_units(const MergeParams& p, const S
     constexpr int B = 32, ML = B * K / 32;               // splits of one round: B per warp, their (m, l) in ML registers per lane
     const int n_units = p.S * p.Hq * CH;
     const int sub = warp % K;
-    const int n_groups = (int)gridDim.x * (NW / K), gid = (int)blockIdx.x * (NW / K) + warp / K;
     const size_t stride = (size_t)kDecRows * D;
-    for (int u = gid; u < n_units; u += n_groups) {
-        const int ch = u % CH, hd = (u / CH) % p.Hq, s = u / (CH * p.Hq);
-        const int kvh = hd / p.G, row = hd % p.G;
-        int first, cnt;
-        if (!p.seg) { cnt = sp.per[s]; first = sp.first[s] + kvh * cnt; }
-        else { const int2 sg = p.seg[s * p.Hkv + kvh]; first = sg.x; cnt = sg.y; }
-        const float* base = p.partial + ((size_t)first * kDecRows + row) * D + ch * 32 + lane;
-        const float2* mlb = p.ml + (size_t)hd * p.max_items + first;
-        float dv[B];
-        float2 ml[ML];
+    const int u = (int)blockIdx.x * (NW / K) + warp / K;      // (there are as many groups as units at least)
+    if (u >= n_units) return;
+    const int ch = u % CH, hd = (u / CH) % p.Hq, s = u / (CH * p.Hq);
+    const int kvh = hd / p.G, row = hd % p.G;
+    int first, cnt;
+    if (!p.seg) { cnt = sp.per[s]; first = sp.first[s] + kvh * cnt; }
+    else { const int2 sg = p.seg[s * p.Hkv + kvh]; first = sg.x; cnt = sg.y; }
+    const float* base = p.partial + ((size_t)first * kDecRows + row) * D + ch * 32 + lane;
+    const float2* mlb = p.ml + (size_t)hd * p.max_items + first;
+    float dv[B];
+    float2 ml[ML];
 #pragma unroll
-        for (int b = 0; b < B; ++b) { const int i = sub + b * K; dv[b] = (i < cnt) ? __ldcg(base + i * stride) : 0.f; }
+    for (int b = 0; b < B; ++b) { const int i = sub + b * K; dv[b] = (i < cnt) ? __ldcg(base + i * stride) : 0.f; }
 #pragma unroll
-        for (int j = 0; j < ML; ++j) { const int i = lane + 32 * j; ml[j] = (i < cnt) ? __ldcg(mlb + i) : make_float2(-INFINITY, 0.f); }
-        float mx = -INFINITY;
+    for (int j = 0; j < ML; ++j) { const int i = lane + 32 * j; ml[j] = (i < cnt) ? __ldcg(mlb + i) : make_float2(-INFINITY, 0.f); }
+    float mx = -INFINITY;
 #pragma unroll
-        for (int j = 0; j < ML; ++j) mx = fmaxf(mx, ml[j].x);
-        for (int i = lane + 32 * ML; i < cnt; i += 32) mx = fmaxf(mx, __ldcg(mlb + i).x);          // more than B * K splits: further rounds
+    for (int j = 0; j < ML; ++j) mx = fmaxf(mx, ml[j].x);
+    for (int i = lane + 32 * ML; i < cnt; i += 32) mx = fmaxf(mx, __ldcg(mlb + i).x);          // more than B * K splits: further rounds
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        float ls = 0.f;
+    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    float ls = 0.f;
 #pragma unroll
-        for (int j = 0; j < ML; ++j) {
-            ml[j].x = exp2f((ml[j].x - mx) * p.scale_log2);     // the split's weight (0 where there is no split)
-            ls = fmaf(ml[j].x, ml[j].y, ls);
-        }
-        for (int i = lane + 32 * ML; i < cnt; i += 32) { const float2 v = __ldcg(mlb + i); ls = fmaf(exp2f((v.x - mx) * p.scale_log2), v.y, ls); }
+    for (int j = 0; j < ML; ++j) {
+        ml[j].x = exp2f((ml[j].x - mx) * p.scale_log2);     // the split's weight (0 where there is no split)
+        ls = fmaf(ml[j].x, ml[j].y, ls);
+    }
+    for (int i = lane + 32 * ML; i < cnt; i += 32) { const float2 v = __ldcg(mlb + i); ls = fmaf(exp2f((v.x - mx) * p.scale_log2), v.y, ls); }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) ls += __shfl_xor_sync(0xffffffffu, ls, o);
-        float acc = 0.f;
+    for (int o = 16; o > 0; o >>= 1) ls += __shfl_xor_sync(0xffffffffu, ls, o);
+    float acc = 0.f;
 #pragma unroll
-        for (int b = 0; b < B; ++b) acc = fmaf(__shfl_sync(0xffffffffu, ml[(b * K) / 32].x, (sub + b * K) & 31), dv[b], acc);
-        for (int i = sub + B * K; i < cnt; i += K) acc = fmaf(exp2f((__ldcg(mlb + i).x - mx) * p.scale_log2), __ldcg(base + i * stride), acc);
-        if (K > 1) {
-            s_acc[warp][lane] = acc;
-            asm volatile("bar.sync %0, %1;" ::"r"(1 + warp / K), "n"(K * 32) : "memory");
-            if (sub == 0) {
-                acc = 0.f;
-#pragma unroll
-                for (int j = 0; j < K; ++j) acc += s_acc[warp + j][lane];
-            }
-            asm volatile("bar.sync %0, %1;" ::"r"(1 + warp / K), "n"(K * 32) : "memory");
-        }
+    for (int b = 0; b < B; ++b) acc = fmaf(__shfl_sync(0xffffffffu, ml[(b * K) / 32].x, (sub + b * K) & 31), dv[b], acc);
+    for (int i = sub + B * K; i < cnt; i += K) acc = fmaf(exp2f((__ldcg(mlb + i).x - mx) * p.scale_log2), __ldcg(base + i * stride), acc);
+    if (K > 1) {
+        s_acc[warp][lane] = acc;
+        asm volatile("bar.sync %0, %1;" ::"r"(1 + warp / K), "n"(K * 32) : "memory");
         if (sub == 0) {
-            const float v = cnt > 0 ? acc / ls : 0.f;
-            p.out[(int64_t)s * p.ldo + (int64_t)hd * D + ch * 32 + lane] = __float2bfloat16(v);
-            if (p.lse && ch == 0 && lane == 0) p.lse[(int64_t)s * p.Hq + hd] = cnt > 0 ? mx * p.scale + logf(ls) : -INFINITY;
+            acc = 0.f;
+#pragma unroll
+            for (int j = 0; j < K; ++j) acc += s_acc[warp + j][lane];
         }
+    }
+    if (sub == 0) {
+        const float v = cnt > 0 ? acc / ls : 0.f;
+        p.out[(int64_t)s * p.ldo + (int64_t)hd * D + ch * 32 + lane] = __float2bfloat16(v);
+        if (p.lse && ch == 0 && lane == 0) p.lse[(int64_t)s * p.Hq + hd] = cnt > 0 ? mx * p.scale + logf(ls) : -INFINITY;
     }
 }
 
@@ -691,7 +691,7 @@ extern "C" int dash_decode_attention(const void* q, const void* Kc, const void* 
     float* partial = (float*)((char*)seq_first + align_up((size_t)S * sizeof(int), 256));
     float2* ml = (float2*)((char*)partial + align_up((size_t)max_items * kDecRows * D * sizeof(float), 256));
     const bool self_plan = S <= kSelfPlanSeqs;
-    const int target = 4 * sm_count();        // items aimed at: four per SM (self-planning CTAs go down to one item each where that keeps them all busy)
+    const int target = 4 * sm_count();        // twice the CTAs: items that the plan kernel aims at, bound of the lengths that self_plan_build looks at
     if (!self_plan) {
         decode_plan_kernel<<<1, 256, 0, st>>>(cu_seqlens, S, Hkv, target, plan, seg, (int*)(w + 4), (unsigned int*)w, max_items, seq_first);
         DASH_CUDA_TRY(cudaGetLastError());
