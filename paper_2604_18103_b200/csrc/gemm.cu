@@ -332,12 +332,6 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
             // own part written and read back as well the last pair of the down projection was done 14 us after its last product at 701 rows, 13 at
             // 1500, now 12 and 10.)
             auto part_col = [&](int k) { return EPI == GEMM_SWIGLU ? (k >> 1) * 128 + half * 64 + (k & 1) * 32 : half * 128 + k * 32; };   // of piece k
-            auto part_of = [&](int grp, int col) {
-                const long long U = (long long)n_tiles * ksteps;
-                const int seg = (int)((grp * U / g.groups) / ksteps) == nt ? 0 : 1;      // the tile its share begins in, or the one it ends in
-                return reinterpret_cast<float4*>(g.part) + (size_t)(2 * (grp * m_tiles + mt) + seg) * (2 * kGM * kGN / 4) + (size_t)(col >> 2) * (2 * kGM) +
-                       rank * kGM + q * 32 + lane;
-            };
             auto leave_part = [&]() -> bool {                     // true: the tile is left to another pair
                 if constexpr (!CUT) return false;
                 const long long U = (long long)n_tiles * ksteps, u0 = (long long)nt * ksteps;
@@ -345,6 +339,15 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                 unsigned int* cnt = g.arrived + (size_t)((nt * m_tiles + mt) * 2 + rank) * kGEpiWarps + (warp - 2);
                 if (row0 >= g.n) return true;                     // no rows here: nothing to add up, nothing to store
                 const int own = pair / m_tiles - first_grp;
+                // Part p of the tile: of the two places of its pair the first (the share begins in this tile) or, p = 0 only, the second (it begins in a tile in
+                // front).  (With that found by 64-bit divisions for every part the four kernels spilled 44 to 120 bytes: RESID now 24, ROPE 8, the others none.
+                // us, a block of 523 rows with output and down projection cut 162.6, now 156.0, with Q | K | V and gate | up cut 149.7 / 143.0, three blocks of
+                // 701 rows of the 7B shape 868 / 863.  Without the last 24 and 8, rows' indices asked for behind this and 16 columns at a time: 158.5, 143.1, 865.)
+                const bool cont = first_grp * U / g.groups < u0;
+                auto part_of = [&](int p, int col) {
+                    return reinterpret_cast<float4*>(g.part) + (size_t)(2 * ((first_grp + p) * m_tiles + mt) + (p == 0 && cont ? 1 : 0)) * (2 * kGM * kGN / 4) + (size_t)(col >> 2) * (2 * kGM) +
+                           rank * kGM + q * 32 + lane;
+                };
                 constexpr unsigned int kLeft = 1u << 16;          // low half of the counter: pairs that are done, high half: parts that are in `part`
                 unsigned int in = 0;
                 if (lane == 0) in = atomicAdd(cnt, 1u) & (kLeft - 1u);
@@ -382,7 +385,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                                 tmem_ld32(tD + col, v);
                                 tmem_wait_ld();
                             } else {
-                                const float4 *s0 = part_of(first_grp + p, col), *s1 = two ? part_of(first_grp + p + 1, col) : s0;
+                                const float4 *s0 = part_of(p, col), *s1 = two ? part_of(p + 1, col) : s0;
 #pragma unroll
                                 for (int c = 0; c < (kTwo ? 16 : 8); ++c) {
                                     if (c < 8 || two) {
@@ -412,7 +415,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                     uint32_t o[32];
                     tmem_ld32(tD + col, o);
                     tmem_wait_ld();
-                    float4* dst = part_of(pair / m_tiles, col);
+                    float4* dst = part_of(own, col);
 #pragma unroll
                     for (int c = 0; c < 8; ++c) st_v4(dst + c * (2 * kGM), make_uint4(o[4 * c], o[4 * c + 1], o[4 * c + 2], o[4 * c + 3]));
                 }
