@@ -328,9 +328,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
             // A tile that was cut along K.  Every pair says that it is done; all but the last to say so leave their partial sums in `part` (a lane's
             // row in 16-byte pieces, so that a warp's piece is 512 contiguous bytes) and say that too.  The last one waits for what the others are
             // writing at that moment -- they wait for nothing -- adds the parts up in the order of K, its own from TMEM, and goes on as with a whole
-            // tile.  Warp by warp: the same warp of every pair holds the same rows and columns.  Bound by that one SM's loads from L2, a few at a time.  (With its
-            // own part written and read back as well the last pair of the down projection was done 14 us after its last product at 701 rows, 13 at
-            // 1500, now 12 and 10.)
+            // tile.  Warp by warp: the same warp of every pair holds the same rows and columns.  Bound by that one SM's loads from L2, a few at a time: from the last
+            // product of the down projection to its last result 9 us at 701 rows, 8 at 1500, 13 at 233, four parts to a tile.  (14, 14 and 18 with 64-bit divisions in
+            // the place of every part, 14 and 13 with its own part written and read back as well.)
             auto part_col = [&](int k) { return EPI == GEMM_SWIGLU ? (k >> 1) * 128 + half * 64 + (k & 1) * 32 : half * 128 + k * 32; };   // of piece k
             auto leave_part = [&]() -> bool {                     // true: the tile is left to another pair
                 if constexpr (!CUT) return false;
@@ -760,11 +760,13 @@ static int launch_tiles(const CUtensorMap& ma, const CUtensorMap& mw, const Gemm
 // fp32, 1024 rows of d = 256, Q | K | V 4.0 / 3.6, output projection 4.2 / 2.4.
 static bool gemm_narrow(int m_tiles, int n_tiles, int P) { return 2LL * m_tiles * n_tiles <= P; }
 
-// Groups of rows of tiles or of columns: the group's operand (16 tiles of 256 x 3584, 29 MB) stays in L2 while the other one streams past it, once
-// per group.  So of the two orders the one that reads less: (groups - 1) times the other operand more than both once.  The gate | up projection of
+// Groups of rows of tiles or of columns: the group's operand (16 tiles of 256 x 3584 are 29 MB, of 256 x 8192 67 MB) stays in L2 while the other one streams past
+// it, once per group; of a K too deep for that (16 tiles of 256 x 18 944 are 155 MB) the pairs of a wave share what they go through side by side.  So of
+// the two orders the one that reads less: (groups - 1) times the other operand more than both once.  The gate | up projection of
 // 8192 rows, 32 x 148 tiles, reads 1.01 GB from HBM in groups of columns, 0.83 in groups of rows (its operands are 0.33 GB); the
 // step runs at the power cap, where bytes are time: three blocks of 701, 6683, 8192 rows in a loop, columns / rows, us 883 / 877, 5772 / 5737,
-// 7817 / 7768.  Groups of 8, 11 and 32: 8192 rows 7812, 7828, 7910.
+// 7817 / 7768.  Groups of 8, 11 and 32: 8192 rows 7812, 7828, 7910.  Blocks of d = 8192, m = 28 672, columns / this rule: 2500 rows 3720 / 3530, 4096
+// 5825 / 5750 (all four projections by rows, the down projection 28 672 deep), 5000 7370 / 7280 (gate | up), 8192 12 115 / 12 040 (Q | K | V, gate | up).
 static bool gemm_by_m(int m_tiles, int n_tiles) {
     auto more = [](int grouped, int swept) { return (int64_t)((grouped + kGGroup - 1) / kGGroup - 1) * swept; };
     return more(m_tiles, n_tiles) < more(n_tiles, m_tiles);

@@ -607,7 +607,8 @@ scatter_kernel(const char* __restrict__ src, int64_t n, int64_t row_bytes, int64
 
 // ---------------------------------------------------------------------------
 // Steps 1-3 of the block step in one pass (threshold rule, every row's H~ written to the full-length
-// buffer): per tile of 32 tokens the 16 warps form r, the keep decision and H~ = H + U, stream H~ to
+// buffer; U and H of more rows than delta_tail_rows_kernel takes, row sums or given decisions of more than
+// delta_given_kernel does): per tile of 32 tokens the 16 warps form r, the keep decision and H~ = H + U, stream H~ to
 // x_full[tok[row]], then the tile finds its output base by decoupled look-back and copies its active
 // rows (just written, still in L2) into the next block's packed buffer.  Reads U and H once, writes
 // x_full and H_next once: no separate scatter and compaction passes over H~.
@@ -680,13 +681,15 @@ __device__ __forceinline__ int tail_decide(const TailArgs& a, int64_t row, float
 }
 
 // The same pass with a warp per row and tiles of eight rows, so that 700 rows are 88 CTAs and not 22: threshold rule on U and H (fp32 tensors, shapes whose
-// projections run plain; the others decide in sums_to_score_kernel, tail_in_two).  Bound by the chain ticket -> rows -> look-back -> copy; for inputs
-// whose tiles are all resident.  So the number of rows is asked for beside the ticket, every tile in front is asked for its count at once, a thread
+// projections run plain; the others decide in sums_to_score_kernel, tail_in_two).  Bound by the chain ticket -> rows -> look-back -> copy.
+// So the number of rows is asked for beside the ticket, every tile in front is asked for its count at once, a thread
 // to each, and a row's last vectors stay in registers for the copy (from the end of the kernel in front, us: fp32 layer of 1024 rows 6.6, 8.3 with these
 // one behind the other).  Loops of seven vectors per lane (two for a row of 3584 bf16), not unrolled: with the whole row in registers and
 // straight-line code the warps waited 14 us for instructions they run once.
 constexpr int kTailRows = 8;
-constexpr int kTailSmallTiles = 3;          // per SM.  fp32 layers (d = 256) in a graph, this kernel / the general one, us: 1200 rows 35.7 / 38.2, 2300 42.2 / 45.6, 3000 45.3 /
+// Tiles per SM up to which it is taken.  Two CTAs are resident (98 registers; bf16 128): tiles of a third round draw their ticket when one of the first
+// two has left, so that what they wait for has run or runs.
+constexpr int kTailSmallTiles = 3;          // fp32 layers (d = 256) in a graph, this kernel / the general one, us: 1200 rows 35.7 / 38.2, 2300 42.2 / 45.6, 3000 45.3 /
                                             // 48.2, 3500 52.6 / 52.9, 5000 63.6 / 63.8.  (Rows of 7 KB, while they came here too: 2368 170 / 180, 3500 267 / 271, 4000 334 / 323)
 template <bool BF16>
 __global__ void __launch_bounds__(32 * kTailRows)
@@ -808,8 +811,10 @@ delta_tail_rows_kernel(const TailArgs a, int64_t n_upper) {
 // stays, to H_next (U null: the rows are in x_full, those that stay are copied, and inv_next comes from sums).  A warp per row, RPW rows one behind the other.  Bound by HBM, for few
 // rows by the chain mask -> rows.  From the end of the kernel in front to its own, us, kernels with look-back / this one: blocks of the 7B shape of 701
 // rows that all stay 15.2 / 9.8, 1500 17.8 / 11.1, 3000 47.8 / 22.9, 6683 53 / 38.5, 8192 61.6 / 51.1 (235 MB), 32 768 245 / 203, of 2728 51 / 23;
-// count rule, 12 345 rows 40.5 / 29.9.  (As many rows to every CTA, all resident at once: 701 11.7, 8192 55.7, 32 768 210.)  Up to kGivenMaxRows:
-// further up the mask in front is too long to be counted by every tile.
+// count rule, 12 345 rows 40.5 / 29.9.  (As many rows to every CTA, all resident at once: 701 11.7, 8192 55.7, 32 768 210.)  Up to kGivenMaxRows, dash_compact's line:
+// further up every tile counts a longer mask, and neither form is ahead everywhere.  The pass alone, kernels with look-back / this one, bf16 rows of 7 KB,
+// 60 % stay: U and H, 40 000 rows 203 / 176, 65 536 313 / 332, 100 000 459 / 434, 131 072 600 / 657; rows moved out of x_full 84 / 82, 127 / 119, 185 / 211,
+// 238 / 233; rows of 1 KB moved, 131 072 125 / 127, 300 000 275 / 832.
 constexpr int kGivenMaxRows = 32768, kGivenThreads = 256;
 template <bool BF16, int RPW>
 __global__ void __launch_bounds__(kGivenThreads)
@@ -1322,8 +1327,8 @@ int launch_sums_to_score(const float4* sums, int n_sum_tiles, int64_t n, dash_no
 }
 
 // Whether a threshold step of n rows whose H~ and row sums the output projection has written decides in a launch of its own (sums_to_score_kernel)
-// and then moves the rows (delta_given_kernel).  Layers of the 7B shape in a loop, 60 % stay, one launch for both / two, us: 700 rows 78.1 / 78.0, 1500
-// 126.2 / 125.0, 2300 171.2 / 170.7, 3000 218 / 212, 5000 364 / 359.5, 8192 827 / 819, 15 000 1494 / 1490, 24 000 3015 / 3017.
+// and then moves the rows (delta_given_kernel), instead of delta_tail_kernel's one launch.  Layers of the 7B shape in a loop, both sides in turn, 60 % stay, one launch /
+// two, us: 700 rows 81.0 / 76.8, 1500 125.5 / 120.3, 3000 213.2 / 208.7, 5000 357.9 / 355.3, 8192 821 / 816, 15 000 1480 / 1478, 24 000 3010 / 2998.
 bool tail_in_two(int64_t n) { return n <= kGivenMaxRows; }
 // Whether launch_delta_tail takes one of the kernels with look-back
 bool tail_looks_back(bool decided, int64_t n) { return !(decided && n <= kGivenMaxRows); }
