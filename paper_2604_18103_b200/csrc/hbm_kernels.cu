@@ -687,7 +687,7 @@ __device__ __forceinline__ int tail_decide(const TailArgs& a, int64_t row, float
 // one behind the other).  Loops of seven vectors per lane (two for a row of 3584 bf16), not unrolled: with the whole row in registers and
 // straight-line code the warps waited 14 us for instructions they run once.
 constexpr int kTailRows = 8;
-// Tiles per SM up to which it is taken.  Two CTAs are resident (98 registers; bf16 128): tiles of a third round draw their ticket when one of the first
+// Tiles per SM up to which it is taken.  Two CTAs are resident (98 registers; bf16 128): tiles of a third wave draw their ticket when one of the first
 // two has left, so that what they wait for has run or runs.
 constexpr int kTailSmallTiles = 3;          // fp32 layers (d = 256) in a graph, this kernel / the general one, us: 1200 rows 35.7 / 38.2, 2300 42.2 / 45.6, 3000 45.3 /
                                             // 48.2, 3500 52.6 / 52.9, 5000 63.6 / 63.8.  (Rows of 7 KB, while they came here too: 2368 170 / 180, 3500 267 / 271, 4000 334 / 323)
